@@ -17,7 +17,6 @@
 namespace bn {
 
 static constexpr double LN10 = 2.302585092994045684017991454684364208;
-static constexpr int BUILD_RANGE = 64;     // consecutive ranks per warp work unit
 static constexpr int BUILD_THREADS = 256;
 
 // ---------------------------------------------------------------------------------
@@ -41,11 +40,14 @@ __device__ __forceinline__ void unrank_dev(int N, int64_t rank, int& j, uint64_t
 __device__ __forceinline__ void next_set(int N, int& j, uint64_t& mask)
 {
     if (j == 0) { j = 1; mask = 1; return; }
+    if (mask == (~0ull >> (64 - j)) << (N - j)) {       // {N - j .. N - 1}, the last of its size
+        ++j;
+        mask = (j >= 64) ? ~0ull : ((1ull << j) - 1);
+        return;
+    }
     uint64_t c = mask & (~mask + 1);
     uint64_t r = mask + c;
-    uint64_t nxt = (((r ^ mask) >> 2) >> (__ffsll((long long)mask) - 1)) | r;
-    if ((nxt >> N) != 0) { ++j; mask = (j >= 64) ? ~0ull : ((1ull << j) - 1); }
-    else mask = nxt;
+    mask = (((r ^ mask) >> 2) >> (__ffsll((long long)mask) - 1)) | r;
 }
 
 // ---------------------------------------------------------------------------------
@@ -118,207 +120,268 @@ __global__ void k_pad_keys(int64_t* __restrict__ keys, int n, int64_t S, int64_t
     keys[i * Sp + S + e] = KEY_NONE;
 }
 
-struct BuildArgs {
+// ---------------------------------------------------------------------------------
+// a2 + a3 by joint tables.  An entry's lgamma terms split into a sum over the cells of the
+// joint count table of U = pi + {i} and a sum over the configurations of pi:
+//     sum_c sum_x L_cell[N_cx] - sum_c L_cfg[N_c] = G(U) - H(pi).
+// G depends on U alone (its lgamma table is the one of alpha = 1 for K2 and of ess over
+// the number of cells for BDeu, whichever member of U is the child) and H on pi and, for
+// K2, the child's arity.  Both are exact 128-bit fixed-point integers, so their difference
+// is the exact sum and the entry's one rounding is unchanged.  So the rows are counted
+// once per set U of at most k + 1 nodes (k_joint) instead of once per (node, parent set):
+// C(60, 5) = 5.5 M tables instead of 29.4 M at n = 60, k = 4; k_assemble forms the entries.
+// Measured at n = 60, k = 4, m = 1000, ternary: 20.0 ms with one count table per entry,
+// 5.05 ms for k_joint and 0.89 ms for k_assemble.
+// ---------------------------------------------------------------------------------
+struct JointArgs {
     const uint32_t* packed;
-    int m, n, mw, k;
-    int64_t S, Sp;
-    int units_per_node;
+    int n, mw;
+    uint32_t pad;             // zero rows of the last word, all in cell 0
+    int k;                    // largest parent set
+    int64_t S0, S1;           // sets of at most k and of at most k + 1 of the n nodes
+    int range;                // consecutive sets per warp work unit
     int cells_cap;
-    int cells_max;           // largest histogram (q * r) of any entry
     const uint8_t* arity;
-    const double* ppf;        // n*n or null
-    double log10g;
     const fx128* lut;
     int lut_stride;           // m + 1
-    const int16_t* cell_lut;  // [(qmax+1) * 5], index q*5 + r
-    const int16_t* cfg_lut;
+    const int16_t* cell_lut;  // [cells] lgamma table of a joint table of that many cells
+    const int16_t* cfg_lut;   // [q * nv + v] of variant v's configuration counts
+    int nv;                   // variants of H: the distinct child arities (K2), 1 (BDeu)
+    fx128* G;                 // [S1]
+    fx128* H;                 // [nv][S0]
+};
+
+// warp sum, exact mod 2^128: five limbs (26, 26, 26, 26, 24 bits) of every lane's value
+// summed by one 32-bit reduction instruction each (32 lanes x 2^26 < 2^32)
+__device__ __forceinline__ fx128 warp_sum_fx(fx128 acc)
+{
+    const uint64_t lo = (uint64_t)acc, hi = (uint64_t)(acc >> 64);
+    constexpr uint64_t M26 = (1ull << 26) - 1;
+    const uint32_t s0 = __reduce_add_sync(0xffffffffu, (uint32_t)(lo & M26));
+    const uint32_t s1 = __reduce_add_sync(0xffffffffu, (uint32_t)((lo >> 26) & M26));
+    const uint32_t s2 = __reduce_add_sync(0xffffffffu, (uint32_t)(((lo >> 52) | (hi << 12)) & M26));
+    const uint32_t s3 = __reduce_add_sync(0xffffffffu, (uint32_t)((hi >> 14) & M26));
+    const uint32_t s4 = __reduce_add_sync(0xffffffffu, (uint32_t)(hi >> 40));
+    return (fx128)s0 + ((fx128)s1 << 26) + ((fx128)s2 << 52) + ((fx128)s3 << 78) + ((fx128)s4 << 104);
+}
+
+// One warp per unit of `range` consecutive sets U (colex order: the lowest node varies
+// fastest).  A set's cell index of a row is base + state(lowest node) * Qp, where base
+// comes from the nodes above the lowest and Qp is the product of their arities; BASE keeps
+// the rows' bases (16 bits a row, scaled by 4) in shared memory while those nodes stay the
+// same (about 12 sets on average at n = 60, k = 4), so a row costs one shift, mask,
+// multiply-add and one shared atomic.  Four rows of a packed word make one item; items run
+// over the lanes, so the base reads are free of bank conflicts.  Shared memory holds the
+// warps' histograms, their bases, then (SMEM_DATA) the packed data.  Bound by the shared
+// atomics (one per row and set, conflicts on a table's frequent cells) and the issue slots.
+template <int KT, bool SMEM_DATA, bool BASE>
+__global__ void __launch_bounds__(BUILD_THREADS) k_joint(JointArgs A)
+{
+    extern __shared__ __align__(16) uint32_t sm[];
+    const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int items = A.mw * 4;
+    uint32_t* hist = sm + warp * A.cells_cap;
+    uint2* base = (uint2*)(sm + nw * A.cells_cap) + (BASE ? warp * items : 0);
+    const uint32_t* D = A.packed;
+    for (int c = lane; c < A.cells_cap; c += 32) hist[c] = 0u;
+    if (SMEM_DATA) {
+        uint32_t* sd = sm + nw * A.cells_cap + (BASE ? nw * items * 2 : 0);
+        for (int t = threadIdx.x; t < A.n * A.mw; t += blockDim.x) sd[t] = A.packed[t];
+        D = sd;
+    }
+    __syncthreads();
+    uint8_t* hb = (uint8_t*)hist;
+    const int64_t units = (A.S1 + A.range - 1) / A.range;
+    for (int64_t u = (int64_t)blockIdx.x * nw + warp; u < units; u += (int64_t)gridDim.x * nw) {
+        const int64_t r0 = u * A.range;
+        const int64_t r1 = min(r0 + (int64_t)A.range, A.S1);
+        int j;
+        uint64_t mask;
+        unrank_dev(A.n, r0, j, mask);
+        uint64_t above = ~0ull;                 // the nodes above the lowest `base` is for
+        int poff[KT];
+        uint32_t cs[KT];
+        int Qp = 1;
+        fx128 my_acc = 0;
+        for (int64_t rho = r0; rho < r1; ++rho) {
+            const uint64_t up = mask & (mask - 1);
+            if (up != above) {                  // (warp-uniform)
+                above = up;
+                Qp = 1;
+                uint64_t mm = up;
+#pragma unroll
+                for (int t = 0; t < KT; ++t) {
+                    poff[t] = 0;
+                    cs[t] = 0u;
+                    if (mm) {
+                        const int p = __ffsll((long long)mm) - 1;
+                        mm &= mm - 1;
+                        poff[t] = p * A.mw;
+                        cs[t] = (uint32_t)(4 * Qp);
+                        Qp *= __ldg(&A.arity[p]);
+                    }
+                }
+                if (BASE) {
+                    __syncwarp();
+                    for (int c = lane; c < items; c += 32) {
+                        const int w = c >> 2, sft = 2 * (c & 3);
+                        uint2 b = make_uint2(0u, 0u);
+#pragma unroll
+                        for (int t = 0; t < KT; ++t) {
+                            const uint32_t x = D[poff[t] + w] >> sft;
+                            b.x += (x & 0x00030003u) * cs[t];
+                            b.y += ((x >> 8) & 0x00030003u) * cs[t];
+                        }
+                        base[c] = b;
+                    }
+                    __syncwarp();
+                }
+            }
+            const int low = mask ? __ffsll((long long)mask) - 1 : 0;
+            const uint32_t scale = mask ? (uint32_t)(4 * Qp) : 0u;
+            const int Q = mask ? Qp * (int)__ldg(&A.arity[low]) : 1;
+            const uint32_t* Dl = D + (size_t)low * A.mw;
+#pragma unroll 4
+            for (int c = lane; c < items; c += 32) {
+                const int w = c >> 2, sft = 2 * (c & 3);
+                uint2 b;
+                if (BASE) b = base[c];
+                else {
+                    b = make_uint2(0u, 0u);
+#pragma unroll
+                    for (int t = 0; t < KT; ++t) {
+                        const uint32_t y = D[poff[t] + w] >> sft;
+                        b.x += (y & 0x00030003u) * cs[t];
+                        b.y += ((y >> 8) & 0x00030003u) * cs[t];
+                    }
+                }
+                const uint32_t x = Dl[w] >> sft;
+                b.x += (x & 0x00030003u) * scale;
+                b.y += ((x >> 8) & 0x00030003u) * scale;
+                atomicAdd((uint32_t*)(hb + (b.x & 0xffffu)), 1u);
+                atomicAdd((uint32_t*)(hb + (b.x >> 16)), 1u);
+                atomicAdd((uint32_t*)(hb + (b.y & 0xffffu)), 1u);
+                atomicAdd((uint32_t*)(hb + (b.y >> 16)), 1u);
+            }
+            __syncwarp();
+            if (lane == 0 && A.pad) hist[0] -= A.pad;
+            __syncwarp();
+            // every cell read is set back to 0 for the next set
+            const fx128* Lx = A.lut + (size_t)A.cell_lut[Q] * A.lut_stride;
+            fx128 acc = 0;
+            if (j > A.k) {
+                for (int c = lane; c < Q; c += 32) {
+                    const uint32_t v = hist[c];
+                    hist[c] = 0u;
+                    acc += Lx[v];
+                }
+            } else {                            // a parent set too: its configuration sums
+                for (int v = 0; v < A.nv; ++v) {
+                    const fx128* Lc = A.lut + (size_t)A.cfg_lut[Q * A.nv + v] * A.lut_stride;
+                    fx128 h = 0;
+                    for (int c = lane; c < Q; c += 32) h += Lc[hist[c]];
+                    h = warp_sum_fx(h);
+                    if (lane == 0) A.H[(size_t)v * A.S0 + rho] = h;
+                }
+                for (int c = lane; c < Q; c += 32) {
+                    const uint32_t v = hist[c];
+                    hist[c] = 0u;
+                    acc += Lx[v];
+                }
+            }
+            acc = warp_sum_fx(acc);
+            // lane (rho - r0) % 32 keeps the set's sum; 32 of them go out at once
+            const int slot = (int)((rho - r0) & 31);
+            if (lane == slot) my_acc = acc;
+            if (slot == 31 || rho + 1 == r1) {
+                if (lane <= slot) A.G[rho - slot + lane] = my_acc;
+                __syncwarp();
+            }
+            __syncwarp();
+            next_set(A.n, j, mask);
+        }
+    }
+}
+
+struct AssembleArgs {
+    const uint64_t* pst;
+    int n, k;
+    int64_t S, Sp, S0;
+    const fx128* G;
+    const fx128* H;
+    const uint8_t* arity;
+    uint32_t vmap;            // byte r - 1: variant of a child of arity r
+    const double* ppf;        // n*n or null
+    double log10g;
     int64_t* keys;
 };
 
-// an entry from its exact lgamma sum: / ln 10, the size penalty, the prior of every
-// parent (candidate mask -> node ids, ascending), as one FP64 value in key form
-__device__ __forceinline__ void finish_entry(const BuildArgs& A, int i, fx128 acc, int j, uint64_t mask, int64_t rho)
+// x / ln 10, correctly rounded, without the division's dependent iterations: z + zl is
+// 1 / ln 10 to twice the working precision, so q0 is within one ulp of the quotient, the
+// remainder x - q0 ln 10 is exact in one fused multiply-add, and one more rounds correctly
+// (Markstein's theorem for a correctly rounded reciprocal z; Brisebarre, Muller and Raina
+// on division by a constant).
+__device__ __forceinline__ double div_ln10(double x)
 {
-    double ls = __dadd_rn(__ddiv_rn(fx_to_double(acc), LN10), __dmul_rn((double)j, A.log10g));
+    constexpr double z = 0x1.bcb7b1526e50dp-2, zl = 0x1.d756d22d31e1ap-56;
+    const double q0 = __fma_rn(x, z, __dmul_rn(x, zl));
+    const double r = __fma_rn(-q0, LN10, x);
+    return __fma_rn(r, z, q0);
+}
+
+// One thread per (node, rank): the node-space ranks of pi and pi + {i}, their sums, one
+// rounding, / ln 10, the size penalty, the prior of every parent (ascending node ids).
+// Consecutive ranks differ in their lowest parents, so both gathers are mostly coalesced.
+// Bound by the FP64 pipe (about ten operations an entry) and the 16-byte gathers.
+__global__ void __launch_bounds__(256) k_assemble(AssembleArgs A)
+{
+    __shared__ int64_t s_bin[65 * (MAXK + 2)];          // C(a, t), t <= k + 1
+    __shared__ int64_t s_base[MAXK + 3];                // first rank of every set size
+    const int T = A.k + 2;
+    for (int q = threadIdx.x; q < 65 * T; q += blockDim.x) s_bin[q] = (int64_t)c_binom.v[q / T][q % T];
+    if (threadIdx.x == 0) {
+        int64_t b = 0;
+        for (int t = 0; t <= A.k + 1; ++t) {
+            s_base[t] = b;
+            b += (int64_t)c_binom.v[A.n][t];
+        }
+    }
+    __syncthreads();
+    const int i = blockIdx.y;
+    const int64_t rho = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (rho >= A.Sp) return;
+    int64_t* out = A.keys + (size_t)i * A.Sp + rho;
+    if (rho >= A.S) {
+        *out = KEY_NONE;                                // padding
+        return;
+    }
+    const uint64_t mask = A.pst[rho];
+    const int j = __popcll(mask);
+    int64_t rp = s_base[j], ru = s_base[j + 1];
+    int t = 0, below = 0;
+    uint64_t mm = mask;
+    while (mm) {
+        const int c = __ffsll((long long)mm) - 1;
+        mm &= mm - 1;
+        const int gt = c >= i;
+        const int64_t* row = s_bin + (c + gt) * T + ++t;
+        rp += row[0];
+        ru += row[gt];
+        below += !gt;
+    }
+    ru += s_bin[i * T + below + 1];
+    const int v = (int)((A.vmap >> (8 * (A.arity[i] - 1))) & 0xffu);
+    const fx128 acc = A.G[ru] - A.H[(size_t)v * A.S0 + rp];
+    double ls = __dadd_rn(div_ln10(fx_to_double(acc)), __dmul_rn((double)j, A.log10g));
     if (A.ppf) {
-        uint64_t mm = mask;
+        mm = mask;
         while (mm) {
             const int c = __ffsll((long long)mm) - 1;
             mm &= mm - 1;
             ls = __dadd_rn(ls, A.ppf[(size_t)i * A.n + c + (c >= i ? 1 : 0)]);
         }
     }
-    A.keys[(size_t)i * A.Sp + rho] = double_to_key(ls);
-}
-
-// Counts of one packed word (16 rows).  cell = child state + sum_t parent state_t * cs[t];
-// with cells <= 256 four rows' cells are formed at once as the bytes of one 32-bit
-// integer (no byte can carry: each is a cell index < 256), otherwise two rows' as 16-bit
-// halves.  Parents past the set's size have cs = 0.
-template <int KT, bool WARP_AGG>
-__device__ __forceinline__ void count_word(uint32_t* hist, uint32_t cw, const uint32_t (&pw)[KT],
-                                           const uint32_t (&cs)[KT], bool bytes, int lane)
-{
-    if (bytes) {
-#pragma unroll
-        for (int sft = 0; sft < 8; sft += 2) {
-            uint32_t c4 = (cw >> sft) & 0x03030303u;
-#pragma unroll
-            for (int t = 0; t < KT; ++t) c4 += ((pw[t] >> sft) & 0x03030303u) * cs[t];
-            if (WARP_AGG) {
-                // tiny histograms: one add per distinct cell of the warp
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const uint32_t cell = (c4 >> (8 * r)) & 0xffu;
-                    const unsigned grp = __match_any_sync(__activemask(), cell);
-                    if ((__ffs(grp) - 1) == lane) atomicAdd(&hist[cell], (uint32_t)__popc(grp));
-                }
-            } else {
-                atomicAdd(&hist[c4 & 0xffu], 1u);
-                atomicAdd(&hist[(c4 >> 8) & 0xffu], 1u);
-                atomicAdd(&hist[(c4 >> 16) & 0xffu], 1u);
-                atomicAdd(&hist[c4 >> 24], 1u);
-            }
-        }
-    } else {
-#pragma unroll
-        for (int h = 0; h < 16; h += 8) {
-#pragma unroll
-            for (int sft = 0; sft < 8; sft += 2) {
-                uint32_t c2 = (cw >> (h + sft)) & 0x00030003u;
-#pragma unroll
-                for (int t = 0; t < KT; ++t) c2 += ((pw[t] >> (h + sft)) & 0x00030003u) * cs[t];
-                atomicAdd(&hist[c2 & 0xffffu], 1u);
-                atomicAdd(&hist[c2 >> 16], 1u);
-            }
-        }
-    }
-}
-
-// The lgamma terms of one count table: per configuration c, sum_x L_cell[N_cx] -
-// L_cfg[sum_x N_cx], exactly in 128-bit fixed point.  Every cell read is set back to 0,
-// so the warp's histogram is all zero again for the next entry.
-template <int RI>
-__device__ __forceinline__ fx128 score_cells(uint32_t* hist, int q, const fx128* __restrict__ Lx,
-                                             const fx128* __restrict__ Lc, int lane)
-{
-    fx128 acc = 0;
-    for (int c = lane; c < q; c += 32) {
-        uint32_t v[RI], Nc = 0;
-#pragma unroll
-        for (int x = 0; x < RI; ++x) {
-            v[x] = hist[c * RI + x];
-            Nc += v[x];
-        }
-#pragma unroll
-        for (int x = 0; x < RI; ++x) {
-            hist[c * RI + x] = 0u;
-            acc += Lx[v[x]];
-        }
-        acc -= Lc[Nc];
-    }
-    return acc;
-}
-
-// a2 + a3: one warp per work unit of BUILD_RANGE consecutive ranks of one node.  Per
-// parent set: a warp-private shared-memory histogram of (parent configuration, child
-// state) counts over all m rows, then the lgamma terms summed exactly in 128-bit fixed
-// point (the sum is independent of the cell order), one rounding to FP64, the
-// structure penalty, and the prior terms in ascending parent id.
-// Shared memory holds the warps' histograms, then (when it fits) the packed data.
-template <int KT, bool SMEM_DATA, bool WARP_AGG>
-__global__ void __launch_bounds__(BUILD_THREADS) k_build(BuildArgs A)
-{
-    extern __shared__ __align__(16) uint32_t sm[];
-    const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t* hist = sm + warp * A.cells_cap;
-    const uint32_t* D = A.packed;
-    for (int c = lane; c < A.cells_cap; c += 32) hist[c] = 0u;
-    if (SMEM_DATA) {
-        uint32_t* sd = sm + nw * A.cells_cap;
-        for (int t = threadIdx.x; t < A.n * A.mw; t += blockDim.x) sd[t] = A.packed[t];
-        D = sd;
-    }
-    __syncthreads();
-    const int N = A.n - 1;
-    const uint32_t pad = (uint32_t)(16 * A.mw - A.m);   // zero rows of the last word, all in cell 0
-    const int64_t units = (int64_t)A.n * A.units_per_node;
-    for (int64_t u = (int64_t)blockIdx.x * nw + warp; u < units; u += (int64_t)gridDim.x * nw) {
-        const int i = (int)(u / A.units_per_node);
-        const int64_t r0 = (u - (int64_t)i * A.units_per_node) * BUILD_RANGE;
-        const int64_t r1 = min(r0 + (int64_t)BUILD_RANGE, A.S);
-        const int ri = A.arity[i];
-        const uint32_t* Di = D + (size_t)i * A.mw;
-        int j;
-        uint64_t mask;
-        unrank_dev(N, r0, j, mask);
-        fx128 my_acc = 0;
-        int my_j = 0;
-        uint64_t my_mask = 0;
-        int64_t my_rho = 0;
-        for (int64_t rho = r0; rho < r1; ++rho) {
-            int poff[KT];
-            uint32_t cs[KT];
-            int q = 1;
-            uint64_t mm = mask;
-#pragma unroll
-            for (int t = 0; t < KT; ++t) {
-                poff[t] = 0;
-                cs[t] = 0u;
-                if (t < j) {
-                    const int c = __ffsll((long long)mm) - 1;
-                    mm &= mm - 1;
-                    const int p = c + (c >= i ? 1 : 0);
-                    poff[t] = p * A.mw;
-                    cs[t] = (uint32_t)(q * ri);
-                    q *= __ldg(&A.arity[p]);
-                }
-            }
-            const bool bytes = q * ri <= 256;
-            for (int w = lane; w < A.mw; w += 32) {
-                const uint32_t cw = Di[w];
-                uint32_t pw[KT];
-#pragma unroll
-                for (int t = 0; t < KT; ++t) pw[t] = D[poff[t] + w];
-                count_word<KT, WARP_AGG>(hist, cw, pw, cs, bytes, lane);
-            }
-            __syncwarp();
-            if (lane == 0 && pad) hist[0] -= pad;
-            const fx128* Lx = A.lut + (size_t)A.cell_lut[q * 5 + ri] * A.lut_stride;
-            const fx128* Lc = A.lut + (size_t)A.cfg_lut[q * 5 + ri] * A.lut_stride;
-            fx128 acc;
-            if (ri == 2) acc = score_cells<2>(hist, q, Lx, Lc, lane);
-            else if (ri == 3) acc = score_cells<3>(hist, q, Lx, Lc, lane);
-            else acc = score_cells<4>(hist, q, Lx, Lc, lane);
-            // warp sum, exact mod 2^128: five limbs (26, 26, 26, 26, 24 bits) of every lane's
-            // value summed by one 32-bit reduction instruction each (32 lanes x 2^26 < 2^32)
-            {
-                const uint64_t lo = (uint64_t)acc, hi = (uint64_t)(acc >> 64);
-                constexpr uint64_t M26 = (1ull << 26) - 1;
-                const uint32_t s0 = __reduce_add_sync(0xffffffffu, (uint32_t)(lo & M26));
-                const uint32_t s1 = __reduce_add_sync(0xffffffffu, (uint32_t)((lo >> 26) & M26));
-                const uint32_t s2 = __reduce_add_sync(0xffffffffu, (uint32_t)(((lo >> 52) | (hi << 12)) & M26));
-                const uint32_t s3 = __reduce_add_sync(0xffffffffu, (uint32_t)((hi >> 14) & M26));
-                const uint32_t s4 = __reduce_add_sync(0xffffffffu, (uint32_t)(hi >> 40));
-                acc = (fx128)s0 + ((fx128)s1 << 26) + ((fx128)s2 << 52) + ((fx128)s3 << 78) + ((fx128)s4 << 104);
-            }
-            // every lane holds the sum; lane (rho - r0) % 32 finishes this entry, 32 entries
-            // at a time (the FP64 tail runs on all lanes instead of on one)
-            const int slot = (int)((rho - r0) & 31);
-            if (lane == slot) {
-                my_acc = acc;
-                my_j = j;
-                my_mask = mask;
-                my_rho = rho;
-            }
-            if (slot == 31 || rho + 1 == r1) {
-                if (lane <= slot) finish_entry(A, i, my_acc, my_j, my_mask, my_rho);
-                __syncwarp();
-            }
-            __syncwarp();
-            next_set(N, j, mask);
-        }
-    }
+    *out = double_to_key(ls);
 }
 
 // score table upload / readout
@@ -374,13 +437,13 @@ static int table_alloc(int n, int k, bn_table** out)
     return BN_OK;
 }
 
-static int build_pst(bn_table* t, cudaStream_t s)
+static int build_pst(bn_table* t, cudaStream_t s, bool pad_keys)
 {
     int thr = 256;
     int64_t blocks = (t->Sp + thr - 1) / thr;
     k_pst<<<(unsigned)blocks, thr, 0, s>>>(t->n - 1, t->S, t->Sp, t->pst);
     BN_LAUNCH_CHECK("k_pst");
-    if (t->Sp > t->S) {
+    if (pad_keys && t->Sp > t->S) {
         int64_t tot = (int64_t)t->n * (t->Sp - t->S);
         k_pad_keys<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(t->keys, t->n, t->S, t->Sp);
         BN_LAUNCH_CHECK("k_pad_keys");
@@ -407,39 +470,31 @@ struct Temps {
         *out = (T*)q;
         return BN_OK;
     }
-    ~Temps()
+    void release()
     {
         for (void* q : p) cudaFreeAsync(q, s);
+        p.clear();
     }
+    ~Temps() { release(); }
 };
 
-// Counting: plain shared-memory atomics, except for tiny histograms (<= 8 cells), where
-// the lanes of a warp collide on a few cells and warp-aggregated adds (one atomic per
-// distinct cell, __match_any_sync) win.  Measured on GB300 at n = 60, k = 4, m = 1000
-// (243-cell histograms): 0.070 s plain against 0.224 s aggregated for the whole table.
-template <int KT>
-static int launch_build_kt(const BuildArgs& A, bool smem_data, size_t smem, int grid, cudaStream_t s)
+template <int KT, bool SMEM_DATA, bool BASE>
+static int launch_joint(const JointArgs& A, size_t smem, int grid, int threads, cudaStream_t s)
 {
-    const bool agg = A.cells_max <= 8;
-    if (smem_data) {
-        if (agg) {
-            cudaFuncSetAttribute(k_build<KT, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k_build<KT, true, true><<<grid, BUILD_THREADS, smem, s>>>(A);
-        } else {
-            cudaFuncSetAttribute(k_build<KT, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k_build<KT, true, false><<<grid, BUILD_THREADS, smem, s>>>(A);
-        }
-    } else {
-        if (agg) {
-            cudaFuncSetAttribute(k_build<KT, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k_build<KT, false, true><<<grid, BUILD_THREADS, smem, s>>>(A);
-        } else {
-            cudaFuncSetAttribute(k_build<KT, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k_build<KT, false, false><<<grid, BUILD_THREADS, smem, s>>>(A);
-        }
-    }
-    BN_LAUNCH_CHECK("k_build");
+    BN_CUDA(cudaFuncSetAttribute(k_joint<KT, SMEM_DATA, BASE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_joint<KT, SMEM_DATA, BASE><<<grid, threads, smem, s>>>(A);
+    BN_LAUNCH_CHECK("k_joint");
     return BN_OK;
+}
+
+template <int KT>
+static int launch_joint_kt(const JointArgs& A, bool smem_data, bool base, size_t smem, int grid, int threads,
+                           cudaStream_t s)
+{
+    if (smem_data) return base ? launch_joint<KT, true, true>(A, smem, grid, threads, s)
+                               : launch_joint<KT, true, false>(A, smem, grid, threads, s);
+    return base ? launch_joint<KT, false, true>(A, smem, grid, threads, s)
+                : launch_joint<KT, false, false>(A, smem, grid, threads, s);
 }
 
 static int copy_in(void* dst, const void* src, size_t bytes, int mem, cudaStream_t s)
@@ -471,6 +526,8 @@ struct BuildPlan {
     std::vector<double> Rh;
     int64_t S = 0;
     int cells_max = 1;
+    int nv = 1;                       // variants of the configuration sums
+    uint32_t vmap = 0;                // byte r - 1: variant of a child of arity r
     std::vector<int16_t> cell_lut, cfg_lut;
     std::vector<double> alpha;
 };
@@ -554,29 +611,43 @@ static int build_plan(const uint8_t* data, int m, int n, const uint8_t* arity, i
                 if ((int64_t)q * a <= MAX_CELLS / 2) nq.insert(q * a);
         qs.swap(nq);
     }
+    // cell_lut[cells of a joint table], cfg_lut[configurations * nv + variant]: a joint
+    // table of Q cells is q * r of some reachable q and child arity r, and its alpha is
+    // ess / Q whichever; K2's configuration alpha is the child's arity (a variant per
+    // arity present), BDeu's is ess / q
     const int qmax = *qs.rbegin();
     std::vector<int16_t>& cell_lut = P->cell_lut;
     std::vector<int16_t>& cfg_lut = P->cfg_lut;
     std::vector<double>& alpha = P->alpha;
-    cell_lut.assign((size_t)(qmax + 1) * 5, 0);
-    cfg_lut.assign((size_t)(qmax + 1) * 5, 0);
+    P->vmap = 0;
+    P->nv = 1;
     if (kind == 0) {
-        alpha = {1.0, 2.0, 3.0, 4.0};
-        for (int q : qs)
-            for (int r = 2; r <= 4; ++r) {
-                cell_lut[(size_t)q * 5 + r] = 0;
-                cfg_lut[(size_t)q * 5 + r] = (int16_t)(r - 1);
+        P->nv = 0;
+        for (int r = 2; r <= 4; ++r)
+            if (std::find(ar.begin(), ar.end(), (uint8_t)r) != ar.end()) {
+                P->vmap |= (uint32_t)P->nv << (8 * (r - 1));
+                ++P->nv;
+                alpha.push_back((double)r);
             }
+        alpha.push_back(1.0);
+        cell_lut.assign((size_t)4 * qmax + 1, (int16_t)(alpha.size() - 1));
+        cfg_lut.assign((size_t)(qmax + 1) * P->nv, 0);
+        for (size_t q = 0; q < cfg_lut.size(); ++q) cfg_lut[q] = (int16_t)(q % P->nv);
     } else {
+        cell_lut.assign((size_t)4 * qmax + 1, 0);
+        cfg_lut.assign((size_t)qmax + 1, 0);
+        auto table = [&](int v) {
+            const double a = ess / (double)v;
+            for (size_t x = 0; x < alpha.size(); ++x)
+                if (alpha[x] == a) return (int16_t)x;
+            alpha.push_back(a);
+            return (int16_t)(alpha.size() - 1);
+        };
         for (int q : qs) {
-            int cfg_id = (int)alpha.size();
-            alpha.push_back(ess / (double)q);
-            for (int r = 2; r <= 4; ++r) {
-                cfg_lut[(size_t)q * 5 + r] = (int16_t)cfg_id;
-                cell_lut[(size_t)q * 5 + r] = (int16_t)alpha.size();
-                alpha.push_back(ess / ((double)q * (double)r));
-            }
+            cfg_lut[q] = table(q);
+            for (int r = 2; r <= 4; ++r) cell_lut[(size_t)q * r] = table(q * r);
         }
+        cell_lut[1] = table(1);
     }
     if (alpha.size() > 32000) return set_error(BN_EUNSUPPORTED, "bn_build_scores: too many lgamma tables");
     return BN_OK;
@@ -626,46 +697,61 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_status, cu
         k_lut<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(d_alpha, (int)alpha.size(), m + 1, d_lut);
         BN_LAUNCH_CHECK("k_lut");
     }
-    if ((rc = build_pst(t, s))) return rc;
+    if ((rc = build_pst(t, s, false))) return rc;
 
-    BuildArgs A;
+    // joint sets over all n nodes; the LUT index of every table size
+    JointArgs A;
     A.packed = d_packed;
-    A.m = m;
     A.n = n;
     A.mw = mw;
+    A.pad = (uint32_t)(16 * mw - m);
     A.k = k;
-    A.S = P.S;
-    A.Sp = t->Sp;
-    A.units_per_node = (int)((P.S + BUILD_RANGE - 1) / BUILD_RANGE);
+    A.S0 = num_sets_host(n, k);
+    A.S1 = num_sets_host(n, k + 1);
     A.cells_cap = (int)round_up(P.cells_max, 32);
-    A.cells_max = (int)P.cells_max;
     A.arity = d_ar;
-    A.ppf = d_ppf;
-    A.log10g = P.log10g;
     A.lut = d_lut;
     A.lut_stride = m + 1;
     A.cell_lut = d_cell;
     A.cfg_lut = d_cfg;
-    A.keys = t->keys;
-    const int nwarps = BUILD_THREADS / 32;
-    size_t data_bytes = sizeof(uint32_t) * (size_t)n * mw;
-    size_t hist_bytes = sizeof(uint32_t) * (size_t)A.cells_cap * nwarps;
-    bool smem_data = data_bytes + hist_bytes <= 160 * 1024;
-    size_t smem = hist_bytes + (smem_data ? data_bytes : 0);   // histograms, then the data
-    int per_sm = std::max(1, std::min(8, (int)((220 * 1024) / std::max<size_t>(smem + 1024, 1))));
-    int64_t units = (int64_t)n * A.units_per_node;
-    int grid = (int)std::min<int64_t>((int64_t)sm_count() * per_sm, (units + nwarps - 1) / nwarps);
-    if (grid < 1) grid = 1;
-    int kt = k <= 2 ? 2 : k <= 4 ? 4 : k <= 8 ? 8 : 12;
-    if (ev0) BN_CUDA(cudaEventRecord(ev0, s));
-    switch (kt) {
-        case 2: rc = launch_build_kt<2>(A, smem_data, smem, grid, s); break;
-        case 4: rc = launch_build_kt<4>(A, smem_data, smem, grid, s); break;
-        case 8: rc = launch_build_kt<8>(A, smem_data, smem, grid, s); break;
-        default: rc = launch_build_kt<12>(A, smem_data, smem, grid, s); break;
+    A.nv = P.nv;
+    Temps sums(s);
+    if ((rc = sums.get(&A.G, (size_t)A.S1)) || (rc = sums.get(&A.H, (size_t)A.S0 * P.nv))) return rc;
+    // Shared memory: the histograms, the row bases and the packed data as long as two blocks
+    // fit an SM with them; fewer warps a block, then no bases, when a block alone does not
+    // fit (counts of thousands of cells, tens of thousands of rows).
+    int nwarps = BUILD_THREADS / 32;
+    const size_t data_bytes = sizeof(uint32_t) * (size_t)n * mw;
+    const size_t per_hist = sizeof(uint32_t) * (size_t)A.cells_cap, per_base = (size_t)mw * 32;
+    const size_t LIM = 220 * 1024;
+    bool base = true;
+    while (nwarps > 2 && nwarps * (per_hist + per_base) > LIM) nwarps /= 2;
+    if (nwarps * (per_hist + per_base) > LIM) {
+        base = false;
+        nwarps = BUILD_THREADS / 32;
+        while (nwarps > 1 && nwarps * per_hist > LIM) nwarps /= 2;
     }
+    size_t smem = nwarps * (per_hist + (base ? per_base : 0));
+    const bool smem_data = smem + data_bytes <= LIM / 2;
+    if (smem_data) smem += data_bytes;
+    const int per_sm = std::max(1, std::min(2048 / (32 * nwarps), (int)((224 * 1024) / std::max<size_t>(smem + 1024, 1))));
+    // 8 to 64 sets a unit: about eight units a resident warp where there are enough sets
+    const int64_t warps = (int64_t)sm_count() * per_sm * nwarps;
+    A.range = (int)std::max<int64_t>(4, std::min<int64_t>(64, A.S1 / (8 * warps)));
+    const int64_t units = (A.S1 + A.range - 1) / A.range;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count() * per_sm, (units + nwarps - 1) / nwarps));
+    if (ev0) BN_CUDA(cudaEventRecord(ev0, s));
+    const int thr = 32 * nwarps;
+    if (k <= 2) rc = launch_joint_kt<2>(A, smem_data, base, smem, grid, thr, s);
+    else if (k <= 4) rc = launch_joint_kt<4>(A, smem_data, base, smem, grid, thr, s);
+    else if (k <= 8) rc = launch_joint_kt<8>(A, smem_data, base, smem, grid, thr, s);
+    else rc = launch_joint_kt<12>(A, smem_data, base, smem, grid, thr, s);
     if (rc) return rc;
+    AssembleArgs B{t->pst, n, k, P.S, t->Sp, A.S0, A.G, A.H, d_ar, P.vmap, d_ppf, P.log10g, t->keys};
+    k_assemble<<<dim3((unsigned)((t->Sp + 255) / 256), (unsigned)n), 256, 0, s>>>(B);
+    BN_LAUNCH_CHECK("k_assemble");
     if (ev1) BN_CUDA(cudaEventRecord(ev1, s));
+    sums.release();
     return rank_entries(t, s);
 }
 
@@ -851,7 +937,7 @@ extern "C" int bn_table_from_scores(const double* scores, int n, int k, int mem,
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { bn_table_free(t); return cuda_fail(e, "k_keys_from_scores", __FILE__, __LINE__); }
     count_launches(1);
-    if ((rc = build_pst(t, s))) { bn_table_free(t); return rc; }
+    if ((rc = build_pst(t, s, true))) { bn_table_free(t); return rc; }
     if ((rc = rank_entries(t, s))) { bn_table_free(t); return rc; }
     uint32_t st = 0;
     if ((rc = read_status(d_status, &st, s))) { bn_table_free(t); return rc; }
