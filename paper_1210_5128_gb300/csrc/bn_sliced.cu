@@ -39,8 +39,7 @@ static constexpr int SL_STAGES = 4;
 static constexpr int SL_PER_WARP = SL_SUB / SL_CWARPS;  // 256 entries of a stage per consumer warp
 static constexpr int SL_ROWS = 66;                  // nodes 0..63, "no parent" (64), "never" (65)
 static constexpr int SL_ROW_BYTES = 256;            // two groups' 32 lanes per row
-static constexpr uint32_t SL_ROW_ONES = 64;
-static constexpr uint32_t SL_WORD_NEVER = 0x41414141u;  // four bytes of row 65 (all zero)
+static_assert(SSET_ONES == 64 && SSET_NEVER == 0x41414141u, "rows 64 (all ones) and 65 (all zero)");
 static constexpr int SL_MAX_K = 4;
 
 // The P copies of up to four groups sit in static shared memory, whose address the
@@ -74,59 +73,41 @@ struct SlicedArgs {
 };
 
 // ---------------------------------------------------------------------------------
-// sset[i][p]: byte j = the j-th smallest parent node id of the entry at sorted position
-// p of node i (node space: candidate c is node c + (c >= i)), SL_ROW_ONES for j >= the
-// set's size; positions at or past S (padding up to the row stride Ssp, a whole number of
-// stages) hold SL_WORD_NEVER, which no order is consistent with.
+// sset[i][p]: the parent nodes of the entry at sorted position p of node i (sset_word);
+// positions at or past S (padding up to the row stride Ssp, a whole number of stages) hold
+// SSET_NEVER.
 // ---------------------------------------------------------------------------------
 __global__ void k_sset(const uint32_t* __restrict__ srank, const uint64_t* __restrict__ pst, int n, int64_t S,
                        int64_t Sp, int64_t Ssp, uint32_t* __restrict__ sset)
 {
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (int64_t)n * Ssp) return;
-    const int i = (int)(g / Ssp);
-    const int64_t p = g - (int64_t)i * Ssp;
-    uint32_t w = SL_WORD_NEVER;
-    if (p < S) {
-        uint64_t m = pst[srank[(size_t)i * Sp + p]];
-        w = 0;
-        for (int j = 0; j < SL_MAX_K; ++j) {
-            uint32_t v = SL_ROW_ONES;
-            if (m) {
-                const int c = __ffsll((long long)m) - 1;
-                m &= m - 1;
-                v = (uint32_t)(c + (c >= i));
-            }
-            w |= v << (8 * j);
-        }
+    if (g >= (int64_t)n * S) return;
+    const int i = (int)(g / S);
+    const int64_t p = g - (int64_t)i * S;
+    sset[(size_t)i * Ssp + p] = sset_word(pst[srank[(size_t)i * Sp + p]], i);
+}
+
+int alloc_sset(bn_table* t)
+{
+    if (t->k > SL_MAX_K || t->n > 64 || t->sset) return BN_OK;   // the mask-test scans serve larger k
+    const int64_t Ssp = round_up(t->S, SL_SUB);
+    cudaError_t e = cudaMalloc(&t->sset, sizeof(uint32_t) * (size_t)t->n * (size_t)Ssp);
+    if (e != cudaSuccess) {
+        t->sset = nullptr;
+        cudaGetLastError();
+        return set_error(BN_ENOMEM, "sorted parent sets: %zu bytes: %s",
+                         sizeof(uint32_t) * (size_t)t->n * (size_t)Ssp, cudaGetErrorString(e));
     }
-    sset[g] = w;
+    t->sset_stride = Ssp;
+    t->bytes += sizeof(uint32_t) * (size_t)t->n * (size_t)Ssp;
+    return BN_OK;
 }
 
 int build_sset(bn_table* t, cudaStream_t s)
 {
-    if (t->k > SL_MAX_K || t->n > 64) return BN_OK;          // the mask-test scans serve these
-    const int64_t Ssp = round_up(t->S, SL_SUB);
-    if (!t->sset) {
-        cudaError_t e = cudaMalloc(&t->sset, sizeof(uint32_t) * (size_t)t->n * (size_t)Ssp);
-        if (e != cudaSuccess) {
-            t->sset = nullptr;
-            cudaGetLastError();
-            return set_error(BN_ENOMEM, "sorted parent sets: %zu bytes: %s",
-                             sizeof(uint32_t) * (size_t)t->n * (size_t)Ssp, cudaGetErrorString(e));
-        }
-        t->sset_stride = Ssp;
-        t->bytes += sizeof(uint32_t) * (size_t)t->n * (size_t)Ssp;
-    }
-    const int64_t tot = (int64_t)t->n * Ssp;
-    k_sset<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(t->srank, t->pst, t->n, t->S, t->Sp, Ssp, t->sset);
+    const int64_t tot = (int64_t)t->n * t->S;
+    k_sset<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(t->srank, t->pst, t->n, t->S, t->Sp, t->sset_stride, t->sset);
     BN_LAUNCH_CHECK("k_sset");
-    // the empty set's sorted position per node, for the sorted mode's launch shape: ranks
-    // 0 and 1 of every node are the first 2 n words of the entry-major copy spos_t
-    uint32_t h[2 * 64];
-    BN_CUDA(cudaMemcpyAsync(h, t->spos_t, sizeof(uint32_t) * 2 * (size_t)t->n, cudaMemcpyDeviceToHost, s));
-    BN_CUDA(cudaStreamSynchronize(s));
-    for (int i = 0; i < t->n; ++i) t->cut[i] = h[2 * i] + 1;
     return BN_OK;
 }
 
@@ -181,7 +162,7 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
     const uint32_t* src = A.sset + (size_t)node * A.Ssp;
     uint64_t pol_stream = 0;
     // the producer stages `it` into buffer st: always a whole stage (the row stride Ssp is
-    // a whole number of stages).  Words past S are SL_WORD_NEVER; in the sorted mode the
+    // a whole number of stages).  Words past S are SSET_NEVER; in the sorted mode the
     // last stage may run past the empty set's position, and those entries cannot win
     // (the empty set, in the same stage, is consistent with every item and ranks above
     // them), so no lane needs a bounds test.

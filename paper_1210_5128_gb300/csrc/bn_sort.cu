@@ -4,13 +4,19 @@
 // by score descending, ties by rank ascending.  spos is unique within a node and
 // "smaller spos" means "higher score, or equal score and lower rank", so the order-score
 // scan's (max score, lowest rank) reduction becomes a single unsigned min over spos.
-// srank[i][p] is the inverse (the rank at sorted position p).
+// srank[i][p] is the inverse (the rank at sorted position p), sset[i][p] its parent nodes.
 //
-// The ordering is a stable least-significant-digit radix sort (8-bit digits) of
-// (node, ~key) with the global index as value: eight passes over the 64-bit
-// order-inverted score keys, then one over the node, each pass = digit histogram per
-// tile, per-digit scan over tiles, stable scatter.  Input order is (node, rank), so
-// stability keeps equal scores in rank order.
+// The order is total (no two entries of a node share score and rank), so no pass has to be
+// stable.  A node's entries are split by sampled splitters -- (score, rank) pairs, so ties
+// split too -- into buckets of about 1,024, and a block sorts each bucket in shared memory
+// and writes all three arrays: the keys are read twice and the pairs written and read once,
+// against nine read-and-scatter passes of a byte-digit radix sort.  Measured at n = 60,
+// k = 4 (60 times 489,406 entries): radix sort and set words 5.43 ms, buckets 1.73 ms
+// (splitters 0.06, bucket of every entry 0.30, scatter 0.52, sorting and writing 0.84);
+// HBM would allow about 0.25 ms.  The count pass is bound by its binary searches in shared
+// memory, the scatter by its 12 scattered bytes an entry.  Tables of more than
+// BS_MAX_BUCKETS * 2,048 sets a node keep the radix sort: their buckets would outgrow a
+// block's shared memory.
 #include <algorithm>
 #include <vector>
 
@@ -160,6 +166,311 @@ __global__ void k_rs_finish(const uint32_t* __restrict__ vals, int64_t N, int64_
     spos[(node0 + i) * Sp + r] = (uint32_t)p;
 }
 
+// ---------------------------------------------------------------------------------
+// bucket sort
+// ---------------------------------------------------------------------------------
+static constexpr int BS_MAX_BUCKETS = 1024;
+static constexpr int BS_AVG = 1024;                  // entries a bucket on average (2,048 above 1 M sets)
+static constexpr int BS_CAP = 4096;                  // entries a block sorts in shared memory
+static constexpr int BS_THREADS = 512;
+static constexpr int BS_PER = BS_CAP / BS_THREADS;
+static constexpr int BS_NSUB = 512;                  // sub-buckets of a bucket
+static constexpr int BS_TILE = 8192;                 // entries of a partition tile
+static constexpr int BS_SAMPLES = 8192;              // at most, of a node
+
+// ascending <=> score descending
+__device__ __forceinline__ uint64_t bs_key(int64_t key) { return (uint64_t)key ^ 0x7FFFFFFFFFFFFFFFull; }
+__device__ __forceinline__ bool bs_less(uint64_t xa, uint32_t ra, uint64_t xb, uint32_t rb)
+{
+    return xa < xb || (xa == xb && ra < rb);
+}
+
+struct BsArgs {
+    const int64_t* keys;      // [n][Sp]
+    const uint64_t* pst;
+    int64_t S, Sp;
+    int node0;                // first node of this batch
+    int NB, tiles;            // buckets and tiles a node
+    int M;                    // samples a node (a power of two, at least 2 NB)
+    uint64_t* split_x;        // [nb][NB] splitters; bucket b holds [splitter b - 1, splitter b)
+    uint32_t* split_r;
+    uint32_t* counts;         // [nb][NB] entries, then [nb][NB] first entries of the buckets
+    uint32_t* tile_base;      // [nb][tiles][NB] the tile's first entry within each bucket
+    uint16_t* bid;            // [nb][S] bucket of each entry
+    uint64_t* bx;             // [nb][S] the entries by bucket
+    uint32_t* br;
+    uint32_t* srank;          // [n][Sp]
+    uint32_t* spos;           // [n][Sp]
+    uint32_t* sset;           // [n][Ssp] or null
+    int64_t Ssp;
+};
+
+// splitters of one node a block: a stratified pseudo-random sample, sorted in shared memory
+// (bitonic), every (M / NB)-th element.  The result of the sort does not depend on them.
+__global__ void __launch_bounds__(1024) k_bs_split(BsArgs A)
+{
+    extern __shared__ __align__(16) uint8_t bs_sm[];
+    uint64_t* x = (uint64_t*)bs_sm;
+    uint32_t* r = (uint32_t*)(x + A.M);
+    const int i = blockIdx.x;
+    const int64_t* K = A.keys + (size_t)(A.node0 + i) * A.Sp;
+    for (int j = threadIdx.x; j < A.M; j += blockDim.x) {
+        const int64_t lo = A.S * j / A.M, hi = A.S * (j + 1) / A.M;      // hi > lo: S >= M
+        uint32_t h = (uint32_t)j * 0x9E3779B9u;
+        h ^= h >> 15;
+        h *= 0x85EBCA6Bu;
+        h ^= h >> 13;
+        const int64_t e = lo + (int64_t)(h % (uint32_t)(hi - lo));
+        x[j] = bs_key(K[e]);
+        r[j] = (uint32_t)e;
+    }
+    for (int len = 2; len <= A.M; len <<= 1)
+        for (int d = len >> 1; d > 0; d >>= 1) {
+            __syncthreads();
+            for (int t = threadIdx.x; t < A.M / 2; t += blockDim.x) {
+                const int lo = 2 * t - (t & (d - 1)), hi = lo + d;       // bit d of lo is 0
+                const bool up = (lo & len) == 0;
+                const uint64_t xa = x[lo], xb = x[hi];
+                const uint32_t ra = r[lo], rb = r[hi];
+                if (bs_less(xb, rb, xa, ra) == up) {
+                    x[lo] = xb; x[hi] = xa;
+                    r[lo] = rb; r[hi] = ra;
+                }
+            }
+        }
+    __syncthreads();
+    for (int b = threadIdx.x; b + 1 < A.NB; b += blockDim.x) {
+        const int q = (int)((int64_t)A.M * (b + 1) / A.NB);
+        A.split_x[(size_t)i * A.NB + b] = x[q];
+        A.split_r[(size_t)i * A.NB + b] = r[q];
+    }
+}
+
+// bucket of every entry of a tile, and the tile's place within each bucket (the tiles take
+// their places in the order they arrive)
+__global__ void __launch_bounds__(512) k_bs_count(BsArgs A)
+{
+    __shared__ uint64_t sx[BS_MAX_BUCKETS];
+    __shared__ uint32_t sr[BS_MAX_BUCKETS];
+    __shared__ uint32_t h[BS_MAX_BUCKETS];
+    const int i = blockIdx.y, tile = blockIdx.x, ns = A.NB - 1;
+    for (int b = threadIdx.x; b < BS_MAX_BUCKETS; b += blockDim.x) {
+        sx[b] = b < ns ? A.split_x[(size_t)i * A.NB + b] : ~0ull;
+        sr[b] = b < ns ? A.split_r[(size_t)i * A.NB + b] : ~0u;
+        h[b] = 0;
+    }
+    __syncthreads();
+    int top = 1;
+    while (2 * top <= A.NB) top *= 2;
+    const int64_t* K = A.keys + (size_t)(A.node0 + i) * A.Sp;
+    uint16_t* B = A.bid + (size_t)i * A.S;
+    const int64_t e1 = min((int64_t)(tile + 1) * BS_TILE, A.S);
+#pragma unroll 4
+    for (int64_t e = (int64_t)tile * BS_TILE + threadIdx.x; e < e1; e += 512) {
+        const uint64_t x = bs_key(K[e]);
+        int b = 0;                                  // splitters below x ...
+        for (int d = top; d > 0; d >>= 1)
+            if (b + d <= ns && sx[b + d - 1] < x) b += d;
+        while (b < ns && sx[b] == x && sr[b] <= (uint32_t)e) ++b;       // ... and ties at or below e
+        B[e] = (uint16_t)b;
+        atomicAdd(&h[b], 1u);
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < A.NB; b += blockDim.x)
+        A.tile_base[((size_t)i * A.tiles + tile) * A.NB + b] = h[b] ? atomicAdd(&A.counts[(size_t)i * A.NB + b], h[b]) : 0u;
+}
+
+// first entry of every bucket (one block a node; the second half of `counts`)
+__global__ void __launch_bounds__(BS_MAX_BUCKETS) k_bs_scan(BsArgs A, int nb)
+{
+    __shared__ uint32_t w[32];
+    const int i = blockIdx.x, b = threadIdx.x, lane = b & 31;
+    const uint32_t c = b < A.NB ? A.counts[(size_t)i * A.NB + b] : 0u;
+    uint32_t s = c;
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, s, d);
+        if (lane >= d) s += y;
+    }
+    if (lane == 31) w[b >> 5] = s;
+    __syncthreads();
+    if (b < 32) {
+        uint32_t v = w[b], t = v;
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, t, d);
+            if (b >= d) t += y;
+        }
+        w[b] = t - v;
+    }
+    __syncthreads();
+    if (b < A.NB) A.counts[(size_t)(nb + i) * A.NB + b] = s - c + w[b >> 5];
+}
+
+__global__ void __launch_bounds__(512) k_bs_scatter(BsArgs A, int nb)
+{
+    __shared__ uint32_t cur[BS_MAX_BUCKETS];
+    const int i = blockIdx.y, tile = blockIdx.x;
+    for (int b = threadIdx.x; b < A.NB; b += blockDim.x)
+        cur[b] = A.counts[(size_t)(nb + i) * A.NB + b] + A.tile_base[((size_t)i * A.tiles + tile) * A.NB + b];
+    __syncthreads();
+    const int64_t* K = A.keys + (size_t)(A.node0 + i) * A.Sp;
+    const uint16_t* B = A.bid + (size_t)i * A.S;
+    const int64_t e1 = min((int64_t)(tile + 1) * BS_TILE, A.S);
+#pragma unroll 4
+    for (int64_t e = (int64_t)tile * BS_TILE + threadIdx.x; e < e1; e += 512) {
+        const uint64_t x = bs_key(K[e]);
+        const size_t at = (size_t)i * A.S + atomicAdd(&cur[B[e]], 1u);
+        A.bx[at] = x;
+        A.br[at] = (uint32_t)e;
+    }
+}
+
+// the outputs of one entry: sorted position p of node i holds rank r
+__device__ __forceinline__ void bs_write(const BsArgs& A, int i, uint32_t p, uint32_t r)
+{
+    A.srank[(size_t)i * A.Sp + p] = r;
+    A.spos[(size_t)i * A.Sp + r] = p;
+    if (A.sset) A.sset[(size_t)i * A.Ssp + p] = sset_word(A.pst[r], i);
+}
+
+// One block a bucket.  The entries are spread over BS_NSUB sub-buckets by their distance from
+// the bucket's smallest key (a shift: the keys of one bucket are close to evenly spread),
+// and an entry's place is its sub-bucket's start plus the entries of it that come before
+// (two to four compares on average; all of them where scores tie).  WHOLE: a node's entries
+// are one bucket, read straight from the table.  Buckets above BS_CAP (rare: four times the
+// average of sampled splitters) are placed by counting, tile by tile.
+template <bool WHOLE>
+__global__ void __launch_bounds__(BS_THREADS) k_bs_sort(BsArgs A, int nb)
+{
+    extern __shared__ __align__(16) uint8_t bs_sm[];
+    uint64_t* sx = (uint64_t*)bs_sm;                    // [CAP] by sub-bucket
+    uint32_t* sr = (uint32_t*)(sx + BS_CAP);            // [CAP]
+    uint32_t* so = sr + BS_CAP;                         // [CAP] ranks in final order
+    uint32_t* sub = so + BS_CAP;                        // [NSUB + 1]
+    __shared__ uint64_t s_min[BS_THREADS / 32], s_max[BS_THREADS / 32];
+    __shared__ uint32_t s_w[BS_THREADS / 32];
+    const int i = blockIdx.y, b = blockIdx.x, node = A.node0 + i;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t p0 = 0;
+    int cnt = (int)A.S;
+    const uint64_t* gx = nullptr;
+    const uint32_t* gr = nullptr;
+    if (!WHOLE) {
+        cnt = (int)A.counts[(size_t)i * A.NB + b];
+        p0 = A.counts[(size_t)(nb + i) * A.NB + b];
+        gx = A.bx + (size_t)i * A.S + p0;
+        gr = A.br + (size_t)i * A.S + p0;
+        if (cnt > BS_CAP) {
+            for (int e0 = 0; e0 < cnt; e0 += BS_THREADS) {                       // (block-uniform)
+                const int e = e0 + threadIdx.x;
+                const uint64_t x = e < cnt ? gx[e] : 0;
+                const uint32_t r = e < cnt ? gr[e] : 0;
+                uint32_t q = 0;
+                for (int t0 = 0; t0 < cnt; t0 += BS_CAP) {
+                    const int m = min(BS_CAP, cnt - t0);
+                    __syncthreads();
+                    for (int t = threadIdx.x; t < m; t += BS_THREADS) {
+                        sx[t] = gx[t0 + t];
+                        sr[t] = gr[t0 + t];
+                    }
+                    __syncthreads();
+                    for (int t = 0; t < m; ++t) q += bs_less(sx[t], sr[t], x, r);
+                }
+                if (e < cnt) bs_write(A, node, p0 + q, r);
+            }
+            return;
+        }
+    }
+    uint64_t x[BS_PER], lo = ~0ull, hi = 0ull;
+    uint32_t r[BS_PER];
+    uint32_t at[BS_PER];
+#pragma unroll
+    for (int u = 0; u < BS_PER; ++u) {
+        const int e = u * BS_THREADS + threadIdx.x;
+        x[u] = 0;
+        r[u] = 0;
+        if (e < cnt) {
+            x[u] = WHOLE ? bs_key(A.keys[(size_t)node * A.Sp + e]) : gx[e];
+            r[u] = WHOLE ? (uint32_t)e : gr[e];
+            lo = min(lo, x[u]);
+            hi = max(hi, x[u]);
+        }
+    }
+    sub[threadIdx.x] = 0;
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
+    }
+    if (lane == 0) {
+        s_min[warp] = lo;
+        s_max[warp] = hi;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < BS_THREADS / 32; ++w) {
+        lo = min(lo, s_min[w]);
+        hi = max(hi, s_max[w]);
+    }
+    const uint64_t range = hi >= lo ? hi - lo : 0ull;                            // (hi < lo: an empty bucket)
+    const int shift = max(0, 64 - __clzll((long long)range) - 9);                // range >> shift < NSUB
+#pragma unroll
+    for (int u = 0; u < BS_PER; ++u)
+        if (u * BS_THREADS + (int)threadIdx.x < cnt) at[u] = atomicAdd(&sub[(x[u] - lo) >> shift], 1u);
+    __syncthreads();
+    {
+        // exclusive scan of the 512 sub-bucket counts, one a thread
+        const uint32_t c = sub[threadIdx.x];
+        uint32_t s = c;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, s, d);
+            if (lane >= d) s += y;
+        }
+        if (lane == 31) s_w[warp] = s;
+        __syncthreads();
+        uint32_t add = 0;
+        for (int w = 0; w < warp; ++w) add += s_w[w];
+        sub[threadIdx.x] = s - c + add;
+        if (threadIdx.x == 0) sub[BS_NSUB] = (uint32_t)cnt;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < BS_PER; ++u)
+        if (u * BS_THREADS + (int)threadIdx.x < cnt) {
+            const uint32_t q = sub[(x[u] - lo) >> shift] + at[u];
+            sx[q] = x[u];
+            sr[q] = r[u];
+        }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < BS_PER; ++u)
+        if (u * BS_THREADS + (int)threadIdx.x < cnt) {
+            const int d = (int)((x[u] - lo) >> shift);
+            const uint32_t s0 = sub[d], s1 = sub[d + 1];
+            uint32_t q = s0;
+            for (uint32_t t = s0; t < s1; ++t) q += bs_less(sx[t], sr[t], x[u], r[u]);
+            so[q] = r[u];
+        }
+    __syncthreads();
+    for (int q = threadIdx.x; q < cnt; q += BS_THREADS) bs_write(A, node, p0 + (uint32_t)q, so[q]);
+}
+
+static constexpr size_t BS_SMEM = (size_t)BS_CAP * 16 + 4 * (BS_NSUB + 1);
+
+// sorted positions at or past S of the parent-node words (padding up to the row stride, a
+// whole number of the sliced scan's stages): never consistent with an order
+__global__ void k_sset_pad(uint32_t* __restrict__ sset, int64_t S, int64_t Ssp)
+{
+    const int64_t p = S + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < Ssp) sset[(size_t)blockIdx.y * Ssp + p] = SSET_NEVER;
+}
+
+// the empty set's sorted position of every node, plus 1
+__global__ void k_cut(const uint32_t* __restrict__ spos, int64_t Sp, int n, uint32_t* __restrict__ cut)
+{
+    if ((int)threadIdx.x < n) cut[threadIdx.x] = spos[(size_t)threadIdx.x * Sp] + 1;
+}
+
 // spos_t[r / 2][i][r % 2] = spos[i][r]: 32 x 32 tiles through shared memory, a thread
 // storing the two positions of a rank pair of one node as one 8-byte word (coalesced both
 // ways)
@@ -191,11 +502,87 @@ __global__ void k_spos_pad(uint32_t* __restrict__ spos, uint32_t* __restrict__ s
     srank[i * Sp + S + e] = 0u;
 }
 
-// Ranks every node's entries (see the file comment).  Temporaries are stream-ordered.
-int rank_entries(bn_table* t, cudaStream_t s)
+// stream-ordered temporaries of one call
+struct SortTemps {
+    cudaStream_t s;
+    std::vector<void*> p;
+    ~SortTemps()
+    {
+        for (void* q : p) cudaFreeAsync(q, s);
+    }
+    template <class T>
+    int get(T** out, size_t count)
+    {
+        void* q = nullptr;
+        cudaError_t e = cudaMallocAsync(&q, std::max<size_t>(count, 1) * sizeof(T), s);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(BN_ENOMEM, "rank_entries: %zu bytes of sort buffers: %s", count * sizeof(T),
+                             cudaGetErrorString(e));
+        }
+        p.push_back(q);
+        *out = (T*)q;
+        return BN_OK;
+    }
+};
+
+static int rank_by_buckets(bn_table* t, cudaStream_t s)
 {
     const int64_t S = t->S;
-    if (S > 0xffffffffLL) return set_error(BN_EUNSUPPORTED, "rank_entries: too many sets per node");
+    const int per = (int)std::max<int64_t>(1, std::min<int64_t>(t->n, 0x7fffffffLL / S));
+    BsArgs A;
+    A.keys = t->keys;
+    A.pst = t->pst;
+    A.S = S;
+    A.Sp = t->Sp;
+    A.srank = t->srank;
+    A.spos = t->spos;
+    A.sset = t->sset;
+    A.Ssp = t->sset_stride;
+    const bool whole = S <= BS_CAP;
+    A.NB = whole ? 1 : (int)std::min<int64_t>(BS_MAX_BUCKETS, (S + BS_AVG - 1) / BS_AVG);
+    A.tiles = (int)((S + BS_TILE - 1) / BS_TILE);
+    A.M = 32;
+    while (A.M < 8 * A.NB && A.M < BS_SAMPLES) A.M *= 2;
+    SortTemps tmp{s, {}};
+    int rc;
+    if (!whole &&
+        ((rc = tmp.get(&A.split_x, (size_t)per * A.NB)) || (rc = tmp.get(&A.split_r, (size_t)per * A.NB)) ||
+         (rc = tmp.get(&A.counts, (size_t)2 * per * A.NB)) ||
+         (rc = tmp.get(&A.tile_base, (size_t)per * A.tiles * A.NB)) || (rc = tmp.get(&A.bid, (size_t)per * S)) ||
+         (rc = tmp.get(&A.bx, (size_t)per * S)) || (rc = tmp.get(&A.br, (size_t)per * S))))
+        return rc;
+    static unsigned long long ctx[64] = {0};
+    if (first_in_context(ctx)) {
+        BN_CUDA(cudaFuncSetAttribute(k_bs_split, cudaFuncAttributeMaxDynamicSharedMemorySize, BS_SAMPLES * 12));
+        BN_CUDA(cudaFuncSetAttribute(k_bs_sort<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SMEM));
+        BN_CUDA(cudaFuncSetAttribute(k_bs_sort<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SMEM));
+    }
+    for (A.node0 = 0; A.node0 < t->n; A.node0 += per) {
+        const int nb = std::min(per, t->n - A.node0);
+        if (whole) {
+            k_bs_sort<true><<<dim3(1, (unsigned)nb), BS_THREADS, BS_SMEM, s>>>(A, nb);
+            BN_LAUNCH_CHECK("k_bs_sort");
+            continue;
+        }
+        BN_CUDA(cudaMemsetAsync(A.counts, 0, sizeof(uint32_t) * (size_t)nb * A.NB, s));
+        k_bs_split<<<nb, 1024, (size_t)A.M * 12, s>>>(A);
+        BN_LAUNCH_CHECK("k_bs_split");
+        k_bs_count<<<dim3((unsigned)A.tiles, (unsigned)nb), 512, 0, s>>>(A);
+        BN_LAUNCH_CHECK("k_bs_count");
+        k_bs_scan<<<nb, BS_MAX_BUCKETS, 0, s>>>(A, nb);
+        BN_LAUNCH_CHECK("k_bs_scan");
+        k_bs_scatter<<<dim3((unsigned)A.tiles, (unsigned)nb), 512, 0, s>>>(A, nb);
+        BN_LAUNCH_CHECK("k_bs_scatter");
+        k_bs_sort<false><<<dim3((unsigned)A.NB, (unsigned)nb), BS_THREADS, BS_SMEM, s>>>(A, nb);
+        BN_LAUNCH_CHECK("k_bs_sort");
+    }
+    return BN_OK;
+}
+
+static int rank_by_radix(bn_table* t, cudaStream_t s)
+{
+    const int64_t S = t->S;
     // nodes per batch so that batch * S fits the 32-bit value
     const int per = (int)std::max<int64_t>(1, std::min<int64_t>(t->n, 0x7fffffffLL / S));
     const int64_t Nmax = (int64_t)per * S;
@@ -256,6 +643,30 @@ int rank_entries(bn_table* t, cudaStream_t s)
         k_rs_finish<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(vi, N, S, t->Sp, node0, t->srank, t->spos);
         BN_LAUNCH_CHECK("k_rs_finish");
     }
+    return BN_OK;
+}
+
+// Ranks every node's entries (see the file comment) and lays out what the scans read:
+// srank, spos, its entry-major copy spos_t and (k <= 4) the parent nodes by sorted
+// position.  d_cut receives each node's empty-set position + 1 (device, n words; the caller
+// copies it to t->cut).  Temporaries are stream-ordered; nothing waits for the device.
+int rank_entries(bn_table* t, uint32_t* d_cut, cudaStream_t s)
+{
+    const int64_t S = t->S;
+    if (S > 0xffffffffLL) return set_error(BN_EUNSUPPORTED, "rank_entries: too many sets per node");
+    int rc = alloc_sset(t);
+    if (rc) return rc;
+    if (S <= (int64_t)BS_MAX_BUCKETS * 2 * BS_AVG) {
+        if ((rc = rank_by_buckets(t, s))) return rc;
+    } else {
+        if ((rc = rank_by_radix(t, s))) return rc;
+        if (t->sset && (rc = build_sset(t, s))) return rc;
+    }
+    if (t->sset && t->sset_stride > S) {
+        k_sset_pad<<<dim3((unsigned)((t->sset_stride - S + 255) / 256), (unsigned)t->n), 256, 0, s>>>(t->sset, S,
+                                                                                                 t->sset_stride);
+        BN_LAUNCH_CHECK("k_sset_pad");
+    }
     if (t->Sp > S) {
         const int64_t tot = (int64_t)t->n * (t->Sp - S);
         k_spos_pad<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(t->spos, t->srank, t->n, S, t->Sp);
@@ -264,7 +675,9 @@ int rank_entries(bn_table* t, cudaStream_t s)
     k_spos_transpose<<<dim3((unsigned)(t->Sp / 32), (unsigned)((t->n + 31) / 32)), dim3(32, 8), 0, s>>>(t->spos, t->n, t->Sp,
                                                                                                     t->spos_t);
     BN_LAUNCH_CHECK("k_spos_transpose");
-    return build_sset(t, s);
+    k_cut<<<1, MAXN, 0, s>>>(t->spos, t->Sp, t->n, d_cut);
+    BN_LAUNCH_CHECK("k_cut");
+    return BN_OK;
 }
 
 }  // namespace bn

@@ -505,12 +505,6 @@ static int copy_in(void* dst, const void* src, size_t bytes, int mem, cudaStream
     return BN_OK;
 }
 
-static int read_status(const uint32_t* d_status, uint32_t* h, cudaStream_t s)
-{
-    BN_CUDA(cudaMemcpyAsync(h, d_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    BN_CUDA(cudaStreamSynchronize(s));
-    return BN_OK;
-}
 
 }  // namespace bn
 
@@ -653,10 +647,12 @@ static int build_plan(const uint8_t* data, int m, int n, const uint8_t* arity, i
     return BN_OK;
 }
 
-// Device half: every kernel of the build on stream s, writing t (allocated) and OR-ing
-// STATUS_BADINPUT into *d_status for a data value at or above its arity.  Temporaries
-// are stream-ordered; nothing here waits for the device.
-static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_status, cudaStream_t s,
+// Device half: every kernel of the build on stream s, writing t (allocated), OR-ing
+// STATUS_BADINPUT into d_meta[0] for a data value at or above its arity and leaving the
+// nodes' empty-set positions + 1 in d_meta[1..n] (META_WORDS words).  Temporaries are
+// stream-ordered; nothing here waits for the device.
+static constexpr int META_WORDS = 1 + MAXN;
+static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cudaStream_t s,
                          cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr)
 {
     const int n = P.n, m = P.m, k = P.k;
@@ -683,7 +679,7 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_status, cu
             if ((rc = tmp.get(&d_data, (size_t)m * n))) return rc;
             if ((rc = copy_in(d_data, P.data, (size_t)m * n, BN_MEM_HOST, s))) return rc;
         }
-        k_pack<<<(n * mw + 255) / 256, 256, 0, s>>>(d_data, m, n, mw, d_ar, d_packed, d_status);
+        k_pack<<<(n * mw + 255) / 256, 256, 0, s>>>(d_data, m, n, mw, d_ar, d_packed, d_meta);
         BN_LAUNCH_CHECK("k_pack");
     }
     if (P.R) {
@@ -752,7 +748,18 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_status, cu
     BN_LAUNCH_CHECK("k_assemble");
     if (ev1) BN_CUDA(cudaEventRecord(ev1, s));
     sums.release();
-    return rank_entries(t, s);
+    return rank_entries(t, d_meta + 1, s);
+}
+
+// the status word and the table's empty-set positions, once the work on s is done
+static int read_meta(const uint32_t* d_meta, bn_table* t, uint32_t* status, cudaStream_t s)
+{
+    uint32_t h[META_WORDS];
+    BN_CUDA(cudaMemcpyAsync(h, d_meta, sizeof(uint32_t) * (1 + t->n), cudaMemcpyDeviceToHost, s));
+    BN_CUDA(cudaStreamSynchronize(s));
+    *status = h[0];
+    memcpy(t->cut, h + 1, sizeof(uint32_t) * t->n);
+    return BN_OK;
 }
 
 static int build_scores_impl(const uint8_t* data, int m, int n, const uint8_t* arity, int k, const double* R,
@@ -776,14 +783,14 @@ static int build_scores_impl(const uint8_t* data, int m, int n, const uint8_t* a
             if (!ok && t) bn_table_free(t);
         }
     } guard{t};
-    uint32_t* d_status = nullptr;
+    uint32_t* d_meta = nullptr;
     {
         Temps tmp(s);
-        if ((rc = tmp.get(&d_status, 1))) return rc;
-        BN_CUDA(cudaMemsetAsync(d_status, 0, sizeof(uint32_t), s));
-        if ((rc = build_enqueue(P, t, d_status, s, ev0, ev1))) return rc;
+        if ((rc = tmp.get(&d_meta, META_WORDS))) return rc;
+        BN_CUDA(cudaMemsetAsync(d_meta, 0, sizeof(uint32_t), s));
+        if ((rc = build_enqueue(P, t, d_meta, s, ev0, ev1))) return rc;
         uint32_t st = 0;
-        if ((rc = read_status(d_status, &st, s))) return rc;
+        if ((rc = read_meta(d_meta, t, &st, s))) return rc;
         if (st & STATUS_BADINPUT) return set_error(BN_EINVAL, "bn_build_scores: a data value is >= its arity");
     }
     guard.ok = true;
@@ -870,14 +877,14 @@ extern "C" int bn_build_scores_batch(int count, const uint8_t* const* data, cons
                 if (x) cudaEventDestroy(x);
         }
     } sg{side, ev};
-    uint32_t* d_status = nullptr;
-    BN_CUDA(cudaMallocAsync((void**)&d_status, sizeof(uint32_t) * count, s));
+    uint32_t* d_meta = nullptr;
+    BN_CUDA(cudaMallocAsync((void**)&d_meta, sizeof(uint32_t) * META_WORDS * count, s));
     struct Free {
         uint32_t* p;
         cudaStream_t s;
         ~Free() { cudaFreeAsync(p, s); }
-    } fr{d_status, s};
-    BN_CUDA(cudaMemsetAsync(d_status, 0, sizeof(uint32_t) * count, s));
+    } fr{d_meta, s};
+    BN_CUDA(cudaMemsetAsync(d_meta, 0, sizeof(uint32_t) * META_WORDS * count, s));
     for (int j = 0; j <= ns; ++j) BN_CUDA(cudaEventCreateWithFlags(&ev[j], cudaEventDisableTiming));
     BN_CUDA(cudaEventRecord(ev[ns], s));
     for (int j = 0; j < ns; ++j) {
@@ -887,7 +894,7 @@ extern "C" int bn_build_scores_batch(int count, const uint8_t* const* data, cons
     int rc = BN_OK;
     for (int q = 0; q < count && !rc; ++q) {
         const int i = order[q];
-        rc = build_enqueue(plans[i], tabs[i], d_status + i, side[q % ns]);
+        rc = build_enqueue(plans[i], tabs[i], d_meta + (size_t)META_WORDS * i, side[q % ns]);
     }
     for (int j = 0; j < ns; ++j) {
         cudaEventRecord(ev[j], side[j]);
@@ -897,11 +904,12 @@ extern "C" int bn_build_scores_batch(int count, const uint8_t* const* data, cons
         cudaStreamSynchronize(s);
         return rc;
     }
-    std::vector<uint32_t> st(count, 0);
-    BN_CUDA(cudaMemcpyAsync(st.data(), d_status, sizeof(uint32_t) * count, cudaMemcpyDeviceToHost, s));
+    std::vector<uint32_t> st((size_t)META_WORDS * count, 0);
+    BN_CUDA(cudaMemcpyAsync(st.data(), d_meta, sizeof(uint32_t) * st.size(), cudaMemcpyDeviceToHost, s));
     BN_CUDA(cudaStreamSynchronize(s));
+    for (int i = 0; i < count; ++i) memcpy(tabs[i]->cut, &st[(size_t)META_WORDS * i + 1], sizeof(uint32_t) * n[i]);
     for (int i = 0; i < count; ++i)
-        if (st[i] & STATUS_BADINPUT)
+        if (st[(size_t)META_WORDS * i] & STATUS_BADINPUT)
             return set_error(BN_EINVAL, "bn_build_scores_batch: network %d: a data value is >= its arity", i);
     guard.ok = true;
     for (int i = 0; i < count; ++i) out[i] = tabs[i];
@@ -924,23 +932,23 @@ extern "C" int bn_table_from_scores(const double* scores, int n, int k, int mem,
     if (rc) return rc;
     Temps tmp(s);
     double* d_sc = nullptr;
-    uint32_t* d_status = nullptr;
-    if ((rc = tmp.get(&d_status, 1))) { bn_table_free(t); return rc; }
+    uint32_t* d_meta = nullptr;
+    if ((rc = tmp.get(&d_meta, META_WORDS))) { bn_table_free(t); return rc; }
     if (mem == BN_MEM_DEVICE) d_sc = (double*)scores;
     else {
         if ((rc = tmp.get(&d_sc, (size_t)n * S))) { bn_table_free(t); return rc; }
         if ((rc = copy_in(d_sc, scores, sizeof(double) * (size_t)n * S, BN_MEM_HOST, s))) { bn_table_free(t); return rc; }
     }
-    if (cudaMemsetAsync(d_status, 0, 4, s) != cudaSuccess) { bn_table_free(t); return cuda_fail(cudaGetLastError(), "memset", __FILE__, __LINE__); }
+    if (cudaMemsetAsync(d_meta, 0, 4, s) != cudaSuccess) { bn_table_free(t); return cuda_fail(cudaGetLastError(), "memset", __FILE__, __LINE__); }
     int64_t tot = (int64_t)n * S;
-    k_keys_from_scores<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(d_sc, n, S, t->Sp, t->keys, d_status);
+    k_keys_from_scores<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(d_sc, n, S, t->Sp, t->keys, d_meta);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { bn_table_free(t); return cuda_fail(e, "k_keys_from_scores", __FILE__, __LINE__); }
     count_launches(1);
     if ((rc = build_pst(t, s, true))) { bn_table_free(t); return rc; }
-    if ((rc = rank_entries(t, s))) { bn_table_free(t); return rc; }
+    if ((rc = rank_entries(t, d_meta + 1, s))) { bn_table_free(t); return rc; }
     uint32_t st = 0;
-    if ((rc = read_status(d_status, &st, s))) { bn_table_free(t); return rc; }
+    if ((rc = read_meta(d_meta, t, &st, s))) { bn_table_free(t); return rc; }
     if (st) { bn_table_free(t); return set_error(BN_EINVAL, "bn_table_from_scores: NaN or +inf score"); }
     *out = t;
     return BN_OK;

@@ -45,12 +45,36 @@ struct bn_table {
 
 namespace bn {
 
-// Sorted positions and their inverse for every node (bn_sort.cu).
-int rank_entries(bn_table* t, cudaStream_t s);
+// Sorted positions and their inverse for every node (bn_sort.cu); d_cut: n words on the
+// device, each node's empty-set position + 1.
+int rank_entries(bn_table* t, uint32_t* d_cut, cudaStream_t s);
 
-// The bit-sliced scans (bn_sliced.cu): the parent sets in sorted-position order (k <= 4;
-// nothing for larger k), and the scan of work lists in the layout of launch_scan, as a
+// The word of a parent set in the sorted parent sets (k <= 4): the parent node ids, ascending,
+// a byte each; SSET_ONES where the set has fewer than four parents.  SSET_NEVER: a
+// padding entry that no order is consistent with.
+constexpr uint32_t SSET_ONES = 64u;
+constexpr uint32_t SSET_NEVER = 0x41414141u;
+__device__ __forceinline__ uint32_t sset_word(uint64_t m, int i)
+{
+    uint32_t w = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        uint32_t v = SSET_ONES;
+        if (m) {
+            const int c = __ffsll((long long)m) - 1;
+            m &= m - 1;
+            v = (uint32_t)(c + (c >= i));
+        }
+        w |= v << (8 * j);
+    }
+    return w;
+}
+
+// The bit-sliced scans (bn_sliced.cu): memory for the parent sets in sorted-position order
+// (k <= 4; none for larger k), their words from srank (the bucket sort writes them itself),
+// and the scan of work lists in the layout of launch_scan, as a
 // full pass (cut = false) or stopping early with identical results (cut = true).
+int alloc_sset(bn_table* t);
 int build_sset(bn_table* t, cudaStream_t s);
 int launch_scan_sliced(const bn_table* t, const uint32_t* list_count, const uint64_t* list_pc, uint32_t* list_best,
                        int cap, bool cut, uint32_t* status, cudaStream_t s);
