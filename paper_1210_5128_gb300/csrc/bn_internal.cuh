@@ -61,6 +61,9 @@ constexpr BinomTable make_binom()
 }
 static __constant__ BinomTable c_binom = make_binom();
 constexpr BinomTable h_binom = make_binom();
+// The same table in global memory: lanes that read different entries (a block copying it to
+// shared memory) are served in one pass, where the constant bank takes them one by one.
+static __device__ const BinomTable g_binom = make_binom();
 
 // sets of size <= k drawn from N candidates
 inline int64_t num_sets_host(int N, int k)

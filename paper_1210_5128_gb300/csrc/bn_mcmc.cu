@@ -439,31 +439,42 @@ __global__ void k_gcache_fill(const int64_t* __restrict__ keys, const uint32_t* 
     if (j <= (uint32_t)n) c_off[j] = j < (uint32_t)n ? aoff[j] : total;
 }
 
-__global__ void k_gcache_first(int n, int cap, const uint8_t* __restrict__ cache, uint16_t* __restrict__ first)
+// One block of 64 threads a node: thread v finds the node's first survivor that contains
+// node v, and the first warp writes the prefix ORs, 32 survivors at a time.
+__global__ void __launch_bounds__(64) k_gcache_index(int cap, uint8_t* __restrict__ cache, uint16_t* __restrict__ first)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * 64) return;
-    const int nd = idx >> 6, v = idx & 63;
-    const uint64_t* c_mask = (const uint64_t*)cache;
-    const uint32_t* c_off = (const uint32_t*)(cache + 28 * (size_t)cap);
-    const uint32_t j0 = c_off[nd], j1 = c_off[nd + 1];
-    uint32_t j = j0;
-    while (j < j1 && ((c_mask[j] >> v) & 1ull) == 0ull) ++j;
-    first[idx] = (uint16_t)min(j - j0, 65535u);
-}
-
-__global__ void k_gcache_orb(int n, int cap, uint8_t* __restrict__ cache)
-{
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= n) return;
+    const int nd = blockIdx.x, v = threadIdx.x, lane = v & 31;
     const uint64_t* c_mask = (const uint64_t*)cache;
     uint64_t* c_orb = (uint64_t*)(cache + 16 * (size_t)cap);
     const uint32_t* c_off = (const uint32_t*)(cache + 28 * (size_t)cap);
-    uint64_t acc = 0ull;
-    for (uint32_t j = c_off[v]; j < c_off[v + 1]; ++j) {
-        c_orb[j] = acc;
-        acc |= c_mask[j];
+    const uint32_t j0 = c_off[nd], j1 = c_off[nd + 1];
+    if (v < 32) {
+        uint64_t run = 0;
+        for (uint32_t b = j0; b < j1; b += 32) {
+            const uint64_t m = b + lane < j1 ? c_mask[b + lane] : 0ull;
+            uint64_t s = m;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint64_t y = __shfl_up_sync(0xffffffffu, s, d);
+                if (lane >= d) s |= y;
+            }
+            const uint64_t up = __shfl_up_sync(0xffffffffu, s, 1);
+            if (b + lane < j1) c_orb[b + lane] = run | (lane ? up : 0ull);
+            run |= __shfl_sync(0xffffffffu, s, 31);
+        }
     }
+    uint32_t j = j0;
+    bool found = false;
+    for (uint32_t b = j0; b < j1; b += 8) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (b + u < j1 && !found) {
+                found = (c_mask[b + u] >> v) & 1ull;
+                j = b + u + (found ? 0 : 1);
+            }
+        if (__all_sync(0xffffffffu, found)) break;
+    }
+    first[nd * 64 + v] = (uint16_t)min(j - j0, 65535u);
 }
 
 // JUMP (global-memory caches): `first` = F.gfirst, the first survivor of every node that
@@ -1416,10 +1427,8 @@ int build_survivor_cache(bn_table* t, cudaStream_t s)
     const unsigned blocks = (unsigned)((std::max<uint32_t>(total, (uint32_t)t->n + 1) + 255) / 256);
     k_gcache_fill<<<blocks, 256, 0, s>>>(t->keys, t->srank, t->Sp, t->n, t->amask, t->aspos, t->aoff, total, cap, g);
     BN_LAUNCH_CHECK("k_gcache_fill");
-    k_gcache_orb<<<(t->n + 63) / 64, 64, 0, s>>>(t->n, cap, g);
-    BN_LAUNCH_CHECK("k_gcache_orb");
-    k_gcache_first<<<(t->n * 64 + 255) / 256, 256, 0, s>>>(t->n, cap, g, (uint16_t*)(g + surv_cache_stride(cap)));
-    BN_LAUNCH_CHECK("k_gcache_first");
+    k_gcache_index<<<t->n, 64, 0, s>>>(cap, g, (uint16_t*)(g + surv_cache_stride(cap)));
+    BN_LAUNCH_CHECK("k_gcache_index");
     t->gcache = g;
     return BN_OK;
 }

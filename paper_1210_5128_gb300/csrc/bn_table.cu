@@ -99,16 +99,41 @@ __global__ void k_lut(const double* __restrict__ alpha, int nlut, int m1, fx128*
 }
 
 // a4: parent-set table, candidate-space mask of every rank; padding ranks get ~0 (they
-// can never be consistent with an order)
-__global__ void k_pst(int N, int64_t S, int64_t Sp, uint64_t* __restrict__ pst)
+// can never be consistent with an order).  A thread unranks the first of PST_RUN
+// consecutive ranks (binomials in shared memory, binary searches) and steps to the others:
+// 55 -> 8 us at n = 60, k = 4 against one unranking from the constant bank per rank.
+static constexpr int PST_RUN = 4;
+__global__ void __launch_bounds__(256) k_pst(int N, int k, int64_t S, int64_t Sp, uint64_t* __restrict__ pst)
 {
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= Sp) return;
-    if (r >= S) { pst[r] = ~0ull; return; }
-    int j;
-    uint64_t m;
-    unrank_dev(N, r, j, m);
-    pst[r] = m;
+    extern __shared__ uint64_t s_bin[];                 // C(a, t), a <= 63, t <= k
+    const int T = k + 1;
+    for (int q = threadIdx.x; q < 64 * T; q += blockDim.x) s_bin[q] = g_binom.v[q / T][q % T];
+    __syncthreads();
+    const int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * PST_RUN;
+    if (r0 >= Sp) return;                               // Sp is a multiple of PST_RUN
+    int j = 0;
+    uint64_t mask = 0;
+    if (r0 < S) {
+        uint64_t r = (uint64_t)r0;
+        while (r >= s_bin[N * T + j]) r -= s_bin[N * T + j++];
+        int hi = N - 1;
+        for (int t = j; t >= 1; --t) {                  // largest a with C(a, t) <= r
+            int lo = t - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (s_bin[mid * T + t] <= r) lo = mid;
+                else hi = mid - 1;
+            }
+            mask |= 1ull << lo;
+            r -= s_bin[lo * T + t];
+            hi = lo - 1;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < PST_RUN; ++u) {
+        pst[r0 + u] = r0 + u < S ? mask : ~0ull;
+        next_set(N, j, mask);
+    }
 }
 
 __global__ void k_pad_keys(int64_t* __restrict__ keys, int n, int64_t S, int64_t Sp)
@@ -131,7 +156,7 @@ __global__ void k_pad_keys(int64_t* __restrict__ keys, int n, int64_t S, int64_t
 // once per set U of at most k + 1 nodes (k_joint) instead of once per (node, parent set):
 // C(60, 5) = 5.5 M tables instead of 29.4 M at n = 60, k = 4; k_assemble forms the entries.
 // Measured at n = 60, k = 4, m = 1000, ternary: 20.0 ms with one count table per entry,
-// 5.05 ms for k_joint and 0.89 ms for k_assemble.
+// 5.05 ms for k_joint and 0.51 ms for k_assemble.
 // ---------------------------------------------------------------------------------
 struct JointArgs {
     const uint32_t* packed;
@@ -329,16 +354,21 @@ __device__ __forceinline__ double div_ln10(double x)
     return __fma_rn(r, z, q0);
 }
 
-// One thread per (node, rank): the node-space ranks of pi and pi + {i}, their sums, one
+static constexpr int ASM_BLOCK = 2048;     // entries of a block (its binomial table is paid once)
+
+// One entry a thread at a time: the node-space ranks of pi and pi + {i}, their sums, one
 // rounding, / ln 10, the size penalty, the prior of every parent (ascending node ids).
 // Consecutive ranks differ in their lowest parents, so both gathers are mostly coalesced.
-// Bound by the FP64 pipe (about ten operations an entry) and the 16-byte gathers.
+// Bound by the FP64 pipe (about ten operations an entry) and the 16-byte gathers: 0.51 ms
+// at n = 60, k = 4 (0.89 ms with 256 entries a block).
 __global__ void __launch_bounds__(256) k_assemble(AssembleArgs A)
 {
     __shared__ int64_t s_bin[65 * (MAXK + 2)];          // C(a, t), t <= k + 1
     __shared__ int64_t s_base[MAXK + 3];                // first rank of every set size
+    __shared__ double s_pen[MAXK + 1];                  // its structure penalty
     const int T = A.k + 2;
-    for (int q = threadIdx.x; q < 65 * T; q += blockDim.x) s_bin[q] = (int64_t)c_binom.v[q / T][q % T];
+    for (int q = threadIdx.x; q < 65 * T; q += blockDim.x) s_bin[q] = (int64_t)g_binom.v[q / T][q % T];
+    if ((int)threadIdx.x <= A.k) s_pen[threadIdx.x] = __dmul_rn((double)threadIdx.x, A.log10g);
     if (threadIdx.x == 0) {
         int64_t b = 0;
         for (int t = 0; t <= A.k + 1; ++t) {
@@ -348,40 +378,43 @@ __global__ void __launch_bounds__(256) k_assemble(AssembleArgs A)
     }
     __syncthreads();
     const int i = blockIdx.y;
-    const int64_t rho = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (rho >= A.Sp) return;
-    int64_t* out = A.keys + (size_t)i * A.Sp + rho;
-    if (rho >= A.S) {
-        *out = KEY_NONE;                                // padding
-        return;
-    }
-    const uint64_t mask = A.pst[rho];
-    const int j = __popcll(mask);
-    int64_t rp = s_base[j], ru = s_base[j + 1];
-    int t = 0, below = 0;
-    uint64_t mm = mask;
-    while (mm) {
-        const int c = __ffsll((long long)mm) - 1;
-        mm &= mm - 1;
-        const int gt = c >= i;
-        const int64_t* row = s_bin + (c + gt) * T + ++t;
-        rp += row[0];
-        ru += row[gt];
-        below += !gt;
-    }
-    ru += s_bin[i * T + below + 1];
     const int v = (int)((A.vmap >> (8 * (A.arity[i] - 1))) & 0xffu);
-    const fx128 acc = A.G[ru] - A.H[(size_t)v * A.S0 + rp];
-    double ls = __dadd_rn(div_ln10(fx_to_double(acc)), __dmul_rn((double)j, A.log10g));
-    if (A.ppf) {
-        mm = mask;
+    const fx128* H = A.H + (size_t)v * A.S0;
+    const int64_t r1 = min((int64_t)(blockIdx.x + 1) * ASM_BLOCK, A.Sp);
+#pragma unroll 2
+    for (int64_t rho = (int64_t)blockIdx.x * ASM_BLOCK + threadIdx.x; rho < r1; rho += 256) {
+        int64_t* out = A.keys + (size_t)i * A.Sp + rho;
+        if (rho >= A.S) {
+            *out = KEY_NONE;                            // padding
+            continue;
+        }
+        const uint64_t mask = A.pst[rho];
+        const int j = __popcll(mask);
+        int64_t rp = s_base[j], ru = s_base[j + 1];
+        int t = 0, below = 0;
+        uint64_t mm = mask;
         while (mm) {
             const int c = __ffsll((long long)mm) - 1;
             mm &= mm - 1;
-            ls = __dadd_rn(ls, A.ppf[(size_t)i * A.n + c + (c >= i ? 1 : 0)]);
+            const int gt = c >= i;
+            const int64_t* row = s_bin + (c + gt) * T + ++t;
+            rp += row[0];
+            ru += row[gt];
+            below += !gt;
         }
+        ru += s_bin[i * T + below + 1];
+        const fx128 acc = A.G[ru] - H[rp];
+        double ls = __dadd_rn(div_ln10(fx_to_double(acc)), s_pen[j]);
+        if (A.ppf) {
+            mm = mask;
+            while (mm) {
+                const int c = __ffsll((long long)mm) - 1;
+                mm &= mm - 1;
+                ls = __dadd_rn(ls, A.ppf[(size_t)i * A.n + c + (c >= i ? 1 : 0)]);
+            }
+        }
+        *out = double_to_key(ls);
     }
-    *out = double_to_key(ls);
 }
 
 // score table upload / readout
@@ -440,8 +473,8 @@ static int table_alloc(int n, int k, bn_table** out)
 static int build_pst(bn_table* t, cudaStream_t s, bool pad_keys)
 {
     int thr = 256;
-    int64_t blocks = (t->Sp + thr - 1) / thr;
-    k_pst<<<(unsigned)blocks, thr, 0, s>>>(t->n - 1, t->S, t->Sp, t->pst);
+    const int64_t blocks = (t->Sp / PST_RUN + thr - 1) / thr;
+    k_pst<<<(unsigned)blocks, thr, sizeof(uint64_t) * 64 * (t->k + 1), s>>>(t->n - 1, t->k, t->S, t->Sp, t->pst);
     BN_LAUNCH_CHECK("k_pst");
     if (pad_keys && t->Sp > t->S) {
         int64_t tot = (int64_t)t->n * (t->Sp - t->S);
@@ -744,7 +777,7 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
     else rc = launch_joint_kt<12>(A, smem_data, base, smem, grid, thr, s);
     if (rc) return rc;
     AssembleArgs B{t->pst, n, k, P.S, t->Sp, A.S0, A.G, A.H, d_ar, P.vmap, d_ppf, P.log10g, t->keys};
-    k_assemble<<<dim3((unsigned)((t->Sp + 255) / 256), (unsigned)n), 256, 0, s>>>(B);
+    k_assemble<<<dim3((unsigned)((t->Sp + ASM_BLOCK - 1) / ASM_BLOCK), (unsigned)n), 256, 0, s>>>(B);
     BN_LAUNCH_CHECK("k_assemble");
     if (ev1) BN_CUDA(cudaEventRecord(ev1, s));
     sums.release();
