@@ -10,9 +10,10 @@
 // entry against 32 orders at once.  Of those items, the ones this warp has not found
 // yet take the entry's sorted position (a shared-memory atomicMin, by the lowest lane of
 // a step that hits the item), and a warp-wide OR marks them found.  Every later entry of
-// the warp lies further down the sorted list, so it can only lose.  Blocks of the same
-// node also trade positions across chunks through the work list: an item that already
-// holds a position above a block's chunk is not tested there at all.
+// the warp lies further down the sorted list, so it can only lose.  A node's stages (2,048
+// entries) go round its blocks, so all of them walk from the top of the list to its end
+// together, and they trade positions through the work list: an item that holds a position
+// above a block's next stage is not tested there any more.
 //
 // The entries reach shared memory as one 4-byte word each (the parent node ids, a byte
 // apiece, in sorted-position order; `sset`), streamed by 1-D bulk (TMA) copies, so a
@@ -20,12 +21,11 @@
 // items per shared-memory word instead of one.  The per-lane copies of the P words
 // (each lane reads its own bank) keep the four loads free of bank conflicts.
 //
-// Two modes.  The full pass tests every entry of the table (Eq. (6) taken literally).
-// The sorted mode (BN_SCAN_SORTED) stops early, with identical results: nothing past the
-// empty set's sorted position can be chosen (the empty set is consistent with every
-// order), a block stops streaming once each of its items has taken an entry (every
-// entry still unread lies further down the list), and a block whose items all hold a
-// position above its chunk already (from blocks of earlier chunks) does nothing.
+// Two modes.  The full pass reads every entry of the table.  The sorted mode
+// (BN_SCAN_SORTED) stops early, with identical results: nothing past the empty set's
+// sorted position can be chosen (the empty set is consistent with every order), and a
+// block stops streaming once each of its items holds a position above the next stage
+// (every entry still unread lies further down the list).
 #include <algorithm>
 
 #include "bn_table.cuh"
@@ -63,8 +63,8 @@ struct SlicedArgs {
     int64_t Sp, S;
     int64_t Ssp;                   // sset row stride: S rounded up to whole stages
     int n;
-    int64_t chunk;                 // entries per block (multiple of SL_SUB)
-    int nchunk;
+    int nchunk;                    // blocks per node and item set
+    int per;                       // sorted mode: consecutive stages per block
     const uint32_t* list_count;
     const uint64_t* list_pc;
     uint32_t* list_best;
@@ -117,22 +117,69 @@ __device__ __forceinline__ int Pw(int g, int v)
     return (g >> 1) * SL_ROWS * (SL_ROW_BYTES / 4) + v * (SL_ROW_BYTES / 4) + (g & 1) * 32;
 }
 
-// Block (chunk c, node i) = blockIdx.x = c * n + i, item set blockIdx.y: items
-// 32 G y .. 32 G y + 32 G - 1 of node i.  Eight consumer warps and one producer warp:
-// consumer warp w tests entries w * 256 .. w * 256 + 255 of every stage, 128 a step, so
-// each warp walks its entries in increasing sorted position; the producer refills a stage
-// as soon as every consumer has released it (an empty mbarrier per stage), so no
-// consumer waits for a refill.
+// bit l of lane r's result = bit r of lane l's x (five exchange steps)
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane)
+{
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        const uint32_t m = d == 16 ? 0x0000ffffu : d == 8 ? 0x00ff00ffu : d == 4 ? 0x0f0f0f0fu : d == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, d);
+        x = (lane & d) ? (x & ~m) | ((y & ~m) >> d) : (x & m) | ((y & m) << d);
+    }
+    return x;
+}
+
+// Records a step's new items of one group: `hit` = the items that this lane's four entries w
+// match, `items` = the OR over the lanes.  Positions run lane-major (lane l holds pos0 +
+// 4 l .. + 3).  A ballot per new item, or a bit-matrix transpose where there are many, hands
+// lane r the lanes that hit item r; it takes the lowest of them, fetches that lane's four
+// words and records the first that holds the item: one conflict-free atomicMin a lane,
+// however dense the hits.
+__device__ __forceinline__ void record_items(uint32_t hit, uint32_t items, uint4 w4, const uint8_t* P,
+                                             uint32_t* best, uint32_t pos0, int lane)
+{
+    uint32_t lanes = 0;
+    if (__popc(items) > 16) {
+        lanes = transpose32(hit, lane);
+    } else {
+        for (uint32_t t = items; t; t &= t - 1) {
+            const int r = __ffs(t) - 1;
+            const uint32_t b = __ballot_sync(0xffffffffu, (hit >> r) & 1u);
+            if (lane == r) lanes = b;
+        }
+    }
+    const int src = lanes ? __ffs(lanes) - 1 : 0;
+    const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+    const uint32_t lane4 = (uint32_t)lane * 4u;
+    int u = 3;
+#pragma unroll
+    for (int v = 3; v >= 0; --v) {
+        uint32_t m = 0xffffffffu;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) m &= *(const uint32_t*)(P + __byte_perm(w[v], lane4, 0x5504u + 0x10u * j));
+        if ((__shfl_sync(0xffffffffu, m, src) >> lane) & 1u) u = v;
+    }
+    if (lanes) atomicMin(best + lane, pos0 + 4 * src + u);
+}
+
+// Block (c, node i) = blockIdx.x = c * n + i, item set blockIdx.y: items 32 G y .. 32 G y +
+// 32 G - 1 of node i, stages c, c + nchunk, c + 2 nchunk, .. of the node's list (sorted
+// mode: stages c per .. c per + per - 1).  Eight
+// consumer warps and one producer warp: consumer warp w tests entries w * 256 .. w * 256 +
+// 255 of every stage, 128 a step, so each warp walks its entries in increasing sorted
+// position; the producer refills a stage as soon as every consumer has released it (an
+// empty mbarrier per stage), so no consumer waits for a refill.
+//
+// With contiguous chunks the lower blocks of a full pass test all their items although the
+// top one finds most of them.  Round-robin stages, the recording of a step's items by one
+// atomicMin a lane and the producer's early end of its trades took the full pass at n = 60
+// from 154 to 60 us for 256 orders and from 533 to 164 for 777.  The sorted mode keeps
+// contiguous chunks (its lower blocks stop as soon as the top one has found everything, and
+// every block that holds some of the top pays for its dense hits): 83 -> 36 us and 132 -> 70
+// by the recording alone.
 template <int G, bool CUT>
 __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
 {
-    // one record per item and step (measured: faster everywhere but in the full pass over
-    // eight groups, where hits are sparse and the prefix ORs cost more than the duplicates)
-    constexpr bool DEDUP = CUT || G <= 4;
-    // positions traded with the node's other chunks after each refill (measured: faster
-    // but for the full pass over eight groups, whose short, load-bound stages the trade's
-    // global round trip would hold back)
-    constexpr bool TRADE = CUT || G <= 4;
     extern __shared__ __align__(128) uint8_t smem[];
     uint32_t* s_ent = (uint32_t*)smem;                                            // [STAGES][SUB]
     // P[v][g] for lane l at word (g / 2) * ROWS * 64 + v * 64 + (g % 2) * 32 + l: a row of
@@ -143,7 +190,7 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
     uint32_t* s_best = s_ent + SL_STAGES * SL_SUB + (sl_static_p(G) ? 0 : sl_p_bytes(G) / 4);   // [32 G]
     uint64_t* bar = (uint64_t*)(s_best + 32 * G);                                 // full, per stage
     uint64_t* ebar = bar + SL_STAGES;                                             // empty, per stage
-    int* s_flags = (int*)(ebar + SL_STAGES);                                      // abort, last, nrec
+    int* s_flags = (int*)(ebar + SL_STAGES);                                      // abort, first stage not issued, done
     uint32_t* s_skip = (uint32_t*)(s_flags + 4);                                  // [G]
 
     const int node = blockIdx.x % A.n;
@@ -151,13 +198,15 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
     const int cnt = (int)A.list_count[node];
     const int g0 = blockIdx.y * 32 * G;
     if (g0 >= cnt) return;                                                        // block-uniform
-    const int64_t e0 = (int64_t)chunk * A.chunk;
-    int64_t e1 = min(e0 + A.chunk, A.S);
-    if (CUT) e1 = min(e1, (int64_t)A.spos[(size_t)node * A.Sp] + 1);              // the empty set's position
-    if (e0 >= e1) return;
+    int64_t end = A.S;
+    if (CUT) end = min(end, (int64_t)A.spos[(size_t)node * A.Sp] + 1);            // the empty set's position
+    const int total = (int)((end + SL_SUB - 1) / SL_SUB);                         // the node's stages
+    const int first = CUT ? chunk * A.per : chunk, stride = CUT ? 1 : A.nchunk;   // this block's
+    if (first >= total) return;
+    const int nsub = CUT ? min(A.per, total - first) : (total - first + stride - 1) / stride;
+    auto stage_base = [&](int it) { return ((int64_t)it * stride + first) * SL_SUB; };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nvalid = min(cnt - g0, 32 * G);
-    const int nsub = (int)((e1 - e0 + SL_SUB - 1) / SL_SUB);
     const bool producer = warp == SL_CWARPS;
     const uint32_t* src = A.sset + (size_t)node * A.Ssp;
     uint64_t pol_stream = 0;
@@ -167,95 +216,71 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
     // (the empty set, in the same stage, is consistent with every item and ranks above
     // them), so no lane needs a bounds test.
     auto issue = [&](int it, int st) {
-        const int64_t base = e0 + (int64_t)it * SL_SUB;
         mbar_arrive_expect_tx(&bar[st], SL_SUB * 4u);
-        bulk_g2s(s_ent + st * SL_SUB, src + base, SL_SUB * 4u, &bar[st], pol_stream);
+        bulk_g2s(s_ent + st * SL_SUB, src + stage_base(it), SL_SUB * 4u, &bar[st], pol_stream);
     };
 
     if (producer) {
-        // Items this block need not test: in the sorted mode those holding a position above
-        // this chunk already (from blocks of earlier chunks).  The producer decides for
-        // every warp, so all skip the same items and the count of items holding a position
-        // stays exact.  Then the first copies go out while the consumers set up.
+        // items that hold a position above this block's first stage already (from blocks that
+        // ran before it) are not tested; then the first copies go out while the consumers
+        // set up
         int pre = 0;
-        if (CUT) {
-            for (int g = 0; g < G; ++g) {
-                const int item = g0 + 32 * g + lane;
-                const bool done = item < cnt && *(volatile const uint32_t*)&A.list_best[(size_t)node * A.cap + item] <
-                                                    (uint32_t)e0;
-                const uint32_t d = __ballot_sync(0xffffffffu, done);
-                if (lane == 0) s_skip[g] = d;
-                pre += __popc(d);
-            }
-        } else if (lane < G) {
-            s_skip[lane] = 0;
+        for (int g = 0; g < G; ++g) {
+            const int item = g0 + 32 * g + lane;
+            const bool done = item < cnt && *(volatile const uint32_t*)&A.list_best[(size_t)node * A.cap + item] <
+                                                (uint32_t)stage_base(0);
+            const uint32_t d = __ballot_sync(0xffffffffu, done);
+            if (lane == 0) s_skip[g] = d;
+            pre += __popc(d);
         }
         if (lane == 0) {
             s_flags[0] = 0;                                                       // abort
             s_flags[1] = 0x7fffffff;                                              // first stage never issued
-            s_flags[2] = pre;                                                     // items holding a position
+            s_flags[2] = CUT && pre == nvalid;                                    // nothing to do
             pol_stream = l2_policy_evict_first();
             for (int s = 0; s < SL_STAGES; ++s) {
                 mbar_init(&bar[s], 1);
                 mbar_init(&ebar[s], SL_CWARPS);
             }
             fence_mbar_init();
-            if (!(CUT && pre == nvalid))
+            if (!s_flags[2])
                 for (int it = 0; it < SL_STAGES && it < nsub; ++it) issue(it, it);
         }
     } else {
-        // the items' predecessor words: warp g builds group g (rows 0..63 from ballots of
-        // the 32 items' masks, row 64 all ones, row 65 zero)
-        if (warp < G) {
-            const int item = g0 + warp * 32 + lane;
-            const uint64_t pc = item < cnt ? A.list_pc[(size_t)node * A.cap + item] : 0ull;
-            for (int v = 0; v < 64; ++v) {
-                const int c = v - (v > node);
-                const bool bit = v < A.n && v != node && ((pc >> c) & 1ull);
-                const uint32_t word = __ballot_sync(0xffffffffu, bit);
-                s_P[Pw(warp, v) + lane] = word;
-            }
-            s_P[Pw(warp, 64) + lane] = 0xffffffffu;
-            s_P[Pw(warp, 65) + lane] = 0u;
+        // the items' predecessor words, the consumer warps spread over (group, node): rows of
+        // the nodes from ballots of the group's masks, row 64 all ones, row 65 zero
+        constexpr int PARTS = SL_CWARPS / G;                                      // warps a group
+        const int g = warp / PARTS, part = warp % PARTS;
+        const int item = g0 + g * 32 + lane;
+        const uint64_t pc = item < cnt ? A.list_pc[(size_t)node * A.cap + item] : 0ull;
+#pragma unroll 4
+        for (int v = part; v < A.n; v += PARTS) {
+            const bool bit = v != node && ((pc >> (v - (v > node))) & 1ull);
+            s_P[Pw(g, v) + lane] = __ballot_sync(0xffffffffu, bit);
+        }
+        if (part == 0) {
+            s_P[Pw(g, 64) + lane] = 0xffffffffu;
+            s_P[Pw(g, 65) + lane] = 0u;
         }
         for (int j = threadIdx.x; j < 32 * G; j += 32 * SL_CWARPS) s_best[j] = SPOS_NONE;
     }
     __syncthreads();
-    if (CUT && s_flags[2] == nvalid) return;                                      // block-uniform; nothing issued
+    if (CUT && s_flags[2]) return;                                      // block-uniform; nothing issued
 
-    if (producer && !TRADE) {
-        // lane 0 alone refills each stage once every consumer has released it
-        if (lane == 0) {
-            int issued = min(SL_STAGES, nsub);
-            for (int it = 0; it + SL_STAGES < nsub; ++it) {
-                const int st = it % SL_STAGES;
-                if (*(volatile int*)&s_flags[0]) break;
-                if (!mbar_wait_bounded(&ebar[st], (uint32_t)((it / SL_STAGES) & 1), WAIT_TIMEOUT_NS)) {
-                    *(volatile int*)&s_flags[0] = 1;
-                    atomicOr(A.status, STATUS_TIMEOUT);
-                    break;
-                }
-                issue(it + SL_STAGES, st);
-                issued = it + SL_STAGES + 1;
-            }
-            // no copy may still be in flight when the block's shared memory goes away
-            for (int j = max(0, issued - SL_STAGES); j < issued; ++j)
-                mbar_wait_bounded(&bar[j % SL_STAGES], (uint32_t)((j / SL_STAGES) & 1), WAIT_TIMEOUT_NS);
-        }
-    } else if (producer) {
+    if (producer) {
         // Lane 0 refills each stage once every consumer has released it.  Then, while the
-        // copy is in flight, the whole warp trades positions with the blocks of the node's
-        // other chunks: it publishes this block's new positions (atomicMin) and marks as
-        // skipped every item that already holds a position above this chunk -- no entry
-        // of the chunk can win for it, so the consumers stop testing it (they still read
-        // every entry).
+        // copy is in flight, the whole warp trades positions with the node's other blocks: it
+        // publishes this block's new positions (atomicMin), marks as skipped every item that
+        // holds a position above the next stage, and (sorted mode) sees whether all of them
+        // hold one above the stage that would be issued next.
         int issued = min(SL_STAGES, nsub);
+        bool all_done = false, settled = false;
         uint32_t pub[G], known[G];         // last published position; items already skipped
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             pub[g] = SPOS_NONE;
-            known[g] = s_skip[g];          // (the sorted mode's items skipped at the start are
-        }                                  // counted already)
+            known[g] = s_skip[g];
+        }
         for (int it = 0; it + SL_STAGES < nsub; ++it) {
             const int st = it % SL_STAGES;
             int go = 1;
@@ -266,9 +291,9 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
                     *(volatile int*)&s_flags[0] = 1;
                     atomicOr(A.status, STATUS_TIMEOUT);
                     go = 0;
-                } else if (CUT && *(volatile int*)&s_flags[2] >= nvalid) {
-                    // every item holds a position: no unread entry can win; release the
-                    // consumers of this buffer's next phase without a copy
+                } else if (CUT && all_done) {
+                    // no unread entry can win; release the consumers of this buffer's next
+                    // phase without a copy
                     *(volatile int*)&s_flags[1] = it + SL_STAGES;
                     mbar_arrive(&bar[st]);
                     issued = it + SL_STAGES + 1;
@@ -279,6 +304,7 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
                 }
             }
             if (!__shfl_sync(0xffffffffu, go, 0)) break;
+            if (settled) continue;         // (a trade's round trip would outlast a stage's copy)
             // every load first (one round trip for all groups), then the updates
             uint32_t mine[G], other[G];
 #pragma unroll
@@ -288,6 +314,8 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
                 mine[g] = live ? *(volatile const uint32_t*)&s_best[g * 32 + lane] : SPOS_NONE;
                 other[g] = live ? *(volatile const uint32_t*)&A.list_best[(size_t)node * A.cap + item] : SPOS_NONE;
             }
+            const uint32_t next = (uint32_t)stage_base(it + 1), after = (uint32_t)stage_base(it + 1 + SL_STAGES);
+            bool open = false;             // an item that the stage to be issued next may serve
 #pragma unroll
             for (int g = 0; g < G; ++g) {
                 const int item = g0 + 32 * g + lane;
@@ -295,12 +323,18 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
                     atomicMin(&A.list_best[(size_t)node * A.cap + item], mine[g]);
                     pub[g] = mine[g];
                 }
-                const bool sk = other[g] < (uint32_t)e0;
-                // in the sorted mode the item now holds a position (for the stop)
-                if (CUT && sk && atomicMin(&s_best[g * 32 + lane], other[g]) == SPOS_NONE) atomicAdd(&s_flags[2], 1);
-                const uint32_t bits = __ballot_sync(0xffffffffu, sk);
+                const uint32_t pos = min(mine[g], other[g]);
+                open |= item < cnt && !((known[g] >> lane) & 1u) && pos >= after;
+                const uint32_t bits = __ballot_sync(0xffffffffu, pos < next);
                 known[g] |= bits;
                 if (lane == 0 && bits) *(volatile uint32_t*)&s_skip[g] |= bits;
+            }
+            all_done = !__any_sync(0xffffffffu, open);
+            settled = true;
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                const int nv = min(max(cnt - g0 - 32 * g, 0), 32);
+                settled &= (known[g] | (nv >= 32 ? 0u : 0xffffffffu << nv)) == 0xffffffffu;
             }
         }
         if (lane == 0) {
@@ -330,12 +364,12 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
                 break;
             }
             if (CUT && it >= __shfl_sync(0xffffffffu, *(volatile int*)&s_flags[1], 0)) break;
-            const int64_t base = e0 + (int64_t)it * SL_SUB + warp * SL_PER_WARP;
+            const int64_t base = stage_base(it) + warp * SL_PER_WARP;
             const uint4* E4 = (const uint4*)(s_ent + st * SL_SUB + warp * SL_PER_WARP);
             uint32_t all_found = 0xffffffffu;
 #pragma unroll
             for (int g = 0; g < G; ++g) {
-                if constexpr (TRADE) found[g] |= *(volatile const uint32_t*)&s_skip[g];
+                found[g] |= *(volatile const uint32_t*)&s_skip[g];
                 all_found &= found[g];
             }
             if (all_found != 0xffffffffu) {
@@ -366,61 +400,15 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
 #pragma unroll
                     for (int g = 0; g < G; ++g) any |= raw[g] & ~found[g];
                     if (__any_sync(0xffffffffu, any != 0)) {
-                        const uint32_t pos0 = (uint32_t)(base + q * 128 + 4 * lane);
-                        if constexpr (DEDUP) {
-                            // rare: record the step's new items.  Positions run lane-major
-                            // (lane l holds pos0 .. pos0 + 3), so of the lanes hitting an
-                            // item only the lowest records it (an exclusive prefix OR over
-                            // the lanes), at its first entry that hits: one atomicMin per
-                            // item and step, however densely the top of a node's list
-                            // matches the orders
+                        // rare past the top of a list, where one entry matches many orders
+                        const uint32_t pos0 = (uint32_t)(base + q * 128);
 #pragma unroll
-                            for (int g = 0; g < G; ++g) {
-                                const uint32_t hit = raw[g] & ~found[g];
-                                uint32_t incl = hit;
-#pragma unroll
-                                for (int d = 1; d < 32; d <<= 1) {
-                                    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
-                                    if (lane >= d) incl |= y;
-                                }
-                                const uint32_t before = __shfl_up_sync(0xffffffffu, incl, 1);   // lanes below
-                                uint32_t mine = lane == 0 ? hit : hit & ~before;
-#pragma unroll
-                                for (int u = 0; u < 4; ++u) {
-                                    if (!mine) break;
-                                    uint32_t m = word(w[u], 0x5504, g) & word(w[u], 0x5514, g) &
-                                                 word(w[u], 0x5524, g) & word(w[u], 0x5534, g) & mine;
-                                    mine &= ~m;
-                                    while (m) {
-                                        const int b = __ffs(m) - 1;
-                                        m &= m - 1;
-                                        const uint32_t old = atomicMin(&s_best[g * 32 + b], pos0 + u);
-                                        if (CUT && old == SPOS_NONE) atomicAdd(&s_flags[2], 1);
-                                    }
-                                }
-                                found[g] |= __shfl_sync(0xffffffffu, incl, 31);
-                            }
-                        } else {
-                            // every lane records its own new items (duplicates of one step
-                            // lose the atomicMin); cheaper where hits are sparse
-#pragma unroll
-                            for (int g = 0; g < G; ++g) {
-                                const uint32_t hit = raw[g] & ~found[g];
-                                if (hit) {
-#pragma unroll
-                                    for (int u = 0; u < 4; ++u) {
-                                        uint32_t m = word(w[u], 0x5504, g) & word(w[u], 0x5514, g) &
-                                                     word(w[u], 0x5524, g) & word(w[u], 0x5534, g) & hit;
-                                        while (m) {
-                                            const int b = __ffs(m) - 1;
-                                            m &= m - 1;
-                                            const uint32_t old = atomicMin(&s_best[g * 32 + b], pos0 + u);
-                                            if (CUT && old == SPOS_NONE) atomicAdd(&s_flags[2], 1);
-                                        }
-                                    }
-                                }
-                                found[g] |= __reduce_or_sync(0xffffffffu, hit);
-                            }
+                        for (int g = 0; g < G; ++g) {
+                            const uint32_t hit = raw[g] & ~found[g];
+                            const uint32_t items = __reduce_or_sync(0xffffffffu, hit);
+                            if (!items) continue;                                 // warp-uniform
+                            found[g] |= items;
+                            record_items(hit, items, w4, Pb + 4 * Pw(g, 0), &s_best[g * 32], pos0, lane);
                         }
                     }
                 }
@@ -439,8 +427,8 @@ __global__ void __launch_bounds__(SL_THREADS) k_scan_sliced(SlicedArgs A)
 
 // Launch shape: as many blocks as are resident at once (the occupancy calculator: threads,
 // registers and shared memory), one wave of long blocks, so each block's set-up is paid
-// once; the sorted mode spreads its chunks (at least four stages each) over the nodes'
-// live ranges [0, cut), and the blocks past a node's cut leave at once.
+// once; the sorted mode counts on at least four stages a block over the nodes' live ranges
+// [0, cut), and the blocks past a node's live stages leave at once.
 template <int G, bool CUT>
 static int sliced_launch(const bn_table* t, const uint32_t* list_count, const uint64_t* list_pc,
                          uint32_t* list_best, int cap, int sets, uint32_t* status, cudaStream_t s)
@@ -457,22 +445,22 @@ static int sliced_launch(const bn_table* t, const uint32_t* list_count, const ui
     }
     const int per_sm = (d >= 0 && d < 64 && resident[d] > 0) ? resident[d] : 1;
     const int64_t want = (int64_t)sm_count() * per_sm;
-    int64_t chunk, nchunk;
+    int64_t nchunk, per = 0;
     if (!CUT) {
         nchunk = std::max<int64_t>(1, want / ((int64_t)t->n * sets));
-        chunk = round_up((t->S + nchunk - 1) / nchunk, SL_SUB);
-        nchunk = (t->S + chunk - 1) / chunk;
+        nchunk = std::min<int64_t>(nchunk, (t->S + SL_SUB - 1) / SL_SUB);
     } else {
         int64_t live = 0, longest = 0;
         for (int i = 0; i < t->n; ++i) {
             live += t->cut[i];
             longest = std::max<int64_t>(longest, t->cut[i]);
         }
-        chunk = std::max<int64_t>(4 * SL_SUB, round_up((live * sets + want - 1) / want, SL_SUB));
+        const int64_t chunk = std::max<int64_t>(4 * SL_SUB, round_up((live * sets + want - 1) / want, SL_SUB));
         nchunk = (longest + chunk - 1) / chunk;
+        per = chunk / SL_SUB;
     }
-    SlicedArgs A{t->sset, t->spos, t->Sp, t->S, t->sset_stride, t->n, chunk, (int)nchunk, list_count, list_pc,
-                 list_best, cap, status};
+    SlicedArgs A{t->sset, t->spos, t->Sp, t->S, t->sset_stride, t->n, (int)nchunk, (int)per, list_count,
+                 list_pc, list_best, cap, status};
     dim3 grid((unsigned)(nchunk * t->n), (unsigned)sets);
     k_scan_sliced<G, CUT><<<grid, SL_THREADS, sl_smem(G), s>>>(A);
     BN_LAUNCH_CHECK("k_scan_sliced");
