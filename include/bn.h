@@ -174,8 +174,11 @@ int bn_score_orders_noalloc(const bn_table* t, const uint8_t* orders, int B,
 
 /* Scan mode of a table (used by bn_score_orders, bn_score_orders_noalloc and samplers
  * whose next step is captured after the change):
- *   BN_SCAN_FULL    every entry of a node's table is tested against every order (the
- *                   default; Eq. (6) taken literally)
+ *   BN_SCAN_FULL    every entry of a node's table is read and competes for every order
+ *                   (the default; Eq. (6) taken literally).  With k <= 4 and thousands of
+ *                   sets a node, batches and samplers are scanned bit-sliced as in
+ *                   BN_SCAN_SLICED; smaller tables, up to three orders and k > 4 by mask
+ *                   tests
  *   BN_SCAN_PRUNED  only entries that no proper subset of their parent set matches or
  *                   beats are tested.  A dominated entry can never be chosen: whenever
  *                   its set lies in a node's predecessors so does the subset, which has
@@ -211,14 +214,14 @@ int bn_table_set_scan(bn_table* t, int mode, void* stream);
 /* surviving entries per node after pruning (n int64) */
 int bn_table_pruned(const bn_table* t, int64_t* survivors_per_node);
 
-/* Autotuner of the full-table scan: times every (shared-memory stage size in
+/* Autotuner of the mask-test scan: times every (shared-memory stage size in
  * {512, 1024, 2048} entries) x (blocks per SM target in {1, 2, 4, 8, 16}) tiling on this
  * table with synthetic work lists of max_items (node, order) items per node, and keeps
  * the fastest for later scans of up to that many items (per 256-item group, up to 2048).
- * It also runs by itself: the first bn_score_orders call that takes the full-table scan
- * and the first bn_chains_create on a table not in BN_SCAN_PRUNED mode tune the tiling
- * for their number of 256-item groups (tens of milliseconds once per table and group
- * count; BN_AUTOTUNE=0 in the environment keeps the fixed tiling).  Results do not depend
+ * It also runs by itself where the mask-test scan serves large batches (k > 4, or
+ * BN_SCAN_UNRANK): the first bn_score_orders call and the first bn_chains_create on such a
+ * table tune the tiling for their number of 256-item groups (tens of milliseconds once per
+ * table and group count; BN_AUTOTUNE=0 in the environment keeps the fixed tiling).  Results do not depend
  * on the tiling.
  * chosen (3 int64, may be NULL): stage size, blocks per node, microseconds per launch.
  * The table's scan mode is unchanged.  Errors: BN_EINVAL, BN_EUNSUPPORTED, BN_ECUDA. */

@@ -78,7 +78,6 @@ extern "C" int bn_score_orders_noalloc(const bn_table* t, const uint8_t* orders,
                          "bn_score_orders_noalloc: B=%d orders of n=%d nodes need %zu bytes of scratch; the "
                          "static scratch holds %zu (at most %zu orders at this n)",
                          B, n, need, NOALLOC_SCRATCH_BYTES, (NOALLOC_SCRATCH_BYTES - 1024 - 4 * (size_t)n) / (12 * (size_t)n));
-    const ScanPlan pl = plan_scan(t, B);
 
     void* base = nullptr;
     int rc = noalloc_scratch(&base);
@@ -93,8 +92,7 @@ extern "C" int bn_score_orders_noalloc(const bn_table* t, const uint8_t* orders,
     // counts, masks and per-item results are rewritten by k_pred_lists before use
     BN_CUDA(cudaMemsetAsync(d_status, 0, sizeof(uint32_t), s));
     if ((rc = launch_pred_lists(orders, B, n, d_pc, d_best, d_cnt, d_status, s))) return rc;
-    rc = scan_nodes_fits(t, B) ? launch_scan_nodes(t, B, d_pc, d_best, d_status, s)
-                               : launch_scan(t, pl, d_cnt, d_pc, d_best, B, d_status, s);
+    rc = launch_scan_orders(t, B, d_cnt, d_pc, d_best, d_status, s);
     if (rc) return rc;
     if ((rc = launch_reduce_orders(t, d_best, B, best_rank, order_score, s))) return rc;
     uint32_t st = 0;

@@ -345,12 +345,9 @@ static int scan_variant(const ScanArgs& A, dim3 grid, cudaStream_t s)
     return BN_OK;
 }
 
-int launch_scan(const bn_table* t, const ScanPlan& pl, const uint32_t* list_count, const uint64_t* list_pc,
-                uint32_t* list_best, int cap, uint32_t* status, cudaStream_t s)
+static int launch_scan_masks(const bn_table* t, const ScanPlan& pl, const uint32_t* list_count, const uint64_t* list_pc,
+                             uint32_t* list_best, int cap, uint32_t* status, cudaStream_t s)
 {
-    if (t->scan_mode == BN_SCAN_PRUNED) return launch_scan_pruned(t, list_count, list_pc, list_best, cap, s);
-    if (t->scan_mode == BN_SCAN_SLICED || t->scan_mode == BN_SCAN_SORTED)
-        return launch_scan_sliced(t, list_count, list_pc, list_best, cap, t->scan_mode == BN_SCAN_SORTED, status, s);
     ScanArgs A;
     A.spos = t->spos;
     A.pst = t->pst;
@@ -370,6 +367,25 @@ int launch_scan(const bn_table* t, const ScanPlan& pl, const uint32_t* list_coun
     if (pl.sub >= 2048) return unrank ? scan_variant<2048, true>(A, grid, s) : scan_variant<2048, false>(A, grid, s);
     if (pl.sub >= 1024) return unrank ? scan_variant<1024, true>(A, grid, s) : scan_variant<1024, false>(A, grid, s);
     return unrank ? scan_variant<512, true>(A, grid, s) : scan_variant<512, false>(A, grid, s);
+}
+
+// Whether work lists of a fully scanned table go to the bit-sliced full pass: it reads the
+// same 4 bytes an entry and tests 32 items at once, but records hits and trades positions,
+// which a table of one or two stages (2,048 entries) a node does not pay back.  Measured, us
+// per sampler step (mask tests / bit-sliced): 10 nodes (256 sets a node) 22 / 32 for 512
+// chains, 20 nodes (5,036) 29 / 33, 30 nodes (27,841) 78 / 40, 60 nodes (489,406) 1,210 /
+// 107 and for one chain 38 / 31.
+static constexpr int64_t SLICED_LIST_SETS = 8192;
+
+int launch_scan(const bn_table* t, const ScanPlan& pl, const uint32_t* list_count, const uint64_t* list_pc,
+                uint32_t* list_best, int cap, uint32_t* status, cudaStream_t s)
+{
+    if (t->scan_mode == BN_SCAN_PRUNED) return launch_scan_pruned(t, list_count, list_pc, list_best, cap, s);
+    if (t->scan_mode == BN_SCAN_SLICED || t->scan_mode == BN_SCAN_SORTED)
+        return launch_scan_sliced(t, list_count, list_pc, list_best, cap, t->scan_mode == BN_SCAN_SORTED, status, s);
+    if (t->scan_mode == BN_SCAN_FULL && t->sset && t->S >= SLICED_LIST_SETS)
+        return launch_scan_sliced(t, list_count, list_pc, list_best, cap, false, status, s);
+    return launch_scan_masks(t, pl, list_count, list_pc, list_best, cap, status, s);
 }
 
 // ---------------------------------------------------------------------------------
@@ -499,9 +515,13 @@ struct NsShape {
     int T, R, threads;
 };
 
-static NsShape ns_shape(int n, int B)
+static bool few_slices(int64_t Sp) { return Sp / NS_SUB < sm_count(); }
+
+static NsShape ns_shape(int n, int B, int64_t Sp)
 {
-    const int BG = (B + NS_RMAX - 1) / NS_RMAX;
+    // as few groups as possible (each staged entry read least); on a table with fewer slices
+    // than SMs one order a thread: there a thread's chain of tests is what the scan takes
+    const int BG = few_slices(Sp) ? B : (B + NS_RMAX - 1) / NS_RMAX;
     const int R = (B + BG - 1) / BG;
     const int items = n * BG;
     int T = 1;
@@ -509,9 +529,22 @@ static NsShape ns_shape(int n, int B)
     return {T, R, items * T <= 256 ? 256 : (int)round_up(items, 32)};
 }
 
-bool scan_nodes_fits(const bn_table* t, int B)
+// (13 nodes, 794 sets: 256 orders 20 us at eight a thread, 11 us by k_scan)
+static bool scan_nodes_fits(const bn_table* t, int B)
 {
-    return t->scan_mode == BN_SCAN_FULL && B >= 1 && (int64_t)t->n * ((B + NS_RMAX - 1) / NS_RMAX) <= NS_MAX_ITEMS;
+    const int64_t groups = few_slices(t->Sp) ? B : (B + NS_RMAX - 1) / NS_RMAX;
+    return t->scan_mode == BN_SCAN_FULL && B >= 1 && t->n * groups <= NS_MAX_ITEMS;
+}
+
+// Whether B orders of a fully scanned table go to the bit-sliced full pass (k <= 4).  Up to
+// three orders the node scan is at least as fast (60 nodes: 19, 21, 25 us against 24), then its
+// tests grow with the orders (4: 31, 8: 53, 32: 183 us against 24 - 25); tables of a few
+// stages a node need many orders to pay for the recorded hits (20 nodes, 5,036 sets: 256
+// orders 13 us by masks and 23 bit-sliced, 777: 23 and 22, 2,048: 48 and 27; 13 nodes, 794
+// sets: mask tests throughout).
+static bool orders_sliced(const bn_table* t, int B)
+{
+    return t->scan_mode == BN_SCAN_FULL && t->sset && ((B >= 4 && t->S >= 8192) || (B >= 512 && t->S >= 4096));
 }
 
 template <int T, int R>
@@ -532,7 +565,7 @@ static void ns_table_row(NsLaunchFn* l, NsKernelFn* k)
     k[4] = k_scan_nodes<T, 5>; k[5] = k_scan_nodes<T, 6>; k[6] = k_scan_nodes<T, 7>; k[7] = k_scan_nodes<T, 8>;
 }
 
-int launch_scan_nodes(const bn_table* t, int B, const uint64_t* list_pc, uint32_t* list_best, uint32_t* status,
+static int launch_scan_nodes(const bn_table* t, int B, const uint64_t* list_pc, uint32_t* list_best, uint32_t* status,
                       cudaStream_t s)
 {
     static_assert(NS_RMAX == 8, "one table row per T holds R = 1..8");
@@ -552,7 +585,7 @@ int launch_scan_nodes(const bn_table* t, int B, const uint64_t* list_pc, uint32_
             for (int r = 0; r < NS_RMAX; ++r)
                 BN_CUDA(cudaFuncSetAttribute(kern[a][r], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)ns_smem(MAXN)));
-    const NsShape sh = ns_shape(t->n, B);
+    const NsShape sh = ns_shape(t->n, B, t->Sp);
     // whole waves: as many blocks per SM as its 2,048 threads and shared memory hold (at
     // most four)
     const int per_sm = (int)std::max<size_t>(
@@ -565,6 +598,14 @@ int launch_scan_nodes(const bn_table* t, int B, const uint64_t* list_pc, uint32_
     launch[a][sh.R - 1](grid, sh.threads, smem, s, A);
     BN_LAUNCH_CHECK("k_scan_nodes");
     return BN_OK;
+}
+
+int launch_scan_orders(const bn_table* t, int B, const uint32_t* list_count, const uint64_t* list_pc,
+                       uint32_t* list_best, uint32_t* status, cudaStream_t s)
+{
+    if (orders_sliced(t, B)) return launch_scan_sliced(t, list_count, list_pc, list_best, B, false, status, s);
+    if (scan_nodes_fits(t, B)) return launch_scan_nodes(t, B, list_pc, list_best, status, s);
+    return launch_scan(t, plan_scan(t, B), list_count, list_pc, list_best, B, status, s);
 }
 
 // synthetic work lists for tuning: every node holds `items` items with pseudo-random
@@ -646,13 +687,16 @@ __global__ void k_reduce_orders(const uint32_t* __restrict__ list_best, const ui
     }
 }
 
-// the full-table scan's tiling for up to max_items items per node, tuned on first use: the
-// first scan with a new number of 256-item groups (<= 8) times every tiling the autotuner
+// the mask-test scan's tiling for up to max_items items per node, tuned on first use (k > 4
+// or the unranking mode; with k <= 4 only tables below SLICED_LIST_SETS reach it, on the
+// fixed plan): the first scan with a new number of 256-item groups (<= 8) times every tiling the autotuner
 // knows on this table (tens of milliseconds once) and keeps the fastest.  BN_AUTOTUNE=0 in
 // the environment keeps the fixed plan.
 int ensure_tuned(const bn_table* t, int max_items, cudaStream_t s)
 {
     if (!t || (t->scan_mode != BN_SCAN_FULL && t->scan_mode != BN_SCAN_UNRANK) || max_items < 1) return BN_OK;
+    // bit-sliced, or too small a table to matter
+    if (t->scan_mode == BN_SCAN_FULL && (t->sset || few_slices(t->Sp))) return BN_OK;
     const int groups = (max_items + SCAN_THREADS - 1) / SCAN_THREADS;
     if (groups > 8 || t->tuned_sub[groups]) return BN_OK;
     static const bool off = [] {
@@ -737,7 +781,6 @@ static int score_orders_impl(const bn_table* t, const uint8_t* orders, int B, ui
         int rt = ensure_tuned(t, B, s);
         if (rt) return rt;
     }
-    const ScanPlan pl = plan_scan(t, B);
     keep_pool_mapped();
 
     // one scratch block: orders | list_pc | list_best | counts | status | ranks | scores
@@ -780,8 +823,7 @@ static int score_orders_impl(const bn_table* t, const uint8_t* orders, int B, ui
     int rc = launch_pred_lists(d_orders, B, n, d_pc, d_best, d_cnt, d_st, s);
     if (rc) return rc;
     if (ev0) BN_CUDA(cudaEventRecord(ev0, s));
-    rc = scan_nodes_fits(t, B) ? launch_scan_nodes(t, B, d_pc, d_best, d_st, s)
-                               : launch_scan(t, pl, d_cnt, d_pc, d_best, B, d_st, s);
+    rc = launch_scan_orders(t, B, d_cnt, d_pc, d_best, d_st, s);
     if (rc) return rc;
     if (ev1) BN_CUDA(cudaEventRecord(ev1, s));
     if ((rc = launch_reduce_orders(t, d_best, B, d_rank, d_score, s))) return rc;
@@ -911,7 +953,7 @@ extern "C" int bn_table_autotune(bn_table* t, int max_items, void* stream, int64
                 if (cudaGetLastError() != cudaSuccess) { rc = set_error(BN_ECUDA, "k_tune_lists"); break; }
                 count_launches(1);
                 if (cudaEventRecord(e0, s) != cudaSuccess) { rc = set_error(BN_ECUDA, "event"); break; }
-                rc = launch_scan(t, pl, cnt, pc, best, items, st, s);
+                rc = launch_scan_masks(t, pl, cnt, pc, best, items, st, s);
                 if (rc) break;
                 if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess) {
                     rc = set_error(BN_ECUDA, "event sync");

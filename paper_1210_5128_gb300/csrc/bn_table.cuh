@@ -107,12 +107,10 @@ int launch_scan(const bn_table* t, const ScanPlan& pl, const uint32_t* list_coun
                 const uint64_t* list_pc, uint32_t* list_best, int cap, uint32_t* status,
                 cudaStream_t s);
 
-// The same for B orders of every node when n * ceil(B / 8) <= 1,024 and the table is
-// scanned in full (scan_nodes_fits): one pass over the rank range for all nodes and
-// orders, up to eight orders a thread (list layout [n][B]).
-bool scan_nodes_fits(const bn_table* t, int B);
-int launch_scan_nodes(const bn_table* t, int B, const uint64_t* list_pc, uint32_t* list_best, uint32_t* status,
-                      cudaStream_t s);
+// The same for B orders of every node (list layout [n][B]), by the scan that suits the
+// table, its mode and B.
+int launch_scan_orders(const bn_table* t, int B, const uint32_t* list_count, const uint64_t* list_pc,
+                       uint32_t* list_best, uint32_t* status, cudaStream_t s);
 
 // Candidate-space predecessor masks of B orders written as node-major work lists:
 // list_pc[i * B + b] (item b of node i is order b), list_best[i * B + b] = SPOS_NONE,
