@@ -29,23 +29,36 @@
 
 namespace bn {
 
-// initial orders: Fisher-Yates from the identity driven by the Philox init stream
-__global__ void k_init_orders(ChainState S)
+// initial orders: Fisher-Yates from the identity driven by the Philox init stream.  A warp
+// per chain: the lanes draw the blocks (four positions each) side by side, one lane swaps
+// in shared memory.
+__global__ void __launch_bounds__(256) k_init_orders(ChainState S)
 {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ uint8_t s_o[8][MAXN], s_j[8][MAXN];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c = blockIdx.x * 8 + warp;
     if (c >= S.C) return;
-    uint8_t o[MAXN];
-    for (int p = 0; p < S.n; ++p) o[p] = (uint8_t)p;
-    U64x4 buf;
-    int used = 4;
-    uint64_t blk = 0;
-    for (int i = S.n - 1; i >= 1; --i) {
-        if (used == 4) { buf = philox4x64(blk++, (uint64_t)c, 1, 0, S.seed, 0); used = 0; }
-        uint64_t x = buf.x[used++];
-        int j = (int)mulhi64(x, (uint64_t)(i + 1));
-        uint8_t tmp = o[i]; o[i] = o[j]; o[j] = tmp;
+    const int n = S.n;
+    for (int p = lane; p < n; p += 32) s_o[warp][p] = (uint8_t)p;
+    // word q of the stream serves position i = n - 1 - q
+    if (4 * lane < n - 1) {
+        const U64x4 x = philox4x64((uint64_t)lane, (uint64_t)c, 1, 0, S.seed, 0);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const int i = n - 1 - (4 * lane + w);
+            if (i >= 1) s_j[warp][i] = (uint8_t)mulhi64(x.x[w], (uint64_t)(i + 1));
+        }
     }
-    for (int p = 0; p < S.n; ++p) S.cur_order[(size_t)c * S.n + p] = o[p];
+    __syncwarp();
+    if (lane == 0)
+        for (int i = n - 1; i >= 1; --i) {
+            const int j = s_j[warp][i];
+            const uint8_t t = s_o[warp][i];
+            s_o[warp][i] = s_o[warp][j];
+            s_o[warp][j] = t;
+        }
+    __syncwarp();
+    for (int p = lane; p < n; p += 32) S.cur_order[(size_t)c * n + p] = s_o[warp][p];
 }
 
 // scan result of one (node, item): the chosen rank and its entry's key
@@ -56,30 +69,40 @@ __device__ __forceinline__ void item_result(const ChainState& S, int i, uint32_t
     bk = S.keys[(size_t)i * S.Sp + br];
 }
 
-// full scoring of the initial orders (items of node i are chains 0..C-1)
-__global__ void k_init_state(ChainState S)
+// full scoring of the initial orders (items of node i are chains 0..C-1): a block takes 32
+// chains, its threads gather (node, chain) pairs side by side, then one thread a chain adds
+// its entries
+static constexpr int IS_CHAINS = 32;
+__global__ void __launch_bounds__(256) k_init_state(ChainState S)
 {
-    __shared__ int64_t s_key[8][MAXN];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int c = blockIdx.x * 8 + warp;
-    if (c >= S.C) return;
-    for (int i = lane; i < S.n; i += 32) {
+    __shared__ int64_t s_key[MAXN][IS_CHAINS + 1];
+    __shared__ uint32_t s_rank[IS_CHAINS][MAXN + 1];
+    const int n = S.n, c0 = blockIdx.x * IS_CHAINS, nc = min(IS_CHAINS, S.C - c0);
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < n * nc; idx += 256) {
+        const int i = idx / nc, q = idx - i * nc;
         int64_t bk;
         uint32_t br;
-        item_result(S, i, S.list_best[(size_t)i * S.C + c], bk, br);
-        s_key[warp][i] = bk;
-        S.cur_key[(size_t)c * S.n + i] = bk;
-        S.cur_rank[(size_t)c * S.n + i] = br;
-        S.best_rank[(size_t)c * S.n + i] = br;
+        item_result(S, i, S.list_best[(size_t)i * S.C + c0 + q], bk, br);
+        s_key[i][q] = bk;
+        s_rank[q][i] = br;
     }
-    for (int p = lane; p < S.n; p += 32) S.best_order[(size_t)c * S.n + p] = S.cur_order[(size_t)c * S.n + p];
-    __syncwarp();
-    if (lane == 0) {
+    __syncthreads();
+    if ((int)threadIdx.x < nc) {
+        const int c = c0 + threadIdx.x;
         double sum = 0.0;
-        for (int i = 0; i < S.n; ++i) sum = __dadd_rn(sum, key_to_double(s_key[warp][i]));
+        for (int i = 0; i < n; ++i) sum = __dadd_rn(sum, key_to_double(s_key[i][threadIdx.x]));
         S.cur_score[c] = sum;
         S.best_score[c] = sum;
         S.accepts[c] = 0;
+    }
+    for (int idx = threadIdx.x; idx < n * nc; idx += 256) {
+        const int q = idx / n, i = idx - q * n;
+        const size_t at = (size_t)c0 * n + idx;
+        S.cur_key[at] = s_key[i][q];
+        S.cur_rank[at] = s_rank[q][i];
+        S.best_rank[at] = s_rank[q][i];
+        S.best_order[at] = S.cur_order[at];
     }
 }
 
@@ -149,9 +172,10 @@ __global__ void k_propose(ChainState S)
 // step 3: combine, MH test, bookkeeping; the last block advances the step counter
 __global__ void k_accept(ChainState S)
 {
-    __shared__ int64_t s_key[8][MAXN];
+    __shared__ int64_t s_key[8][MAXN + 1];
     __shared__ uint32_t s_rank[8][MAXN];
     __shared__ int s_acc[8];
+    __shared__ double s_lu[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = blockIdx.x * 8 + warp;
     const int n = S.n;
@@ -159,50 +183,74 @@ __global__ void k_accept(ChainState S)
     if (c < S.C) {
         const int a = S.prop_ab[2 * c], b = S.prop_ab[2 * c + 1];
         const uint8_t* po = S.prop_order + (size_t)c * n;
+        // both of a lane's positions together, the chain of dependent loads (slot, scan
+        // result, rank, key) once; the current entries and the logarithm in its shadow
         bool moved = false;
-        for (int p = lane; p < n; p += 32) {
-            const int v = po[p];
-            int64_t bk;
-            uint32_t br;
-            if (p >= a && p <= b) {
-                const uint32_t slot = S.slot_of[(size_t)c * n + v];
-                item_result(S, v, S.list_best[(size_t)v * S.C + slot], bk, br);
-                moved |= br != S.cur_rank[(size_t)c * n + v];
-            } else {
-                bk = S.cur_key[(size_t)c * n + v];
-                br = S.cur_rank[(size_t)c * n + v];
+        int v[2];
+        bool act[2], in[2];
+        uint32_t slot[2], cr[2];
+        int64_t ck[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int p = lane + 32 * h;
+            act[h] = p < n;
+            in[h] = act[h] && p >= a && p <= b;
+            v[h] = act[h] ? po[p] : 0;
+            slot[h] = in[h] ? S.slot_of[(size_t)c * n + v[h]] : 0u;
+            cr[h] = act[h] ? S.cur_rank[(size_t)c * n + v[h]] : 0u;
+            ck[h] = act[h] && !in[h] ? S.cur_key[(size_t)c * n + v[h]] : 0;
+        }
+        if (lane == 0) s_lu[warp] = log(S.prop_u[c]);
+        uint32_t bp[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) bp[h] = in[h] ? S.list_best[(size_t)v[h] * S.C + slot[h]] : 0u;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            int64_t bk = ck[h];
+            uint32_t br = cr[h];
+            if (in[h]) {
+                item_result(S, v[h], bp[h], bk, br);
+                moved |= br != cr[h];
             }
-            s_key[warp][v] = bk;
-            s_rank[warp][v] = br;
+            if (act[h]) {
+                s_key[warp][v[h]] = bk;
+                s_rank[warp][v[h]] = br;
+            }
         }
         moved = __any_sync(0xffffffffu, moved);
         if (S.changed && lane == 0) S.changed[c] = moved ? 1 : 0;
-        __syncwarp();
-        if (lane == 0) {
-            double s2 = 0.0;
-            for (int i = 0; i < n; ++i) s2 = __dadd_rn(s2, key_to_double(s_key[warp][i]));
-            const double s1 = S.cur_score[c];
-            const double delta = __dsub_rn(s2, s1);
-            const double lu = log(S.prop_u[c]);
-            // learned proposal: ln q(pair | proposed) - ln q(pair | current)
-            const double corr = S.mode == BN_PROPOSAL_LEARNED
-                                    ? (double)S.prop_lq[(size_t)c * S.P + S.prop_pair[c]] - (double)S.prop_lqf[c]
-                                    : 0.0;
-            const bool acc = S.literal_log ? (lu < __dadd_rn(delta, corr))
-                                           : (lu < __dadd_rn(__dmul_rn(LN10, delta), corr));
-            if (S.delta) S.delta[c] = (float)delta;
-            s_acc[warp] = acc ? 1 : 0;
-            if (acc) {
-                S.cur_score[c] = s2;
-                S.accepts[c] += 1;
-                if (s2 > S.best_score[c]) { S.best_score[c] = s2; s_acc[warp] = 2; }
-            }
-            if (t < S.trace_cap) {
-                S.trace_score[(size_t)c * S.trace_cap + t] = acc ? s2 : s1;
-                S.trace_accept[(size_t)c * S.trace_cap + t] = acc ? 1 : 0;
-            }
+    }
+    __syncthreads();
+    // the sums of the block's eight chains on eight lanes of one warp: an FP64 instruction
+    // holds the pipe for the whole warp whatever lanes are on
+    if (threadIdx.x < 8 && blockIdx.x * 8 + (int)threadIdx.x < S.C) {
+        const int q = threadIdx.x, cq = blockIdx.x * 8 + q;
+        const double lu = s_lu[q];
+        double s2 = 0.0;
+        for (int i = 0; i < n; ++i) s2 = __dadd_rn(s2, key_to_double(s_key[q][i]));
+        const double s1 = S.cur_score[cq];
+        const double delta = __dsub_rn(s2, s1);
+        // learned proposal: ln q(pair | proposed) - ln q(pair | current)
+        const double corr = S.mode == BN_PROPOSAL_LEARNED
+                                ? (double)S.prop_lq[(size_t)cq * S.P + S.prop_pair[cq]] - (double)S.prop_lqf[cq]
+                                : 0.0;
+        const bool acc = S.literal_log ? (lu < __dadd_rn(delta, corr))
+                                       : (lu < __dadd_rn(__dmul_rn(LN10, delta), corr));
+        if (S.delta) S.delta[cq] = (float)delta;
+        s_acc[q] = acc ? 1 : 0;
+        if (acc) {
+            S.cur_score[cq] = s2;
+            S.accepts[cq] += 1;
+            if (s2 > S.best_score[cq]) { S.best_score[cq] = s2; s_acc[q] = 2; }
         }
-        __syncwarp();
+        if (t < S.trace_cap) {
+            S.trace_score[(size_t)cq * S.trace_cap + t] = acc ? s2 : s1;
+            S.trace_accept[(size_t)cq * S.trace_cap + t] = acc ? 1 : 0;
+        }
+    }
+    __syncthreads();
+    if (c < S.C) {
+        const uint8_t* po = S.prop_order + (size_t)c * n;
         const int acc = s_acc[warp];
         if (acc && S.mode == BN_PROPOSAL_LEARNED) {
             for (int j = lane; j < S.P; j += 32) S.cur_lq[(size_t)c * S.P + j] = S.prop_lq[(size_t)c * S.P + j];
@@ -231,7 +279,7 @@ __global__ void k_accept(ChainState S)
                     const int slot = __ffsll((long long)m) - 1;
                     m &= m - 1;
                     const int par = slot + (slot >= i ? 1 : 0);
-                    E[par] += 1u;
+                    atomicAdd(&E[par], 1u);          // no read-back: nothing waits for it
                     if (rec) {
                         S.rec_bits[(((size_t)c * n + i) * n + par) * S.rec_words + (ridx >> 6)] |= 1ull << (ridx & 63);
                     }
@@ -240,16 +288,21 @@ __global__ void k_accept(ChainState S)
         }
     }
     // the last block to finish advances the step and clears the work lists
+    __shared__ int s_last;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const uint32_t ticket = atomicAdd(S.done, 1u);
-        if (ticket == gridDim.x - 1) {
-            int64_t items = 0;
-            for (int i = 0; i < n; ++i) {
-                items += S.list_count[i];
-                S.list_count[i] = 0;
-            }
+        s_last = atomicAdd(S.done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (s_last && warp == 0) {
+        uint32_t items = 0;
+        for (int i = lane; i < n; i += 32) {
+            items += S.list_count[i];
+            S.list_count[i] = 0;
+        }
+        items = __reduce_add_sync(0xffffffffu, items);
+        if (lane == 0) {
             *S.items_total += items;
             if (t >= S.burn_in && S.record_every > 0 && ((t - S.burn_in) % S.record_every) == 0 &&
                 (t - S.burn_in) / S.record_every < S.record_cap)
@@ -1625,33 +1678,71 @@ __global__ void k_ess(const uint64_t* __restrict__ bits, int C, int n, int words
     out[e] = any ? total : NAN;
 }
 
-__global__ void k_edge_freq(const uint32_t* __restrict__ edge, int C, int n, double denom, double* __restrict__ out)
+// edge frequencies: 32 edges a block, 16 threads an edge over the chains (whole numbers, so
+// any order of the sum gives the same)
+static constexpr int EF_ROWS = 16;
+__global__ void __launch_bounds__(32 * EF_ROWS) k_edge_freq(const uint32_t* __restrict__ edge, int C, int n,
+                                                           double denom, double* __restrict__ out)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n * n) return;
+    __shared__ uint64_t s_s[EF_ROWS][32];
+    const int e = blockIdx.x * 32 + threadIdx.x;
     uint64_t s = 0;
-    for (int c = 0; c < C; ++c) s += edge[(size_t)c * n * n + e];
-    out[e] = denom > 0 ? (double)s / denom : 0.0;
+    if (e < n * n) {
+#pragma unroll 8
+        for (int c = threadIdx.y; c < C; c += EF_ROWS) s += edge[(size_t)c * n * n + e];
+    }
+    s_s[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y == 0 && e < n * n) {
+        for (int r = 1; r < EF_ROWS; ++r) s += s_s[r][threadIdx.x];
+        out[e] = denom > 0 ? (double)s / denom : 0.0;
+    }
 }
 
-// best chain (highest best score, lowest chain id on ties) and its greedy DAG
-__global__ void k_pick_best(const double* __restrict__ best_score, const uint8_t* __restrict__ best_order,
-                            const uint32_t* __restrict__ best_rank, const uint64_t* __restrict__ pst, int C, int n,
-                            uint8_t* __restrict__ out_order, uint8_t* __restrict__ out_dag, double* __restrict__ out_score)
+// best chain (highest best score, lowest chain id on ties) and its greedy DAG, one block
+__global__ void __launch_bounds__(256) k_pick_best(const double* __restrict__ best_score,
+                                                   const uint8_t* __restrict__ best_order,
+                                                   const uint32_t* __restrict__ best_rank,
+                                                   const uint64_t* __restrict__ pst, int C, int n,
+                                                   uint8_t* __restrict__ out_order, uint8_t* __restrict__ out_dag,
+                                                   double* __restrict__ out_score)
 {
-    __shared__ int s_c;
-    if (threadIdx.x == 0) {
-        int bc = 0;
-        for (int c = 1; c < C; ++c)
-            if (best_score[c] > best_score[bc]) bc = c;
-        s_c = bc;
-        *out_score = best_score[bc];
+    __shared__ double s_v[8];
+    __shared__ int s_c[8];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int bc = min(tid, C - 1);
+    double bv = best_score[bc];
+    for (int c = tid + 256; c < C; c += 256) {
+        const double v = best_score[c];
+        if (v > bv) {
+            bv = v;
+            bc = c;
+        }
     }
+    auto better = [](double v, int c, double w, int d) { return v > w || (v == w && c < d); };
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, bv, d);
+        const int c = __shfl_xor_sync(0xffffffffu, bc, d);
+        if (better(v, c, bv, bc)) {
+            bv = v;
+            bc = c;
+        }
+    }
+    if (lane == 0) {
+        s_v[warp] = bv;
+        s_c[warp] = bc;
+    }
+    for (int e = tid; e < n * n; e += 256) out_dag[e] = 0;
     __syncthreads();
-    const int bc = s_c;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int w = 0; w < 8; ++w)
+        if (better(s_v[w], s_c[w], bv, bc)) {
+            bv = s_v[w];
+            bc = s_c[w];
+        }
+    if (tid == 0) *out_score = bv;
+    for (int i = tid; i < n; i += 256) {
         out_order[i] = best_order[(size_t)bc * n + i];
-        for (int m = 0; m < n; ++m) out_dag[(size_t)i * n + m] = 0;
         uint64_t msk = pst[best_rank[(size_t)bc * n + i]];
         while (msk) {
             const int slot = __ffsll((long long)msk) - 1;
@@ -1847,7 +1938,7 @@ extern "C" int bn_chains_create(const bn_table* t, const bn_mcmc_params* p, cons
         if (cudaMemcpyAsync(S.cur_order, src, Cn, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
             return fail(cuda_fail(cudaGetLastError(), "copy init orders", __FILE__, __LINE__));
     } else {
-        k_init_orders<<<(C + 127) / 128, 128, 0, s>>>(S);
+        k_init_orders<<<(C + 7) / 8, 256, 0, s>>>(S);
         cudaError_t le = cudaGetLastError();
         if (le != cudaSuccess) return fail(cuda_fail(le, "k_init_orders", __FILE__, __LINE__));
         count_launches(1);
@@ -1856,7 +1947,7 @@ extern "C" int bn_chains_create(const bn_table* t, const bn_mcmc_params* p, cons
     int rc = launch_pred_lists(S.cur_order, C, n, S.list_pc, S.list_best, S.list_count, S.status, s);
     if (rc) return fail(rc);
     if ((rc = launch_scan(t, ch->plan, S.list_count, S.list_pc, S.list_best, C, S.status, s))) return fail(rc);
-    k_init_state<<<(C + 7) / 8, 256, 0, s>>>(S);
+    k_init_state<<<(C + IS_CHAINS - 1) / IS_CHAINS, 256, 0, s>>>(S);
     {
         cudaError_t le = cudaGetLastError();
         if (le != cudaSuccess) return fail(cuda_fail(le, "k_init_state", __FILE__, __LINE__));
@@ -2230,10 +2321,10 @@ static int run_collect(bn_chains* ch, const bn_mcmc_params* p, int64_t total, in
     BN_CUDA(cudaMallocAsync((void**)&d_dag, (size_t)n * n, s));
     BN_CUDA(cudaMallocAsync((void**)&d_s, 8, s));
     BN_CUDA(cudaMallocAsync((void**)&d_f, 8 * (size_t)n * n, s));
-    k_pick_best<<<1, 64, 0, s>>>(ch->S.best_score, ch->S.best_order, ch->S.best_rank, t->pst, C, n, d_o, d_dag, d_s);
+    k_pick_best<<<1, 256, 0, s>>>(ch->S.best_score, ch->S.best_order, ch->S.best_rank, t->pst, C, n, d_o, d_dag, d_s);
     BN_LAUNCH_CHECK("k_pick_best");
     const double denom = (double)C * (double)std::max<int64_t>(0, total - p->burn_in);
-    k_edge_freq<<<(n * n + 127) / 128, 128, 0, s>>>(ch->S.edge, C, n, denom, d_f);
+    k_edge_freq<<<(n * n + 31) / 32, dim3(32, EF_ROWS), 0, s>>>(ch->S.edge, C, n, denom, d_f);
     BN_LAUNCH_CHECK("k_edge_freq");
     std::vector<double> f((size_t)n * n);
     std::vector<int64_t> acc1(C);
