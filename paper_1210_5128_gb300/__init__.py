@@ -187,12 +187,20 @@ class Table:
 
     def __init__(self, handle):
         self._h = handle
+        self._n = None
 
     @property
     def handle(self):
         if not self._h:
             raise ValueError("table already freed")
         return self._h
+
+    @property
+    def n(self):
+        """Nodes of the network (fixed for a table's life)."""
+        if self._n is None:
+            self._n = table_info(self)["n"]
+        return self._n
 
     def free(self):
         if self._h:
@@ -307,7 +315,7 @@ def table_scores(t: Table, node: int = -1, device=None):
 
 def score_orders(t: Table, orders):
     """Eq. (6) for a batch of orders (bn_score_orders) -> (best_rank (B,n), score (B,))."""
-    n = table_info(t)["n"]
+    n = t.n
     if _is_cuda(orders):
         import torch
         o = _dev(orders, torch.uint8)
@@ -328,7 +336,7 @@ def score_orders_profiled(t: Table, orders):
     """score_orders on device tensors with the scan kernel's device time (ms, CUDA events
     around its launch): (best_rank, score, scan_ms)."""
     import torch
-    n = table_info(t)["n"]
+    n = t.n
     o = _dev(orders, torch.uint8)
     B = o.shape[0]
     br = torch.empty((B, n), dtype=torch.int32, device=o.device)
@@ -342,7 +350,7 @@ def score_orders_profiled(t: Table, orders):
 def score_orders_sum(t: Table, orders):
     """The sum-based order score (bn_score_orders_sum) -> (order score (B,), node terms (B, n));
     device tensors in, device tensors out; host arrays in, numpy arrays out."""
-    n = table_info(t)["n"]
+    n = t.n
     if _is_cuda(orders):
         import torch
         o = _dev(orders, torch.uint8)
@@ -431,7 +439,7 @@ class Chains:
 
 def chains_create(t: Table, chains, seed, burn_in=0, init_orders=None, literal_log=False,
                   record_every=0, record_cap=0, trace_cap=0) -> Chains:
-    n = table_info(t)["n"]
+    n = t.n
     p = MCMCParams(chains, burn_in, seed, 1 if literal_log else 0, record_every, record_cap,
                    1 if trace_cap else 0, trace_cap, 0, 0.0, 0, 0, None)
     h = _vp()
@@ -478,7 +486,7 @@ def mcmc_run(t: Table, chains, steps, seed, burn_in=0, literal_log=False, propos
     frequencies and the run's summary (acceptance, edge-posterior ESS when thin > 0,
     device times).  proposal = PROPOSAL_LEARNED trains the network (given, or one the
     call creates) for train_iters steps first."""
-    n = table_info(t)["n"]
+    n = t.n
     p = MCMCParams(chains, burn_in, seed, 1 if literal_log else 0, 0, 0, 0, 0,
                    proposal, eps_mix, train_iters, thin, net.handle if net is not None else None)
     bo = np.empty(n, np.uint8)

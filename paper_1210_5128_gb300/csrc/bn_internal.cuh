@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
+
 #include "bn.h"
 
 namespace bn {
@@ -27,6 +29,30 @@ unsigned long long context_id();
 // this call site's `slots` (64 zero-initialised entries): per-context set-up, such as a
 // kernel's shared-memory attribute, which a context destroyed and created again loses.
 bool first_in_context(unsigned long long* slots);
+
+// Device memory from the library's own pool of the current device (bn_api.cu).  dev_alloc /
+// dev_free are ordered by stream s; obj_alloc's memory is usable on every stream when it
+// returns, and obj_free waits for the device first, as cudaMalloc and cudaFree would.
+cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t s);
+void dev_free(void* p, cudaStream_t s);
+cudaError_t obj_alloc(void** p, size_t bytes);
+template <class T>
+cudaError_t obj_alloc(T** p, size_t bytes) { return obj_alloc((void**)p, bytes); }
+void obj_free(std::initializer_list<void*> ps);
+// A small pinned host block, readable and writable by kernels at its host address, for the
+// duration of one synchronous call: a zeroed status word, then SLOT_BYTES of staging.
+struct HostSlot {
+    static constexpr size_t SLOT_BYTES = 64 * 1024;
+    uint32_t* status = nullptr;
+    uint8_t* buf = nullptr;
+    HostSlot();
+    ~HostSlot();
+    HostSlot(const HostSlot&) = delete;
+    HostSlot& operator=(const HostSlot&) = delete;
+
+private:
+    unsigned long long ctx = 0;
+};
 
 #define BN_CUDA(call)                                                                  \
     do {                                                                               \

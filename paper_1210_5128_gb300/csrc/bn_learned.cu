@@ -1041,7 +1041,7 @@ void bn::learned_free(LearnedPath* lp)
 {
     if (!lp) return;
     if (lp->exec) cudaGraphExecDestroy(lp->exec);
-    cudaFree(lp->block);
+    obj_free({lp->block});
     delete lp;
 }
 
@@ -1089,7 +1089,7 @@ static int learned_alloc(bn_chains* ch)
                  r_off = r_rk + (size_t)round_up((int64_t)(4 * alive), 16),
                  r_end = r_off + (size_t)round_up((int64_t)(4 * (n + 1)), 16);
     const size_t o_sreg = take(r_end);
-    cudaError_t e = cudaMalloc(&lp->block, off);
+    cudaError_t e = obj_alloc(&lp->block, off);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete lp;
@@ -1432,14 +1432,14 @@ int bn::learned_read_logits(const bn_chains* ch, float* out, int mem, cudaStream
     float* d = out;
     float* tmp = nullptr;
     if (mem == BN_MEM_HOST) {
-        BN_CUDA(cudaMallocAsync((void**)&tmp, 4 * (size_t)cnt, s));
+        BN_CUDA(dev_alloc((void**)&tmp, 4 * (size_t)cnt, s));
         d = tmp;
     }
     k_gather_logits<<<blocks_of(cnt), 256, 0, s>>>(lp->L.logits, lp->L.cur_buf, lp->C, lp->P, lp->Pp, d);
     BN_LAUNCH_CHECK("k_gather_logits");
     if (mem == BN_MEM_HOST) {
         BN_CUDA(cudaMemcpyAsync(out, tmp, 4 * (size_t)cnt, cudaMemcpyDeviceToHost, s));
-        BN_CUDA(cudaFreeAsync(tmp, s));
+        dev_free(tmp, s);
     }
     BN_CUDA(cudaStreamSynchronize(s));
     return BN_OK;

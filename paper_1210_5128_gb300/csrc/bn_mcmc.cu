@@ -1471,7 +1471,7 @@ int build_survivor_cache(bn_table* t, cudaStream_t s)
     const int cap = (int)t->alive_total;
     uint8_t* g = nullptr;
     // the cache, then the [n][64] first-survivor table (16-bit offsets within a node)
-    cudaError_t e = cudaMalloc((void**)&g, surv_cache_stride(cap) + sizeof(uint16_t) * 64 * MAXN);
+    cudaError_t e = obj_alloc((void**)&g, surv_cache_stride(cap) + sizeof(uint16_t) * 64 * MAXN);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return BN_OK;                       // no cache: the uncached walk still works
@@ -1894,7 +1894,7 @@ extern "C" int bn_chains_create(const bn_table* t, const bn_mcmc_params* p, cons
     size_t o_ts = take(8 * (size_t)C * S.trace_cap), o_ta = take((size_t)C * S.trace_cap);
     size_t o_rec = take(8 * Cn * n * S.rec_words);
     size_t o_init = take(mem == BN_MEM_HOST && init_orders ? Cn : 0);
-    cudaError_t e = cudaMalloc(&ch->block, off);
+    cudaError_t e = obj_alloc(&ch->block, off);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete ch;
@@ -2132,7 +2132,7 @@ extern "C" int bn_chains_read(const bn_chains* ch, int what, void* out, int mem,
             double* d = (double*)out;
             double* tmp = nullptr;
             if (mem == BN_MEM_HOST) {
-                BN_CUDA(cudaMallocAsync((void**)&tmp, 8 * (size_t)S.n * S.n, s));
+                BN_CUDA(dev_alloc((void**)&tmp, 8 * (size_t)S.n * S.n, s));
                 d = tmp;
             }
             const int nn = S.n * S.n;
@@ -2140,7 +2140,7 @@ extern "C" int bn_chains_read(const bn_chains* ch, int what, void* out, int mem,
             BN_LAUNCH_CHECK("k_ess");
             if (mem == BN_MEM_HOST) {
                 BN_CUDA(cudaMemcpyAsync(out, tmp, 8 * (size_t)nn, cudaMemcpyDeviceToHost, s));
-                BN_CUDA(cudaFreeAsync(tmp, s));
+                dev_free(tmp, s);
             }
             BN_CUDA(cudaStreamSynchronize(s));
             return BN_OK;
@@ -2158,8 +2158,7 @@ extern "C" void bn_chains_free(bn_chains* ch)
     if (!ch) return;
     if (ch->exec) cudaGraphExecDestroy(ch->exec);
     learned_free(ch->lp);
-    cudaFree(ch->block);
-    cudaFree(ch->prop_block);
+    obj_free({ch->block, ch->prop_block});
     delete ch;
 }
 
@@ -2193,7 +2192,7 @@ extern "C" int bn_chains_set_proposal(bn_chains* ch, bn_mlp* m, int mode, double
         const size_t o_cur = take(4 * C * P), o_prop = take(4 * C * P), o_pair = take(4 * C), o_lqf = take(4 * C),
                      o_delta = take(4 * C), o_to = take(C * S.n), o_tp = take(4 * C), o_ta = take(4 * C),
                      o_ch = take(C);
-        cudaError_t e = cudaMalloc(&ch->prop_block, off);
+        cudaError_t e = obj_alloc(&ch->prop_block, off);
         if (e != cudaSuccess) {
             cudaGetLastError();
             ch->prop_block = nullptr;
@@ -2315,30 +2314,33 @@ static int run_collect(bn_chains* ch, const bn_mcmc_params* p, int64_t total, in
     cudaStream_t s = (cudaStream_t)stream;
     const bn_table* t = ch->t;
     const int n = t->n, C = p->chains;
-    uint8_t *d_o = nullptr, *d_dag = nullptr;
-    double *d_s = nullptr, *d_f = nullptr;
-    BN_CUDA(cudaMallocAsync((void**)&d_o, n, s));
-    BN_CUDA(cudaMallocAsync((void**)&d_dag, (size_t)n * n, s));
-    BN_CUDA(cudaMallocAsync((void**)&d_s, 8, s));
-    BN_CUDA(cudaMallocAsync((void**)&d_f, 8 * (size_t)n * n, s));
+    // one block back to the host: score | frequencies | accepts | order | DAG
+    const size_t o_f = 8, o_acc = o_f + 8 * (size_t)n * n, o_o = o_acc + 8 * (size_t)C, o_dag = o_o + n,
+                 bytes = o_dag + (size_t)n * n;
+    uint8_t* d = nullptr;
+    BN_CUDA(dev_alloc((void**)&d, bytes, s));
+    struct Free {
+        uint8_t* p;
+        cudaStream_t s;
+        ~Free() { dev_free(p, s); }
+    } fr{d, s};
+    double *d_s = (double*)d, *d_f = (double*)(d + o_f);
+    uint8_t *d_o = d + o_o, *d_dag = d + o_dag;
     k_pick_best<<<1, 256, 0, s>>>(ch->S.best_score, ch->S.best_order, ch->S.best_rank, t->pst, C, n, d_o, d_dag, d_s);
     BN_LAUNCH_CHECK("k_pick_best");
     const double denom = (double)C * (double)std::max<int64_t>(0, total - p->burn_in);
     k_edge_freq<<<(n * n + 31) / 32, dim3(32, EF_ROWS), 0, s>>>(ch->S.edge, C, n, denom, d_f);
     BN_LAUNCH_CHECK("k_edge_freq");
-    std::vector<double> f((size_t)n * n);
-    std::vector<int64_t> acc1(C);
-    if (best_order) BN_CUDA(cudaMemcpyAsync(best_order, d_o, n, cudaMemcpyDeviceToHost, s));
-    if (best_dag) BN_CUDA(cudaMemcpyAsync(best_dag, d_dag, (size_t)n * n, cudaMemcpyDeviceToHost, s));
-    if (best_score) BN_CUDA(cudaMemcpyAsync(best_score, d_s, 8, cudaMemcpyDeviceToHost, s));
-    BN_CUDA(cudaMemcpyAsync(f.data(), d_f, 8 * (size_t)n * n, cudaMemcpyDeviceToHost, s));
-    if (stats) BN_CUDA(cudaMemcpyAsync(acc1.data(), ch->S.accepts, 8 * (size_t)C, cudaMemcpyDeviceToHost, s));
-    cudaFreeAsync(d_o, s);
-    cudaFreeAsync(d_dag, s);
-    cudaFreeAsync(d_s, s);
-    cudaFreeAsync(d_f, s);
+    BN_CUDA(cudaMemcpyAsync(d + o_acc, ch->S.accepts, 8 * (size_t)C, cudaMemcpyDeviceToDevice, s));
+    std::vector<uint8_t> h(bytes);
+    BN_CUDA(cudaMemcpyAsync(h.data(), d, bytes, cudaMemcpyDeviceToHost, s));
     BN_CUDA(cudaStreamSynchronize(s));
-    if (edge_freq) std::copy(f.begin(), f.end(), edge_freq);
+    const double* f = (const double*)(h.data() + o_f);
+    const int64_t* acc1 = (const int64_t*)(h.data() + o_acc);
+    if (best_order) memcpy(best_order, h.data() + o_o, n);
+    if (best_dag) memcpy(best_dag, h.data() + o_dag, (size_t)n * n);
+    if (best_score) memcpy(best_score, h.data(), 8);
+    if (edge_freq) memcpy(edge_freq, f, 8 * (size_t)n * n);
     if (stats) {
         bn_mcmc_stats st;
         int64_t acc = 0;
@@ -2454,7 +2456,7 @@ extern "C" int bn_batch_create(int count, const bn_table* const* tables, const b
         b->chains.push_back(c);
     }
     const size_t bytes = (sizeof(ChainState) + sizeof(FusedArgs) + 2 * sizeof(int64_t)) * (size_t)(count + 1) + 1024;
-    cudaError_t e = cudaMalloc(&b->dev, bytes);
+    cudaError_t e = obj_alloc(&b->dev, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         bn_batch_free(b);
@@ -2547,11 +2549,11 @@ extern "C" int bn_batch_step(bn_batch* b, int64_t steps, void* stream)
     }
     uint8_t* args = nullptr;
     const size_t fbytes = sizeof(FusedArgs) * hf.size(), ibytes = sizeof(int) * hit.size();
-    BN_CUDA(cudaMallocAsync((void**)&args, fbytes + ibytes + 16, s));
+    BN_CUDA(dev_alloc((void**)&args, fbytes + ibytes + 16, s));
     struct Free {
         uint8_t* p;
         cudaStream_t s;
-        ~Free() { cudaFreeAsync(p, s); }
+        ~Free() { dev_free(p, s); }
     } fr{args, s};
     FusedArgs* d_fargs = (FusedArgs*)args;
     int* d_iters = (int*)(args + fbytes);
@@ -2572,7 +2574,7 @@ extern "C" void bn_batch_free(bn_batch* b)
 {
     if (!b) return;
     for (bn_chains* c : b->chains) bn_chains_free(c);
-    cudaFree(b->dev);
+    obj_free({b->dev});
     delete b;
 }
 

@@ -520,7 +520,7 @@ extern "C" int bn_mlp_create(int n, const bn_mlp_params* p, const float* E, cons
     off += (size_t)round_up((int64_t)cap * n, 256) + (size_t)round_up((int64_t)cap * 4, 256) * 2;
     const size_t o_inv = off;                        // inverse orders of a training batch
     off += (size_t)round_up((int64_t)cap * 64, 256);
-    cudaError_t e = cudaMalloc(&m->block, off);
+    cudaError_t e = obj_alloc(&m->block, off);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete m;
@@ -646,7 +646,7 @@ extern "C" int bn_mlp_read(const bn_mlp* m, int what, float* out, int mem, void*
 extern "C" void bn_mlp_free(bn_mlp* m)
 {
     if (!m) return;
-    cudaFree(m->block);
+    obj_free({m->block});
     delete m;
 }
 
@@ -656,14 +656,14 @@ extern "C" int bn_gemm_bf16(const uint16_t* A, const uint16_t* B, float* C, int 
     if (!A || !B || !C) return set_error(BN_EINVAL, "bn_gemm_bf16: NULL");
     cudaStream_t s = (cudaStream_t)stream;
     uint32_t* st = nullptr;
-    BN_CUDA(cudaMallocAsync((void**)&st, 4, s));
+    BN_CUDA(dev_alloc((void**)&st, 4, s));
     BN_CUDA(cudaMemsetAsync(st, 0, 4, s));
     int rc = gemm_tc((const bf16*)A, K, (const bf16*)B, K, C, N, M, N, K, st, s, nullptr, 0);
     uint32_t h = 0;
     if (!rc) {
         BN_CUDA(cudaMemcpyAsync(&h, st, 4, cudaMemcpyDeviceToHost, s));
     }
-    cudaFreeAsync(st, s);
+    dev_free(st, s);
     BN_CUDA(cudaStreamSynchronize(s));
     if (rc) return rc;
     if (h & STATUS_TIMEOUT) return set_error(BN_ETIMEOUT, "bn_gemm_bf16: a bounded device wait expired");

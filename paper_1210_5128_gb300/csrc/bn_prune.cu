@@ -264,7 +264,7 @@ int prune_table(bn_table* t, cudaStream_t s)
     const size_t o_bits = take(4 * (size_t)n * words), o_max = take(8), o_aoff = take(4 * (size_t)n),
                  o_acnt = take(4 * (size_t)n), o_cnt = take(4 * (size_t)n * nch), o_le = take(8 * (size_t)n * below);
     uint8_t* work = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&work, off, s);
+    cudaError_t e = dev_alloc((void**)&work, off, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(BN_ENOMEM, "prune: %zu bytes of work space", off);
@@ -272,7 +272,7 @@ int prune_table(bn_table* t, cudaStream_t s)
     struct F {
         void* p;
         cudaStream_t s;
-        ~F() { cudaFreeAsync(p, s); }
+        ~F() { dev_free(p, s); }
     } fr{work, s};
     uint32_t* alive = (uint32_t*)(work + o_bits);
     uint32_t* counts = (uint32_t*)(work + o_cnt);
@@ -314,7 +314,7 @@ int prune_table(bn_table* t, cudaStream_t s)
     if (run >= 0xffffffffull) return set_error(BN_EUNSUPPORTED, "prune: too many surviving entries");
     uint8_t* blk = nullptr;
     const size_t m1 = (size_t)std::max<uint64_t>(run, 1);
-    BN_CUDA(cudaMalloc((void**)&blk, 12 * m1 + 8 * (size_t)n + 64));
+    BN_CUDA(obj_alloc((void**)&blk, 12 * m1 + 8 * (size_t)n + 64));
     t->alive_block = blk;
     t->aspos = (uint32_t*)(blk + 8 * m1);
     t->aoff = (uint32_t*)(blk + 12 * m1);

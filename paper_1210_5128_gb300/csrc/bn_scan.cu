@@ -781,21 +781,6 @@ int launch_reduce_orders(const bn_table* t, const uint32_t* list_best, int B, ui
 
 using namespace bn;
 
-// the stream-ordered pool keeps freed scratch mapped (its default release threshold of 0
-// would unmap it at every synchronisation and map it again on the next call)
-static void keep_pool_mapped()
-{
-    static unsigned long long ctx[64] = {0};
-    if (!first_in_context(ctx)) return;
-    const int d = device_id();
-    cudaMemPool_t pool;
-    if (cudaDeviceGetDefaultMemPool(&pool, d) == cudaSuccess) {
-        uint64_t thr = (uint64_t)256 << 20;
-        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
-    }
-    cudaGetLastError();
-}
-
 static int score_orders_impl(const bn_table* t, const uint8_t* orders, int B, uint32_t* best_rank,
                              double* order_score, int mem, void* stream, cudaEvent_t ev0, cudaEvent_t ev1)
 {
@@ -811,24 +796,32 @@ static int score_orders_impl(const bn_table* t, const uint8_t* orders, int B, ui
         int rt = ensure_tuned(t, B, s);
         if (rt) return rt;
     }
-    keep_pool_mapped();
+    // The status word lies in pinned host memory, where only an error writes it.  Small host
+    // arrays go through the slot too: the list builder reads the orders there (once each)
+    // and the reduction writes its results there, with no copies in between.
+    HostSlot slot;
+    if (!slot.status) return set_error(BN_ENOMEM, "bn_score_orders: pinned memory for the call's status");
+    const size_t out_rank = best_rank ? (size_t)round_up((int64_t)(sizeof(uint32_t) * (size_t)B * n), 16) : 0;
+    const size_t in_bytes = (size_t)round_up((int64_t)((size_t)B * n), 16);
+    const bool staged = mem == BN_MEM_HOST &&
+                        in_bytes + out_rank + (order_score ? sizeof(double) * (size_t)B : 0) <= HostSlot::SLOT_BYTES;
+    const bool copied = mem == BN_MEM_HOST && !staged;
 
-    // one scratch block: orders | list_pc | list_best | counts | status | ranks | scores
+    // one scratch block: orders | list_pc | list_best | counts | ranks | scores
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
         off = (size_t)round_up((int64_t)(off + bytes), 256);
         return o;
     };
-    const size_t o_orders = take(mem == BN_MEM_HOST ? (size_t)B * n : 0);
+    const size_t o_orders = take(copied ? (size_t)B * n : 0);
     const size_t o_pc = take(sizeof(uint64_t) * (size_t)n * B);
     const size_t o_best = take(sizeof(uint32_t) * (size_t)n * B);
     const size_t o_cnt = take(sizeof(uint32_t) * n);
-    const size_t o_st = take(sizeof(uint32_t));
-    const size_t o_rank = take(mem == BN_MEM_HOST && best_rank ? sizeof(uint32_t) * (size_t)B * n : 0);
-    const size_t o_score = take(mem == BN_MEM_HOST && order_score ? sizeof(double) * B : 0);
+    const size_t o_rank = take(copied && best_rank ? sizeof(uint32_t) * (size_t)B * n : 0);
+    const size_t o_score = take(copied && order_score ? sizeof(double) * B : 0);
     uint8_t* base = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&base, off, s);
+    cudaError_t e = dev_alloc((void**)&base, off, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(BN_ENOMEM, "bn_score_orders: scratch of %zu bytes: %s", off, cudaGetErrorString(e));
@@ -836,20 +829,35 @@ static int score_orders_impl(const bn_table* t, const uint8_t* orders, int B, ui
     struct Free {
         uint8_t* p;
         cudaStream_t s;
-        ~Free() { cudaFreeAsync(p, s); }
+        ~Free() { dev_free(p, s); }
     } fr{base, s};
     const uint8_t* d_orders = orders;
-    if (mem == BN_MEM_HOST) {
+    uint32_t* d_rank = best_rank;
+    double* d_score = order_score;
+    if (copied) {
         BN_CUDA(cudaMemcpyAsync(base + o_orders, orders, (size_t)B * n, cudaMemcpyHostToDevice, s));
         d_orders = base + o_orders;
+        d_rank = best_rank ? (uint32_t*)(base + o_rank) : nullptr;
+        d_score = order_score ? (double*)(base + o_score) : nullptr;
+    } else if (staged) {
+        memcpy(slot.buf, orders, (size_t)B * n);
+        d_orders = slot.buf;
+        d_rank = best_rank ? (uint32_t*)(slot.buf + in_bytes) : nullptr;
+        d_score = order_score ? (double*)(slot.buf + in_bytes + out_rank) : nullptr;
     }
     uint64_t* d_pc = (uint64_t*)(base + o_pc);
     uint32_t* d_best = (uint32_t*)(base + o_best);
     uint32_t* d_cnt = (uint32_t*)(base + o_cnt);
-    uint32_t* d_st = (uint32_t*)(base + o_st);
-    uint32_t* d_rank = mem == BN_MEM_HOST ? (best_rank ? (uint32_t*)(base + o_rank) : nullptr) : best_rank;
-    double* d_score = mem == BN_MEM_HOST ? (order_score ? (double*)(base + o_score) : nullptr) : order_score;
-    BN_CUDA(cudaMemsetAsync(d_st, 0, sizeof(uint32_t), s));
+    uint32_t* d_st = slot.status;
+    // the slot goes back to the next call only when nothing on s can still write it
+    struct Drain {
+        cudaStream_t s;
+        bool done = false;
+        ~Drain()
+        {
+            if (!done) cudaStreamSynchronize(s);
+        }
+    } drain{s};
     int rc = launch_pred_lists(d_orders, B, n, d_pc, d_best, d_cnt, d_st, s);
     if (rc) return rc;
     if (ev0) BN_CUDA(cudaEventRecord(ev0, s));
@@ -857,14 +865,18 @@ static int score_orders_impl(const bn_table* t, const uint8_t* orders, int B, ui
     if (rc) return rc;
     if (ev1) BN_CUDA(cudaEventRecord(ev1, s));
     if ((rc = launch_reduce_orders(t, d_best, B, d_rank, d_score, s))) return rc;
-    if (mem == BN_MEM_HOST) {
+    if (copied) {
         if (best_rank)
             BN_CUDA(cudaMemcpyAsync(best_rank, d_rank, sizeof(uint32_t) * (size_t)B * n, cudaMemcpyDeviceToHost, s));
         if (order_score) BN_CUDA(cudaMemcpyAsync(order_score, d_score, sizeof(double) * B, cudaMemcpyDeviceToHost, s));
     }
-    uint32_t st = 0;
-    BN_CUDA(cudaMemcpyAsync(&st, d_st, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     BN_CUDA(cudaStreamSynchronize(s));
+    drain.done = true;
+    if (staged) {
+        if (best_rank) memcpy(best_rank, d_rank, sizeof(uint32_t) * (size_t)B * n);
+        if (order_score) memcpy(order_score, d_score, sizeof(double) * B);
+    }
+    const uint32_t st = *(volatile uint32_t*)slot.status;
     if (st & STATUS_BADINPUT) return set_error(BN_EINVAL, "bn_score_orders: an order is not a permutation of 0..n-1");
     if (st & STATUS_TIMEOUT) return set_error(BN_ETIMEOUT, "bn_score_orders: a bounded device wait expired");
     return BN_OK;
@@ -900,11 +912,11 @@ extern "C" int bn_measure_test_rate(void* stream, double* tests_per_s)
     if (!tests_per_s) return set_error(BN_EINVAL, "bn_measure_test_rate: NULL output");
     cudaStream_t s = (cudaStream_t)stream;
     uint32_t* sink = nullptr;
-    BN_CUDA(cudaMallocAsync((void**)&sink, 4, s));
+    BN_CUDA(dev_alloc((void**)&sink, 4, s));
     struct Free {
         uint32_t* p;
         cudaStream_t s;
-        ~Free() { cudaFreeAsync(p, s); }
+        ~Free() { dev_free(p, s); }
     } fr{sink, s};
     cudaEvent_t e0, e1;
     BN_CUDA(cudaEventCreate(&e0));
@@ -945,11 +957,11 @@ extern "C" int bn_table_autotune(bn_table* t, int max_items, void* stream, int64
     uint8_t* blk = nullptr;
     const size_t o_pc = 0, o_best = (size_t)round_up(8 * (int64_t)n * items, 256),
                  o_cnt = o_best + (size_t)round_up(4 * (int64_t)n * items, 256), o_st = o_cnt + 256;
-    BN_CUDA(cudaMallocAsync((void**)&blk, o_st + 256, s));
+    BN_CUDA(dev_alloc((void**)&blk, o_st + 256, s));
     struct Free {
         uint8_t* p;
         cudaStream_t s;
-        ~Free() { cudaFreeAsync(p, s); }
+        ~Free() { dev_free(p, s); }
     } fr{blk, s};
     uint64_t* pc = (uint64_t*)(blk + o_pc);
     uint32_t* best = (uint32_t*)(blk + o_best);

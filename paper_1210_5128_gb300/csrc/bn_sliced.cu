@@ -91,7 +91,7 @@ int alloc_sset(bn_table* t)
 {
     if (t->k > SL_MAX_K || t->n > 64 || t->sset) return BN_OK;   // the mask-test scans serve larger k
     const int64_t Ssp = round_up(t->S, SL_SUB);
-    cudaError_t e = cudaMalloc(&t->sset, sizeof(uint32_t) * (size_t)t->n * (size_t)Ssp);
+    cudaError_t e = obj_alloc(&t->sset, sizeof(uint32_t) * (size_t)t->n * (size_t)Ssp);
     if (e != cudaSuccess) {
         t->sset = nullptr;
         cudaGetLastError();

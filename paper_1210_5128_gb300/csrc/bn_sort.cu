@@ -508,13 +508,13 @@ struct SortTemps {
     std::vector<void*> p;
     ~SortTemps()
     {
-        for (void* q : p) cudaFreeAsync(q, s);
+        for (void* q : p) dev_free(q, s);
     }
     template <class T>
     int get(T** out, size_t count)
     {
         void* q = nullptr;
-        cudaError_t e = cudaMallocAsync(&q, std::max<size_t>(count, 1) * sizeof(T), s);
+        cudaError_t e = dev_alloc(&q, std::max<size_t>(count, 1) * sizeof(T), s);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return set_error(BN_ENOMEM, "rank_entries: %zu bytes of sort buffers: %s", count * sizeof(T),
@@ -589,19 +589,19 @@ static int rank_by_radix(bn_table* t, cudaStream_t s)
     const int Tmax = (int)((Nmax + RS_TILE - 1) / RS_TILE);
     uint64_t *k0 = nullptr, *k1 = nullptr;
     uint32_t *v0 = nullptr, *v1 = nullptr, *counts = nullptr, *totals = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&k0, 8 * (size_t)Nmax, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&k1, 8 * (size_t)Nmax, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&v0, 4 * (size_t)Nmax, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&v1, 4 * (size_t)Nmax, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&counts, 4 * (size_t)256 * Tmax, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&totals, 4 * 256, s);
+    cudaError_t e = dev_alloc((void**)&k0, 8 * (size_t)Nmax, s);
+    if (e == cudaSuccess) e = dev_alloc((void**)&k1, 8 * (size_t)Nmax, s);
+    if (e == cudaSuccess) e = dev_alloc((void**)&v0, 4 * (size_t)Nmax, s);
+    if (e == cudaSuccess) e = dev_alloc((void**)&v1, 4 * (size_t)Nmax, s);
+    if (e == cudaSuccess) e = dev_alloc((void**)&counts, 4 * (size_t)256 * Tmax, s);
+    if (e == cudaSuccess) e = dev_alloc((void**)&totals, 4 * 256, s);
     struct F {
         cudaStream_t s;
         void* p[6];
         ~F()
         {
             for (void* q : p)
-                if (q) cudaFreeAsync(q, s);
+                if (q) dev_free(q, s);
         }
     } fr{s, {k0, k1, v0, v1, counts, totals}};
     if (e != cudaSuccess) {

@@ -207,7 +207,7 @@ extern "C" int bn_score_orders_sum(const bn_table* t, const uint8_t* orders, int
     const size_t o_os = take(mem == BN_MEM_HOST && order_score ? sizeof(double) * B : 0);
     const size_t o_ns = take(mem == BN_MEM_HOST && node_score ? sizeof(double) * (size_t)B * n : 0);
     uint8_t* base = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&base, off, s);
+    cudaError_t e = dev_alloc((void**)&base, off, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(BN_ENOMEM, "bn_score_orders_sum: scratch of %zu bytes: %s", off, cudaGetErrorString(e));
@@ -215,7 +215,7 @@ extern "C" int bn_score_orders_sum(const bn_table* t, const uint8_t* orders, int
     struct Free {
         uint8_t* p;
         cudaStream_t s;
-        ~Free() { cudaFreeAsync(p, s); }
+        ~Free() { dev_free(p, s); }
     } fr{base, s};
     const uint8_t* d_orders = orders;
     if (mem == BN_MEM_HOST) {

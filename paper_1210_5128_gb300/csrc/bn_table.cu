@@ -449,17 +449,13 @@ static int table_alloc(int n, int k, bn_table** out)
     t->dev = device_id();
     t->S = num_sets_host(n - 1, k);
     t->Sp = round_up(t->S, SUBQ);
-    cudaError_t e = cudaMalloc(&t->keys, sizeof(int64_t) * (size_t)n * (size_t)t->Sp);
-    if (e == cudaSuccess) e = cudaMalloc(&t->pst, sizeof(uint64_t) * (size_t)t->Sp);
-    if (e == cudaSuccess) e = cudaMalloc(&t->spos, sizeof(uint32_t) * (size_t)n * (size_t)t->Sp);
-    if (e == cudaSuccess) e = cudaMalloc(&t->srank, sizeof(uint32_t) * (size_t)n * (size_t)t->Sp);
-    if (e == cudaSuccess) e = cudaMalloc(&t->spos_t, sizeof(uint32_t) * (size_t)n * (size_t)t->Sp);
+    cudaError_t e = obj_alloc(&t->keys, sizeof(int64_t) * (size_t)n * (size_t)t->Sp);
+    if (e == cudaSuccess) e = obj_alloc(&t->pst, sizeof(uint64_t) * (size_t)t->Sp);
+    if (e == cudaSuccess) e = obj_alloc(&t->spos, sizeof(uint32_t) * (size_t)n * (size_t)t->Sp);
+    if (e == cudaSuccess) e = obj_alloc(&t->srank, sizeof(uint32_t) * (size_t)n * (size_t)t->Sp);
+    if (e == cudaSuccess) e = obj_alloc(&t->spos_t, sizeof(uint32_t) * (size_t)n * (size_t)t->Sp);
     if (e != cudaSuccess) {
-        cudaFree(t->keys);
-        cudaFree(t->pst);
-        cudaFree(t->spos);
-        cudaFree(t->srank);
-        cudaFree(t->spos_t);
+        obj_free({t->keys, t->pst, t->spos, t->srank, t->spos_t});
         delete t;
         cudaGetLastError();
         return set_error(BN_ENOMEM, "table allocation of %lld entries failed: %s",
@@ -493,10 +489,10 @@ struct Temps {
     int get(T** out, size_t count)
     {
         void* q = nullptr;
-        cudaError_t e = cudaMallocAsync(&q, std::max<size_t>(count, 1) * sizeof(T), s);
+        cudaError_t e = dev_alloc(&q, std::max<size_t>(count, 1) * sizeof(T), s);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            return set_error(BN_ENOMEM, "cudaMallocAsync(%zu bytes) failed: %s", count * sizeof(T),
+            return set_error(BN_ENOMEM, "device memory (%zu bytes) failed: %s", count * sizeof(T),
                              cudaGetErrorString(e));
         }
         p.push_back(q);
@@ -505,7 +501,7 @@ struct Temps {
     }
     void release()
     {
-        for (void* q : p) cudaFreeAsync(q, s);
+        for (void* q : p) dev_free(q, s);
         p.clear();
     }
     ~Temps() { release(); }
@@ -911,11 +907,11 @@ extern "C" int bn_build_scores_batch(int count, const uint8_t* const* data, cons
         }
     } sg{side, ev};
     uint32_t* d_meta = nullptr;
-    BN_CUDA(cudaMallocAsync((void**)&d_meta, sizeof(uint32_t) * META_WORDS * count, s));
+    BN_CUDA(dev_alloc((void**)&d_meta, sizeof(uint32_t) * META_WORDS * count, s));
     struct Free {
         uint32_t* p;
         cudaStream_t s;
-        ~Free() { cudaFreeAsync(p, s); }
+        ~Free() { dev_free(p, s); }
     } fr{d_meta, s};
     BN_CUDA(cudaMemsetAsync(d_meta, 0, sizeof(uint32_t) * META_WORDS * count, s));
     for (int j = 0; j <= ns; ++j) BN_CUDA(cudaEventCreateWithFlags(&ev[j], cudaEventDisableTiming));
@@ -1021,13 +1017,6 @@ extern "C" int bn_table_scores(const bn_table* t, int node, double* out, int mem
 extern "C" void bn_table_free(bn_table* t)
 {
     if (!t) return;
-    cudaFree(t->keys);
-    cudaFree(t->pst);
-    cudaFree(t->spos);
-    cudaFree(t->srank);
-    cudaFree(t->spos_t);
-    cudaFree(t->sset);
-    cudaFree(t->alive_block);
-    cudaFree(t->gcache);
+    obj_free({t->keys, t->pst, t->spos, t->srank, t->spos_t, t->sset, t->alive_block, t->gcache});
     delete t;
 }
