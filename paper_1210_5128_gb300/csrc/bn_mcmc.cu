@@ -1810,7 +1810,7 @@ static int sweep_launch(bn_chains* ch, cudaStream_t s, cudaEvent_t ev0 = nullptr
     if (S.mode == BN_PROPOSAL_LEARNED) {
         k_propose_learned<<<(S.C + 7) / 8, 256, 0, s>>>(S);
         BN_LAUNCH_CHECK("k_propose_learned");
-        if ((rc = mlp_forward_dev(ch->mlp, S.prop_order, S.C, false, s))) return rc;
+        if ((rc = mlp_forward_dev(ch->mlp, S.prop_order, S.C, s))) return rc;
         k_log_q<<<(S.C + 7) / 8, 256, 0, s>>>(ch->mlp->L, ch->mlp->Pp, S.C, S.P, S.eps_mix, S.prop_lq);
         BN_LAUNCH_CHECK("k_log_q");
     } else {
@@ -1837,7 +1837,7 @@ static int sweep_launch(bn_chains* ch, cudaStream_t s, cudaEvent_t ev0 = nullptr
 static int refresh_lq(bn_chains* ch, cudaStream_t s)
 {
     ChainState& S = ch->S;
-    int rc = mlp_forward_dev(ch->mlp, S.cur_order, S.C, false, s);
+    int rc = mlp_forward_dev(ch->mlp, S.cur_order, S.C, s);
     if (rc) return rc;
     k_log_q<<<(S.C + 7) / 8, 256, 0, s>>>(ch->mlp->L, ch->mlp->Pp, S.C, S.P, S.eps_mix, S.cur_lq);
     BN_LAUNCH_CHECK("k_log_q");

@@ -40,8 +40,22 @@ struct GemmArgs {
 // core-matrix layout of a 128 x 64 bf16 tile: row r, 16-byte chunk kc of the row
 __device__ __forceinline__ uint32_t tc_tile_off(int r, int kc) { return (r >> 3) * 1024 + kc * 128 + (r & 7) * 16; }
 
-__global__ void __launch_bounds__(128) k_gemm_tc(GemmArgs g)
+// Up to two independent products in one launch (the weight and the input gradient of a
+// layer): blocks below `blocks0` belong to the first.
+struct GemmPair {
+    GemmArgs g[2];
+    int blocks0;
+};
+
+__global__ void __launch_bounds__(128) k_gemm_tc(GemmPair gp)
 {
+    const bool second = (int)blockIdx.x >= gp.blocks0;
+    const GemmArgs& g = gp.g[second];
+    int tile = blockIdx.x - (second ? gp.blocks0 : 0);
+    const int tn = g.N / TC_BN, tm = g.M / TC_BM;
+    const int bx = tile % tn;
+    tile /= tn;
+    const int by = tile % tm, bz = tile / tm;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* sA = smem;
@@ -49,11 +63,11 @@ __global__ void __launch_bounds__(128) k_gemm_tc(GemmArgs g)
     uint64_t* bar = (uint64_t*)(smem + 2 * TC_STAGES * TC_TILE);
     uint32_t* tslot = (uint32_t*)(bar + TC_STAGES);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * TC_BM, n0 = blockIdx.x * TC_BN;
+    const int m0 = by * TC_BM, n0 = bx * TC_BN;
     const int kpart = g.K / g.ksplit;               // this CTA's K range (multiple of 64)
-    const int kbase = blockIdx.z * kpart;
+    const int kbase = bz * kpart;
     const int nk = kpart / TC_BK;
-    float* Cz = g.C + (size_t)blockIdx.z * g.M * g.ldc;
+    float* Cz = g.C + (size_t)bz * g.M * g.ldc;
 
     if (warp == 0) {
         tc_alloc(tslot, 128);
@@ -149,30 +163,39 @@ __global__ void k_splitk_reduce(const float* __restrict__ ws, int ksplit, int M,
     C[(size_t)r * ldc + c] = s;
 }
 
-// C = A B^T.  Few output tiles and a long K split K over grid z (each CTA at least four
-// 64-wide stages) into the workspace, then one reduction; ws == nullptr disables it.
-int gemm_tc(const bf16* A, int lda, const bf16* B, int ldb, float* C, int ldc, int M, int N, int K,
-            uint32_t* status, cudaStream_t s, float* ws, size_t ws_elems)
+// Few output tiles and a long K split K (each part at least four 64-wide stages) into
+// partials that the consumer adds in split order
+static int gemm_split(int M, int N, int K, size_t ws_elems)
 {
-    if (M % TC_BM || N % TC_BN || K % TC_BK)
-        return set_error(BN_EINVAL, "gemm: M=%d N=%d K=%d must be multiples of 128, 128, 64", M, N, K);
+    const int tiles = (M / TC_BM) * (N / TC_BN), stages = K / TC_BK;
+    const int lim = std::min(sm_count() / std::max(tiles, 1), stages / 4);
+    for (int dv = lim; dv >= 2; --dv)
+        if (stages % dv == 0 && (size_t)dv * M * N <= ws_elems) return dv;
+    return 1;
+}
+
+static int gemm_launch(const GemmArgs& a, const GemmArgs* b, cudaStream_t s)
+{
     static unsigned long long ctx[64] = {0};
     if (first_in_context(ctx))
         BN_CUDA(cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
-    const int tiles = (M / TC_BM) * (N / TC_BN);
-    int split = 1;
-    if (ws) {
-        const int stages = K / TC_BK;
-        const int lim = std::min(sm_count() / std::max(tiles, 1), stages / 4);
-        for (int dv = lim; dv >= 2; --dv)
-            if (stages % dv == 0 && (size_t)dv * M * N <= ws_elems) {
-                split = dv;
-                break;
-            }
-    }
-    GemmArgs g{A, B, split > 1 ? ws : C, M, N, K, lda, ldb, split > 1 ? N : ldc, split, status};
-    k_gemm_tc<<<dim3(N / TC_BN, M / TC_BM, split), 128, TC_SMEM, s>>>(g);
+    auto blocks = [](const GemmArgs& g) { return (g.M / TC_BM) * (g.N / TC_BN) * g.ksplit; };
+    GemmPair gp{{a, b ? *b : a}, blocks(a)};
+    k_gemm_tc<<<(unsigned)(gp.blocks0 + (b ? blocks(*b) : 0)), 128, TC_SMEM, s>>>(gp);
     BN_LAUNCH_CHECK("k_gemm_tc");
+    return BN_OK;
+}
+
+// C = A B^T, whole
+static int gemm_tc(const bf16* A, int lda, const bf16* B, int ldb, float* C, int ldc, int M, int N, int K,
+                   uint32_t* status, cudaStream_t s, float* ws, size_t ws_elems)
+{
+    if (M % TC_BM || N % TC_BN || K % TC_BK)
+        return set_error(BN_EINVAL, "gemm: M=%d N=%d K=%d must be multiples of 128, 128, 64", M, N, K);
+    const int split = ws ? gemm_split(M, N, K, ws_elems) : 1;
+    GemmArgs g{A, B, split > 1 ? ws : C, M, N, K, lda, ldb, split > 1 ? N : ldc, split, status};
+    const int rc = gemm_launch(g, nullptr, s);
+    if (rc) return rc;
     if (split > 1) {
         const int64_t tot = (int64_t)M * N;
         k_splitk_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(ws, split, M, N, C, ldc);
@@ -181,45 +204,98 @@ int gemm_tc(const bf16* A, int lda, const bf16* B, int ldb, float* C, int ldc, i
     return BN_OK;
 }
 
+// An M x N product as the GEMM left it: C, or the split partials the reader has to add
+struct Product {
+    const float* p;
+    int split;
+    int64_t stride;              // elements between partials
+    __device__ __forceinline__ float at(int64_t idx) const
+    {
+        if (split == 1) return p[idx];
+        float s = 0.f;
+        for (int z0 = 0; z0 < split; z0 += 8) {
+            float a[8];                                             // eight loads in flight
+#pragma unroll
+            for (int z = 0; z < 8; ++z) a[z] = z0 + z < split ? p[(size_t)(z0 + z) * stride + idx] : 0.f;
+#pragma unroll
+            for (int z = 0; z < 8; ++z)
+                if (z0 + z < split) s += a[z];
+        }
+        return s;
+    }
+};
+
 // ---------------------------------------------------------------------------------
 // elementwise kernels
 // ---------------------------------------------------------------------------------
 
-// x rows: X[r][p*d + j] = E[order_r(p)][j] (bf16), zero padding; XT optional (transposed)
-__global__ void k_embed(const uint8_t* __restrict__ orders, int B, int n, int d, int ndp, int Mp,
-                        const bf16* __restrict__ Eb, bf16* __restrict__ X, bf16* __restrict__ XT)
+// The elementwise kernels of the dense layers work on 32 x 32 tiles, 32 x 8 threads, so that
+// the transposed copies the weight gradients read go out coalesced through shared memory.
+// dst [.., ld] natural, dstT [.., ldt] transposed (may be null).
+__device__ __forceinline__ void store_tile(bf16 (&tile)[32][33], const bf16 (&v)[4], int r0, int c0, bf16* dst, int ld,
+                                           bf16* dstT, int ldt)
 {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)Mp * ndp) return;
-    const int r = (int)(idx / ndp), col = (int)(idx - (int64_t)r * ndp);
-    bf16 v = __float2bfloat16_rn(0.f);
-    if (r < B && col < n * d) {
-        const int p = col / d, j = col - p * d;
-        v = Eb[(size_t)orders[(size_t)r * n + p] * d + j];
+    const int x = threadIdx.x, y = threadIdx.y;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dst[(size_t)(r0 + y + 8 * k) * ld + c0 + x] = v[k];
+    if (!dstT) return;                                              // block-uniform
+#pragma unroll
+    for (int k = 0; k < 4; ++k) tile[y + 8 * k][x] = v[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dstT[(size_t)(c0 + y + 8 * k) * ldt + r0 + x] = tile[x][y + 8 * k];
+}
+
+// x rows: X[r][p*d + j] = E[order_r(p)][j] (bf16), zero padding; XT and inv (the inverse
+// orders: inv[r * 64 + v] = position of node v in order r) for training
+__global__ void __launch_bounds__(256) k_embed(const uint8_t* __restrict__ orders, int B, int n, int d, int ndp, int Mp,
+                                               const bf16* __restrict__ Eb, bf16* __restrict__ X, bf16* __restrict__ XT,
+                                               uint8_t* __restrict__ inv)
+{
+    __shared__ bf16 tile[32][33];
+    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, col = c0 + threadIdx.x;
+    const int p = col / d, j = col - p * d;
+    bf16 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = r0 + threadIdx.y + 8 * k;
+        v[k] = __float2bfloat16_rn(0.f);
+        if (r < B && p < n) {
+            const int o = orders[(size_t)r * n + p];
+            v[k] = Eb[(size_t)o * d + j];
+            if (inv && j == 0) inv[(size_t)r * 64 + o] = (uint8_t)p;
+        }
     }
-    X[idx] = v;
-    if (XT) XT[(size_t)col * Mp + r] = v;
+    store_tile(tile, v, r0, c0, X, ndp, XT, Mp);
 }
 
-// Z += bias; H = bf16(relu(Z)) (rows >= B -> 0); HT optional
-__global__ void k_bias_relu(float* __restrict__ Z, const float* __restrict__ bias, int Mp, int N, int B,
-                            bf16* __restrict__ H, bf16* __restrict__ HT)
+// Z = the product + bias; H = bf16(relu(Z)) (rows >= B -> 0); HT optional
+__global__ void __launch_bounds__(256) k_bias_relu(Product in, float* __restrict__ Z, const float* __restrict__ bias,
+                                                   int Mp, int N, int B, bf16* __restrict__ H, bf16* __restrict__ HT)
 {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)Mp * N) return;
-    const int r = (int)(idx / N), c = (int)(idx - (int64_t)r * N);
-    const float z = Z[idx] + bias[c];
-    Z[idx] = z;
-    const bf16 h = __float2bfloat16_rn(r < B ? fmaxf(z, 0.f) : 0.f);
-    H[idx] = h;
-    if (HT) HT[(size_t)c * Mp + r] = h;
+    __shared__ bf16 tile[32][33];
+    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, c = c0 + threadIdx.x;
+    bf16 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = r0 + threadIdx.y + 8 * k;
+        const int64_t idx = (int64_t)r * N + c;
+        const float z = in.at(idx) + bias[c];
+        Z[idx] = z;
+        v[k] = __float2bfloat16_rn(r < B ? fmaxf(z, 0.f) : 0.f);
+    }
+    store_tile(tile, v, r0, c0, H, N, HT, Mp);
 }
 
-__global__ void k_bias(float* __restrict__ Z, const float* __restrict__ bias, int Mp, int N)
+// Z = the product + bias; for training the rest of the grid clears the output layer's
+// gradients (only the rows of the batch's pairs are written later)
+__global__ void __launch_bounds__(256) k_bias(Product in, float* __restrict__ Z, const float* __restrict__ bias, int Mp,
+                                              int N, float4* __restrict__ zero, int64_t zeros)
 {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)Mp * N) return;
-    Z[idx] += bias[idx % N];
+    const int64_t tot = (int64_t)Mp * N;
+    if (idx < tot) Z[idx] = in.at(idx) + bias[idx % N];
+    else if (idx - tot < zeros) zero[idx - tot] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // output layer gradient of the BCE loss (one logit per row): block per row.  The row's
@@ -255,100 +331,208 @@ __global__ void k_out_grad(const float* __restrict__ L, int ldl, const uint32_t*
     }
 }
 
-// gW3 and gb3 rows of the pairs the batch touches: the block of the first row holding a
-// pair sums that pair's rows in row order (the other rows of the pair leave it)
-__global__ void k_out_grad_w(const uint32_t* __restrict__ pairs, const float* __restrict__ grow, int B, int H,
-                             const bf16* __restrict__ H2, float* __restrict__ gW3, float* __restrict__ gb3)
+// Column sums over the first B rows of a bf16 matrix (a bias gradient), 32 columns a block:
+// the rows come in side by side through shared memory, each column adds them in row order.
+static constexpr int CS_ROWS = 128;
+__device__ __forceinline__ void colsum_block(float (&s_t)[CS_ROWS][33], const bf16* __restrict__ M, int N, int B, int c0,
+                                             float* __restrict__ out)
 {
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    float s = 0.f;
+    for (int r0 = 0; r0 < B; r0 += CS_ROWS) {
+        const int rows = min(CS_ROWS, B - r0);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < CS_ROWS / 8; ++k) {
+            const int r = y + 8 * k;
+            if (r < rows) s_t[r][x] = __bfloat162float(M[(size_t)(r0 + r) * N + c0 + x]);
+        }
+        __syncthreads();
+        if (y == 0) {
+#pragma unroll 8
+            for (int r = 0; r < rows; ++r) s += s_t[r][x];
+        }
+    }
+    if (y == 0) out[c0 + x] = s;
+}
+
+// What follows from the output layer's row gradients, one launch: blocks below B the gW3 and
+// gb3 rows of the pairs the batch touches (the block of the first row holding a pair sums
+// that pair's rows in row order, the others of the pair leave it), then H / 32 blocks the
+// column sums of dZ2 (gb2), the last block the batch loss (per thread a strided run, then a
+// fixed shared-memory tree).
+__global__ void __launch_bounds__(256) k_out_sums(const uint32_t* __restrict__ pairs, const float* __restrict__ grow,
+                                                  const float* __restrict__ lrow, int B, int H,
+                                                  const bf16* __restrict__ H2, const bf16* __restrict__ dZ2,
+                                                  float* __restrict__ gW3, float* __restrict__ gb3,
+                                                  float* __restrict__ gb2, float* __restrict__ loss)
+{
+    __shared__ float s_t[CS_ROWS][33];
+    __shared__ int s_list[256];
+    __shared__ int s_w[8];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if ((int)blockIdx.x >= B + H / 32) {
+        float* red = &s_t[0][0];
+        float s = 0.f;
+        for (int r = tid; r < B; r += 256) s += lrow[r];
+        red[tid] = s;
+        __syncthreads();
+        for (int w = 128; w > 0; w >>= 1) {
+            if (tid < w) red[tid] += red[tid + w];
+            __syncthreads();
+        }
+        if (tid == 0) *loss = red[0];
+        return;
+    }
+    if ((int)blockIdx.x >= B) {
+        colsum_block(s_t, dZ2, H, B, ((int)blockIdx.x - B) * 32, gb2);
+        return;
+    }
     const int r = blockIdx.x;
     const uint32_t p = pairs[r];
     bool dup = false;
-    for (int q = threadIdx.x; q < r; q += blockDim.x) dup |= pairs[q] == p;
+    for (int q = tid; q < r; q += 256) dup |= pairs[q] == p;
     if (__syncthreads_or(dup)) return;                                  // block-uniform
-    for (int c = threadIdx.x; c < H; c += blockDim.x) {
+    float sb = 0.f;
+    for (int c0 = 0; c0 < H; c0 += 256) {
+        const int c = c0 + tid;
         float s = 0.f;
-        for (int q = r; q < B; ++q)
-            if (pairs[q] == p) s += grow[q] * __bfloat162float(H2[(size_t)q * H + c]);
-        gW3[(size_t)p * H + c] = s;
+        for (int q0 = r; q0 < B; q0 += 256) {
+            // this chunk's rows of the pair, in row order
+            const bool hit = q0 + tid < B && pairs[q0 + tid] == p;
+            const unsigned bal = __ballot_sync(0xffffffffu, hit);
+            if (lane == 0) s_w[warp] = __popc(bal);
+            __syncthreads();
+            int before = 0, cnt = 0;
+            for (int w = 0; w < 8; ++w) {
+                before += w < warp ? s_w[w] : 0;
+                cnt += s_w[w];
+            }
+            if (hit) s_list[before + __popc(bal & ((1u << lane) - 1u))] = q0 + tid;
+            __syncthreads();
+            for (int k = 0; k < cnt; ++k) {
+                const int q = s_list[k];
+                if (c < H) s += grow[q] * __bfloat162float(H2[(size_t)q * H + c]);
+                if (c0 == 0 && tid == 0) sb += grow[q];
+            }
+            __syncthreads();
+        }
+        if (c < H) gW3[(size_t)p * H + c] = s;
     }
-    if (threadIdx.x == 0) {
-        float s = 0.f;
-        for (int q = r; q < B; ++q)
-            if (pairs[q] == p) s += grow[q];
-        gb3[p] = s;
-    }
-}
-
-// the batch loss: the rows' terms in a fixed order (per thread a strided run, then a
-// fixed shared-memory tree)
-__global__ void k_loss_sum(const float* __restrict__ lrow, int B, float* __restrict__ loss)
-{
-    __shared__ float red[256];
-    float s = 0.f;
-    for (int r = threadIdx.x; r < B; r += 256) s += lrow[r];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *loss = red[0];
+    if (tid == 0) gb3[p] = sb;
 }
 
 // dZ = bf16(dH * (Z > 0)), rows >= B -> 0, with the transposed copy
-__global__ void k_relu_grad(const float* __restrict__ dH, const float* __restrict__ Z, int Mp, int N, int B,
-                            bf16* __restrict__ dZ, bf16* __restrict__ dZT)
+__global__ void __launch_bounds__(256) k_relu_grad(Product dH, const float* __restrict__ Z, int Mp, int N, int B,
+                                                   bf16* __restrict__ dZ, bf16* __restrict__ dZT)
 {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)Mp * N) return;
-    const int r = (int)(idx / N), c = (int)(idx - (int64_t)r * N);
-    const bf16 v = __float2bfloat16_rn((r < B && Z[idx] > 0.f) ? dH[idx] : 0.f);
-    dZ[idx] = v;
-    dZT[(size_t)c * Mp + r] = v;
+    __shared__ bf16 tile[32][33];
+    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+    bf16 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = r0 + threadIdx.y + 8 * k;
+        const int64_t idx = (int64_t)r * N + c0 + threadIdx.x;
+        v[k] = __float2bfloat16_rn((r < B && Z[idx] > 0.f) ? dH.at(idx) : 0.f);
+    }
+    store_tile(tile, v, r0, c0, dZ, N, dZT, Mp);
 }
 
-// column sums over the first B rows of a bf16 matrix (bias gradients)
-__global__ void k_colsum(const bf16* __restrict__ M, int N, int B, float* __restrict__ out)
+// Blocks below n * ceil(d / 32): dE[v][j] = sum over the rows r, in row order, of
+// dX[r][inv_r(v) d + j], 32 columns j of one node a block, the rows side by side through
+// shared memory as in colsum_block.  The rest: the column sums of dZ1 (gb1).
+__global__ void __launch_bounds__(256) k_embed_grad(const uint8_t* __restrict__ inv, Product dX, int B, int n, int d,
+                                                    int ndp, float* __restrict__ gE, const bf16* __restrict__ dZ1, int H,
+                                                    float* __restrict__ gb1)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
+    __shared__ float s_t[CS_ROWS][33];
+    const int jb = (d + 31) / 32;
+    if ((int)blockIdx.x >= n * jb) {
+        colsum_block(s_t, dZ1, H, B, ((int)blockIdx.x - n * jb) * 32, gb1);
+        return;
+    }
+    const int v = blockIdx.x / jb, j = (blockIdx.x - v * jb) * 32 + (threadIdx.x & 31), x = threadIdx.x & 31,
+              y = threadIdx.x >> 5;
     float s = 0.f;
-    for (int r = 0; r < B; ++r) s += __bfloat162float(M[(size_t)r * N + c]);
-    out[c] = s;
-}
-
-// inverse of each order: inv[r * 64 + v] = position of node v in order r
-__global__ void k_inv_orders(const uint8_t* __restrict__ orders, int n, uint8_t* __restrict__ inv)
-{
-    const int r = blockIdx.x, p = threadIdx.x;
-    if (p < n) inv[(size_t)r * 64 + orders[(size_t)r * n + p]] = (uint8_t)p;
-}
-
-// dE[v][j] = sum over the rows r, in row order, of dX[r][inv_r(v) d + j]
-__global__ void k_embed_grad(const uint8_t* __restrict__ inv, const float* __restrict__ dX, int B, int n, int d,
-                             int ndp, float* __restrict__ gE)
-{
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * d) return;
-    const int v = idx / d, j = idx - v * d;
-    float s = 0.f;
-    for (int r = 0; r < B; ++r) s += dX[(size_t)r * ndp + (size_t)inv[(size_t)r * 64 + v] * d + j];
-    gE[idx] = s;
+    for (int r0 = 0; r0 < B; r0 += CS_ROWS) {
+        const int rows = min(CS_ROWS, B - r0);
+        __syncthreads();
+        int at[CS_ROWS / 8];
+#pragma unroll
+        for (int k = 0; k < CS_ROWS / 8; ++k) {
+            const int r = y + 8 * k;
+            at[k] = r < rows ? inv[(size_t)(r0 + r) * 64 + v] : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < CS_ROWS / 8; ++k) {
+            const int r = y + 8 * k;
+            if (r < rows && j < d) s_t[r][x] = dX.at((int64_t)(r0 + r) * ndp + (int64_t)at[k] * d + j);
+        }
+        __syncthreads();
+        if (y == 0) {
+#pragma unroll 8
+            for (int r = 0; r < rows; ++r) s += s_t[r][x];
+        }
+    }
+    if (y == 0 && j < d) gE[(size_t)v * d + j] = s;
 }
 
 // Adam (Kingma & Ba): moments and the FP32 master weight
-__global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, int64_t count, float lr, float b1, float b2, float eps, float c1,
-                       float c2)
+struct AdamRates {
+    float lr, b1, b2, eps, c1, c2;
+};
+__device__ __forceinline__ float adam_at(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
+                                         float* __restrict__ v, int64_t i, const AdamRates& R)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
+    // (the fused multiply-adds written out, so that inlining cannot change which is fused)
     const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+    const float mi = __fmaf_rn(1.f - R.b1, gi, __fmul_rn(R.b1, m[i]));
+    const float vi = __fmaf_rn(__fmul_rn(1.f - R.b2, gi), gi, __fmul_rn(R.b2, v[i]));
     m[i] = mi;
     v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float x = w[i] - R.lr * (mi / R.c1) / (sqrtf(vi / R.c2) + R.eps);
+    w[i] = x;
+    return x;
+}
+struct AdamTensor {
+    float *w, *g, *m, *v;
+    bf16 *b, *bT;               // bf16 copy and its transpose, or null
+    int rows, cols;             // tiled (bT): multiples of 32; else rows = 1, cols = elements
+    int blocks;                 // of this tensor, after those of the tensors before it
+};
+struct AdamArgs {
+    AdamTensor t[7];
+    AdamRates R;
+};
+
+// Every parameter in one launch, with the bf16 copies the GEMMs read: 1,024 elements a block,
+// W1 and W2 by 32 x 32 tiles for their transposes.  Bound by the weights' and moments'
+// traffic, 24 bytes a parameter and step; seven launches for the step and four for the
+// copies took 61 us of kernels at n = 60, H = 512, this one 18.
+__global__ void __launch_bounds__(256) k_adam(AdamArgs A)
+{
+    __shared__ bf16 tile[32][33];
+    int blk = blockIdx.x, k = 0;
+    while (blk >= A.t[k].blocks) blk -= A.t[k++].blocks;
+    const AdamTensor& T = A.t[k];
+    const int x = threadIdx.x, y = threadIdx.y;
+    if (T.bT) {
+        const int tc = T.cols / 32, r0 = blk / tc * 32, c0 = blk % tc * 32;
+        bf16 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            v[q] = __float2bfloat16_rn(adam_at(T.w, T.g, T.m, T.v, (int64_t)(r0 + y + 8 * q) * T.cols + c0 + x, A.R));
+        store_tile(tile, v, r0, c0, T.b, T.cols, T.bT, T.rows);
+        return;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t i = (int64_t)blk * 1024 + q * 256 + y * 32 + x;
+        if (i < T.cols) {
+            const float w = adam_at(T.w, T.g, T.m, T.v, i, A.R);
+            if (T.b) T.b[i] = __float2bfloat16_rn(w);
+        }
+    }
 }
 
 // bf16 copy of a rows x cols FP32 matrix (row stride ld), zero-padded to prow x pcol,
@@ -373,6 +557,16 @@ using namespace bn;
 // ---------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------
+// A B^T of the network's buffers, left in partials where K is split
+static int gemm_part(bn_mlp* m, const bf16* A, int lda, const bf16* B, int ldb, float* C, int ldc, int M, int N, int K,
+                     cudaStream_t s, Product* out)
+{
+    const int split = gemm_split(M, N, K, m->ws_elems);
+    const GemmArgs g{A, B, split > 1 ? m->ws : C, M, N, K, lda, ldb, split > 1 ? N : ldc, split, m->status};
+    *out = Product{g.C, split, (int64_t)M * N};
+    return gemm_launch(g, nullptr, s);
+}
+
 static int mlp_refresh_bf16(bn_mlp* m, cudaStream_t s)
 {
     k_to_bf16<<<nblk((int64_t)m->n * m->d), 256, 0, s>>>(m->E, m->d, m->n, m->d, m->n, m->d, m->Eb, nullptr);
@@ -387,60 +581,79 @@ static int mlp_refresh_bf16(bn_mlp* m, cudaStream_t s)
     return BN_OK;
 }
 
-// forward of B <= cap orders already staged in m->orders_dev
-int bn::mlp_forward_dev(bn_mlp* m, const uint8_t* d_orders, int B, bool keep_transposes, cudaStream_t s)
+static dim3 tiles_of(int rows, int cols) { return dim3((unsigned)(cols / 32), (unsigned)(rows / 32)); }
+static const dim3 TILE(32, 8);
+
+// forward of B <= cap orders; `train` also leaves the transposed operands and the inverse
+// orders, and clears the output layer's gradients
+static int mlp_forward(bn_mlp* m, const uint8_t* d_orders, int B, bool train, cudaStream_t s)
 {
-    const int Mp = (int)round_up(std::max(B, 1), 128);
+    const int Mp = (int)round_up(std::max(B, 1), 128), H = m->H;
     if (Mp > m->cap) return set_error(BN_EINVAL, "mlp: batch %d above capacity %d", B, m->cap);
     m->Mp = Mp;
-    k_embed<<<nblk((int64_t)Mp * m->ndp), 256, 0, s>>>(d_orders, B, m->n, m->d, m->ndp, Mp, m->Eb, m->X,
-                                                      keep_transposes ? m->XT : nullptr);
+    k_embed<<<tiles_of(Mp, m->ndp), TILE, 0, s>>>(d_orders, B, m->n, m->d, m->ndp, Mp, m->Eb, m->X, train ? m->XT : nullptr,
+                                                 train ? m->inv : nullptr);
     BN_LAUNCH_CHECK("k_embed");
     int rc;
-    if ((rc = gemm_tc(m->X, m->ndp, m->W1b, m->ndp, m->Z1, m->H, Mp, m->H, m->ndp, m->status, s, m->ws, m->ws_elems))) return rc;
-    k_bias_relu<<<nblk((int64_t)Mp * m->H), 256, 0, s>>>(m->Z1, m->b1, Mp, m->H, B, m->H1,
-                                                        keep_transposes ? m->H1T : nullptr);
+    Product z;
+    if ((rc = gemm_part(m, m->X, m->ndp, m->W1b, m->ndp, m->Z1, H, Mp, H, m->ndp, s, &z))) return rc;
+    k_bias_relu<<<tiles_of(Mp, H), TILE, 0, s>>>(z, m->Z1, m->b1, Mp, H, B, m->H1, train ? m->H1T : nullptr);
     BN_LAUNCH_CHECK("k_bias_relu");
-    if ((rc = gemm_tc(m->H1, m->H, m->W2b, m->H, m->Z2, m->H, Mp, m->H, m->H, m->status, s, m->ws, m->ws_elems))) return rc;
-    k_bias_relu<<<nblk((int64_t)Mp * m->H), 256, 0, s>>>(m->Z2, m->b2, Mp, m->H, B, m->H2, nullptr);
+    if ((rc = gemm_part(m, m->H1, H, m->W2b, H, m->Z2, H, Mp, H, H, s, &z))) return rc;
+    k_bias_relu<<<tiles_of(Mp, H), TILE, 0, s>>>(z, m->Z2, m->b2, Mp, H, B, m->H2, nullptr);
     BN_LAUNCH_CHECK("k_bias_relu");
-    if ((rc = gemm_tc(m->H2, m->H, m->W3b, m->H, m->L, m->Pp, Mp, m->Pp, m->H, m->status, s, m->ws, m->ws_elems))) return rc;
-    k_bias<<<nblk((int64_t)Mp * m->Pp), 256, 0, s>>>(m->L, m->b3, Mp, m->Pp);
+    if ((rc = gemm_part(m, m->H2, H, m->W3b, H, m->L, m->Pp, Mp, m->Pp, H, s, &z))) return rc;
+    // gW3 and gb3 lie side by side, in multiples of 256 bytes
+    const int64_t zeros = train ? ((m->gb3 + m->Pp) - m->gW3) / 4 : 0;
+    k_bias<<<nblk((int64_t)Mp * m->Pp + zeros), 256, 0, s>>>(z, m->L, m->b3, Mp, m->Pp, (float4*)m->gW3, zeros);
     BN_LAUNCH_CHECK("k_bias");
     return BN_OK;
+}
+
+int bn::mlp_forward_dev(bn_mlp* m, const uint8_t* d_orders, int B, cudaStream_t s)
+{
+    return mlp_forward(m, d_orders, B, false, s);
+}
+
+// A layer's weight gradient gW = dZT actT^T and input gradient dA = dZ WT^T, in one launch
+// unless the weight gradient's K is split (large batches)
+static int grad_pair(bn_mlp* m, const bf16* dZT, const bf16* actT, float* gW, int ldg, int cols, const bf16* dZ,
+                     const bf16* WT, float* dA, cudaStream_t s, Product* out)
+{
+    const int Mp = m->Mp, H = m->H;
+    if (gemm_split(H, cols, Mp, m->ws_elems) > 1) {
+        int rc = gemm_tc(dZT, Mp, actT, Mp, gW, ldg, H, cols, Mp, m->status, s, m->ws, m->ws_elems);
+        if (rc) return rc;
+        return gemm_part(m, dZ, H, WT, H, dA, cols, Mp, cols, H, s, out);
+    }
+    const GemmArgs a{dZT, actT, gW, H, cols, Mp, Mp, Mp, ldg, 1, m->status};
+    const int split = gemm_split(Mp, cols, H, m->ws_elems);
+    const GemmArgs b{dZ, WT, split > 1 ? m->ws : dA, Mp, cols, H, H, H, cols, split, m->status};
+    *out = Product{b.C, split, (int64_t)Mp * cols};
+    return gemm_launch(a, &b, s);
 }
 
 int bn::mlp_loss_grad_dev(bn_mlp* m, const uint8_t* d_orders, const uint32_t* d_pairs, const float* d_alpha, int B,
                           cudaStream_t s)
 {
-    int rc = mlp_forward_dev(m, d_orders, B, true, s);
+    int rc = mlp_forward(m, d_orders, B, true, s);
     if (rc) return rc;
     const int Mp = m->Mp, H = m->H;
-    BN_CUDA(cudaMemsetAsync(m->gE, 0, sizeof(float) * (size_t)m->n * m->d, s));
-    BN_CUDA(cudaMemsetAsync(m->gW3, 0, sizeof(float) * (size_t)m->P * H, s));
-    BN_CUDA(cudaMemsetAsync(m->gb3, 0, sizeof(float) * (size_t)m->P, s));
     k_out_grad<<<Mp, 256, 0, s>>>(m->L, m->Pp, d_pairs, d_alpha, B, Mp, H, m->Z2, m->W3b, m->dZ2, m->dZ2T,
                                   m->grow, m->lrow);
     BN_LAUNCH_CHECK("k_out_grad");
-    k_out_grad_w<<<B, 256, 0, s>>>(d_pairs, m->grow, B, H, m->H2, m->gW3, m->gb3);
-    BN_LAUNCH_CHECK("k_out_grad_w");
-    k_loss_sum<<<1, 256, 0, s>>>(m->lrow, B, m->loss);
-    BN_LAUNCH_CHECK("k_loss_sum");
-    k_colsum<<<nblk(H), 256, 0, s>>>(m->dZ2, H, B, m->gb2);
-    BN_LAUNCH_CHECK("k_colsum");
+    k_out_sums<<<(unsigned)(B + H / 32 + 1), 256, 0, s>>>(d_pairs, m->grow, m->lrow, B, H, m->H2, m->dZ2, m->gW3, m->gb3,
+                                                        m->gb2, m->loss);
+    BN_LAUNCH_CHECK("k_out_sums");
+    Product dH, dX;
     // dW2 = dZ2^T H1 ; dH1 = dZ2 W2
-    if ((rc = gemm_tc(m->dZ2T, Mp, m->H1T, Mp, m->gW2, H, H, H, Mp, m->status, s, m->ws, m->ws_elems))) return rc;
-    if ((rc = gemm_tc(m->dZ2, H, m->W2T, H, m->dH1, H, Mp, H, H, m->status, s, m->ws, m->ws_elems))) return rc;
-    k_relu_grad<<<nblk((int64_t)Mp * H), 256, 0, s>>>(m->dH1, m->Z1, Mp, H, B, m->dZ1, m->dZ1T);
+    if ((rc = grad_pair(m, m->dZ2T, m->H1T, m->gW2, H, H, m->dZ2, m->W2T, m->dH1, s, &dH))) return rc;
+    k_relu_grad<<<tiles_of(Mp, H), TILE, 0, s>>>(dH, m->Z1, Mp, H, B, m->dZ1, m->dZ1T);
     BN_LAUNCH_CHECK("k_relu_grad");
-    k_colsum<<<nblk(H), 256, 0, s>>>(m->dZ1, H, B, m->gb1);
-    BN_LAUNCH_CHECK("k_colsum");
     // dW1 = dZ1^T X ; dX = dZ1 W1
-    if ((rc = gemm_tc(m->dZ1T, Mp, m->XT, Mp, m->gW1, m->ndp, H, m->ndp, Mp, m->status, s, m->ws, m->ws_elems))) return rc;
-    if ((rc = gemm_tc(m->dZ1, H, m->W1T, H, m->dX, m->ndp, Mp, m->ndp, H, m->status, s, m->ws, m->ws_elems))) return rc;
-    k_inv_orders<<<B, 64, 0, s>>>(d_orders, m->n, m->inv);
-    BN_LAUNCH_CHECK("k_inv_orders");
-    k_embed_grad<<<nblk((int64_t)m->n * m->d), 256, 0, s>>>(m->inv, m->dX, B, m->n, m->d, m->ndp, m->gE);
+    if ((rc = grad_pair(m, m->dZ1T, m->XT, m->gW1, m->ndp, m->ndp, m->dZ1, m->W1T, m->dX, s, &dX))) return rc;
+    k_embed_grad<<<(unsigned)(m->n * ((m->d + 31) / 32) + H / 32), 256, 0, s>>>(m->inv, dX, B, m->n, m->d, m->ndp, m->gE,
+                                                                              m->dZ1, H, m->gb1);
     BN_LAUNCH_CHECK("k_embed_grad");
     return BN_OK;
 }
@@ -449,21 +662,24 @@ int bn::mlp_adam_dev(bn_mlp* m, cudaStream_t s)
 {
     m->t += 1;
     const float c1 = 1.f - powf(m->beta1, (float)m->t), c2 = 1.f - powf(m->beta2, (float)m->t);
-    struct P {
-        float *w, *g, *mm, *vv;
-        int64_t cnt;
-    } ps[7] = {{m->E, m->gE, m->mE, m->vE, (int64_t)m->n * m->d},
-               {m->W1, m->gW1, m->mW1, m->vW1, (int64_t)m->H * m->ndp},
-               {m->b1, m->gb1, m->mb1, m->vb1, (int64_t)m->H},
-               {m->W2, m->gW2, m->mW2, m->vW2, (int64_t)m->H * m->H},
-               {m->b2, m->gb2, m->mb2, m->vb2, (int64_t)m->H},
-               {m->W3, m->gW3, m->mW3, m->vW3, (int64_t)m->P * m->H},
-               {m->b3, m->gb3, m->mb3, m->vb3, (int64_t)m->P}};
-    for (auto& p : ps) {
-        k_adam<<<nblk(p.cnt), 256, 0, s>>>(p.w, p.g, p.mm, p.vv, p.cnt, m->lr, m->beta1, m->beta2, m->adam_eps, c1, c2);
-        BN_LAUNCH_CHECK("k_adam");
-    }
-    return mlp_refresh_bf16(m, s);
+    auto flat = [](float* w, float* g, float* mm, float* v, bf16* b, int64_t cnt) {
+        return AdamTensor{w, g, mm, v, b, nullptr, 1, (int)cnt, (int)((cnt + 1023) / 1024)};
+    };
+    auto tiled = [](float* w, float* g, float* mm, float* v, bf16* b, bf16* bT, int rows, int cols) {
+        return AdamTensor{w, g, mm, v, b, bT, rows, cols, rows / 32 * (cols / 32)};
+    };
+    AdamArgs A{{tiled(m->W1, m->gW1, m->mW1, m->vW1, m->W1b, m->W1T, m->H, m->ndp),
+                tiled(m->W2, m->gW2, m->mW2, m->vW2, m->W2b, m->W2T, m->H, m->H),
+                flat(m->W3, m->gW3, m->mW3, m->vW3, m->W3b, (int64_t)m->P * m->H),
+                flat(m->E, m->gE, m->mE, m->vE, m->Eb, (int64_t)m->n * m->d),
+                flat(m->b1, m->gb1, m->mb1, m->vb1, nullptr, m->H), flat(m->b2, m->gb2, m->mb2, m->vb2, nullptr, m->H),
+                flat(m->b3, m->gb3, m->mb3, m->vb3, nullptr, m->P)},
+               {m->lr, m->beta1, m->beta2, m->adam_eps, c1, c2}};
+    int blocks = 0;
+    for (const AdamTensor& t : A.t) blocks += t.blocks;
+    k_adam<<<(unsigned)blocks, TILE, 0, s>>>(A);
+    BN_LAUNCH_CHECK("k_adam");
+    return BN_OK;
 }
 
 extern "C" int bn_mlp_create(int n, const bn_mlp_params* p, const float* E, const float* W1, const float* b1,
@@ -582,7 +798,7 @@ extern "C" int bn_mlp_forward(bn_mlp* m, const uint8_t* orders, int B, float* lo
     const void* d_o = nullptr;
     int rc = stage_in(m->stage_orders, orders, (size_t)B * m->n, mem, s, &d_o);
     if (rc) return rc;
-    if ((rc = mlp_forward_dev(m, (const uint8_t*)d_o, B, false, s))) return rc;
+    if ((rc = mlp_forward_dev(m, (const uint8_t*)d_o, B, s))) return rc;
     BN_CUDA(cudaMemcpy2DAsync(logits, 4 * (size_t)m->P, m->L, 4 * (size_t)m->Pp, 4 * (size_t)m->P, B,
                               mem == BN_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     return check_status(m, s, "bn_mlp_forward");

@@ -32,10 +32,8 @@ struct bn_mlp {
 };
 
 namespace bn {
-int gemm_tc(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, float* C, int ldc, int M, int N,
-            int K, uint32_t* status, cudaStream_t s, float* ws, size_t ws_elems);
 // forward of B orders (device pointer); logits land in m->L (row stride Pp)
-int mlp_forward_dev(bn_mlp* m, const uint8_t* d_orders, int B, bool keep_transposes, cudaStream_t s);
+int mlp_forward_dev(bn_mlp* m, const uint8_t* d_orders, int B, cudaStream_t s);
 int mlp_loss_grad_dev(bn_mlp* m, const uint8_t* d_orders, const uint32_t* d_pairs, const float* d_alpha, int B,
                       cudaStream_t s);
 int mlp_adam_dev(bn_mlp* m, cudaStream_t s);
