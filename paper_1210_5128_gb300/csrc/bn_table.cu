@@ -78,6 +78,53 @@ __global__ void k_pack(const uint8_t* __restrict__ data, int m, int n, int mw,
     packed[idx] = word;
 }
 
+// Per variable the rows that are not in its most frequent state, ascending, as row * 4 +
+// (the state's index among the others): one block a variable, states from the packed words.
+static constexpr int LIST_ROWS = 1 << 14;          // rows a 16-bit list entry can name
+__global__ void __launch_bounds__(256) k_minor_rows(const uint32_t* __restrict__ packed, int m, int mw,
+                                                    uint16_t* __restrict__ rows, uint32_t* __restrict__ len)
+{
+    __shared__ uint32_t s_cnt[4], s_w[8];
+    const int v = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t* D = packed + (size_t)v * mw;
+    auto state = [&](int r) { return (D[r >> 4] >> (8 * (r & 3) + 2 * ((r & 15) >> 2))) & 3u; };
+    if (tid < 4) s_cnt[tid] = 0;
+    __syncthreads();
+    uint32_t c[4] = {0, 0, 0, 0};
+    for (int r = tid; r < m; r += 256) {
+        const uint32_t x = state(r);
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q) c[q] += x == q;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t t = __reduce_add_sync(0xffffffffu, c[q]);
+        if (lane == 0 && t) atomicAdd(&s_cnt[q], t);
+    }
+    __syncthreads();
+    uint32_t mode = 0;
+    for (uint32_t q = 1; q < 4; ++q)
+        if (s_cnt[q] > s_cnt[mode]) mode = q;
+    uint32_t at = 0;
+    for (int r0 = 0; r0 < m; r0 += 256) {
+        const int r = r0 + tid;
+        const uint32_t x = r < m ? state(r) : mode;
+        const unsigned bal = __ballot_sync(0xffffffffu, x != mode);
+        if (lane == 0) s_w[warp] = __popc(bal);
+        __syncthreads();
+        uint32_t before = 0, all = 0;
+        for (int w = 0; w < 8; ++w) {
+            before += w < warp ? s_w[w] : 0u;
+            all += s_w[w];
+        }
+        if (x != mode)
+            rows[(size_t)v * m + at + before + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(r * 4 + x - (x > mode));
+        at += all;
+        __syncthreads();
+    }
+    if (tid == 0) len[v] = at;
+}
+
 // PPF of Eq. (10): ppf[i][m] = 100 (R[i][m] - 0.5)^3, evaluated left to right.
 __global__ void k_ppf(const double* __restrict__ R, int n, double* __restrict__ ppf)
 {
@@ -156,11 +203,13 @@ __global__ void k_pad_keys(int64_t* __restrict__ keys, int n, int64_t S, int64_t
 // once per set U of at most k + 1 nodes (k_joint) instead of once per (node, parent set):
 // C(60, 5) = 5.5 M tables instead of 29.4 M at n = 60, k = 4; k_assemble forms the entries.
 // Measured at n = 60, k = 4, m = 1000, ternary: 20.0 ms with one count table per entry,
-// 5.05 ms for k_joint and 0.51 ms for k_assemble.
+// 4.51 ms for k_joint and 0.51 ms for k_assemble.
 // ---------------------------------------------------------------------------------
 struct JointArgs {
     const uint32_t* packed;
-    int n, mw;
+    const uint16_t* minor;    // [n][m] rows not in the variable's most frequent state
+    const uint32_t* minor_len;
+    int n, m, mw;
     uint32_t pad;             // zero rows of the last word, all in cell 0
     int k;                    // largest parent set
     int64_t S0, S1;           // sets of at most k and of at most k + 1 of the n nodes
@@ -190,27 +239,71 @@ __device__ __forceinline__ fx128 warp_sum_fx(fx128 acc)
     return (fx128)s0 + ((fx128)s1 << 26) + ((fx128)s2 << 52) + ((fx128)s3 << 78) + ((fx128)s4 << 104);
 }
 
+// the lgamma terms of one cell count for the joint sum and, if the set is a parent set too,
+// for every variant of its configuration sum
+struct JointLuts {
+    const fx128* x;
+    const fx128* c[3];
+};
+template <bool PARENT>
+__device__ __forceinline__ void add_cell(uint32_t v, const JointLuts& L, int nv, fx128& g, fx128 (&h)[3])
+{
+    g += L.x[v];
+    if (PARENT) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (q < nv) h[q] += L.c[q][v];
+    }
+}
+
+// The counts of the cells hist[q * Qp + c] (q-th of the lowest node's RI - 1 minor states,
+// configuration c of the nodes above) and, as what is left of pre[c], of its most frequent
+// state.  Every cell read is set back to 0 for the next set.
+template <int RI, bool PARENT>
+__device__ __forceinline__ void minor_cells(uint32_t* hist, const uint32_t* pre, int Qp, const JointLuts& L, int nv,
+                                            int lane, fx128& g, fx128 (&h)[3])
+{
+    for (int c = lane; c < Qp; c += 32) {
+        uint32_t v[RI > 1 ? RI - 1 : 1], rest = pre[c];
+#pragma unroll
+        for (int q = 0; q < RI - 1; ++q) {
+            v[q] = hist[q * Qp + c];
+            rest -= v[q];
+        }
+#pragma unroll
+        for (int q = 0; q < RI - 1; ++q) {
+            hist[q * Qp + c] = 0u;
+            add_cell<PARENT>(v[q], L, nv, g, h);
+        }
+        add_cell<PARENT>(rest, L, nv, g, h);
+    }
+}
+
 // One warp per unit of `range` consecutive sets U (colex order: the lowest node varies
-// fastest).  A set's cell index of a row is base + state(lowest node) * Qp, where base
-// comes from the nodes above the lowest and Qp is the product of their arities; BASE keeps
-// the rows' bases (16 bits a row, scaled by 4) in shared memory while those nodes stay the
-// same (about 12 sets on average at n = 60, k = 4), so a row costs one shift, mask,
-// multiply-add and one shared atomic.  Four rows of a packed word make one item; items run
-// over the lanes, so the base reads are free of bank conflicts.  Shared memory holds the
-// warps' histograms, their bases, then (SMEM_DATA) the packed data.  Bound by the shared
-// atomics (one per row and set, conflicts on a table's frequent cells) and the issue slots.
-template <int KT, bool SMEM_DATA, bool BASE>
+// fastest).  MINOR keeps, while the nodes above the lowest stay the same (about 12 sets on
+// average at n = 60, k = 4), every row's configuration of them (16 bits a row, as a byte
+// offset) and the configurations' counts; a set then visits only the rows in which its
+// lowest node is not in its most frequent state -- about half -- and the frequent state's
+// cells are what is left of the configurations' counts.  A visit is two 16-bit loads (the
+// list ascends, so the second is nearly consecutive over the lanes), a multiply-add and a
+// shared atomic; the hottest cells take no atomics at all.  Without MINOR (more rows than a
+// list entry names, or no room) every row's cell is formed from all nodes.  Shared memory
+// holds the warps' histograms, the rows' offsets (MINOR), then (SMEM_DATA) the packed data.
+// n = 60, k = 4, m = 1000: 4.51 ms against 5.05 with every row visited; 628 warp
+// instructions a set at two thirds of the issue slots, and the shared-memory pipe 72 % busy
+// with atomics (a third of it) and the lgamma lookups.
+template <int KT, bool SMEM_DATA, bool MINOR>
 __global__ void __launch_bounds__(BUILD_THREADS) k_joint(JointArgs A)
 {
     extern __shared__ __align__(16) uint32_t sm[];
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int items = A.mw * 4;
+    const int items = A.mw * 4;                 // of four rows
     uint32_t* hist = sm + warp * A.cells_cap;
-    uint2* base = (uint2*)(sm + nw * A.cells_cap) + (BASE ? warp * items : 0);
+    uint2* base = (uint2*)(sm + nw * A.cells_cap) + (MINOR ? warp * items : 0);
     const uint32_t* D = A.packed;
     for (int c = lane; c < A.cells_cap; c += 32) hist[c] = 0u;
     if (SMEM_DATA) {
-        uint32_t* sd = sm + nw * A.cells_cap + (BASE ? nw * items * 2 : 0);
+        uint32_t* sd = sm + nw * A.cells_cap + (MINOR ? nw * items * 2 : 0);
         for (int t = threadIdx.x; t < A.n * A.mw; t += blockDim.x) sd[t] = A.packed[t];
         D = sd;
     }
@@ -223,15 +316,19 @@ __global__ void __launch_bounds__(BUILD_THREADS) k_joint(JointArgs A)
         int j;
         uint64_t mask;
         unrank_dev(A.n, r0, j, mask);
-        uint64_t above = ~0ull;                 // the nodes above the lowest `base` is for
+        uint64_t above = ~0ull;                 // the nodes above the lowest that `base` is for
         int poff[KT];
         uint32_t cs[KT];
         int Qp = 1;
+        uint32_t* pre = hist;                   // (MINOR) configuration counts, the histogram's last Qp words
         fx128 my_acc = 0;
         for (int64_t rho = r0; rho < r1; ++rho) {
             const uint64_t up = mask & (mask - 1);
             if (up != above) {                  // (warp-uniform)
                 above = up;
+                if (MINOR) {
+                    for (int c = lane; c < Qp; c += 32) pre[c] = 0u;
+                }
                 Qp = 1;
                 uint64_t mm = up;
 #pragma unroll
@@ -246,73 +343,100 @@ __global__ void __launch_bounds__(BUILD_THREADS) k_joint(JointArgs A)
                         Qp *= __ldg(&A.arity[p]);
                     }
                 }
-                if (BASE) {
+                if (MINOR) {
+                    pre = hist + A.cells_cap - Qp;
+                    uint8_t* pb = (uint8_t*)pre;
                     __syncwarp();
                     for (int c = lane; c < items; c += 32) {
                         const int w = c >> 2, sft = 2 * (c & 3);
-                        uint2 b = make_uint2(0u, 0u);
+                        uint32_t e = 0u, o = 0u;             // rows 4 c, 4 c + 2 and 4 c + 1, 4 c + 3
 #pragma unroll
                         for (int t = 0; t < KT; ++t) {
                             const uint32_t x = D[poff[t] + w] >> sft;
-                            b.x += (x & 0x00030003u) * cs[t];
-                            b.y += ((x >> 8) & 0x00030003u) * cs[t];
+                            e += (x & 0x00030003u) * cs[t];
+                            o += ((x >> 8) & 0x00030003u) * cs[t];
                         }
-                        base[c] = b;
+                        base[c] = make_uint2(__byte_perm(e, o, 0x5410), __byte_perm(e, o, 0x7632));
+                        atomicAdd((uint32_t*)(pb + (e & 0xffffu)), 1u);
+                        atomicAdd((uint32_t*)(pb + (e >> 16)), 1u);
+                        atomicAdd((uint32_t*)(pb + (o & 0xffffu)), 1u);
+                        atomicAdd((uint32_t*)(pb + (o >> 16)), 1u);
                     }
+                    __syncwarp();
+                    if (lane == 0) pre[0] -= A.pad;
                     __syncwarp();
                 }
             }
             const int low = mask ? __ffsll((long long)mask) - 1 : 0;
+            const int ri = mask ? (int)__ldg(&A.arity[low]) : 1;
+            const int Q = Qp * ri;
             const uint32_t scale = mask ? (uint32_t)(4 * Qp) : 0u;
-            const int Q = mask ? Qp * (int)__ldg(&A.arity[low]) : 1;
-            const uint32_t* Dl = D + (size_t)low * A.mw;
+            if (MINOR) {
+                const uint16_t* L = A.minor + (size_t)low * A.m;
+                const int len = mask ? (int)__ldg(&A.minor_len[low]) : 0;
+                const uint16_t* rowoff = (const uint16_t*)base;
 #pragma unroll 4
-            for (int c = lane; c < items; c += 32) {
-                const int w = c >> 2, sft = 2 * (c & 3);
-                uint2 b;
-                if (BASE) b = base[c];
-                else {
-                    b = make_uint2(0u, 0u);
+                for (int i = lane; i < len; i += 32) {
+                    const uint32_t e = __ldg(L + i);
+                    const uint32_t off = rowoff[e >> 2] + (e & 3u) * scale;
+                    atomicAdd((uint32_t*)(hb + off), 1u);
+                }
+            } else {
+                const uint32_t* Dl = D + (size_t)low * A.mw;
+                for (int c = lane; c < items; c += 32) {
+                    const int w = c >> 2, sft = 2 * (c & 3);
+                    const uint32_t x = Dl[w] >> sft;
+                    uint32_t e = (x & 0x00030003u) * scale, o = ((x >> 8) & 0x00030003u) * scale;
 #pragma unroll
                     for (int t = 0; t < KT; ++t) {
                         const uint32_t y = D[poff[t] + w] >> sft;
-                        b.x += (y & 0x00030003u) * cs[t];
-                        b.y += ((y >> 8) & 0x00030003u) * cs[t];
+                        e += (y & 0x00030003u) * cs[t];
+                        o += ((y >> 8) & 0x00030003u) * cs[t];
                     }
+                    atomicAdd((uint32_t*)(hb + (e & 0xffffu)), 1u);
+                    atomicAdd((uint32_t*)(hb + (e >> 16)), 1u);
+                    atomicAdd((uint32_t*)(hb + (o & 0xffffu)), 1u);
+                    atomicAdd((uint32_t*)(hb + (o >> 16)), 1u);
                 }
-                const uint32_t x = Dl[w] >> sft;
-                b.x += (x & 0x00030003u) * scale;
-                b.y += ((x >> 8) & 0x00030003u) * scale;
-                atomicAdd((uint32_t*)(hb + (b.x & 0xffffu)), 1u);
-                atomicAdd((uint32_t*)(hb + (b.x >> 16)), 1u);
-                atomicAdd((uint32_t*)(hb + (b.y & 0xffffu)), 1u);
-                atomicAdd((uint32_t*)(hb + (b.y >> 16)), 1u);
+                __syncwarp();
+                if (lane == 0 && A.pad) hist[0] -= A.pad;
             }
             __syncwarp();
-            if (lane == 0 && A.pad) hist[0] -= A.pad;
-            __syncwarp();
-            // every cell read is set back to 0 for the next set
-            const fx128* Lx = A.lut + (size_t)A.cell_lut[Q] * A.lut_stride;
-            fx128 acc = 0;
-            if (j > A.k) {
+            JointLuts L;
+            L.x = A.lut + (size_t)A.cell_lut[Q] * A.lut_stride;
+            fx128 acc = 0, h[3] = {0, 0, 0};
+            const bool parent = j <= A.k;       // a parent set too
+            if (parent) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (q < A.nv) L.c[q] = A.lut + (size_t)A.cfg_lut[Q * A.nv + q] * A.lut_stride;
+            }
+            if (MINOR) {
+                if (parent) {
+                    if (ri == 1) minor_cells<1, true>(hist, pre, Qp, L, A.nv, lane, acc, h);
+                    else if (ri == 2) minor_cells<2, true>(hist, pre, Qp, L, A.nv, lane, acc, h);
+                    else if (ri == 3) minor_cells<3, true>(hist, pre, Qp, L, A.nv, lane, acc, h);
+                    else minor_cells<4, true>(hist, pre, Qp, L, A.nv, lane, acc, h);
+                } else {
+                    if (ri == 2) minor_cells<2, false>(hist, pre, Qp, L, A.nv, lane, acc, h);
+                    else if (ri == 3) minor_cells<3, false>(hist, pre, Qp, L, A.nv, lane, acc, h);
+                    else minor_cells<4, false>(hist, pre, Qp, L, A.nv, lane, acc, h);
+                }
+            } else {
                 for (int c = lane; c < Q; c += 32) {
                     const uint32_t v = hist[c];
                     hist[c] = 0u;
-                    acc += Lx[v];
+                    if (parent) add_cell<true>(v, L, A.nv, acc, h);
+                    else add_cell<false>(v, L, A.nv, acc, h);
                 }
-            } else {                            // a parent set too: its configuration sums
-                for (int v = 0; v < A.nv; ++v) {
-                    const fx128* Lc = A.lut + (size_t)A.cfg_lut[Q * A.nv + v] * A.lut_stride;
-                    fx128 h = 0;
-                    for (int c = lane; c < Q; c += 32) h += Lc[hist[c]];
-                    h = warp_sum_fx(h);
-                    if (lane == 0) A.H[(size_t)v * A.S0 + rho] = h;
-                }
-                for (int c = lane; c < Q; c += 32) {
-                    const uint32_t v = hist[c];
-                    hist[c] = 0u;
-                    acc += Lx[v];
-                }
+            }
+            if (parent) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (q < A.nv) {
+                        h[q] = warp_sum_fx(h[q]);
+                        if (lane == 0) A.H[(size_t)q * A.S0 + rho] = h[q];
+                    }
             }
             acc = warp_sum_fx(acc);
             // lane (rho - r0) % 32 keeps the set's sum; 32 of them go out at once
@@ -324,6 +448,10 @@ __global__ void __launch_bounds__(BUILD_THREADS) k_joint(JointArgs A)
             }
             __syncwarp();
             next_set(A.n, j, mask);
+        }
+        if (MINOR) {
+            for (int c = lane; c < Qp; c += 32) pre[c] = 0u;
+            __syncwarp();
         }
     }
 }
@@ -507,11 +635,11 @@ struct Temps {
     ~Temps() { release(); }
 };
 
-template <int KT, bool SMEM_DATA, bool BASE>
+template <int KT, bool SMEM_DATA, bool MINOR>
 static int launch_joint(const JointArgs& A, size_t smem, int grid, int threads, cudaStream_t s)
 {
-    BN_CUDA(cudaFuncSetAttribute(k_joint<KT, SMEM_DATA, BASE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_joint<KT, SMEM_DATA, BASE><<<grid, threads, smem, s>>>(A);
+    BN_CUDA(cudaFuncSetAttribute(k_joint<KT, SMEM_DATA, MINOR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_joint<KT, SMEM_DATA, MINOR><<<grid, threads, smem, s>>>(A);
     BN_LAUNCH_CHECK("k_joint");
     return BN_OK;
 }
@@ -740,18 +868,21 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
     A.cell_lut = d_cell;
     A.cfg_lut = d_cfg;
     A.nv = P.nv;
+    A.m = m;
+    uint16_t* d_minor = nullptr;
+    uint32_t* d_len = nullptr;
     Temps sums(s);
     if ((rc = sums.get(&A.G, (size_t)A.S1)) || (rc = sums.get(&A.H, (size_t)A.S0 * P.nv))) return rc;
-    // Shared memory: the histograms, the row bases and the packed data as long as two blocks
-    // fit an SM with them; fewer warps a block, then no bases, when a block alone does not
-    // fit (counts of thousands of cells, tens of thousands of rows).
+    // Shared memory: the histograms, the rows' offsets and the packed data as long as two
+    // blocks fit an SM with them; fewer warps a block, then every row of every set, when a
+    // block alone does not fit (counts of thousands of cells).
     int nwarps = BUILD_THREADS / 32;
     const size_t data_bytes = sizeof(uint32_t) * (size_t)n * mw;
     const size_t per_hist = sizeof(uint32_t) * (size_t)A.cells_cap, per_base = (size_t)mw * 32;
     const size_t LIM = 220 * 1024;
-    bool base = true;
-    while (nwarps > 2 && nwarps * (per_hist + per_base) > LIM) nwarps /= 2;
-    if (nwarps * (per_hist + per_base) > LIM) {
+    bool base = m <= LIST_ROWS;
+    while (base && nwarps > 2 && nwarps * (per_hist + per_base) > LIM) nwarps /= 2;
+    if (!base || nwarps * (per_hist + per_base) > LIM) {
         base = false;
         nwarps = BUILD_THREADS / 32;
         while (nwarps > 1 && nwarps * per_hist > LIM) nwarps /= 2;
@@ -766,6 +897,13 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
     const int64_t units = (A.S1 + A.range - 1) / A.range;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count() * per_sm, (units + nwarps - 1) / nwarps));
     if (ev0) BN_CUDA(cudaEventRecord(ev0, s));
+    if (base) {
+        if ((rc = sums.get(&d_minor, (size_t)n * m)) || (rc = sums.get(&d_len, (size_t)n))) return rc;
+        k_minor_rows<<<n, 256, 0, s>>>(d_packed, m, mw, d_minor, d_len);
+        BN_LAUNCH_CHECK("k_minor_rows");
+    }
+    A.minor = d_minor;
+    A.minor_len = d_len;
     const int thr = 32 * nwarps;
     if (k <= 2) rc = launch_joint_kt<2>(A, smem_data, base, smem, grid, thr, s);
     else if (k <= 4) rc = launch_joint_kt<4>(A, smem_data, base, smem, grid, thr, s);
