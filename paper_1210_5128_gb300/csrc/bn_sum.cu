@@ -10,10 +10,21 @@
 // (order, node) comes from the max-based scan; then the entries are walked by sorted
 // position (score descending) from the best one down to m - D, D = log10(S 2^60) decades:
 // the entries below sum to less than S 10^-D = 2^-60 of the sum, 1/128 of its last bit, so
-// leaving their terms out changes the result by less than its rounding does.  A block owns a
-// chunk of a node's list and up to SUM_OB orders; blocks outside every order's window
-// leave at once.  The shift is the same for every partial sum of an (order, node), and the
-// partials merge in a fixed order, so results are deterministic for a given launch shape.
+// leaving their terms out changes the result by less than its rounding does.  A warp owns a
+// run of a node's list for up to SUM_OB orders; runs outside every order's window are
+// skipped.  Partials merge in a fixed order, so results are deterministic for a given
+// launch shape.
+//
+// The cost is the exponentials: most consistent entries lie within D of the best, and an
+// FP64 exp10 is some thirty instructions on a pipe that takes 64 cycles for a warp's one.  So
+// an entry's 10^(entry - ref) is formed once for all orders of the block, in 64-bit integer
+// arithmetic (exp10_fx), relative to the first entry ref of a stretch of the list no longer
+// than one decade; a consistent order adds it as an integer, and only the stretch's sums
+// are brought to FP64 and scaled by 10^(ref - m) -- one exp10 on eight lanes per 1,024
+// entries.  Every term is good to 2^-55 of itself, as from FP64.  Steps of 32 entries that
+// span more than a decade or two binades of scores (short lists, the ends of long ones)
+// take FP64 exponentials per (entry, order).  8 orders at n = 60: 484 us with one exp10 per
+// (entry, order), 208 so; 6.1 ms with every entry's.
 #include <algorithm>
 #include <cmath>
 
@@ -24,7 +35,6 @@ namespace bn {
 static constexpr int SUM_OB = 8;          // orders per block
 static constexpr int SUM_THREADS = 256;
 static constexpr int SUM_WARPS = SUM_THREADS / 32;
-static constexpr int SUM_CHUNK = 2048;    // sorted positions per block
 static constexpr int SUM_BATCH = 256;     // orders whose partials are held at a time
 
 struct SumScanArgs {
@@ -33,6 +43,7 @@ struct SumScanArgs {
     const uint32_t* srank;
     int64_t S, Sp;
     int n, B, b0, b1;                     // all orders; the batch [b0, b1)
+    int run;                              // sorted positions per warp (256 or 1,024)
     int nchunk;
     double reach;                         // D
     const uint64_t* list_pc;              // [n][B] candidate-space predecessor masks
@@ -45,19 +56,65 @@ __device__ __forceinline__ int64_t sorted_key(const SumScanArgs& A, int i, int64
     return A.keys[(size_t)i * A.Sp + A.srank[(size_t)i * A.Sp + p]];
 }
 
-// Terms wait in a short queue per (warp, order) so that the exponentials -- the cost of this
-// score: some forty FP64 operations each -- run on full warps: at n = 60 about one entry in
-// five is consistent with an order, and a warp takes the exponential for one lane as for 32.
+// 2^(-j / 64), 2^(-j / 4096) and 2^(-j / 262144), j < 64, with 63 fractional bits, from the
+// exponential series in integer arithmetic
+struct Exp2Tables {
+    uint64_t v[3][64];
+};
+constexpr uint64_t LN2_64 = 0xB17217F7D1CF79ACull;        // ln 2 in 2^-64
+constexpr uint64_t mulhi_c(uint64_t a, uint64_t b) { return (uint64_t)(((unsigned __int128)a * b) >> 64); }
+constexpr Exp2Tables make_exp2()
+{
+    Exp2Tables T{};
+    for (int t = 0; t < 3; ++t)
+        for (int j = 0; j < 64; ++j) {
+            // e^-z, z = ln 2 * j / 64^(t + 1), as sum (-z)^k / k! in 2^-64 with 128-bit sums
+            const uint64_t x = (uint64_t)j << (58 - 6 * t);                  // j / 64^(t + 1) in 2^-64
+            const uint64_t z = mulhi_c(x, LN2_64);
+            unsigned __int128 pos = (unsigned __int128)1 << 64, neg = 0;
+            uint64_t term = z;
+            for (int k = 1; k < 24; ++k) {
+                if (k & 1) neg += term;
+                else pos += term;
+                term = mulhi_c(term, z) / (uint64_t)(k + 1);
+            }
+            T.v[t][j] = (uint64_t)((pos - neg + 1) >> 1);
+        }
+    return T;
+}
+static __device__ const Exp2Tables g_exp2 = make_exp2();
+
+// 10^-d in 2^-58 for d in [0, 1] given in 2^-60: d log2 10 = whole + three table digits of
+// six bits + a rest below 2^-18, whose 2^-r = 1 - z + z^2 / 2 up to z^3 / 6 < 2^-58
+__device__ __forceinline__ uint64_t exp10_fx(uint64_t d, const uint64_t (&T)[3][64])
+{
+    constexpr uint64_t LOG2_10 = 0x6A4D3C25E68DC57Full;                      // log2 10 in 2^-61
+    const uint64_t y = __umul64hi(d, LOG2_10);                               // in 2^-57
+    const uint32_t whole = (uint32_t)(y >> 57);
+    const uint64_t t1 = T[0][(y >> 51) & 63], t2 = T[1][(y >> 45) & 63], t3 = T[2][(y >> 39) & 63];
+    const uint64_t r = y & ((1ull << 39) - 1);                               // in 2^-57, below 2^-18
+    const uint64_t z = __umul64hi(r << 25, LN2_64);                          // in 2^-82, below 2^63.5
+    const uint32_t zh = (uint32_t)(z >> 32);                                 // z in 2^-50
+    const uint64_t sq = (uint64_t)zh * zh;                                   // z^2 in 2^-100
+    // 1 - z + z^2 / 2 in 2^-63
+    const uint64_t e = (1ull << 63) - (z >> 19) + (sq >> 38);
+    uint64_t p = __umul64hi(t1, t2) << 1;                                    // 2^-63 each
+    p = __umul64hi(p, t3) << 1;
+    p = __umul64hi(p, e);                                                    // 2^-62
+    return (p >> 4) >> whole;                                                // 2^-58
+}
+
 __global__ void __launch_bounds__(SUM_THREADS) k_sum_window(SumScanArgs A)
 {
-    __shared__ double s_q[SUM_WARPS][SUM_OB][64];
+    __shared__ uint64_t s_T[3][64];
+    __shared__ double s_slow[SUM_WARPS][SUM_OB][32];      // FP64 terms of a lane's wide steps
     __shared__ uint64_t s_npc[SUM_OB];
     __shared__ int64_t s_thr[SUM_OB];
     __shared__ double s_m[SUM_OB], s_s[SUM_WARPS][SUM_OB];
     __shared__ uint32_t s_p0[SUM_OB];
     const int chunk = blockIdx.x, node = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int b0 = A.b0 + (int)blockIdx.z * SUM_OB, nb = min(SUM_OB, A.b1 - b0);
-    const int64_t e0 = (int64_t)chunk * SUM_CHUNK, e1 = min(e0 + SUM_CHUNK, A.S);
+    if (tid < 192) s_T[tid >> 6][tid & 63] = g_exp2.v[tid >> 6][tid & 63];
     if (tid < SUM_OB) {
         uint32_t p0 = SPOS_NONE;
         int64_t thr = 0x7fffffffffffffffLL;
@@ -65,13 +122,16 @@ __global__ void __launch_bounds__(SUM_THREADS) k_sum_window(SumScanArgs A)
         uint64_t npc = ~0ull;
         if (tid < nb) {
             const size_t at = (size_t)node * A.B + b0 + tid;
-            npc = ~A.list_pc[at];
             p0 = A.list_best[at];
             if ((int64_t)p0 >= A.S) p0 = SPOS_NONE;                     // only after a timed-out scan
             else m = key_to_double(sorted_key(A, node, p0));
             // (a best entry of -inf: every consistent one is, the sum stays empty)
-            if (m > -INFINITY) thr = double_to_key(__dsub_rn(m, A.reach));
-            else p0 = SPOS_NONE;
+            if (m > -INFINITY) {
+                thr = double_to_key(__dsub_rn(m, A.reach));
+                npc = ~A.list_pc[at];
+            } else {
+                p0 = SPOS_NONE;
+            }
         }
         s_npc[tid] = npc;
         s_p0[tid] = p0;
@@ -81,63 +141,103 @@ __global__ void __launch_bounds__(SUM_THREADS) k_sum_window(SumScanArgs A)
     __syncthreads();
     uint32_t first = SPOS_NONE;
     int64_t low = 0x7fffffffffffffffLL;
+    uint64_t npc[SUM_OB];
 #pragma unroll
     for (int b = 0; b < SUM_OB; ++b) {
         first = min(first, s_p0[b]);
         low = min(low, s_thr[b]);
+        npc[b] = s_npc[b];
     }
-    double acc[SUM_OB];
+    const int64_t e0 = ((int64_t)chunk * SUM_WARPS + warp) * A.run, e1 = min(e0 + A.run, A.S);
+    double acc = 0.0;                                     // lane b: order b's sum over this run
+    if (e0 < e1 && e1 > (int64_t)first && sorted_key(A, node, e0) >= low) {          // warp-uniform
+        const double my_m = lane < SUM_OB ? s_m[lane] : 0.0;
+        uint64_t sum[SUM_OB];
 #pragma unroll
-    for (int b = 0; b < SUM_OB; ++b) acc[b] = 0.0;
-    if (e1 > (int64_t)first && sorted_key(A, node, e0) >= low) {        // block-uniform
-        int cnt[SUM_OB];
-#pragma unroll
-        for (int b = 0; b < SUM_OB; ++b) cnt[b] = 0;
-        const uint32_t lt = (1u << lane) - 1u;
-        for (int64_t p = e0 + tid; p - lane < e1; p += SUM_THREADS) {
-            uint32_t ok = 0;
-            uint32_t r = 0;
-            if (p < e1) {
-                r = A.srank[(size_t)node * A.Sp + p];
-                const uint64_t mask = A.pst[r];
-#pragma unroll
-                for (int b = 0; b < SUM_OB; ++b)
-                    ok |= (uint32_t)((uint32_t)p >= s_p0[b] && (mask & s_npc[b]) == 0ull) << b;
-            }
-            const int64_t key = ok ? A.keys[(size_t)node * A.Sp + r] : KEY_NONE;
-            const double v = key_to_double(key);
+        for (int b = 0; b < SUM_OB; ++b) sum[b] = 0;
+        int64_t ref = 0;
+        int ref_exp = 0, held = 0;                        // steps summed relative to ref
+        bool slow_used = false;
+        // the stretch's sums over the warp, 22 bits at a time, to lane b's FP64 sum
+        auto flush = [&]() {
+            uint64_t mine = 0;
+            uint32_t top = 0;
 #pragma unroll
             for (int b = 0; b < SUM_OB; ++b) {
-                const bool take = ((ok >> b) & 1u) && key >= s_thr[b];
-                const uint32_t bal = __ballot_sync(0xffffffffu, take);
-                if (bal) {
-                    double* q = s_q[warp][b];
-                    if (take) q[cnt[b] + __popc(bal & lt)] = __dsub_rn(v, s_m[b]);
-                    cnt[b] += __popc(bal);
-                    if (cnt[b] >= 32) {
-                        __syncwarp();
-                        acc[b] += exp10(q[lane]);
-                        cnt[b] -= 32;
-                        const double rest = q[32 + lane];
-                        __syncwarp();
-                        if (lane < cnt[b]) q[lane] = rest;
-                        __syncwarp();
+                const uint32_t l0 = __reduce_add_sync(0xffffffffu, (uint32_t)sum[b] & 0x3fffffu);
+                const uint32_t l1 = __reduce_add_sync(0xffffffffu, (uint32_t)(sum[b] >> 22) & 0x3fffffu);
+                const uint32_t l2 = __reduce_add_sync(0xffffffffu, (uint32_t)(sum[b] >> 44));
+                if (lane == b) {
+                    mine = ((uint64_t)l1 << 22) + l0;
+                    top = l2;
+                }
+                sum[b] = 0;
+            }
+            if (lane < nb && my_m > -INFINITY) {
+                const double t = __fma_rn((double)top, 0x1p44, (double)mine) * 0x1p-58;
+                if (t != 0.0) acc += t * exp10(key_to_double(ref) - my_m);
+            }
+            held = 0;
+        };
+        for (int64_t p = e0 + lane; p - lane < e1; p += 32) {
+            uint32_t ok = 0;
+            int64_t key = KEY_NONE;
+            const bool in = p < e1;
+            if (in) {
+                const uint32_t r = A.srank[(size_t)node * A.Sp + p];
+                const uint64_t mask = A.pst[r];
+                key = A.keys[(size_t)node * A.Sp + r];
+#pragma unroll
+                for (int b = 0; b < SUM_OB; ++b) ok |= (uint32_t)((mask & npc[b]) == 0ull) << b;
+            }
+            if (!__any_sync(0xffffffffu, ok != 0)) continue;
+            const int last = (int)min((int64_t)31, e1 - 1 - (p - lane));
+            const int64_t k0 = __shfl_sync(0xffffffffu, key, 0), kl = __shfl_sync(0xffffffffu, key, last);
+            // one binade and at most a decade between k0 and kl: key differences are
+            // differences of the scores in units of their last place, 2^(exp - 1075)
+            const uint64_t bits0 = bits_from_key(k0), bitsl = bits_from_key(kl);
+            const int ex = (int)(bits0 >> 52) & 0x7ff;
+            const bool one = (bits0 >> 52) == (bitsl >> 52) && ex > 1015 && ex < 1075;
+            const uint64_t decade = 1ull << (1075 - min(max(ex, 1015), 1075));
+            if (one && (uint64_t)(k0 - kl) <= decade) {
+                const int se = (int)(bits0 >> 52);                           // sign and exponent
+                if (held && (held == 32 || se != ref_exp || (uint64_t)(ref - kl) > decade)) flush();
+                if (!held) {
+                    ref = k0;
+                    ref_exp = se;
+                }
+                ++held;
+                const uint64_t E = in ? exp10_fx((uint64_t)(ref - key) << (ex - 1015), s_T) : 0ull;
+#pragma unroll
+                for (int b = 0; b < SUM_OB; ++b)
+                    if ((ok >> b) & 1u) sum[b] += E;
+            } else {
+                if (!slow_used) {
+#pragma unroll
+                    for (int b = 0; b < SUM_OB; ++b) s_slow[warp][b][lane] = 0.0;
+                    slow_used = true;
+                }
+                // each lane its remaining orders in turn, those whose window holds the entry
+#pragma unroll
+                for (int b = 0; b < SUM_OB; ++b)
+                    if (key < s_thr[b]) ok &= ~(1u << b);
+                while (__any_sync(0xffffffffu, ok != 0)) {
+                    if (ok) {
+                        const int b = __ffs((int)ok) - 1;
+                        ok &= ok - 1;
+                        s_slow[warp][b][lane] += exp10(key_to_double(key) - s_m[b]);
                     }
                 }
             }
         }
-        __syncwarp();
-#pragma unroll
-        for (int b = 0; b < SUM_OB; ++b)
-            if (lane < cnt[b]) acc[b] += exp10(s_q[warp][b][lane]);
+        if (held) flush();
+        if (slow_used) {
+            __syncwarp();
+            if (lane < nb)
+                for (int l = 0; l < 32; ++l) acc += s_slow[warp][lane][l];
+        }
     }
-#pragma unroll
-    for (int b = 0; b < SUM_OB; ++b) {
-        double s = acc[b];
-#pragma unroll
-        for (int off = 16; off; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        if (lane == 0) s_s[warp][b] = s;
-    }
+    if (lane < SUM_OB) s_s[warp][lane] = acc;
     __syncthreads();
     if (tid < nb) {
         double s = 0.0;
@@ -146,29 +246,35 @@ __global__ void __launch_bounds__(SUM_THREADS) k_sum_window(SumScanArgs A)
     }
 }
 
-// One block an order: a warp per node sums the chunks (lane-strided, then a fixed tree), the
-// node terms, then their sum in ascending node id.
+// One block an order: a warp per node sums the chunks (lane-strided, then a fixed tree), a
+// thread per node takes the logarithm, one adds the node terms in ascending node id.
 __global__ void __launch_bounds__(SUM_THREADS) k_sum_finish(SumScanArgs A, double* __restrict__ node_score,
                                                             double* __restrict__ order_score)
 {
     __shared__ double s_v[MAXN];
-    const int b = A.b0 + blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b = A.b0 + blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    double top = 0.0;
+    if (tid < A.n) {
+        uint32_t best = A.list_best[(size_t)tid * A.B + b];
+        if ((int64_t)best >= A.S) best = 0;                            // only after a timed-out scan
+        top = key_to_double(sorted_key(A, tid, best));
+    }
     for (int i = warp; i < A.n; i += SUM_WARPS) {
         const double* p = A.part + ((size_t)i * (A.b1 - A.b0) + blockIdx.x) * A.nchunk;
         double s = 0.0;
         for (int c = lane; c < A.nchunk; c += 32) s += p[c];
 #pragma unroll
         for (int off = 16; off; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        if (lane == 0) {
-            uint32_t best = A.list_best[(size_t)i * A.B + b];
-            if ((int64_t)best >= A.S) best = 0;                        // only after a timed-out scan
-            const double v = key_to_double(sorted_key(A, i, best)) + log10(s);
-            s_v[i] = v;
-            if (node_score) node_score[(size_t)b * A.n + i] = v;
-        }
+        if (lane == 0) s_v[i] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0 && order_score) {
+    if (tid < A.n) {
+        const double v = top + log10(s_v[tid]);
+        s_v[tid] = v;
+        if (node_score) node_score[(size_t)b * A.n + tid] = v;
+    }
+    __syncthreads();
+    if (tid == 0 && order_score) {
         double total = 0.0;
         for (int i = 0; i < A.n; ++i) total += s_v[i];
         order_score[b] = total;
@@ -190,7 +296,9 @@ extern "C" int bn_score_orders_sum(const bn_table* t, const uint8_t* orders, int
     if (!orders) return set_error(BN_EINVAL, "bn_score_orders_sum: orders is NULL");
     cudaStream_t s = (cudaStream_t)stream;
     const int n = t->n;
-    const int nchunk = (int)((t->S + SUM_CHUNK - 1) / SUM_CHUNK);
+    // short runs where there are few: a warp's steps are its latency
+    const int run = t->S >= 65536 ? 1024 : 256;
+    const int nchunk = (int)((t->S + SUM_WARPS * run - 1) / (SUM_WARPS * run));
     const int batch = std::min(B, SUM_BATCH);
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -239,7 +347,7 @@ extern "C" int bn_score_orders_sum(const bn_table* t, const uint8_t* orders, int
     if (rc) return rc;
     const double reach = std::log10((double)t->S) + 60.0 * 0.30102999566398120;
     for (int b0 = 0; b0 < B; b0 += batch) {
-        SumScanArgs A{t->keys, t->pst, t->srank, t->S, t->Sp, n, B, b0, std::min(B, b0 + batch), nchunk, reach, d_pc,
+        SumScanArgs A{t->keys, t->pst, t->srank, t->S, t->Sp, n, B, b0, std::min(B, b0 + batch), run, nchunk, reach, d_pc,
                       d_best, d_part};
         const int groups = (A.b1 - b0 + SUM_OB - 1) / SUM_OB;
         k_sum_window<<<dim3((unsigned)nchunk, (unsigned)n, (unsigned)groups), SUM_THREADS, 0, s>>>(A);
