@@ -91,10 +91,13 @@ extern "C" int bn_score_orders_noalloc(const bn_table* t, const uint8_t* orders,
     // the array keeps the previous call's contents: the status word must start at zero;
     // counts, masks and per-item results are rewritten by k_pred_lists before use
     BN_CUDA(cudaMemsetAsync(d_status, 0, sizeof(uint32_t), s));
-    if ((rc = launch_pred_lists(orders, B, n, d_pc, d_best, d_cnt, d_status, s))) return rc;
-    rc = launch_scan_orders(t, B, d_cnt, d_pc, d_best, d_status, s);
-    if (rc) return rc;
-    if ((rc = launch_reduce_orders(t, d_best, B, best_rank, order_score, s))) return rc;
+    if (score_small_fits(t, B)) {
+        if ((rc = launch_score_small(t, orders, B, best_rank, order_score, d_status, s))) return rc;
+    } else {
+        if ((rc = launch_pred_lists(orders, B, n, d_pc, d_best, d_cnt, d_status, s))) return rc;
+        if ((rc = launch_scan_orders(t, B, d_cnt, d_pc, d_best, d_status, s))) return rc;
+        if ((rc = launch_reduce_orders(t, d_best, B, best_rank, order_score, s))) return rc;
+    }
     uint32_t st = 0;
     BN_CUDA(cudaMemcpyAsync(&st, d_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     BN_CUDA(cudaStreamSynchronize(s));

@@ -623,6 +623,39 @@ __global__ void k_tune_lists(int n, int items, uint64_t* list_pc, uint32_t* list
     list_best[idx] = SPOS_NONE;
 }
 
+// A warp's order: put(i, mask) for every node i, the candidate-space mask of the nodes before
+// it; lane l holds positions l and l + 32.  A row that is no permutation sets STATUS_BADINPUT.
+template <class F>
+__device__ __forceinline__ void order_masks(const uint8_t* __restrict__ o, int n, int lane, uint32_t* status, F put)
+{
+    const uint64_t full = (n == 64) ? ~0ull : ((1ull << n) - 1);
+    int v[2];
+    uint64_t bit[2], s[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int p = lane + 32 * h;
+        v[h] = p < n ? o[p] : MAXN;
+        bit[h] = s[h] = v[h] < n ? 1ull << v[h] : 0ull;
+    }
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint64_t t0 = __shfl_up_sync(0xffffffffu, s[0], d), t1 = __shfl_up_sync(0xffffffffu, s[1], d);
+        if (lane >= d) {
+            s[0] |= t0;
+            s[1] |= t1;
+        }
+    }
+    s[1] |= __shfl_sync(0xffffffffu, s[0], 31);
+    if (lane == 31 && s[1] != full) atomicOr(status, STATUS_BADINPUT);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (v[h] < n) {
+            const uint64_t pred = s[h] & ~bit[h];
+            const int i = v[h];
+            put(i, (pred & ((1ull << i) - 1)) | ((i + 1 < 64) ? ((pred >> (i + 1)) << i) : 0ull));
+        }
+}
+
 // a5: candidate-space predecessor masks, written straight into the node-major work lists
 // (item b of node i is order b); also checks each row is a permutation.  A block takes 32
 // orders: a warp per order reads it once and ORs prefixes by shuffles, and the masks go out
@@ -636,36 +669,8 @@ __global__ void __launch_bounds__(256) k_pred_lists(const uint8_t* __restrict__ 
     __shared__ uint64_t s_pc[MAXN][PL_ORDERS + 1];
     const int b0 = blockIdx.x * PL_ORDERS, nb = min(PL_ORDERS, B - b0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint64_t full = (n == 64) ? ~0ull : ((1ull << n) - 1);
     for (int q = warp; q < nb; q += 8) {
-        const uint8_t* o = orders + (size_t)(b0 + q) * n;
-        int v[2];
-        uint64_t bit[2], s[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int p = lane + 32 * h;
-            v[h] = p < n ? o[p] : MAXN;
-            bit[h] = s[h] = v[h] < n ? 1ull << v[h] : 0ull;
-        }
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint64_t t0 = __shfl_up_sync(0xffffffffu, s[0], d), t1 = __shfl_up_sync(0xffffffffu, s[1], d);
-            if (lane >= d) {
-                s[0] |= t0;
-                s[1] |= t1;
-            }
-        }
-        const uint64_t half = __shfl_sync(0xffffffffu, s[0], 31);
-        s[1] |= half;
-        if (lane == 31 && s[1] != full) atomicOr(status, STATUS_BADINPUT);
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-            if (v[h] < n) {
-                const uint64_t pred = s[h] & ~bit[h];
-                const int i = v[h];
-                const uint64_t lowm = (1ull << i) - 1;
-                s_pc[i][q] = (pred & lowm) | ((i + 1 < 64) ? ((pred >> (i + 1)) << i) : 0ull);
-            }
+        order_masks(orders + (size_t)(b0 + q) * n, n, lane, status, [&](int i, uint64_t pc) { s_pc[i][q] = pc; });
     }
     __syncthreads();
     for (int idx = threadIdx.x; idx < n * nb; idx += 256) {
@@ -715,6 +720,133 @@ __global__ void __launch_bounds__(256) k_reduce_orders(const uint32_t* __restric
     if (best_rank)
         for (int idx = threadIdx.x; idx < n * nb; idx += 256)
             best_rank[(size_t)b0 * n + idx] = s_rank[idx / n][idx % n];
+}
+
+// ---------------------------------------------------------------------------------
+// A whole call in one kernel where the scan itself is short: a pruned table, or the full
+// table of a small network.  A block takes up to 32 orders from predecessor masks to scores,
+// with no work lists in global memory: three dependent launches and their lists cost more
+// than the scan (one order of 13 nodes 30 us a call by three kernels, 22 by one; 4,096
+// orders of 60 nodes on a pruned table, host arrays, 79 and 74).
+// ---------------------------------------------------------------------------------
+static constexpr int SC_THREADS = 512;
+static constexpr int SC_WARPS = SC_THREADS / 32;
+
+struct ScoreArgs {
+    const uint8_t* orders;
+    int B, n, ob;                  // ob: orders a block, at most 32
+    int64_t S, Sp;
+    const uint64_t* pst;
+    const uint32_t* spos;
+    const uint32_t* srank;
+    const int64_t* keys;
+    const uint64_t* amask;         // pruned: survivors in score order
+    const uint32_t* aspos;
+    const uint32_t* aoff;
+    const uint32_t* acnt;
+    uint32_t* best_rank;           // may be null
+    double* score;                 // may be null
+    uint32_t* status;
+};
+static constexpr int SC_SURVIVORS = 8192;          // survivors a block stages (64 KB)
+
+template <bool PRUNED>
+__global__ void __launch_bounds__(SC_THREADS) k_score_small(ScoreArgs A)
+{
+    extern __shared__ uint64_t s_m[];              // pruned: every node's survivors
+    __shared__ uint64_t s_pc[MAXN][33];            // predecessor masks, then the entries' keys
+    __shared__ uint32_t s_best[MAXN][33];          // sorted positions, then ranks
+    const int n = A.n, b0 = blockIdx.x * A.ob, nb = min(A.ob, A.B - b0);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (PRUNED) {
+        const int total = (int)(A.aoff[n - 1] + A.acnt[n - 1]);
+#pragma unroll 4
+        for (int e = tid; e < total; e += SC_THREADS) s_m[e] = A.amask[e];
+    }
+    for (int q = warp; q < nb; q += SC_WARPS)
+        order_masks(A.orders + (size_t)(b0 + q) * n, n, lane, A.status, [&](int i, uint64_t pc) { s_pc[i][q] = pc; });
+    __syncthreads();
+    if (PRUNED) {
+        // a warp per node, a lane per order: the first survivor inside the predecessors
+        for (int i = warp; i < n; i += SC_WARPS) {
+            const uint64_t npc = lane < nb ? ~s_pc[i][lane] : 0ull;
+            const uint64_t* M = s_m + A.aoff[i];
+            const int m = (int)A.acnt[i];
+            int best = lane < nb ? -1 : 0;
+            for (int e = 0; e < m; e += 8) {
+                uint32_t hit = 0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (e + u < m) hit |= (uint32_t)((M[e + u] & npc) == 0ull) << u;
+                if (best < 0 && hit) best = e + __ffs((int)hit) - 1;
+                if (__all_sync(0xffffffffu, best >= 0)) break;
+            }
+            if (lane < nb) s_best[i][lane] = A.aspos[A.aoff[i] + (uint32_t)max(best, 0)];
+        }
+    } else {
+        // a warp per (node, order), the entries over its lanes
+        for (int it = warp; it < n * nb; it += SC_WARPS) {
+            const int i = it / nb, q = it - i * nb;
+            const uint64_t npc = ~s_pc[i][q];
+            const uint32_t* P = A.spos + (size_t)i * A.Sp;
+            uint32_t best = SPOS_NONE;
+#pragma unroll 8
+            for (int e = lane; e < (int)A.S; e += 32) {
+                const uint64_t m = __ldg(A.pst + e);
+                const uint32_t p = __ldg(P + e);
+                if ((m & npc) == 0ull) best = min(best, p);
+            }
+            best = __reduce_min_sync(0xffffffffu, best);
+            if (lane == 0) s_best[i][q] = best;
+        }
+    }
+    __syncthreads();
+    int64_t(*s_key)[33] = (int64_t(*)[33])s_pc;
+#pragma unroll 4
+    for (int idx = tid; idx < n * nb; idx += SC_THREADS) {
+        const int i = idx / nb, q = idx - i * nb;
+        const uint32_t r = A.srank[(size_t)i * A.Sp + s_best[i][q]];
+        s_key[i][q] = A.keys[(size_t)i * A.Sp + r];
+        s_best[i][q] = r;
+    }
+    __syncthreads();
+    if (A.score && tid < nb) {
+        double sum = 0.0;
+        for (int i = 0; i < n; ++i) sum = __dadd_rn(sum, key_to_double(s_key[i][tid]));
+        A.score[b0 + tid] = sum;
+    }
+    if (A.best_rank)
+        for (int idx = tid; idx < n * nb; idx += SC_THREADS)
+            A.best_rank[(size_t)b0 * n + idx] = s_best[idx % n][idx / n];
+}
+
+// Pruned tables whose survivors fit a block's shared memory, whatever B; full tables of up to
+// 65,536 entries with at most 4 M tests (17 nodes and k = 4: 2,517 sets a node, 93 orders),
+// beyond which the scans that spread entries and orders over the GPU are faster.
+bool score_small_fits(const bn_table* t, int B)
+{
+    if (t->scan_mode == BN_SCAN_PRUNED) return t->alive_total <= SC_SURVIVORS;
+    const int64_t entries = (int64_t)t->n * t->S;
+    return t->scan_mode == BN_SCAN_FULL && entries <= 65536 && entries * B <= (int64_t)4 << 20;
+}
+
+int launch_score_small(const bn_table* t, const uint8_t* orders, int B, uint32_t* best_rank, double* score,
+                       uint32_t* status, cudaStream_t s)
+{
+    // one wave while 32 orders a block allow it
+    const int ob = std::max(1, std::min(32, (B + sm_count() - 1) / sm_count()));
+    ScoreArgs A{orders, B, t->n, ob, t->S, t->Sp, t->pst, t->spos, t->srank, t->keys, t->amask, t->aspos, t->aoff, t->acnt,
+                best_rank, score, status};
+    const unsigned grid = (unsigned)((B + ob - 1) / ob);
+    if (t->scan_mode == BN_SCAN_PRUNED) {
+        static unsigned long long ctx[64] = {0};
+        if (first_in_context(ctx))
+            BN_CUDA(cudaFuncSetAttribute(k_score_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * SC_SURVIVORS));
+        k_score_small<true><<<grid, SC_THREADS, sizeof(uint64_t) * (size_t)t->alive_total, s>>>(A);
+    } else
+        k_score_small<false><<<grid, SC_THREADS, 0, s>>>(A);
+    BN_LAUNCH_CHECK("k_score_small");
+    return BN_OK;
 }
 
 // the mask-test scan's tiling for up to max_items items per node, tuned on first use (k > 4
@@ -792,7 +924,8 @@ static int score_orders_impl(const bn_table* t, const uint8_t* orders, int B, ui
     if (!orders) return set_error(BN_EINVAL, "bn_score_orders: orders is NULL");
     cudaStream_t s = (cudaStream_t)stream;
     const int n = t->n;
-    if (!scan_nodes_fits(t, B)) {
+    const bool small = score_small_fits(t, B);
+    if (!small && !scan_nodes_fits(t, B)) {
         int rt = ensure_tuned(t, B, s);
         if (rt) return rt;
     }
@@ -815,13 +948,13 @@ static int score_orders_impl(const bn_table* t, const uint8_t* orders, int B, ui
         return o;
     };
     const size_t o_orders = take(copied ? (size_t)B * n : 0);
-    const size_t o_pc = take(sizeof(uint64_t) * (size_t)n * B);
-    const size_t o_best = take(sizeof(uint32_t) * (size_t)n * B);
-    const size_t o_cnt = take(sizeof(uint32_t) * n);
+    const size_t o_pc = take(small ? 0 : sizeof(uint64_t) * (size_t)n * B);
+    const size_t o_best = take(small ? 0 : sizeof(uint32_t) * (size_t)n * B);
+    const size_t o_cnt = take(small ? 0 : sizeof(uint32_t) * n);
     const size_t o_rank = take(copied && best_rank ? sizeof(uint32_t) * (size_t)B * n : 0);
     const size_t o_score = take(copied && order_score ? sizeof(double) * B : 0);
     uint8_t* base = nullptr;
-    cudaError_t e = dev_alloc((void**)&base, off, s);
+    cudaError_t e = off ? dev_alloc((void**)&base, off, s) : cudaSuccess;
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(BN_ENOMEM, "bn_score_orders: scratch of %zu bytes: %s", off, cudaGetErrorString(e));
@@ -858,13 +991,18 @@ static int score_orders_impl(const bn_table* t, const uint8_t* orders, int B, ui
             if (!done) cudaStreamSynchronize(s);
         }
     } drain{s};
-    int rc = launch_pred_lists(d_orders, B, n, d_pc, d_best, d_cnt, d_st, s);
-    if (rc) return rc;
-    if (ev0) BN_CUDA(cudaEventRecord(ev0, s));
-    rc = launch_scan_orders(t, B, d_cnt, d_pc, d_best, d_st, s);
-    if (rc) return rc;
-    if (ev1) BN_CUDA(cudaEventRecord(ev1, s));
-    if ((rc = launch_reduce_orders(t, d_best, B, d_rank, d_score, s))) return rc;
+    int rc;
+    if (small) {
+        if (ev0) BN_CUDA(cudaEventRecord(ev0, s));
+        if ((rc = launch_score_small(t, d_orders, B, d_rank, d_score, d_st, s))) return rc;
+        if (ev1) BN_CUDA(cudaEventRecord(ev1, s));
+    } else {
+        if ((rc = launch_pred_lists(d_orders, B, n, d_pc, d_best, d_cnt, d_st, s))) return rc;
+        if (ev0) BN_CUDA(cudaEventRecord(ev0, s));
+        if ((rc = launch_scan_orders(t, B, d_cnt, d_pc, d_best, d_st, s))) return rc;
+        if (ev1) BN_CUDA(cudaEventRecord(ev1, s));
+        if ((rc = launch_reduce_orders(t, d_best, B, d_rank, d_score, s))) return rc;
+    }
     if (copied) {
         if (best_rank)
             BN_CUDA(cudaMemcpyAsync(best_rank, d_rank, sizeof(uint32_t) * (size_t)B * n, cudaMemcpyDeviceToHost, s));

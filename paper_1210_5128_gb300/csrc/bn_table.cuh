@@ -118,6 +118,12 @@ int launch_scan_orders(const bn_table* t, int B, const uint32_t* list_count, con
 int launch_pred_lists(const uint8_t* orders, int B, int n, uint64_t* list_pc, uint32_t* list_best,
                       uint32_t* list_count, uint32_t* status, cudaStream_t s);
 
+// Orders to results in one kernel where the scan is short (score_small_fits): a pruned table,
+// or a small full one; the same results as lists, scan and reduction.
+bool score_small_fits(const bn_table* t, int B);
+int launch_score_small(const bn_table* t, const uint8_t* orders, int B, uint32_t* best_rank, double* score,
+                       uint32_t* status, cudaStream_t s);
+
 // a7: per order b, the chosen rank of every node (best_rank[b * n + i], may be null) and
 // the FP64 sum over nodes, ascending node id, of their entries (score[b], may be null),
 // from the scan's smallest sorted positions list_best[i * B + b]
