@@ -140,32 +140,69 @@ __device__ __forceinline__ void store_h1(const LearnArgs& L, int c, int h0, cons
 // set-up kernels
 // ---------------------------------------------------------------------------------
 
-// T[p][v][h] = sum_j W1[h][p d + j] E[v][j]  (bf16 products are exact in FP32; j ascending)
-__global__ void k_l1_table(const bf16* __restrict__ W1b, int ndp, const bf16* __restrict__ Eb, int n, int d, int H,
-                           float* __restrict__ T)
+// T[p][v][h] = sum_j W1[h][p d + j] E[v][j]  (bf16 products are exact in FP32; j ascending).
+// A block takes position p, 128 hidden units and a share of the nodes: the units' weights
+// come in coalesced along j once and stay in shared memory, a thread per unit, for all its
+// nodes (n = 60, H = 512: 206 us with every (p, v) reading its column of W1, 28 so).
+static constexpr int L1_UNITS = 128, L1_SPLIT = 8, L1_MAX_D = 64;
+__global__ void __launch_bounds__(L1_UNITS) k_l1_table(const bf16* __restrict__ W1b, int ndp, const bf16* __restrict__ Eb,
+                                                       int n, int d, int H, float* __restrict__ T)
 {
-    const int pv = blockIdx.x, p = pv / n, v = pv - p * n;
-    for (int h = threadIdx.x; h < H; h += blockDim.x) {
-        float acc = 0.f;
-        for (int j = 0; j < d; ++j)
-            acc = fmaf(__bfloat162float(W1b[(size_t)h * ndp + p * d + j]), __bfloat162float(Eb[(size_t)v * d + j]), acc);
-        T[((size_t)p * n + v) * H + h] = acc;
+    __shared__ float s_w[L1_UNITS][L1_MAX_D + 1];
+    __shared__ float s_e[L1_MAX_D];
+    const int p = blockIdx.x, h0 = blockIdx.y * L1_UNITS, tid = threadIdx.x;
+    const int per = (n + L1_SPLIT - 1) / L1_SPLIT, v0 = blockIdx.z * per, v1 = min(n, v0 + per);
+    float acc[(MAXN + L1_SPLIT - 1) / L1_SPLIT];
+#pragma unroll
+    for (int q = 0; q < (MAXN + L1_SPLIT - 1) / L1_SPLIT; ++q) acc[q] = 0.f;
+    for (int j0 = 0; j0 < d; j0 += L1_MAX_D) {
+        const int w = min(L1_MAX_D, d - j0);
+        __syncthreads();
+        for (int e = tid; e < L1_UNITS * w; e += L1_UNITS) {
+            const int u = e / w, j = e - u * w;
+            s_w[u][j] = h0 + u < H ? __bfloat162float(W1b[(size_t)(h0 + u) * ndp + p * d + j0 + j]) : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < (MAXN + L1_SPLIT - 1) / L1_SPLIT; ++q) {
+            if (v0 + q >= v1) break;                                // block-uniform
+            __syncthreads();
+            for (int j = tid; j < w; j += L1_UNITS) s_e[j] = __bfloat162float(Eb[(size_t)(v0 + q) * d + j0 + j]);
+            __syncthreads();
+            float a = acc[q];
+#pragma unroll 8
+            for (int j = 0; j < w; ++j) a = fmaf(s_w[tid][j], s_e[j], a);
+            acc[q] = a;
+        }
+    }
+    if (h0 + tid < H) {
+#pragma unroll
+        for (int q = 0; q < (MAXN + L1_SPLIT - 1) / L1_SPLIT; ++q)
+            if (v0 + q < v1) T[((size_t)p * n + v0 + q) * H + h0 + tid] = acc[q];
     }
 }
 
 // bound on |z1| before the bias: max over h of sum_p max_v |T[p][v][h]| (float bits of a
-// non-negative value order like unsigned integers)
-__global__ void k_l1_bound(const float* __restrict__ T, int n, int H, uint32_t* __restrict__ out)
+// non-negative value order like unsigned integers).  32 hidden units a block; the positions'
+// maxima side by side, then one thread a unit adds them in position order (495 us with a
+// thread per unit over all n^2 rows, XX so).
+__global__ void __launch_bounds__(1024) k_l1_bound(const float* __restrict__ T, int n, int H, uint32_t* __restrict__ out)
 {
-    const int h = blockIdx.x * blockDim.x + threadIdx.x;
-    if (h >= H) return;
-    float s = 0.f;
-    for (int p = 0; p < n; ++p) {
+    __shared__ float s_m[MAXN][33];
+    const int h = blockIdx.x * 32 + threadIdx.x;
+    for (int p = threadIdx.y; p < n; p += 32) {
         float m = 0.f;
-        for (int v = 0; v < n; ++v) m = fmaxf(m, fabsf(T[((size_t)p * n + v) * H + h]));
-        s += m;
+        if (h < H) {
+#pragma unroll 8
+            for (int v = 0; v < n; ++v) m = fmaxf(m, fabsf(T[((size_t)p * n + v) * H + h]));
+        }
+        s_m[p][threadIdx.x] = m;
     }
-    atomicMax(out, __float_as_uint(s));
+    __syncthreads();
+    if (threadIdx.y == 0 && h < H) {
+        float s = 0.f;
+        for (int p = 0; p < n; ++p) s += s_m[p][threadIdx.x];
+        atomicMax(out, __float_as_uint(s));
+    }
 }
 
 // in place: float -> round-to-nearest integer of value * 2^shift
@@ -1152,9 +1189,9 @@ static int learned_weights(bn_chains* ch, cudaStream_t s)
     const int n = lp->n, H = lp->H;
     BN_CUDA(cudaMemsetAsync(lp->block, 0, lp->bytes, s));
     float* Tf = (float*)lp->L.T;
-    k_l1_table<<<n * n, 256, 0, s>>>(m->W1b, m->ndp, m->Eb, n, m->d, H, Tf);
+    k_l1_table<<<dim3((unsigned)n, (unsigned)((H + L1_UNITS - 1) / L1_UNITS), L1_SPLIT), L1_UNITS, 0, s>>>(m->W1b, m->ndp, m->Eb, n, m->d, H, Tf);
     BN_LAUNCH_CHECK("k_l1_table");
-    k_l1_bound<<<blocks_of(H), 256, 0, s>>>(Tf, n, H, lp->bound);
+    k_l1_bound<<<(unsigned)((H + 31) / 32), dim3(32, 32), 0, s>>>(Tf, n, H, lp->bound);
     BN_LAUNCH_CHECK("k_l1_bound");
     uint32_t hb = 0;
     BN_CUDA(cudaMemcpyAsync(&hb, lp->bound, 4, cudaMemcpyDeviceToHost, s));
