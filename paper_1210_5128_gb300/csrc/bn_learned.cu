@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(L1_UNITS) k_l1_table(const bf16* __restrict__ 
 // bound on |z1| before the bias: max over h of sum_p max_v |T[p][v][h]| (float bits of a
 // non-negative value order like unsigned integers).  32 hidden units a block; the positions'
 // maxima side by side, then one thread a unit adds them in position order (495 us with a
-// thread per unit over all n^2 rows, XX so).
+// thread per unit over all n^2 rows, 27 so).
 __global__ void __launch_bounds__(1024) k_l1_bound(const float* __restrict__ T, int n, int H, uint32_t* __restrict__ out)
 {
     __shared__ float s_m[MAXN][33];

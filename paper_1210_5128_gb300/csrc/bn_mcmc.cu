@@ -351,7 +351,8 @@ __host__ __device__ constexpr size_t surv_cache_bytes(int cap)
 {
     return (size_t)cap * (8 + 8 + 8 + 4) + 4 * (MAXN + 1);
 }
-static constexpr int SURV_CAP_MAX = 2400;
+static constexpr int SURV_CAP_MAX = 2400;   // staged by a many-network launch, or without a global copy
+static constexpr int SPEC_CAP_MAX = 7000;   // staged by a single network's sampler (196 KB)
 // cached networks sum entry changes in 64-bit fixed point (2^-32 units): entries below 2^22
 // in magnitude keep every sum of up to 2 x 64 changes inside int64
 static constexpr double FX_LIMIT = 4194304.0;
@@ -1456,7 +1457,12 @@ __global__ void __launch_bounds__(32 * SPEC_WARPS, 1) k_chain_spec(ChainState S,
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = blockIdx.x;
     if (MODE == 1) {
-        fill_surv_cache(S, F, fcache, threadIdx.x, blockDim.x);
+        if (F.gcache) {                                    // the same layout: a straight copy
+            const uint4* src = (const uint4*)F.gcache;
+            for (size_t i = threadIdx.x; i < surv_cache_stride(F.cap) / 16; i += blockDim.x) ((uint4*)fcache)[i] = src[i];
+        } else {
+            fill_surv_cache(S, F, fcache, threadIdx.x, blockDim.x);
+        }
         __syncthreads();
     }
     if (c >= S.C) return;                                  // block-uniform
@@ -1492,7 +1498,8 @@ static int fused_smem_setup(int cap, size_t* smem)
     const size_t mx = surv_cache_stride(SURV_CAP_MAX);
     if (first_in_context(ctx)) {
         BN_CUDA(cudaFuncSetAttribute(k_chain_fused<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
-        BN_CUDA(cudaFuncSetAttribute(k_chain_spec<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
+        BN_CUDA(cudaFuncSetAttribute(k_chain_spec<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)surv_cache_stride(SPEC_CAP_MAX)));
         BN_CUDA(cudaFuncSetAttribute(k_batch_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
     }
     *smem = surv_cache_stride(cap);
@@ -1763,6 +1770,32 @@ static bool fused_path(const bn_chains* ch)
     return ch->S.mode == BN_PROPOSAL_UNIFORM && ch->t->scan_mode == BN_SCAN_PRUNED;
 }
 
+// Whether a single network's sampler keeps its survivors in shared memory: when that leaves
+// every chain's block resident at once, or as many as its registers allow (a second wave
+// costs a whole run; walking the global-memory copy about a fifth: 60 nodes, 2,767
+// survivors, 256 chains 0.93 us an iteration against 0.85 staged).
+static bool spec_staged(const bn_chains* ch)
+{
+    const int64_t total = ch->t->alive_total;
+    if (!ch->t->gcache) return total <= SURV_CAP_MAX;
+    static unsigned long long ctx[64] = {0};
+    static int by_regs[64] = {0};
+    const int d = device_id();
+    if (first_in_context(ctx) && d >= 0 && d < 64) {
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chain_spec<2>, 32 * SPEC_WARPS, 0) != cudaSuccess) {
+            cudaGetLastError();
+            nb = 4;
+        }
+        by_regs[d] = std::max(1, nb);
+    }
+    const int want = (ch->S.C + sm_count() - 1) / sm_count();
+    const int per_sm = std::min(want, d >= 0 && d < 64 && by_regs[d] > 0 ? by_regs[d] : 4);
+    const int64_t room = 227 * 1024 / per_sm - 1024 - (int64_t)(sizeof(FusedSmem) + sizeof(SpecBatch) + sizeof(SpecChain) +
+                                                               sizeof(SpecTasks) + 256);
+    return total <= SPEC_CAP_MAX && (int64_t)surv_cache_stride((int)total) <= room;
+}
+
 // `iters` fused steps starting at step t0; ev0/ev1 (optional) bracket the fused kernel
 static int fused_launch(bn_chains* ch, int64_t t0, int iters, cudaStream_t s, cudaEvent_t ev0 = nullptr,
                         cudaEvent_t ev1 = nullptr)
@@ -1774,8 +1807,8 @@ static int fused_launch(bn_chains* ch, int64_t t0, int iters, cudaStream_t s, cu
     F.acnt = ch->t->acnt;
     F.t0 = t0;
     F.iters = iters;
-    F.staged = ch->t->alive_total <= SURV_CAP_MAX && ch->t->max_abs_survivor < FX_LIMIT ? 1 : 0;
-    F.gcache = F.staged ? nullptr : ch->t->gcache;
+    F.gcache = ch->t->gcache;
+    F.staged = ch->t->max_abs_survivor < FX_LIMIT && spec_staged(ch) ? 1 : 0;
     F.gfirst = F.gcache ? (const uint16_t*)(F.gcache + surv_cache_stride((int)ch->t->alive_total)) : nullptr;
     F.cap = (F.staged || F.gcache) ? (int)ch->t->alive_total : 0;
     F.margin_x = mh_margin(ch->S.n, ch->t->max_abs_survivor);
