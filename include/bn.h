@@ -74,7 +74,8 @@ typedef struct {
  * exactly (128-bit fixed point) before one rounding to FP64.
  * Errors: BN_EINVAL for n, k, arity, data or R out of range (R NaN included);
  * BN_EUNSUPPORTED if S(n-1,k) >= 2^31 or a count table needs more than 4096 cells;
- * BN_ENOMEM; BN_ECUDA.  On error *out is NULL. */
+ * BN_ENOMEM; BN_ETIMEOUT (a bounded wait of the tensor-core counting expired); BN_ECUDA.
+ * On error *out is NULL. */
 int bn_build_scores(const uint8_t* data, int m, int n, const uint8_t* arity, int k,
                     const double* R, const bn_score_params* params, int mem,
                     void* stream, bn_table** out);
@@ -145,7 +146,8 @@ int bn_score_orders_profiled(const bn_table* t, const uint8_t* orders, int B, ui
  *   orders      B x n uint8 permutations (position -> node)
  *   order_score B float64 out (may be NULL)
  *   node_score  B x n float64 out, [b][i] = node i's term (may be NULL)
- * Scratch is allocated per call.  Errors: BN_EINVAL, BN_ENOMEM, BN_ECUDA. */
+ * Scratch is allocated per call.  Errors: BN_EINVAL, BN_ENOMEM, BN_ETIMEOUT (a bounded
+ * device wait expired), BN_ECUDA. */
 int bn_score_orders_sum(const bn_table* t, const uint8_t* orders, int B, double* order_score,
                         double* node_score, int mem, void* stream);
 

@@ -1,0 +1,33 @@
+// bn_joint_tc.cuh -- joint count tables of the largest sets on the tensor cores
+// (bn_joint_tc.cu), called by the table build.
+#pragma once
+
+#include <vector>
+
+#include "bn_internal.cuh"
+
+namespace bn {
+
+struct TcJoint {
+    int n, m, mw, k;               // sets of k + 1 nodes
+    const uint8_t* arity;          // device
+    const uint32_t* packed;        // device, [n][mw]
+    const fx128* lut;              // device, [m + 1]: lgamma terms of a cell count, one table
+                                   // for every set
+    fx128* G;                      // device, by rank over sets of at most k + 1 nodes
+    uint32_t* status;
+    uint8_t* scratch;              // joint_tc_scratch bytes
+};
+
+// the work of one (n, k, arities): row tiles of pairs, column tiles of low sets
+struct TcPlan {
+    std::vector<uint32_t> pairs, rowinfo, mt_first, nt_start;
+    uint32_t items = 0;
+};
+
+// plans the sets of k + 1 nodes; false where the histogram kernel is the better one
+bool joint_tc_plan(int n, int m, int k, const uint8_t* arity_host, TcPlan* P);
+size_t joint_tc_scratch(const TcPlan& P, int m);
+int launch_joint_tc(const TcJoint& J, const TcPlan& P, cudaStream_t s);
+
+}  // namespace bn

@@ -12,6 +12,7 @@
 #include <string>
 #include <vector>
 
+#include "bn_joint_tc.cuh"
 #include "bn_table.cuh"
 
 namespace bn {
@@ -677,6 +678,7 @@ struct BuildPlan {
     std::vector<double> Rh;
     int64_t S = 0;
     int cells_max = 1;
+    bool one_arity = true;
     int nv = 1;                       // variants of the configuration sums
     uint32_t vmap = 0;                // byte r - 1: variant of a child of arity r
     std::vector<int16_t> cell_lut, cfg_lut;
@@ -751,6 +753,7 @@ static int build_plan(const uint8_t* data, int m, int n, const uint8_t* arity, i
         cells_max = std::max<int>(cells_max, (int)c);
     }
     P->cells_max = cells_max;
+    P->one_arity = std::count(ar.begin(), ar.end(), ar[0]) == n;
 
     // LUT plan: K2 uses alpha = 1 for cells and alpha = r for configurations; BDeu uses
     // ess/(q r) and ess/q for every reachable q (products of <= k arities)
@@ -891,6 +894,16 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
     const bool smem_data = smem + data_bytes <= LIM / 2;
     if (smem_data) smem += data_bytes;
     const int per_sm = std::max(1, std::min(2048 / (32 * nwarps), (int)((224 * 1024) / std::max<size_t>(smem + 1024, 1))));
+    // the largest sets -- nearly all of them -- on the tensor cores where they are many and
+    // one lgamma table serves them all (K2; BDeu with one arity)
+    TcPlan tcp;
+    bool tc = (P.kind == 0 || P.one_arity) && joint_tc_plan(n, m, k, P.ar.data(), &tcp);
+    uint8_t* d_tc = nullptr;
+    if (tc && sums.get(&d_tc, joint_tc_scratch(tcp, m))) {      // no room: count them as the others
+        set_error(BN_OK, "");
+        tc = false;
+    }
+    if (tc) A.S1 = A.S0;
     // 8 to 64 sets a unit: about eight units a resident warp where there are enough sets
     const int64_t warps = (int64_t)sm_count() * per_sm * nwarps;
     A.range = (int)std::max<int64_t>(4, std::min<int64_t>(64, A.S1 / (8 * warps)));
@@ -910,6 +923,13 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
     else if (k <= 8) rc = launch_joint_kt<8>(A, smem_data, base, smem, grid, thr, s);
     else rc = launch_joint_kt<12>(A, smem_data, base, smem, grid, thr, s);
     if (rc) return rc;
+    if (tc) {
+        int Q = 1;
+        for (int q = 0; q <= k; ++q) Q *= P.ar[0];       // (K2's table serves any size)
+        const size_t lut = P.kind == 0 ? (size_t)P.cell_lut[1] : (size_t)P.cell_lut[Q];
+        const TcJoint J{n, m, mw, k, d_ar, d_packed, d_lut + lut * (size_t)(m + 1), A.G, d_meta, d_tc};
+        if ((rc = launch_joint_tc(J, tcp, s))) return rc;
+    }
     AssembleArgs B{t->pst, n, k, P.S, t->Sp, A.S0, A.G, A.H, d_ar, P.vmap, d_ppf, P.log10g, t->keys};
     k_assemble<<<dim3((unsigned)((t->Sp + ASM_BLOCK - 1) / ASM_BLOCK), (unsigned)n), 256, 0, s>>>(B);
     BN_LAUNCH_CHECK("k_assemble");
@@ -959,6 +979,7 @@ static int build_scores_impl(const uint8_t* data, int m, int n, const uint8_t* a
         uint32_t st = 0;
         if ((rc = read_meta(d_meta, t, &st, s))) return rc;
         if (st & STATUS_BADINPUT) return set_error(BN_EINVAL, "bn_build_scores: a data value is >= its arity");
+        if (st & STATUS_TIMEOUT) return set_error(BN_ETIMEOUT, "bn_build_scores: a bounded device wait expired");
     }
     guard.ok = true;
     *out = t;
@@ -1078,6 +1099,9 @@ extern "C" int bn_build_scores_batch(int count, const uint8_t* const* data, cons
     for (int i = 0; i < count; ++i)
         if (st[(size_t)META_WORDS * i] & STATUS_BADINPUT)
             return set_error(BN_EINVAL, "bn_build_scores_batch: network %d: a data value is >= its arity", i);
+    for (int i = 0; i < count; ++i)
+        if (st[(size_t)META_WORDS * i] & STATUS_TIMEOUT)
+            return set_error(BN_ETIMEOUT, "bn_build_scores_batch: network %d: a bounded device wait expired", i);
     guard.ok = true;
     for (int i = 0; i < count; ++i) out[i] = tabs[i];
     return BN_OK;
