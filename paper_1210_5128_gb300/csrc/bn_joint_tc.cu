@@ -9,19 +9,21 @@
 // products 4.0, and the FP32 sums 4 x count are exact up to 2^22 rows.
 //
 // A persistent CTA per SM walks (pair tile, low-set tile) items: twelve warps write the
-// indicators of 128 rows at a time into shared memory (a thread per tile row, three
-// stages), one thread issues tcgen05.mma kind::f8f6f4 into one of two 256-column TMEM
-// accumulators, four warps turn the other accumulator's counts into lgamma terms (96-bit
+// indicators of 128 rows at a time into shared memory (a thread per four tile rows and 32
+// rows of the data, three stages), one thread issues tcgen05.mma kind::f8f6f4 into one of two 256-column TMEM
+// accumulators, eight warps turn the other accumulator's counts into lgamma terms (96-bit
 // fixed point, an eight-byte and a four-byte lookup whose small indices are free of bank
 // conflicts), add them over each table and store G.  Sets whose pair does not lie above
 // the low set are computed and dropped; pairs come in order of falling d, so those are few.
 //
-// What bounds it is the LSU: the states read, the indicators written, three wavefronts of
-// lookups a warp and cell (570 M wavefronts at n = 60, 1.9 ms).  Against the histogram kernel
+// What bounds it is the shared-memory port: the indicators written (165 M wavefronts at
+// n = 60) and read by the products (the tensor pipe is 27 % busy), three wavefronts of lookups
+// a warp and cell (204 M); the LSU alone keeps it 64 % busy.  Against the histogram kernel
 // (k_joint: 628 warp instructions a set, 4.1 ms for the 5.46 M 5-node sets of n = 60,
-// m = 1000) it takes 2.81 ms, the build 6.20 ms instead of 7.08, 12 networks learned together
-// 22.0 ms instead of 23.7.  (With lookups behind a branch per cell, which serialises their
-// latency, it took 5.5 ms; through generic addresses and with spills 3.9.)
+// m = 1000) it takes 2.69 ms, the build 6.1 ms instead of 7.08.  (With lookups behind a branch
+// per cell, which serialises their latency, it took 5.5 ms; through generic addresses and
+// with spills 3.9; with a thread per tile row, which loads the states of a set once for each
+// of its cells, 2.81.)
 #include <algorithm>
 #include <vector>
 
@@ -33,7 +35,7 @@ namespace bn {
 static constexpr int TJ_M = 128, TJ_N = 256;
 static constexpr int TJ_KC = 128;                       // rows of the data per stage
 static constexpr int TJ_STAGES = 3;
-static constexpr int TJ_GEN = TJ_M + TJ_N;              // generator threads, one per tile row
+static constexpr int TJ_GEN = TJ_M + TJ_N;              // generator threads
 static constexpr int TJ_GEN_WARPS = TJ_GEN / 32;
 static constexpr int TJ_EPI_WARPS = 8;                 // two for every quarter of the TMEM lanes
 static constexpr int TJ_THREADS = TJ_GEN + 32 + 32 * TJ_EPI_WARPS;
@@ -213,55 +215,98 @@ __global__ void __launch_bounds__(TJ_THREADS, 1) k_joint_tc(TcJointArgs A)
     };
 
     if (warp < TJ_GEN_WARPS) {
-        // ---- indicators: a thread per tile row
-        const bool isA = tid < TJ_M;
-        const int row = isA ? tid : tid - TJ_M;
-        const uint32_t dst0 = smem_u32(isA ? sA : sB) + tj_off(row, 0);
+        // ---- indicators: a thread writes four consecutive rows of 32 (two pieces of 16) rows of
+        // the data; they belong to two sets at most (a set has four states or more), so it
+        // loads two pieces a stage, seldom four, for the eight it stores.  Its rows come in an
+        // order turned by its piece: eight lanes of a store phase then meet eight banks.
+        const int quad = (warp >> 1) * 16 + (warp & 1) * 8 + (lane >> 2);   // (96 quads, A's first)
+        const int piece = lane & 3;                     // and piece + 4
+        const bool isA = quad < TJ_M / 4;
+        const int row = 4 * (isA ? quad : quad - TJ_M / 4);
+        const uint32_t dst0 = smem_u32(isA ? sA : sB) + tj_off(row, piece);
         const uint32_t stage_bytes = isA ? TJ_A_BYTES : TJ_B_BYTES;
         uint32_t st = 0, ph = 0;                        // stage and its phase
         bool go = true;
         for (uint32_t item = blockIdx.x; go && item < A.items; item += gridDim.x) {
             uint32_t t0, t1;
             locate(item, t0, t1);
-            const uint4* src = (const uint4*)(isA ? A.thigh : A.tlow);
-            uint32_t s4 = 0, on = 0;                    // (rows of no pair or set are zeros)
+            const uint8_t* src[2] = {isA ? A.thigh : A.tlow, nullptr};      // first and last row's set
+            int split = 4;                              // rows of the first
+            uint32_t s4[4], on = 0;                     // state of row (i + piece) % 4; bit i: it has one
             if (isA) {
-                const uint32_t info = __ldg(A.rowinfo + (size_t)mt * TJ_M + row);
-                if (info != TJ_NO_ROW) {
-                    src = (const uint4*)(A.thigh + (size_t)(info >> 8) * A.mp);
-                    s4 = (info & 0xffu) * 0x01010101u;
-                    on = 0x40404040u;
+                const uint4 x = __ldg((const uint4*)(A.rowinfo + (size_t)mt * TJ_M + row));
+                const uint32_t info[4] = {x.x, x.y, x.z, x.w};
+                if (info[0] != TJ_NO_ROW) src[0] += (size_t)(info[0] >> 8) * A.mp;
+#pragma unroll
+                for (int i = 3; i >= 1; --i)
+                    if (info[i] != TJ_NO_ROW && info[i] >> 8 != info[0] >> 8) {
+                        split = i;
+                        src[1] = A.thigh + (size_t)(info[i] >> 8) * A.mp;
+                    }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int q = (i + piece) & 3;
+                    const uint32_t f = q == 0 ? info[0] : q == 1 ? info[1] : q == 2 ? info[2] : info[3];
+                    s4[i] = (f & 0xffu) * 0x01010101u;
+                    if (f != TJ_NO_ROW) on |= 1u << i;
                 }
             } else {
-                int o = 0;
-                for (uint32_t t = t0; t < t1; ++t) {
-                    const int w = (int)__ldg(A.low + t);
-                    if (row < o + w) {
-                        src = (const uint4*)(A.tlow + (size_t)t * A.mp);
-                        s4 = (uint32_t)(row - o) * 0x01010101u;
-                        on = 0x40404040u;
-                        break;
-                    }
+                int o = 0, first = 0;                   // columns before the set; states of row 0
+                uint32_t t = t0;
+                int w = (int)__ldg(A.low + t);
+                while (t < t1 && row >= o + w) {
                     o += w;
+                    w = ++t < t1 ? (int)__ldg(A.low + t) : 0;
+                }
+                int n1 = 0;                             // rows with a set
+                if (t < t1) {
+                    src[0] += (size_t)t * A.mp;
+                    first = row - o;
+                    n1 = 4;
+                    if (first + 4 > w) {
+                        split = w - first;
+                        if (t + 1 < t1) src[1] = A.tlow + (size_t)(t + 1) * A.mp;
+                        else n1 = split;
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int q = (i + piece) & 3;
+                    s4[i] = (uint32_t)(q < split ? first + q : q - split) * 0x01010101u;
+                    if (q < n1) on |= 1u << i;
                 }
             }
-            // the states of a stage are loaded while the one before is written
-            uint4 v[TJ_KC / 16];
+            const bool two = src[1] != nullptr;
+            const uint4* p0 = (const uint4*)src[0] + piece;
+            const uint4* p1 = (const uint4*)src[1] + piece;
+            // the states of a stage are loaded while the one before is multiplied
+            uint4 v[2], u[2];
+            auto fetch = [&](int k) {
 #pragma unroll
-            for (int q = 0; q < TJ_KC / 16; ++q) v[q] = __ldg(src + q);
+                for (int h = 0; h < 2; ++h) {
+                    v[h] = __ldg(p0 + k * (TJ_KC / 16) + 4 * h);
+                    u[h] = two ? __ldg(p1 + k * (TJ_KC / 16) + 4 * h) : v[h];
+                }
+            };
+            fetch(0);
             for (int k = 0; k < nst; ++k) {
                 if (!wait(&S.empty[st], ph ^ 1u)) {     // (the first pass over the stages is free)
                     go = false;
                     break;
                 }
-                src += TJ_KC / 16;
                 const uint32_t dst = dst0 + st * stage_bytes;
 #pragma unroll
-                for (int q = 0; q < TJ_KC / 16; ++q) {
-                    st_shared_v4(dst + q * 128, indicator(v[q].x, s4, on), indicator(v[q].y, s4, on),
-                                 indicator(v[q].z, s4, on), indicator(v[q].w, s4, on));
-                    if (k + 1 < nst) v[q] = __ldg(src + q);
+                for (int i = 0; i < 4; ++i) {
+                    const int q = (i + piece) & 3;
+                    const uint32_t bits = on >> i & 1u ? 0x40404040u : 0u;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint4 x = q < split ? v[h] : u[h];
+                        st_shared_v4(dst + q * 16 + h * 512, indicator(x.x, s4[i], bits), indicator(x.y, s4[i], bits),
+                                     indicator(x.z, s4[i], bits), indicator(x.w, s4[i], bits));
+                    }
                 }
+                if (k + 1 < nst) fetch(k + 1);
                 fence_proxy_async_smem();               // visible to the tensor core's async proxy
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.full[st]);
@@ -353,23 +398,23 @@ __global__ void __launch_bounds__(TJ_THREADS, 1) k_joint_tc(TcJointArgs A)
                     tc_wait_ld();
                     const int j1 = min(32, w - c0 + back);
 #pragma unroll
-                    for (int j8 = 0; j8 < 32; j8 += 8) {
-                        if (j8 + 8 <= back || j8 >= j1) continue;           // warp-uniform
-                        if (j8 < back || j8 + 8 > j1) {
+                    for (int j4 = 0; j4 < 32; j4 += 4) {
+                        if (j4 + 4 <= back || j4 >= j1) continue;           // warp-uniform
+                        if (j4 < back || j4 + 4 > j1) {
 #pragma unroll
-                            for (int j = j8; j < j8 + 8; ++j)
+                            for (int j = j4; j < j4 + 4; ++j)
                                 if (j < back || j >= j1) r[j] = 0u;
                         }
-                        uint32_t x[8][3];
+                        uint32_t x[4][3];
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
+                        for (int q = 0; q < 4; ++q) {
                             // 4 x count as the low bits of the float 2^23 + 4 x count
-                            const uint32_t i4 = __float_as_uint(__uint_as_float(r[j8 + q]) + 8388608.0f);
+                            const uint32_t i4 = __float_as_uint(__uint_as_float(r[j4 + q]) + 8388608.0f);
                             asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x[q][0]), "=r"(x[q][1]) : "r"(2 * i4 + at_lo));
                             asm("ld.shared.u32 %0, [%1];" : "=r"(x[q][2]) : "r"(i4 + at_hi));
                         }
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) add_term(sum, x[q]);
+                        for (int q = 0; q < 4; ++q) add_term(sum, x[q]);
                     }
                 }
                 // the pair's rows (lanes pos = 0 .. g - 1 of one group), to the first
@@ -485,13 +530,13 @@ int launch_joint_tc(const TcJoint& J, const TcPlan& P, cudaStream_t s)
     uint8_t* base = J.scratch;
     std::vector<uint32_t> lists;
     lists.reserve(nt_start.size() + mt_first.size() + rowinfo.size() + pairs.size());
-    for (const auto* v : {&nt_start, &mt_first, &rowinfo, &pairs}) lists.insert(lists.end(), v->begin(), v->end());
+    for (const auto* v : {&rowinfo, &nt_start, &mt_first, &pairs}) lists.insert(lists.end(), v->begin(), v->end());
     BN_CUDA(cudaMemcpyAsync(base + o_lists, lists.data(), 4 * lists.size(), cudaMemcpyHostToDevice, s));
     TcJointArgs A;
-    A.nt_start = (const uint32_t*)(base + o_lists);
+    A.rowinfo = (const uint32_t*)(base + o_lists);      // (first: read in pieces of 16 bytes)
+    A.nt_start = A.rowinfo + rowinfo.size();
     A.mt_first = A.nt_start + nt_start.size();
-    A.rowinfo = A.mt_first + mt_first.size();
-    A.pairs = A.rowinfo + rowinfo.size();
+    A.pairs = A.mt_first + mt_first.size();
     A.low = (const uint32_t*)(base + o_low);
     A.tlow = base + o_tl;
     A.thigh = base + o_th;
