@@ -178,12 +178,6 @@ __device__ __forceinline__ fx128 fx_from_double(double v)
     fx128 u = ((fx128)hi << 64) | (fx128)lo;
     return neg ? (fx128)0 - u : u;
 }
-__device__ __forceinline__ double fx_to_double(fx128 u)
-{
-    int64_t hi = (int64_t)(uint64_t)(u >> 64);
-    uint64_t lo = (uint64_t)u;
-    return __dadd_rn((double)hi, __dmul_rn(__ull2double_rn(lo), 5.421010862427522170037e-20));
-}
 
 // ---------------------------------------------------------------------------------
 // Bounded waits, mbarriers and 1-D bulk (TMA) copies

@@ -12,12 +12,12 @@
 #include <string>
 #include <vector>
 
+#include "bn_fx.cuh"
 #include "bn_joint_tc.cuh"
 #include "bn_table.cuh"
 
 namespace bn {
 
-static constexpr double LN10 = 2.302585092994045684017991454684364208;
 static constexpr int BUILD_THREADS = 256;
 
 // ---------------------------------------------------------------------------------
@@ -470,26 +470,13 @@ struct AssembleArgs {
     int64_t* keys;
 };
 
-// x / ln 10, correctly rounded, without the division's dependent iterations: z + zl is
-// 1 / ln 10 to twice the working precision, so q0 is within one ulp of the quotient, the
-// remainder x - q0 ln 10 is exact in one fused multiply-add, and one more rounds correctly
-// (Markstein's theorem for a correctly rounded reciprocal z; Brisebarre, Muller and Raina
-// on division by a constant).
-__device__ __forceinline__ double div_ln10(double x)
-{
-    constexpr double z = 0x1.bcb7b1526e50dp-2, zl = 0x1.d756d22d31e1ap-56;
-    const double q0 = __fma_rn(x, z, __dmul_rn(x, zl));
-    const double r = __fma_rn(-q0, LN10, x);
-    return __fma_rn(r, z, q0);
-}
-
 static constexpr int ASM_BLOCK = 2048;     // entries of a block (its binomial table is paid once)
 
 // One entry a thread at a time: the node-space ranks of pi and pi + {i}, their sums, one
 // rounding, / ln 10, the size penalty, the prior of every parent (ascending node ids).
 // Consecutive ranks differ in their lowest parents, so both gathers are mostly coalesced.
-// Bound by the FP64 pipe (about ten operations an entry) and the 16-byte gathers: 0.51 ms
-// at n = 60, k = 4 (0.89 ms with 256 entries a block).
+// Bound by integer instructions and the 16-byte gathers: 0.34 ms at n = 60, k = 4 (0.51 ms
+// with the rounding and the division on the FP64 pipe, 0.89 ms with 256 entries a block too).
 __global__ void __launch_bounds__(256) k_assemble(AssembleArgs A)
 {
     __shared__ int64_t s_bin[65 * (MAXK + 2)];          // C(a, t), t <= k + 1
@@ -509,6 +496,7 @@ __global__ void __launch_bounds__(256) k_assemble(AssembleArgs A)
     const int i = blockIdx.y;
     const int v = (int)((A.vmap >> (8 * (A.arity[i] - 1))) & 0xffu);
     const fx128* H = A.H + (size_t)v * A.S0;
+    const bool penalty = A.log10g != 0.0;
     const int64_t r1 = min((int64_t)(blockIdx.x + 1) * ASM_BLOCK, A.Sp);
 #pragma unroll 2
     for (int64_t rho = (int64_t)blockIdx.x * ASM_BLOCK + threadIdx.x; rho < r1; rho += 256) {
@@ -533,7 +521,13 @@ __global__ void __launch_bounds__(256) k_assemble(AssembleArgs A)
         }
         ru += s_bin[i * T + below + 1];
         const fx128 acc = A.G[ru] - H[rp];
-        double ls = __dadd_rn(div_ln10(fx_to_double(acc)), s_pen[j]);
+        uint64_t bits = fx_div_ln10(acc);
+        if (!penalty && !A.ppf) {                       // (adding a zero changes no entry's value)
+            *out = key_from_bits(bits);
+            continue;
+        }
+        double ls = __longlong_as_double((long long)bits);
+        if (penalty) ls = __dadd_rn(ls, s_pen[j]);
         if (A.ppf) {
             mm = mask;
             while (mm) {
