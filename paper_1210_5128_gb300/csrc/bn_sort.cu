@@ -11,10 +11,14 @@
 // split too -- into buckets of about 1,024, and a block sorts each bucket in shared memory
 // and writes all three arrays: the keys are read twice and the pairs written and read once,
 // against nine read-and-scatter passes of a byte-digit radix sort.  Measured at n = 60,
-// k = 4 (60 times 489,406 entries): radix sort and set words 5.43 ms, buckets 1.73 ms
-// (splitters 0.06, bucket of every entry 0.30, scatter 0.52, sorting and writing 0.84);
-// HBM would allow about 0.25 ms.  The count pass is bound by its binary searches in shared
-// memory, the scatter by its 12 scattered bytes an entry.  Tables of more than
+// k = 4 (60 times 489,406 entries): radix sort and set words 5.43 ms, buckets 0.91 ms
+// (splitters 0.07, bucket of every entry 0.11, scatter 0.15, sorting and writing 0.57);
+// HBM would allow about 0.25 ms.  What made the difference between that and a first 1.73 ms:
+// the count pass looks a key's cell up and searches the few splitters there (0.30 with a
+// binary search of all), the scatter orders a tile in shared memory and writes runs (0.51
+// entry by entry), the sort takes a bucket's range from its splitters and 2,048 evenly cut
+// sub-buckets (0.84 with a reduction and 256 to 512 of them).  The sort is bound by its
+// instructions, of which the fixed work of a block is a large part.  Tables of more than
 // BS_MAX_BUCKETS * 2,048 sets a node keep the radix sort: their buckets would outgrow a
 // block's shared memory.
 #include <algorithm>
@@ -174,7 +178,8 @@ static constexpr int BS_AVG = 1024;                  // entries a bucket on aver
 static constexpr int BS_CAP = 4096;                  // entries a block sorts in shared memory
 static constexpr int BS_THREADS = 512;
 static constexpr int BS_PER = BS_CAP / BS_THREADS;
-static constexpr int BS_NSUB = 512;                  // sub-buckets of a bucket
+static constexpr int BS_NSUB = 2048;                 // sub-buckets of a bucket
+static constexpr int BS_CELLS = 2048;                // cells of a node's key range, for the count pass
 static constexpr int BS_TILE = 8192;                 // entries of a partition tile
 static constexpr int BS_SAMPLES = 8192;              // at most, of a node
 
@@ -185,6 +190,25 @@ __device__ __forceinline__ bool bs_less(uint64_t xa, uint32_t ra, uint64_t xb, u
     return xa < xb || (xa == xb && ra < rb);
 }
 
+// Monotone map of the keys of [lo, hi] to N cells of equal width (keys outside: the first or
+// the last cell).  The float's error only moves the cells' ends: 0.999998 keeps the last
+// key below cell N.
+struct BsCells {
+    uint64_t lo, hi, scale;
+    int sh;
+    __device__ __forceinline__ BsCells(uint64_t lo_, uint64_t hi_, int N) : lo(lo_), hi(hi_)
+    {
+        const uint64_t range = hi - lo;
+        sh = max(0, 32 - __clzll((long long)range));
+        scale = __float2ull_rd((float)N * 4294967296.0f / ((float)(uint32_t)(range >> sh) + 1.0f) * 0.999998f);
+    }
+    __device__ __forceinline__ uint32_t operator()(uint64_t x) const
+    {
+        const uint64_t y = min(max(x, lo), hi);
+        return (uint32_t)(((y - lo) >> sh) * scale >> 32);
+    }
+};
+
 struct BsArgs {
     const int64_t* keys;      // [n][Sp]
     const uint64_t* pst;
@@ -194,6 +218,7 @@ struct BsArgs {
     int M;                    // samples a node (a power of two, at least 2 NB)
     uint64_t* split_x;        // [nb][NB] splitters; bucket b holds [splitter b - 1, splitter b)
     uint32_t* split_r;
+    uint32_t* cells;          // [nb][BS_CELLS] splitters below a cell | splitters below the next << 16
     uint32_t* counts;         // [nb][NB] entries, then [nb][NB] first entries of the buckets
     uint32_t* tile_base;      // [nb][tiles][NB] the tile's first entry within each bucket
     uint16_t* bid;            // [nb][S] bucket of each entry
@@ -244,6 +269,24 @@ __global__ void __launch_bounds__(1024) k_bs_split(BsArgs A)
         A.split_x[(size_t)i * A.NB + b] = x[q];
         A.split_r[(size_t)i * A.NB + b] = r[q];
     }
+    // where the splitters of every cell of the key range begin and end
+    const int ns = A.NB - 1;
+    auto splitter = [&](int b) { return x[(int)((int64_t)A.M * (b + 1) / A.NB)]; };
+    const BsCells cell(splitter(0), splitter(ns - 1), BS_CELLS);
+    for (uint32_t c = threadIdx.x; c < BS_CELLS; c += blockDim.x) {
+        int e[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            int lo = 0, hi = ns;                        // splitters of the cells before c + h
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (cell(splitter(mid)) < c + h) lo = mid + 1;
+                else hi = mid;
+            }
+            e[h] = lo;
+        }
+        A.cells[(size_t)i * BS_CELLS + c] = (uint32_t)e[0] | (uint32_t)e[1] << 16;
+    }
 }
 
 // bucket of every entry of a tile, and the tile's place within each bucket (the tiles take
@@ -253,24 +296,29 @@ __global__ void __launch_bounds__(512) k_bs_count(BsArgs A)
     __shared__ uint64_t sx[BS_MAX_BUCKETS];
     __shared__ uint32_t sr[BS_MAX_BUCKETS];
     __shared__ uint32_t h[BS_MAX_BUCKETS];
+    __shared__ uint32_t sc[BS_CELLS];
     const int i = blockIdx.y, tile = blockIdx.x, ns = A.NB - 1;
+    for (int c = threadIdx.x; c < BS_CELLS; c += blockDim.x) sc[c] = A.cells[(size_t)i * BS_CELLS + c];
     for (int b = threadIdx.x; b < BS_MAX_BUCKETS; b += blockDim.x) {
         sx[b] = b < ns ? A.split_x[(size_t)i * A.NB + b] : ~0ull;
         sr[b] = b < ns ? A.split_r[(size_t)i * A.NB + b] : ~0u;
         h[b] = 0;
     }
     __syncthreads();
-    int top = 1;
-    while (2 * top <= A.NB) top *= 2;
+    const BsCells cell(sx[0], sx[ns - 1], BS_CELLS);
     const int64_t* K = A.keys + (size_t)(A.node0 + i) * A.Sp;
     uint16_t* B = A.bid + (size_t)i * A.S;
     const int64_t e1 = min((int64_t)(tile + 1) * BS_TILE, A.S);
 #pragma unroll 4
     for (int64_t e = (int64_t)tile * BS_TILE + threadIdx.x; e < e1; e += 512) {
         const uint64_t x = bs_key(K[e]);
-        int b = 0;                                  // splitters below x ...
-        for (int d = top; d > 0; d >>= 1)
-            if (b + d <= ns && sx[b + d - 1] < x) b += d;
+        const uint32_t range = sc[cell(x)];
+        int b = (int)(range & 0xffffu), b1 = (int)(range >> 16);        // splitters below x ...
+        while (b < b1) {
+            const int mid = (b + b1) >> 1;
+            if (sx[mid] < x) b = mid + 1;
+            else b1 = mid;
+        }
         while (b < ns && sx[b] == x && sr[b] <= (uint32_t)e) ++b;       // ... and ties at or below e
         B[e] = (uint16_t)b;
         atomicAdd(&h[b], 1u);
@@ -305,22 +353,75 @@ __global__ void __launch_bounds__(BS_MAX_BUCKETS) k_bs_scan(BsArgs A, int nb)
     if (b < A.NB) A.counts[(size_t)(nb + i) * A.NB + b] = s - c + w[b >> 5];
 }
 
+// Moves a tile's entries to their buckets.  They are put in bucket order in shared memory
+// first: the tile's entries of one bucket (17 on average at n = 60) then leave as one run of
+// 8-byte and one of 4-byte words instead of one by one.
+static constexpr int BS_ROUNDS = BS_TILE / 512;
+static constexpr size_t BS_SCATTER_SMEM = (size_t)BS_TILE * 12;
 __global__ void __launch_bounds__(512) k_bs_scatter(BsArgs A, int nb)
 {
-    __shared__ uint32_t cur[BS_MAX_BUCKETS];
-    const int i = blockIdx.y, tile = blockIdx.x;
-    for (int b = threadIdx.x; b < A.NB; b += blockDim.x)
-        cur[b] = A.counts[(size_t)(nb + i) * A.NB + b] + A.tile_base[((size_t)i * A.tiles + tile) * A.NB + b];
+    extern __shared__ __align__(16) uint8_t bs_sm[];
+    uint64_t* sx = (uint64_t*)bs_sm;                    // [TILE] keys in bucket order
+    uint32_t* sv = (uint32_t*)(sx + BS_TILE);           // [TILE] entry of the tile | bucket << 16
+    __shared__ uint32_t h[BS_MAX_BUCKETS];              // entries of a bucket, then its first place here
+    __shared__ uint32_t to[BS_MAX_BUCKETS];             // its first place among the node's, less that
+    __shared__ uint32_t w[16];
+    const int i = blockIdx.y, tile = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t e0 = (int64_t)tile * BS_TILE;
+    const int cnt = (int)min((int64_t)BS_TILE, A.S - e0);
+    const int64_t* K = A.keys + (size_t)(A.node0 + i) * A.Sp + e0;
+    const uint16_t* B = A.bid + (size_t)i * A.S + e0;
+    h[tid] = 0;
+    h[tid + 512] = 0;
     __syncthreads();
-    const int64_t* K = A.keys + (size_t)(A.node0 + i) * A.Sp;
-    const uint16_t* B = A.bid + (size_t)i * A.S;
-    const int64_t e1 = min((int64_t)(tile + 1) * BS_TILE, A.S);
+    uint32_t v[BS_ROUNDS];                              // bucket << 16 | place within the tile's bucket
+#pragma unroll
+    for (int u = 0; u < BS_ROUNDS; ++u) {
+        const int e = u * 512 + tid;
+        v[u] = e < cnt ? (uint32_t)B[e] << 16 : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < BS_ROUNDS; ++u)
+        if (u * 512 + tid < cnt) v[u] |= atomicAdd(&h[v[u] >> 16], 1u);
+    __syncthreads();
+    // exclusive scan of the 1,024 counts, two a thread
+    const uint32_t c0 = h[2 * tid], c1 = h[2 * tid + 1];
+    uint32_t s = c0 + c1;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, s, d);
+        if (lane >= d) s += y;
+    }
+    if (lane == 31) w[warp] = s;
+    __syncthreads();
+    s += __reduce_add_sync(0xffffffffu, lane < warp ? w[lane] : 0u) - (c0 + c1);
+    h[2 * tid] = s;
+    h[2 * tid + 1] = s + c0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int b = 2 * tid + q;
+        if (b < A.NB)
+            to[b] = A.counts[(size_t)(nb + i) * A.NB + b] + A.tile_base[((size_t)i * A.tiles + tile) * A.NB + b] -
+                    (q ? s + c0 : s);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < BS_ROUNDS; ++u) {
+        const int e = u * 512 + tid;
+        if (e < cnt) {
+            const uint32_t b = v[u] >> 16, p = h[b] + (v[u] & 0xffffu);
+            sx[p] = bs_key(K[e]);
+            sv[p] = (uint32_t)e | b << 16;
+        }
+    }
+    __syncthreads();
+    uint64_t* X = A.bx + (size_t)i * A.S;
+    uint32_t* R = A.br + (size_t)i * A.S;
 #pragma unroll 4
-    for (int64_t e = (int64_t)tile * BS_TILE + threadIdx.x; e < e1; e += 512) {
-        const uint64_t x = bs_key(K[e]);
-        const size_t at = (size_t)i * A.S + atomicAdd(&cur[B[e]], 1u);
-        A.bx[at] = x;
-        A.br[at] = (uint32_t)e;
+    for (int p = tid; p < cnt; p += 512) {
+        const uint32_t y = sv[p], at = to[y >> 16] + (uint32_t)p;
+        X[at] = sx[p];
+        R[at] = (uint32_t)e0 + (y & 0xffffu);
     }
 }
 
@@ -332,20 +433,21 @@ __device__ __forceinline__ void bs_write(const BsArgs& A, int i, uint32_t p, uin
     if (A.sset) A.sset[(size_t)i * A.Ssp + p] = sset_word(A.pst[r], i);
 }
 
-// One block a bucket.  The entries are spread over BS_NSUB sub-buckets by their distance from
-// the bucket's smallest key (a shift: the keys of one bucket are close to evenly spread),
-// and an entry's place is its sub-bucket's start plus the entries of it that come before
-// (two to four compares on average; all of them where scores tie).  WHOLE: a node's entries
-// are one bucket, read straight from the table.  Buckets above BS_CAP (rare: four times the
-// average of sampled splitters) are placed by counting, tile by tile.
+// One block a bucket.  The entries are spread over BS_NSUB sub-buckets of equal width (the
+// keys of one bucket are close to evenly spread), and an entry's place is its sub-bucket's
+// start plus the entries of it that come before (one compare on average; all of them where
+// scores tie).  The last pass takes the entries by sub-bucket, so that its writes of srank
+// and sset stay nearly in order.  Three blocks an SM (two spill nothing and take 10 %
+// longer).  WHOLE: a node's entries are one bucket, read straight from the table.  Buckets
+// above BS_CAP (rare: four times the average of sampled splitters) are placed by counting,
+// tile by tile.
 template <bool WHOLE>
-__global__ void __launch_bounds__(BS_THREADS) k_bs_sort(BsArgs A, int nb)
+__global__ void __launch_bounds__(BS_THREADS, 3) k_bs_sort(BsArgs A, int nb)
 {
     extern __shared__ __align__(16) uint8_t bs_sm[];
     uint64_t* sx = (uint64_t*)bs_sm;                    // [CAP] by sub-bucket
     uint32_t* sr = (uint32_t*)(sx + BS_CAP);            // [CAP]
-    uint32_t* so = sr + BS_CAP;                         // [CAP] ranks in final order
-    uint32_t* sub = so + BS_CAP;                        // [NSUB + 1]
+    uint32_t* sub = sr + BS_CAP;                        // [NSUB + 1]
     __shared__ uint64_t s_min[BS_THREADS / 32], s_max[BS_THREADS / 32];
     __shared__ uint32_t s_w[BS_THREADS / 32];
     const int i = blockIdx.y, b = blockIdx.x, node = A.node0 + i;
@@ -381,46 +483,59 @@ __global__ void __launch_bounds__(BS_THREADS) k_bs_sort(BsArgs A, int nb)
         }
     }
     uint64_t x[BS_PER], lo = ~0ull, hi = 0ull;
-    uint32_t r[BS_PER];
-    uint32_t at[BS_PER];
+    uint32_t at[BS_PER];                                // sub-bucket << 16 | place within it
 #pragma unroll
     for (int u = 0; u < BS_PER; ++u) {
         const int e = u * BS_THREADS + threadIdx.x;
         x[u] = 0;
-        r[u] = 0;
-        if (e < cnt) {
-            x[u] = WHOLE ? bs_key(A.keys[(size_t)node * A.Sp + e]) : gx[e];
-            r[u] = WHOLE ? (uint32_t)e : gr[e];
-            lo = min(lo, x[u]);
-            hi = max(hi, x[u]);
+        if (e < cnt) x[u] = WHOLE ? bs_key(A.keys[(size_t)node * A.Sp + e]) : gx[e];
+    }
+    for (int q = threadIdx.x; q < BS_NSUB; q += BS_THREADS) sub[q] = 0;
+    if (!WHOLE && b > 0 && b + 1 < A.NB) {              // between two splitters
+        lo = A.split_x[(size_t)i * A.NB + b - 1];
+        hi = A.split_x[(size_t)i * A.NB + b];
+    } else {
+#pragma unroll
+        for (int u = 0; u < BS_PER; ++u)
+            if (u * BS_THREADS + (int)threadIdx.x < cnt) {
+                lo = min(lo, x[u]);
+                hi = max(hi, x[u]);
+            }
+#pragma unroll
+        for (int d = 16; d; d >>= 1) {
+            lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
+            hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
+        }
+        if (lane == 0) {
+            s_min[warp] = lo;
+            s_max[warp] = hi;
+        }
+        __syncthreads();
+        for (int w = 0; w < BS_THREADS / 32; ++w) {
+            lo = min(lo, s_min[w]);
+            hi = max(hi, s_max[w]);
         }
     }
-    sub[threadIdx.x] = 0;
-#pragma unroll
-    for (int d = 16; d; d >>= 1) {
-        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
-        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
-    }
-    if (lane == 0) {
-        s_min[warp] = lo;
-        s_max[warp] = hi;
-    }
     __syncthreads();
-#pragma unroll
-    for (int w = 0; w < BS_THREADS / 32; ++w) {
-        lo = min(lo, s_min[w]);
-        hi = max(hi, s_max[w]);
-    }
-    const uint64_t range = hi >= lo ? hi - lo : 0ull;                            // (hi < lo: an empty bucket)
-    const int shift = max(0, 64 - __clzll((long long)range) - 9);                // range >> shift < NSUB
+    if (hi < lo) return;                                                         // an empty bucket
+    const BsCells cell(lo, hi, BS_NSUB);
 #pragma unroll
     for (int u = 0; u < BS_PER; ++u)
-        if (u * BS_THREADS + (int)threadIdx.x < cnt) at[u] = atomicAdd(&sub[(x[u] - lo) >> shift], 1u);
+        if (u * BS_THREADS + (int)threadIdx.x < cnt) {
+            const uint32_t d = cell(x[u]);
+            at[u] = d << 16 | atomicAdd(&sub[d], 1u);
+        }
     __syncthreads();
     {
-        // exclusive scan of the 512 sub-bucket counts, one a thread
-        const uint32_t c = sub[threadIdx.x];
-        uint32_t s = c;
+        // exclusive scan of the sub-bucket counts, four a thread
+        static_assert(BS_NSUB == 4 * BS_THREADS, "four sub-buckets a thread");
+        uint32_t c[4], s = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            c[q] = sub[4 * threadIdx.x + q];
+            s += c[q];
+        }
+        const uint32_t mine = s;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const uint32_t y = __shfl_up_sync(0xffffffffu, s, d);
@@ -428,34 +543,36 @@ __global__ void __launch_bounds__(BS_THREADS) k_bs_sort(BsArgs A, int nb)
         }
         if (lane == 31) s_w[warp] = s;
         __syncthreads();
-        uint32_t add = 0;
-        for (int w = 0; w < warp; ++w) add += s_w[w];
-        sub[threadIdx.x] = s - c + add;
+        s += __reduce_add_sync(0xffffffffu, lane < warp ? s_w[lane] : 0u) - mine;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            sub[4 * threadIdx.x + q] = s;
+            s += c[q];
+        }
         if (threadIdx.x == 0) sub[BS_NSUB] = (uint32_t)cnt;
     }
     __syncthreads();
 #pragma unroll
-    for (int u = 0; u < BS_PER; ++u)
-        if (u * BS_THREADS + (int)threadIdx.x < cnt) {
-            const uint32_t q = sub[(x[u] - lo) >> shift] + at[u];
+    for (int u = 0; u < BS_PER; ++u) {
+        const int e = u * BS_THREADS + threadIdx.x;
+        if (e < cnt) {
+            const uint32_t q = sub[at[u] >> 16] + (at[u] & 0xffffu);
             sx[q] = x[u];
-            sr[q] = r[u];
+            sr[q] = WHOLE ? (uint32_t)e : gr[e];
         }
+    }
     __syncthreads();
-#pragma unroll
-    for (int u = 0; u < BS_PER; ++u)
-        if (u * BS_THREADS + (int)threadIdx.x < cnt) {
-            const int d = (int)((x[u] - lo) >> shift);
-            const uint32_t s0 = sub[d], s1 = sub[d + 1];
-            uint32_t q = s0;
-            for (uint32_t t = s0; t < s1; ++t) q += bs_less(sx[t], sr[t], x[u], r[u]);
-            so[q] = r[u];
-        }
-    __syncthreads();
-    for (int q = threadIdx.x; q < cnt; q += BS_THREADS) bs_write(A, node, p0 + (uint32_t)q, so[q]);
+    for (int t = threadIdx.x; t < cnt; t += BS_THREADS) {
+        const uint64_t y = sx[t];
+        const uint32_t r = sr[t], d = cell(y);
+        const uint32_t s0 = sub[d], s1 = sub[d + 1];
+        uint32_t q = s0;
+        for (uint32_t o = s0; o < s1; ++o) q += bs_less(sx[o], sr[o], y, r);
+        bs_write(A, node, p0 + q, r);
+    }
 }
 
-static constexpr size_t BS_SMEM = (size_t)BS_CAP * 16 + 4 * (BS_NSUB + 1);
+static constexpr size_t BS_SMEM = (size_t)BS_CAP * 12 + 4 * (BS_NSUB + 1);
 
 // sorted positions at or past S of the parent-node words (padding up to the row stride, a
 // whole number of the sliced scan's stages): never consistent with an order
@@ -548,6 +665,7 @@ static int rank_by_buckets(bn_table* t, cudaStream_t s)
     int rc;
     if (!whole &&
         ((rc = tmp.get(&A.split_x, (size_t)per * A.NB)) || (rc = tmp.get(&A.split_r, (size_t)per * A.NB)) ||
+         (rc = tmp.get(&A.cells, (size_t)per * BS_CELLS)) ||
          (rc = tmp.get(&A.counts, (size_t)2 * per * A.NB)) ||
          (rc = tmp.get(&A.tile_base, (size_t)per * A.tiles * A.NB)) || (rc = tmp.get(&A.bid, (size_t)per * S)) ||
          (rc = tmp.get(&A.bx, (size_t)per * S)) || (rc = tmp.get(&A.br, (size_t)per * S))))
@@ -555,6 +673,7 @@ static int rank_by_buckets(bn_table* t, cudaStream_t s)
     static unsigned long long ctx[64] = {0};
     if (first_in_context(ctx)) {
         BN_CUDA(cudaFuncSetAttribute(k_bs_split, cudaFuncAttributeMaxDynamicSharedMemorySize, BS_SAMPLES * 12));
+        BN_CUDA(cudaFuncSetAttribute(k_bs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SCATTER_SMEM));
         BN_CUDA(cudaFuncSetAttribute(k_bs_sort<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SMEM));
         BN_CUDA(cudaFuncSetAttribute(k_bs_sort<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SMEM));
     }
@@ -572,7 +691,7 @@ static int rank_by_buckets(bn_table* t, cudaStream_t s)
         BN_LAUNCH_CHECK("k_bs_count");
         k_bs_scan<<<nb, BS_MAX_BUCKETS, 0, s>>>(A, nb);
         BN_LAUNCH_CHECK("k_bs_scan");
-        k_bs_scatter<<<dim3((unsigned)A.tiles, (unsigned)nb), 512, 0, s>>>(A, nb);
+        k_bs_scatter<<<dim3((unsigned)A.tiles, (unsigned)nb), 512, BS_SCATTER_SMEM, s>>>(A, nb);
         BN_LAUNCH_CHECK("k_bs_scatter");
         k_bs_sort<false><<<dim3((unsigned)A.NB, (unsigned)nb), BS_THREADS, BS_SMEM, s>>>(A, nb);
         BN_LAUNCH_CHECK("k_bs_sort");
