@@ -1,10 +1,10 @@
-// bn_joint_tc.cu -- joint count tables of the largest sets on the tensor cores.
+// bn_joint_tc.cu -- joint count tables of five and four nodes on the tensor cores.
 //
 // The count of a cell of the joint table of U = {a < b < c < d < e} is the number of rows in
 // which (a, b, c) are in one given state and (d, e) in another: one entry of a product of
 // two 0/1 matrices over the rows, features of pairs by features of low sets.  All tables of
-// the largest size (k + 1 = 4 or 5 nodes) are blocks of that product: a 128 x 256 tile holds
-// up to twelve ternary pairs against nine ternary triples.  The indicators are 8-bit floats
+// one size (4 or 5 nodes; low sets of 2 or 3) are blocks of that product: a 128 x 256 tile
+// holds up to twelve ternary pairs against nine ternary triples.  The indicators are 8-bit floats
 // of 2.0 (one logic op, one add, one logic op make four of them from a row of states), the
 // products 4.0, and the FP32 sums 4 x count are exact up to 2^22 rows.
 //
@@ -13,7 +13,8 @@
 // rows of the data, three stages), one thread issues tcgen05.mma kind::f8f6f4 into one of two 256-column TMEM
 // accumulators, eight warps turn the other accumulator's counts into lgamma terms (96-bit
 // fixed point, an eight-byte and a four-byte lookup whose small indices are free of bank
-// conflicts), add them over each table and store G.  Sets whose pair does not lie above
+// conflicts), add them over each table and store G -- and, for sets that are parent sets
+// too, the configuration sums H of every variant from the same counts.  Sets whose pair does not lie above
 // the low set are computed and dropped; pairs come in order of falling d, so those are few.
 //
 // What bounds it is the shared-memory port: the indicators written (165 M wavefronts at
@@ -23,7 +24,8 @@
 // m = 1000) it takes 2.69 ms, the build 6.1 ms instead of 7.08.  (With lookups behind a branch
 // per cell, which serialises their latency, it took 5.5 ms; through generic addresses and
 // with spills 3.9; with a thread per tile row, which loads the states of a set once for each
-// of its cells, 2.81.)
+// of its cells, 2.81.)  The 487,635 sets of four nodes: 0.20 ms against 0.59, the build 4.87
+// ms against 5.14 with the histograms for those.
 #include <algorithm>
 #include <vector>
 
@@ -40,7 +42,7 @@ static constexpr int TJ_GEN_WARPS = TJ_GEN / 32;
 static constexpr int TJ_EPI_WARPS = 8;                 // two for every quarter of the TMEM lanes
 static constexpr int TJ_THREADS = TJ_GEN + 32 + 32 * TJ_EPI_WARPS;
 static constexpr int TJ_A_BYTES = TJ_M * TJ_KC, TJ_B_BYTES = TJ_N * TJ_KC;
-static constexpr int TJ_LUT_ROWS = 3600;                // m + 1 entries kept in shared memory
+static constexpr int TJ_LUT_ROWS = 6300;                // entries of the lgamma tables in shared memory
 static constexpr uint32_t TJ_NO_ROW = 0xffffffffu;
 static constexpr int TJ_PAD_STATE = 0x3f;               // a state no feature has
 
@@ -56,9 +58,11 @@ struct TcJointArgs {
     int m1;                        // m + 1
     uint32_t items, MT;
     int lowk;                      // nodes of a low set (2 or 3)
-    int64_t base;                  // first rank of the largest size
-    const fx128* lut;              // lgamma terms of a cell count
+    int64_t base;                  // first rank of the sets' size
+    const fx128* lut[4];           // lgamma terms of a cell count; configuration counts' variants
     fx128* G;
+    fx128* H;                      // [variant][H_stride] by rank
+    int64_t H_stride;
     uint32_t* status;
 };
 
@@ -160,21 +164,25 @@ struct TjBars {
     int abort;
 };
 
+// NH: variants of the configuration sums (sets that are parent sets too), or 0
+template <int NH>
 __global__ void __launch_bounds__(TJ_THREADS, 1) k_joint_tc(TcJointArgs A)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ TjBars S;
     uint8_t* sA = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* sB = sA + TJ_STAGES * TJ_A_BYTES;
-    uint64_t* lut_lo = (uint64_t*)(sB + TJ_STAGES * TJ_B_BYTES);       // [m1] low 64 bits
-    uint32_t* lut_hi = (uint32_t*)(lut_lo + A.m1);                     // [m1] next 32 bits
+    uint64_t* lut_lo = (uint64_t*)(sB + TJ_STAGES * TJ_B_BYTES);       // [1 + NH][m1] low 64 bits
+    uint32_t* lut_hi = (uint32_t*)(lut_lo + (1 + NH) * A.m1);          // [1 + NH][m1] next 32 bits
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nst = A.mp / TJ_KC;
 
-    for (int i = tid; i < A.m1; i += TJ_THREADS) {
-        lut_lo[i] = (uint64_t)A.lut[i];
-        lut_hi[i] = (uint32_t)(A.lut[i] >> 64);
-    }
+#pragma unroll
+    for (int l = 0; l <= NH; ++l)
+        for (int i = tid; i < A.m1; i += TJ_THREADS) {
+            lut_lo[l * A.m1 + i] = (uint64_t)A.lut[l][i];
+            lut_hi[l * A.m1 + i] = (uint32_t)(A.lut[l][i] >> 64);
+        }
     if (warp == TJ_GEN_WARPS) {
         tc_alloc(&S.tmem, 512);
         tc_relinquish();
@@ -362,6 +370,7 @@ __global__ void __launch_bounds__(TJ_THREADS, 1) k_joint_tc(TcJointArgs A)
         const uint32_t half = (uint32_t)(warp - TJ_GEN_WARPS - 1) >> 2;
         // where the entry of count 0 lies, less the bits of the float 2^23
         const uint32_t at_lo = smem_u32(lut_lo) - 2u * 0x4b000000u, at_hi = smem_u32(lut_hi) - 0x4b000000u;
+        const uint32_t step = 4u * (uint32_t)A.m1;      // bytes of one table's high words
         uint32_t done = 0;
         for (uint32_t item = blockIdx.x; item < A.items; item += gridDim.x, ++done) {
             uint32_t t0, t1;
@@ -388,7 +397,7 @@ __global__ void __launch_bounds__(TJ_THREADS, 1) k_joint_tc(TcJointArgs A)
                 const int o0 = o;
                 o += w;
                 if (((t - t0) & 1u) != half) continue;  // the quarter's other warp takes it
-                uint32_t sum[3] = {0, 0, 0};
+                uint32_t sum[1 + NH][3] = {};
                 for (int c0 = 0; c0 < w; c0 += 32) {
                     // 32 columns, moved back where they would leave this accumulator; those
                     // of other sets count as 0, whose term is 0
@@ -405,29 +414,39 @@ __global__ void __launch_bounds__(TJ_THREADS, 1) k_joint_tc(TcJointArgs A)
                             for (int j = j4; j < j4 + 4; ++j)
                                 if (j < back || j >= j1) r[j] = 0u;
                         }
-                        uint32_t x[4][3];
+                        uint32_t x[1 + NH][4][3];
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             // 4 x count as the low bits of the float 2^23 + 4 x count
                             const uint32_t i4 = __float_as_uint(__uint_as_float(r[j4 + q]) + 8388608.0f);
-                            asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x[q][0]), "=r"(x[q][1]) : "r"(2 * i4 + at_lo));
-                            asm("ld.shared.u32 %0, [%1];" : "=r"(x[q][2]) : "r"(i4 + at_hi));
+#pragma unroll
+                            for (int l = 0; l <= NH; ++l) {
+                                asm("ld.shared.v2.u32 {%0, %1}, [%2];"
+                                    : "=r"(x[l][q][0]), "=r"(x[l][q][1]) : "r"(2 * i4 + at_lo + 2 * l * step));
+                                asm("ld.shared.u32 %0, [%1];" : "=r"(x[l][q][2]) : "r"(i4 + at_hi + l * step));
+                            }
                         }
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) add_term(sum, x[q]);
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int l = 0; l <= NH; ++l) add_term(sum[l], x[l][q]);
                     }
                 }
                 // the pair's rows (lanes pos = 0 .. g - 1 of one group), to the first
 #pragma unroll
-                for (int off = 8; off; off >>= 1) {
-                    const uint32_t x[3] = {__shfl_down_sync(0xffffffffu, sum[0], off),
-                                           __shfl_down_sync(0xffffffffu, sum[1], off),
-                                           __shfl_down_sync(0xffffffffu, sum[2], off)};
-                    if (pos < off && pos + off < g) add_term(sum, x);
+                for (int l = 0; l <= NH; ++l) {
+#pragma unroll
+                    for (int off = 8; off; off >>= 1) {
+                        const uint32_t x[3] = {__shfl_down_sync(0xffffffffu, sum[l][0], off),
+                                               __shfl_down_sync(0xffffffffu, sum[l][1], off),
+                                               __shfl_down_sync(0xffffffffu, sum[l][2], off)};
+                        if (pos < off && pos + off < g) add_term(sum[l], x);
+                    }
+                    fx128* out = l ? A.H + (size_t)(l - 1) * A.H_stride : A.G;
+                    if (pos == 0 && t < limit)
+                        out[at + t] = ((fx128)(uint64_t)(int64_t)(int32_t)sum[l][2] << 64) |
+                                      (fx128)((uint64_t)sum[l][1] << 32 | sum[l][0]);
                 }
-                if (pos == 0 && t < limit)
-                    A.G[at + t] = ((fx128)(uint64_t)(int64_t)(int32_t)sum[2] << 64) |
-                                  (fx128)((uint64_t)sum[1] << 32 | sum[0]);
             }
             tc_fence_before();
             __syncwarp();
@@ -439,13 +458,13 @@ __global__ void __launch_bounds__(TJ_THREADS, 1) k_joint_tc(TcJointArgs A)
     if (warp == TJ_GEN_WARPS) tc_dealloc(tmem, 512);
 }
 
-bool joint_tc_plan(int n, int m, int k, const uint8_t* ar, TcPlan* P)
+bool joint_tc_plan(int n, int m, int size, int luts, const uint8_t* ar, TcPlan* P)
 {
     // Few sets: the set-up costs what the products save (26 nodes, 65,780 sets: build 347 us
-    // against 365; 20 nodes, 15,504 sets: equal).  The lgamma table has to fit beside the stages.
-    const int lowk = k - 1;
-    if ((k != 3 && k != 4) || n < k + 2 || n > MAXN || m < 64 || m + 1 > TJ_LUT_ROWS) return false;
-    const int64_t sets = (int64_t)h_binom.v[n][k + 1];
+    // against 365; 20 nodes, 15,504 sets: equal).  The lgamma tables have to fit beside the stages.
+    const int lowk = size - 2;
+    if ((size != 4 && size != 5) || n <= size || n > MAXN || m < 64 || luts * (m + 1) > TJ_LUT_ROWS) return false;
+    const int64_t sets = (int64_t)h_binom.v[n][size];
     if (sets < 20000) return false;
     std::vector<uint32_t>&pairs = P->pairs, &rowinfo = P->rowinfo, &mt_first = P->mt_first, &nt_start = P->nt_start;
     // pairs d < e with room for a low set below d, d falling; 32-row blocks, no pair astride
@@ -506,61 +525,79 @@ bool joint_tc_plan(int n, int m, int k, const uint8_t* ar, TcPlan* P)
     return sets >= 48 * (int64_t)items;
 }
 
-size_t joint_tc_scratch(const TcPlan& P, int m)
+template <int NH>
+static int launch(const TcJointArgs& A, cudaStream_t s)
 {
-    const size_t lists = P.nt_start.size() + P.mt_first.size() + P.rowinfo.size() + P.pairs.size();
-    return 4 * (lists + P.nt_start.back()) + (size_t)(P.nt_start.back() + P.pairs.size()) * round_up(m, TJ_KC) + 4 * 256;
+    static unsigned long long ctx[64] = {0};
+    constexpr size_t fixed = (size_t)TJ_STAGES * (TJ_A_BYTES + TJ_B_BYTES) + 1024 + 16;
+    if (first_in_context(ctx))
+        BN_CUDA(cudaFuncSetAttribute(k_joint_tc<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(fixed + 12 * (size_t)TJ_LUT_ROWS)));
+    const size_t smem = fixed + 12 * (size_t)(1 + NH) * A.m1;
+    k_joint_tc<NH><<<std::min<uint32_t>((uint32_t)sm_count(), A.items), TJ_THREADS, smem, s>>>(A);
+    BN_LAUNCH_CHECK("k_joint_tc");
+    return BN_OK;
+}
+
+// the scratch block: lists | cells | states
+struct TcScratch {
+    size_t lists = 0, low, tlow, thigh, bytes;
+    TcScratch(const TcPlan& P, int mp)
+    {
+        const size_t NL = P.nt_start.back(), NH = P.pairs.size();
+        auto after = [](size_t at, size_t b) { return (size_t)round_up((int64_t)(at + b), 256); };
+        low = after(0, 4 * (P.rowinfo.size() + P.nt_start.size() + P.mt_first.size() + NH));
+        tlow = after(low, 4 * NL);
+        thigh = after(tlow, NL * mp);
+        bytes = after(thigh, NH * mp);
+    }
+};
+
+size_t joint_tc_scratch(const TcPlan& P, int m) { return TcScratch(P, (int)round_up(m, TJ_KC)).bytes; }
+
+int joint_tc_upload(const TcPlan& P, uint8_t* scratch, cudaStream_t s)
+{
+    std::vector<uint32_t> lists;
+    lists.reserve(P.rowinfo.size() + P.nt_start.size() + P.mt_first.size() + P.pairs.size());
+    for (const auto* v : {&P.rowinfo, &P.nt_start, &P.mt_first, &P.pairs}) lists.insert(lists.end(), v->begin(), v->end());
+    BN_CUDA(cudaMemcpyAsync(scratch, lists.data(), 4 * lists.size(), cudaMemcpyHostToDevice, s));
+    return BN_OK;
 }
 
 int launch_joint_tc(const TcJoint& J, const TcPlan& P, cudaStream_t s)
 {
-    const int n = J.n, lowk = J.k - 1, mp = (int)round_up(J.m, TJ_KC);
-    const std::vector<uint32_t>&pairs = P.pairs, &rowinfo = P.rowinfo, &mt_first = P.mt_first, &nt_start = P.nt_start;
-    const uint32_t items = P.items, MT = (uint32_t)mt_first.size() - 1, NL = nt_start.back();
-    const uint32_t NH = (uint32_t)pairs.size();
-    // one block: lists | cells | states
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        const size_t o = off;
-        off = (size_t)round_up((int64_t)(off + bytes), 256);
-        return o;
-    };
-    const size_t o_lists = take(4 * (nt_start.size() + mt_first.size() + rowinfo.size() + pairs.size()));
-    const size_t o_low = take(4 * (size_t)NL), o_tl = take((size_t)NL * mp), o_th = take((size_t)NH * mp);
+    const int n = J.n, lowk = J.size - 2, mp = (int)round_up(J.m, TJ_KC);
+    const uint32_t NL = P.nt_start.back(), NH = (uint32_t)P.pairs.size();
+    const TcScratch at(P, mp);
     uint8_t* base = J.scratch;
-    std::vector<uint32_t> lists;
-    lists.reserve(nt_start.size() + mt_first.size() + rowinfo.size() + pairs.size());
-    for (const auto* v : {&rowinfo, &nt_start, &mt_first, &pairs}) lists.insert(lists.end(), v->begin(), v->end());
-    BN_CUDA(cudaMemcpyAsync(base + o_lists, lists.data(), 4 * lists.size(), cudaMemcpyHostToDevice, s));
     TcJointArgs A;
-    A.rowinfo = (const uint32_t*)(base + o_lists);      // (first: read in pieces of 16 bytes)
-    A.nt_start = A.rowinfo + rowinfo.size();
-    A.mt_first = A.nt_start + nt_start.size();
-    A.pairs = A.mt_first + mt_first.size();
-    A.low = (const uint32_t*)(base + o_low);
-    A.tlow = base + o_tl;
-    A.thigh = base + o_th;
+    A.rowinfo = (const uint32_t*)base;                  // (first: read in pieces of 16 bytes)
+    A.nt_start = A.rowinfo + P.rowinfo.size();
+    A.mt_first = A.nt_start + P.nt_start.size();
+    A.pairs = A.mt_first + P.mt_first.size();
+    A.low = (const uint32_t*)(base + at.low);
+    A.tlow = base + at.tlow;
+    A.thigh = base + at.thigh;
     A.mp = mp;
     A.m1 = J.m + 1;
-    A.items = items;
-    A.MT = MT;
+    A.items = P.items;
+    A.MT = (uint32_t)P.mt_first.size() - 1;
     A.lowk = lowk;
-    A.base = num_sets_host(n, J.k);
-    A.lut = J.lut;
+    A.base = num_sets_host(n, J.size - 1);
+    for (int l = 0; l < 4; ++l) A.lut[l] = J.lut[l];
     A.G = J.G;
+    A.H = J.H;
+    A.H_stride = J.H_stride;
     A.status = J.status;
-    k_tc_rows<<<NL + NH, 128, 0, s>>>(J.packed, J.m, J.mw, mp, J.arity, lowk, NL, A.pairs, (uint32_t*)(base + o_low),
-                                     base + o_tl, base + o_th);
+    k_tc_rows<<<NL + NH, 128, 0, s>>>(J.packed, J.m, J.mw, mp, J.arity, lowk, NL, A.pairs, (uint32_t*)(base + at.low),
+                                     base + at.tlow, base + at.thigh);
     BN_LAUNCH_CHECK("k_tc_rows");
-    static unsigned long long ctx[64] = {0};
-    constexpr size_t fixed = (size_t)TJ_STAGES * (TJ_A_BYTES + TJ_B_BYTES) + 1024 + 16;
-    if (first_in_context(ctx))
-        BN_CUDA(cudaFuncSetAttribute(k_joint_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(fixed + 12 * (size_t)TJ_LUT_ROWS)));
-    const size_t smem = fixed + 12 * (size_t)A.m1;
-    k_joint_tc<<<std::min<uint32_t>((uint32_t)sm_count(), items), TJ_THREADS, smem, s>>>(A);
-    BN_LAUNCH_CHECK("k_joint_tc");
-    return BN_OK;
+    switch (J.nh) {
+    case 0: return launch<0>(A, s);
+    case 1: return launch<1>(A, s);
+    case 2: return launch<2>(A, s);
+    default: return launch<3>(A, s);
+    }
 }
 
 }  // namespace bn

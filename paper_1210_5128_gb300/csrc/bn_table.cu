@@ -204,7 +204,8 @@ __global__ void k_pad_keys(int64_t* __restrict__ keys, int n, int64_t S, int64_t
 // once per set U of at most k + 1 nodes (k_joint) instead of once per (node, parent set):
 // C(60, 5) = 5.5 M tables instead of 29.4 M at n = 60, k = 4; k_assemble forms the entries.
 // Measured at n = 60, k = 4, m = 1000, ternary: 20.0 ms with one count table per entry,
-// 4.51 ms for k_joint and 0.51 ms for k_assemble.
+// 4.51 ms for k_joint over all of them; with the sets of four and five nodes on the tensor
+// cores (bn_joint_tc.cu) 2.90 ms for those, 0.03 for k_joint and 0.34 for k_assemble.
 // ---------------------------------------------------------------------------------
 struct JointArgs {
     const uint32_t* packed;
@@ -888,16 +889,25 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
     const bool smem_data = smem + data_bytes <= LIM / 2;
     if (smem_data) smem += data_bytes;
     const int per_sm = std::max(1, std::min(2048 / (32 * nwarps), (int)((224 * 1024) / std::max<size_t>(smem + 1024, 1))));
-    // the largest sets -- nearly all of them -- on the tensor cores where they are many and
-    // one lgamma table serves them all (K2; BDeu with one arity)
-    TcPlan tcp;
-    bool tc = (P.kind == 0 || P.one_arity) && joint_tc_plan(n, m, k, P.ar.data(), &tcp);
-    uint8_t* d_tc = nullptr;
-    if (tc && sums.get(&d_tc, joint_tc_scratch(tcp, m))) {      // no room: count them as the others
-        set_error(BN_OK, "");
-        tc = false;
+    // the largest sets -- nearly all of them -- and those of four nodes on the tensor cores
+    // where they are many and one set of lgamma tables serves them all (K2; BDeu with one arity)
+    TcPlan tcp[2];                    // k + 1 nodes; four nodes where they are parent sets too
+    bool tc[2] = {false, false};
+    uint8_t* d_tc[2] = {nullptr, nullptr};
+    if (P.kind == 0 || P.one_arity) {
+        tc[0] = joint_tc_plan(n, m, k + 1, 1, P.ar.data(), &tcp[0]);
+        tc[1] = tc[0] && k == 4 && joint_tc_plan(n, m, k, 1 + P.nv, P.ar.data(), &tcp[1]);
     }
-    if (tc) A.S1 = A.S0;
+    for (int q = 0; q < 2; ++q) {
+        if (!tc[q]) continue;
+        if (sums.get(&d_tc[q], joint_tc_scratch(tcp[q], m))) {      // no room: count them as the others
+            set_error(BN_OK, "");
+            tc[q] = false;
+            if (!q) tc[1] = false;
+        } else if ((rc = joint_tc_upload(tcp[q], d_tc[q], s)))
+            return rc;
+    }
+    if (tc[0]) A.S1 = tc[1] ? num_sets_host(n, k - 1) : A.S0;
     // 8 to 64 sets a unit: about eight units a resident warp where there are enough sets
     const int64_t warps = (int64_t)sm_count() * per_sm * nwarps;
     A.range = (int)std::max<int64_t>(4, std::min<int64_t>(64, A.S1 / (8 * warps)));
@@ -917,12 +927,15 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
     else if (k <= 8) rc = launch_joint_kt<8>(A, smem_data, base, smem, grid, thr, s);
     else rc = launch_joint_kt<12>(A, smem_data, base, smem, grid, thr, s);
     if (rc) return rc;
-    if (tc) {
-        int Q = 1;
-        for (int q = 0; q <= k; ++q) Q *= P.ar[0];       // (K2's table serves any size)
-        const size_t lut = P.kind == 0 ? (size_t)P.cell_lut[1] : (size_t)P.cell_lut[Q];
-        const TcJoint J{n, m, mw, k, d_ar, d_packed, d_lut + lut * (size_t)(m + 1), A.G, d_meta, d_tc};
-        if ((rc = launch_joint_tc(J, tcp, s))) return rc;
+    for (int q = 0; q < 2; ++q) {
+        if (!tc[q]) continue;
+        int Q = 1;                    // cells of a set (K2's tables serve any number)
+        for (int j = 0; j < k + 1 - q; ++j) Q *= P.ar[0];
+        TcJoint J{n, m, mw, k + 1 - q, q ? P.nv : 0, d_ar, d_packed, {}, A.G, A.H, A.S0, d_meta, d_tc[q]};
+        J.lut[0] = d_lut + (size_t)P.cell_lut[P.kind == 0 ? 1 : Q] * (m + 1);
+        for (int v = 0; v < J.nh; ++v)
+            J.lut[1 + v] = d_lut + (size_t)P.cfg_lut[(P.kind == 0 ? 1 : Q) * P.nv + v] * (m + 1);
+        if ((rc = launch_joint_tc(J, tcp[q], s))) return rc;
     }
     AssembleArgs B{t->pst, n, k, P.S, t->Sp, A.S0, A.G, A.H, d_ar, P.vmap, d_ppf, P.log10g, t->keys};
     k_assemble<<<dim3((unsigned)((t->Sp + ASM_BLOCK - 1) / ASM_BLOCK), (unsigned)n), 256, 0, s>>>(B);

@@ -1,8 +1,10 @@
 """The joint counts of the largest sets on the tensor cores where their tiles can go wrong:
 row counts around a stage (128) and a word, every mix of arities (pairs of 4 to 16 and low
 sets of 4 to 64 states, tiles that end inside a pair block or a set), both set sizes
-(k = 3: pairs by pairs, k = 4: pairs by triples), one lgamma table for all (K2, BDeu with
-one arity) and the networks around the size from which they are used.
+(k = 3: pairs by pairs, k = 4: pairs by triples, and pairs by pairs once more for the parent
+sets of four nodes, with one to three variants of the configuration sums), one lgamma table
+for all (K2, BDeu with one arity), rows up to where the tables fill the shared memory, and
+the networks around the size from which they are used.
 
 Every entry against the oracle: 1e-12 relative, as for every table entry (counts and
 fixed-point sums are exact; one rounding)."""
@@ -17,7 +19,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("n,k,m,arities,kind", [
     (22, 4, 64, (2, 3, 4), 0), (22, 4, 127, (3,), 1), (22, 4, 128, (2,), 1), (23, 4, 129, (4,), 0),
     (21, 4, 300, (3,), 0), (24, 4, 1000, (2, 4), 0), (30, 3, 65, (2, 3, 4), 0), (30, 3, 500, (4,), 1),
-    (28, 3, 255, (2,), 0), (33, 3, 3599, (3, 4), 0), (30, 3, 3600, (2, 3), 0)])
+    (28, 3, 255, (2,), 0), (29, 4, 1574, (2, 3, 4), 0), (28, 4, 2099, (2, 3), 0), (27, 4, 3149, (3,), 1),
+    (27, 4, 1575, (2, 3, 4), 0), (28, 3, 6299, (2, 3), 0), (28, 3, 6300, (3,), 0),
+    (33, 3, 3599, (3, 4), 0), (30, 3, 3600, (2, 3), 0)])
 def test_tensor_core_counts(gpu, n, k, m, arities, kind):
     rng = np.random.default_rng(n * 1000 + m)
     ar = rng.choice(arities, n).astype(np.uint8)
