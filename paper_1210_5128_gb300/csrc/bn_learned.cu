@@ -444,91 +444,118 @@ __device__ __forceinline__ void load_z(const int32_t* row, int lane, int H, int3
     }
 }
 
-// One block's share of a learned MH step: warp w runs chain block * LR_WARPS + w; it
-// finishes the previous step (LF_FINISH) and starts the next (LF_START).  The survivors
-// are read from `sreg` once the staged copy has landed on `s_bar` (when `staged`), else
-// from global memory.  Thread 0 adds the block's re-scored items, and the last of the
-// `nblocks` blocks to finish advances the step counter.
-__device__ __forceinline__ void learned_chain_block(const ChainState& S, const LearnArgs& L, int flags, int block,
-                                                    int nblocks, const uint8_t* sreg, LWarp* sw, int64_t* s_items,
-                                                    uint64_t* s_bar, bool staged, bool stage_wait_at_end)
+// One block's share of a learned MH step: warp w runs chain block * LR_WARPS + w.  It is
+// three functions, so that a launch that runs many steps can move what does not lie on
+// the chain from the network's outputs to the next proposal into its waits:
+//   load    what the step reads besides the network's outputs (the proposal in hand, its
+//           layer-1 sums, the random numbers);
+//   step    finishes the previous step's MH test (LF_FINISH) and starts the next (LF_START);
+//   commit  what the test leaves to be written: the accepted state's exact score (a
+//           sequential FP64 sum: 60 dependent additions are 2.8 us), edge credit, best
+//           state, trace, records, the step counter.
+struct LChain {
+    int64_t t_dev;
+    int cb;
+    int32_t zc[LR_HCH][8], zq[LR_HCH][8];
+    int af, bf;
+    uint32_t pairf;
+    float lqff;
+    double uf, dpf;
+    int64_t pk[2];
+    uint32_t prk[2];
+    U64x4 x;
+    // what commit needs of the test
+    int acc;
+    bool moved, have_s2;
+    double s2;
+    int node[2];                // nodes whose parent set changes (or -1) and the set they leave
+    uint32_t old_rank[2];
+};
+
+__device__ __forceinline__ void learned_chain_load(const ChainState& S, const LearnArgs& L, int flags, int block, LWarp* sw,
+                                                   LChain& D)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c = block * LR_WARPS + warp;
+    const int n = S.n, H = L.H;
+    D.t_dev = *S.step;
+    if (c >= S.C) return;
+    LWarp& W = sw[warp];
+    for (int i = lane; i < n; i += 32) {
+        W.ord[i] = S.cur_order[(size_t)c * n + i];
+        W.rank[i] = S.cur_rank[(size_t)c * n + i];
+        W.key[i] = S.cur_key[(size_t)c * n + i];
+    }
+    D.cb = L.cur_buf[c];
+    load_z(L.z1 + (size_t)c * H, lane, H, D.zc);
+    const bool fin = (flags & LF_FINISH) != 0;
+    D.pk[0] = D.pk[1] = 0;
+    D.prk[0] = D.prk[1] = 0;
+    if (fin) {
+        load_z(L.z1p + (size_t)c * H, lane, H, D.zq);
+        D.af = L.pab[2 * c];
+        D.bf = L.pab[2 * c + 1];
+        D.pairf = L.ppair[c];
+        D.lqff = L.plqf[c];
+        D.uf = L.pu[c];
+        D.dpf = L.pdpart[c];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int p = lane + 32 * h;
+            if (p < n) {
+                D.pk[h] = L.pkey[(size_t)c * n + p];
+                D.prk[h] = L.prank[(size_t)c * n + p];
+            }
+        }
+    }
+    if (flags & LF_START)
+        D.x = philox4x64((uint64_t)(fin ? D.t_dev + 1 : D.t_dev), (uint64_t)c, 0, 0, S.seed, 0);
+    __syncwarp();
+}
+
+// The survivors are read from `sreg` once the staged copy has landed on `s_bar` (when
+// `staged`), else from global memory.
+__device__ __forceinline__ void learned_chain_step(const ChainState& S, const LearnArgs& L, int flags, int block,
+                                                   const uint8_t* sreg, LWarp* sw, uint64_t* s_bar, bool staged, LChain& D)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = block * LR_WARPS + warp;
     const int n = S.n, H = L.H, NT = L.NT;
-    const int64_t t_dev = *S.step;
-    int64_t items = 0;
     if (c < S.C) {
         LWarp& W = sw[warp];
-        // ---------------- every load that depends on nothing computed here -------------
-        for (int i = lane; i < n; i += 32) {
-            W.ord[i] = S.cur_order[(size_t)c * n + i];
-            W.rank[i] = S.cur_rank[(size_t)c * n + i];
-            W.key[i] = S.cur_key[(size_t)c * n + i];
-        }
-        double score = S.cur_score[c];
-        const double best = S.best_score[c];   // read once: lane 0 updates it below
-        int cb = L.cur_buf[c];
+        int cb = D.cb;
+        auto& zc = D.zc;
+        const auto& x = D.x;
         const float2 none = make_float2(-INFINITY, 0.f);
         const float2* pr0 = L.part + (size_t)c * NT;
         const float2* pr1 = L.part + ((size_t)S.C + c) * NT;
         const float2 q00 = lane < NT ? pr0[lane] : none, q01 = lane + 32 < NT ? pr0[lane + 32] : none;
         const float2 q10 = lane < NT ? pr1[lane] : none, q11 = lane + 32 < NT ? pr1[lane + 32] : none;
-        int32_t zc[LR_HCH][8], zq[LR_HCH][8];
-        load_z(L.z1 + (size_t)c * H, lane, H, zc);
-        const bool fin = (flags & LF_FINISH) != 0;
-        int af = 0, bf = 0;
-        uint32_t pairf = 0;
-        float lf0 = 0.f, lf1 = 0.f, lqff = 0.f;
-        double uf = 0.0, dpf = 0.0;
-        int64_t pk[2] = {0, 0};
-        uint32_t prk[2] = {0, 0};
-        if (fin) {
-            load_z(L.z1p + (size_t)c * H, lane, H, zq);
-            af = L.pab[2 * c];
-            bf = L.pab[2 * c + 1];
-            pairf = L.ppair[c];
-            lf0 = L.logits[(size_t)c * L.Pp + pairf];
-            lf1 = L.logits[((size_t)S.C + c) * L.Pp + pairf];
-            lqff = L.plqf[c];
-            uf = L.pu[c];
-            dpf = L.pdpart[c];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int p = lane + 32 * h;
-                if (p < n) {
-                    pk[h] = L.pkey[(size_t)c * n + p];
-                    prk[h] = L.prank[(size_t)c * n + p];
-                }
-            }
-        }
-        const int64_t ts = fin ? t_dev + 1 : t_dev;
-        U64x4 x;
-        if (flags & LF_START) x = philox4x64((uint64_t)ts, (uint64_t)c, 0, 0, S.seed, 0);
-        __syncwarp();
-        // ---------------- finish step tf: the MH test with the reverse proposal ----------
-        if (fin) {
-            const int64_t tf = t_dev;
-            const int a = af, b = bf;
+        // ---------------- finish step t_dev: the MH test with the reverse proposal ----------
+        if (flags & LF_FINISH) {
+            const float lf = L.logits[((size_t)(1 - cb) * S.C + c) * L.Pp + D.pairf];
+            const int a = D.af, b = D.bf;
+            const double uf = D.uf, dpf = D.dpf;
             const int nb = 1 - cb;
             float M, w[2];
             const float lse = nb ? row_lse_v(q10, q11, M, w) : row_lse_v(q00, q01, M, w);
-            const float lrev = log_q(nb ? lf1 : lf0, lse, L.eps, L.P);
-            const double corr = (double)lrev - (double)lqff;
+            const float lrev = log_q(lf, lse, L.eps, L.P);
+            const double corr = (double)lrev - (double)D.lqff;
             // the proposal's keys: positions a..b hold its re-scored nodes, the rest keep theirs
-            uint32_t nrank[2] = {0, 0};
-            int node[2] = {-1, -1};
             bool mv = false;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int p = lane + 32 * h;
+                D.node[h] = -1;
                 if (p < n) {
                     if (p >= a && p <= b) {
                         const int v = (p == a) ? W.ord[b] : (p == b) ? W.ord[a] : W.ord[p];
-                        node[h] = v;
-                        nrank[h] = prk[h];
-                        W.nkey[v] = pk[h];
-                        mv |= prk[h] != W.rank[v];
+                        W.nkey[v] = D.pk[h];
+                        if (D.prk[h] != W.rank[v]) {
+                            mv = true;
+                            D.node[h] = v;
+                            D.old_rank[h] = W.rank[v];
+                        }
                     } else {
                         const int v = W.ord[p];
                         W.nkey[v] = W.key[v];
@@ -537,110 +564,62 @@ __device__ __forceinline__ void learned_chain_block(const ChainState& S, const L
             }
             const bool moved = __any_sync(0xffffffffu, mv);
             __syncwarp();
-            int acc = 0;
+            int acc = 0, exact = 0;
             double s2 = 0.0;
             if (lane == 0) {
                 const float luf = logf((float)uf);
                 const double xa = (S.literal_log ? dpf : LN10 * dpf) + corr;
                 const double margin = 1e-6 * (1.0 + fabs((double)luf)) + (moved ? L.margin_x : 0.0);
                 const double gap = (double)luf - xa;
-                int exact = 0;
                 if (gap > margin) acc = 0;
-                else if (gap < -margin) { acc = 1; exact = 1; }
-                else exact = 2;
+                else if (gap < -margin) acc = 1;
+                else exact = 1;
                 if (exact && !moved) {
                     // no parent set changes: s' = s bit for bit, the test is ln u < corr
-                    s2 = score;
-                    if (exact == 2) acc = log(uf) < __dadd_rn(S.literal_log ? 0.0 : __dmul_rn(LN10, 0.0), corr);
+                    acc = log(uf) < __dadd_rn(S.literal_log ? 0.0 : __dmul_rn(LN10, 0.0), corr);
                 } else if (exact) {
                     for (int i = 0; i < n; ++i) s2 = __dadd_rn(s2, key_to_double(W.nkey[i]));
-                    if (exact == 2) {
-                        const double delta = __dsub_rn(s2, score);
-                        const double lu = log(uf);
-                        acc = S.literal_log ? (lu < __dadd_rn(delta, corr))
-                                            : (lu < __dadd_rn(__dmul_rn(LN10, delta), corr));
-                    }
+                    const double delta = __dsub_rn(s2, S.cur_score[c]);
+                    const double lu = log(uf);
+                    acc = S.literal_log ? (lu < __dadd_rn(delta, corr)) : (lu < __dadd_rn(__dmul_rn(LN10, delta), corr));
                 }
             }
             acc = __shfl_sync(0xffffffffu, acc, 0);
-            s2 = __shfl_sync(0xffffffffu, s2, 0);
-            items = b - a + 1;
+            D.acc = acc;
+            D.moved = moved;
+            D.have_s2 = exact && moved;                 // (lane 0)
+            D.s2 = s2;
             if (acc) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int v = node[h];
-                    if (v >= 0 && nrank[h] != W.rank[v]) {
-                        const size_t si = (size_t)c * n + v;
-                        credit_edges(S, c, v, W.rank[v], L.since[si], tf);
-                        L.since[si] = tf;
-                        W.rank[v] = nrank[h];
+                    const int v = D.node[h];
+                    if (v >= 0) {
+                        W.rank[v] = D.prk[h];
                         W.key[v] = W.nkey[v];
                     }
                 }
-                __syncwarp();
                 if (lane == 0) {
                     const uint8_t oa = W.ord[a];
                     W.ord[a] = W.ord[b];
                     W.ord[b] = oa;
                 }
-                __syncwarp();
                 // the proposal's layer-1 sums and network outputs become the current ones
 #pragma unroll
                 for (int q = 0; q < LR_HCH; ++q) {
                     const int h0 = lane * 8 + 256 * q;
                     if (h0 < H) {
                         int32_t* dst = L.z1 + (size_t)c * H + h0;
-                        *(int4*)dst = make_int4(zq[q][0], zq[q][1], zq[q][2], zq[q][3]);
-                        *(int4*)(dst + 4) = make_int4(zq[q][4], zq[q][5], zq[q][6], zq[q][7]);
+                        *(int4*)dst = make_int4(D.zq[q][0], D.zq[q][1], D.zq[q][2], D.zq[q][3]);
+                        *(int4*)(dst + 4) = make_int4(D.zq[q][4], D.zq[q][5], D.zq[q][6], D.zq[q][7]);
+                    }
+                }
+            }
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) zc[q][j] = zq[q][j];
-                    }
-                }
-                cb = nb;
-                score = s2;
-                for (int i = lane; i < n; i += 32) {
-                    S.cur_order[(size_t)c * n + i] = W.ord[i];
-                    S.cur_rank[(size_t)c * n + i] = W.rank[i];
-                    S.cur_key[(size_t)c * n + i] = W.key[i];
-                }
-                if (s2 > best) {
-                    for (int i = lane; i < n; i += 32) {
-                        S.best_order[(size_t)c * n + i] = W.ord[i];
-                        S.best_rank[(size_t)c * n + i] = W.rank[i];
-                    }
-                    if (lane == 0) S.best_score[c] = s2;
-                }
-                if (lane == 0) {
-                    L.cur_buf[c] = (uint8_t)cb;
-                    S.cur_score[c] = s2;
-                    S.accepts[c] += 1;
-                }
-            }
-            if (lane == 0 && tf < S.trace_cap) {
-                S.trace_score[(size_t)c * S.trace_cap + tf] = score;
-                S.trace_accept[(size_t)c * S.trace_cap + tf] = (uint8_t)acc;
-            }
-            if (tf >= S.burn_in && S.record_every > 0 && ((tf - S.burn_in) % S.record_every) == 0 &&
-                (tf - S.burn_in) / S.record_every < S.record_cap) {
-                const int64_t ridx = (tf - S.burn_in) / S.record_every;
-                for (int i = lane; i < n; i += 32) {
-                    uint64_t m = S.pst[W.rank[i]];
-                    while (m) {
-                        const int slot = __ffsll((long long)m) - 1;
-                        m &= m - 1;
-                        const int par = slot + (slot >= i ? 1 : 0);
-                        atomicOr((unsigned long long*)&S.rec_bits[(((size_t)c * n + i) * n + par) * S.rec_words + (ridx >> 6)],
-                                 1ull << (ridx & 63));
-                    }
-                }
-            }
-            if (flags & LF_FLUSH) {
-                for (int i = lane; i < n; i += 32) {
-                    const size_t si = (size_t)c * n + i;
-                    credit_edges(S, c, i, W.rank[i], L.since[si], tf + 1);
-                    L.since[si] = tf + 1;
-                }
-            }
+            for (int q = 0; q < LR_HCH; ++q)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) zc[q][j] = acc ? D.zq[q][j] : zc[q][j];
+            cb = acc ? nb : cb;
+            D.cb = cb;
             __syncwarp();
         }
         // ---------------- start step ts: draw, swap, re-score, layer 1 ---------------------
@@ -807,31 +786,107 @@ __device__ __forceinline__ void learned_chain_block(const ChainState& S, const L
             }
         }
     }
+}
+
+// Thread 0 adds the block's re-scored items, and the last of the `nblocks` blocks to finish
+// advances the step counter.
+__device__ __forceinline__ void learned_chain_commit(const ChainState& S, const LearnArgs& L, int flags, int block,
+                                                     int nblocks, LWarp* sw, int64_t* s_items, const LChain& D)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c = block * LR_WARPS + warp;
+    const int n = S.n;
+    int64_t items = 0;
+    if (c < S.C && (flags & LF_FINISH)) {
+        const LWarp& W = sw[warp];
+        const int64_t tf = D.t_dev;
+        items = D.bf - D.af + 1;
+        double score = S.cur_score[c];
+        if (D.acc) {
+            const double best = S.best_score[c];   // read once: lane 0 updates it below
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int v = D.node[h];
+                if (v >= 0) {
+                    const size_t si = (size_t)c * n + v;
+                    credit_edges(S, c, v, D.old_rank[h], L.since[si], tf);
+                    L.since[si] = tf;
+                }
+            }
+            double s2 = score;                          // no parent set changes: s' = s bit for bit
+            if (D.moved && lane == 0) {
+                s2 = D.s2;
+                if (!D.have_s2)
+                    for (int i = 0; i < n; ++i) s2 = __dadd_rn(s2, key_to_double(W.key[i]));
+            }
+            s2 = __shfl_sync(0xffffffffu, s2, 0);
+            score = s2;
+            for (int i = lane; i < n; i += 32) {
+                S.cur_order[(size_t)c * n + i] = W.ord[i];
+                S.cur_rank[(size_t)c * n + i] = W.rank[i];
+                S.cur_key[(size_t)c * n + i] = W.key[i];
+            }
+            if (s2 > best) {
+                for (int i = lane; i < n; i += 32) {
+                    S.best_order[(size_t)c * n + i] = W.ord[i];
+                    S.best_rank[(size_t)c * n + i] = W.rank[i];
+                }
+                if (lane == 0) S.best_score[c] = s2;
+            }
+            if (lane == 0) {
+                L.cur_buf[c] = (uint8_t)D.cb;
+                S.cur_score[c] = s2;
+                S.accepts[c] += 1;
+            }
+        }
+        if (lane == 0 && tf < S.trace_cap) {
+            S.trace_score[(size_t)c * S.trace_cap + tf] = score;
+            S.trace_accept[(size_t)c * S.trace_cap + tf] = (uint8_t)D.acc;
+        }
+        if (tf >= S.burn_in && S.record_every > 0 && ((tf - S.burn_in) % S.record_every) == 0 &&
+            (tf - S.burn_in) / S.record_every < S.record_cap) {
+            const int64_t ridx = (tf - S.burn_in) / S.record_every;
+            for (int i = lane; i < n; i += 32) {
+                uint64_t m = S.pst[W.rank[i]];
+                while (m) {
+                    const int slot = __ffsll((long long)m) - 1;
+                    m &= m - 1;
+                    const int par = slot + (slot >= i ? 1 : 0);
+                    atomicOr((unsigned long long*)&S.rec_bits[(((size_t)c * n + i) * n + par) * S.rec_words + (ridx >> 6)],
+                             1ull << (ridx & 63));
+                }
+            }
+        }
+        if (flags & LF_FLUSH) {
+            for (int i = lane; i < n; i += 32) {
+                const size_t si = (size_t)c * n + i;
+                credit_edges(S, c, i, W.rank[i], L.since[si], tf + 1);
+                L.since[si] = tf + 1;
+            }
+        }
+        __syncwarp();
+    }
     if (lane == 0) s_items[warp] = items;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        if (staged && stage_wait_at_end) mbar_wait_bounded(s_bar, 0, WAIT_TIMEOUT_NS);   // no copy left in flight
-        if (flags & LF_FINISH) {
-            int64_t tot = 0;
-            for (int w = 0; w < LR_WARPS; ++w) tot += s_items[w];
-            if (tot) atomicAdd((unsigned long long*)S.items_total, (unsigned long long)tot);
-            // the last block advances the step counter
-            __threadfence();
-            const uint32_t ticket = atomicAdd(L.done, 1u);
-            if (ticket == (uint32_t)nblocks - 1) {
-                const int64_t t_end = t_dev + 1;
-                *S.step = t_end;
-                if (S.record_every > 0 && t_end > S.burn_in) {
-                    const int64_t r = (t_end - 1 - S.burn_in) / S.record_every + 1;
-                    *S.rec_count = r < S.record_cap ? r : S.record_cap;
-                }
-                *L.done = 0;
-                __threadfence();
+    if (threadIdx.x == 0 && (flags & LF_FINISH)) {
+        int64_t tot = 0;
+        for (int w = 0; w < LR_WARPS; ++w) tot += s_items[w];
+        if (tot) atomicAdd((unsigned long long*)S.items_total, (unsigned long long)tot);
+        // the last block advances the step counter
+        __threadfence();
+        const uint32_t ticket = atomicAdd(L.done, 1u);
+        if (ticket == (uint32_t)nblocks - 1) {
+            const int64_t t_end = D.t_dev + 1;
+            *S.step = t_end;
+            if (S.record_every > 0 && t_end > S.burn_in) {
+                const int64_t r = (t_end - 1 - S.burn_in) / S.record_every + 1;
+                *S.rec_count = r < S.record_cap ? r : S.record_cap;
             }
+            *L.done = 0;
+            __threadfence();
         }
     }
 }
-
 
 __global__ void __launch_bounds__(32 * LR_WARPS) k_learned_chain(ChainState S, LearnArgs L, int flags)
 {
@@ -850,7 +905,11 @@ __global__ void __launch_bounds__(32 * LR_WARPS) k_learned_chain(ChainState S, L
     griddep_wait();
     griddep_launch();
     __syncthreads();
-    learned_chain_block(S, L, flags, blockIdx.x, gridDim.x, sreg, sw, s_items, &s_bar, staged, true);
+    LChain D;
+    learned_chain_load(S, L, flags, blockIdx.x, sw, D);
+    learned_chain_step(S, L, flags, blockIdx.x, sreg, sw, &s_bar, staged, D);
+    learned_chain_commit(S, L, flags, blockIdx.x, gridDim.x, sw, s_items, D);
+    if (threadIdx.x == 0 && staged) mbar_wait_bounded(&s_bar, 0, WAIT_TIMEOUT_NS);   // no copy left in flight
 }
 
 // ---------------------------------------------------------------------------------
@@ -861,7 +920,11 @@ __global__ void __launch_bounds__(32 * LR_WARPS) k_learned_chain(ChainState S, L
 // the next) -- separated by grid-wide barriers instead of kernel boundaries.  Every CTA
 // keeps its layer-2 or output-layer weight tile in shared memory and its TMEM columns for
 // the whole launch, and the chain CTAs keep the survivors staged; only the activations
-// and the chains' outputs pass through L2.  CTAs [0, n3) own output-layer tiles, CTAs
+// and the chains' outputs pass through L2.  What the chains' phase does not owe the next
+// GEMM waits: its inputs are loaded before the barrier in front of it, its bookkeeping
+// written behind the arrival after it (256 chains, n = 60, H = 512: 37 -> 26 us a step; of
+// 50,000 cycles of the step's slowest chain 25,000 went to the exact score, the edge credit
+// and to code that only accepting chains run).  CTAs [0, n3) own output-layer tiles, CTAs
 // [n3, n3 + n2) layer-2 tiles, and CTAs [0, nc) four chains each.
 struct PersistArgs {
     int iters;
@@ -879,16 +942,22 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p)
     return v;
 }
 
-// grid-wide barrier number k (1, 2, ...) of the launch: every CTA's writes before it are
-// visible after it, to generic loads and to the bulk copies (async proxy) issued after
-// it.  Bounded: false once the wait has run out (status gets STATUS_TIMEOUT).
-__device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target, uint32_t* status, int* s_ok)
+// grid-wide barrier number k (1, 2, ...) of the launch in two halves: every CTA's writes
+// before its arrival are visible after the wait, to generic loads and to the bulk copies
+// (async proxy) issued after it.  Bounded: false once the wait has run out (status gets
+// STATUS_TIMEOUT).
+__device__ __forceinline__ void grid_arrive(uint32_t* counter)
 {
     asm volatile("fence.proxy.async.global;" ::: "memory");
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(counter, 1u);
+    }
+}
+__device__ __forceinline__ bool grid_wait(uint32_t* counter, uint32_t target, uint32_t* status, int* s_ok)
+{
+    if (threadIdx.x == 0) {
         bool ok = true;
         if (ld_acquire_gpu(counter) < target) {
             const uint64_t t0 = global_timer_ns();
@@ -1005,13 +1074,19 @@ __global__ void __launch_bounds__(32 * LR_WARPS, 1)
         for (int it = 0; it < P.iters; ++it) {
             const uint32_t parity = (uint32_t)(it & 1);
             if (is2 && !persist_gemm(g2, mt, nt, sA, sB, bar, parity, tmem, &s_okg)) ok = false;
-            if (!grid_barrier(P.gsync, G * ++nb, g2.status, &s_okb) || !ok) break;
+            grid_arrive(P.gsync);
+            if (!grid_wait(P.gsync, G * ++nb, g2.status, &s_okb) || !ok) break;
             if (is3 && !persist_gemm(g3, mt, nt, sA, sB, bar, parity, tmem, &s_okg)) ok = false;
-            if (!grid_barrier(P.gsync, G * ++nb, g2.status, &s_okb) || !ok) break;
-            if (isc)
-                learned_chain_block(S, L, LF_FINISH | LF_START, cta, P.nc, psm, sw, s_items, &bar[KB + 2], staged,
-                                    false);
-            if (it + 1 < P.iters && !grid_barrier(P.gsync, G * ++nb, g2.status, &s_okb)) break;
+            grid_arrive(P.gsync);
+            LChain D;
+            if (isc) learned_chain_load(S, L, LF_FINISH | LF_START, cta, sw, D);
+            if (!grid_wait(P.gsync, G * ++nb, g2.status, &s_okb) || !ok) break;
+            if (isc) learned_chain_step(S, L, LF_FINISH | LF_START, cta, psm, sw, &bar[KB + 2], staged, D);
+            if (it + 1 < P.iters) grid_arrive(P.gsync);
+            // the state's bookkeeping while layer 2 runs on other CTAs; this CTA's next arrival
+            // comes after it
+            if (isc) learned_chain_commit(S, L, LF_FINISH | LF_START, cta, P.nc, sw, s_items, D);
+            if (it + 1 < P.iters && !grid_wait(P.gsync, G * ++nb, g2.status, &s_okb)) break;
         }
     }
     if (tid == 0 && staged) mbar_wait_bounded(&bar[KB + 2], 0, WAIT_TIMEOUT_NS);   // no copy left in flight
