@@ -285,8 +285,15 @@ __host__ __device__ constexpr size_t lgemm_smem(int K)
 }
 
 // epilogue of one 128 x 32 tile: TMEM -> bias (+ ReLU -> bf16 operand of the next layer, or
-// logits + per-tile softmax partials of the output layer); warp w holds rows 32w..32w+31
-__device__ __forceinline__ void lgemm_epilogue(const LGemmArgs& g, uint32_t tmem, int warp, int lane, int mt, int nt)
+// logits + per-tile softmax partials of the output layer); warp w holds rows 32w..32w+31.
+// bias: of the tile's 32 columns; cb: the row's current buffer (output layer).
+__device__ __forceinline__ int lgemm_cur_buf(const LGemmArgs& g, int mt)
+{
+    const int row = mt * LR_TM + (int)threadIdx.x;
+    return g.mode != 0 && row < g.C ? g.cur_buf[row] : 0;
+}
+__device__ __forceinline__ void lgemm_epilogue(const LGemmArgs& g, uint32_t tmem, int warp, int lane, int mt, int nt,
+                                               const float* bias, int cb)
 {
     uint32_t r[32];
     tc_ld_32x32b_x32(tmem + ((uint32_t)(warp * 32) << 16), r);
@@ -298,7 +305,7 @@ __device__ __forceinline__ void lgemm_epilogue(const LGemmArgs& g, uint32_t tmem
         for (int q = 0; q < 4; ++q) {
             float v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = fmaxf(__uint_as_float(r[q * 8 + j]) + g.bias[n0 + q * 8 + j], 0.f);
+            for (int j = 0; j < 8; ++j) v[j] = fmaxf(__uint_as_float(r[q * 8 + j]) + bias[q * 8 + j], 0.f);
             uint4 o;
             o.x = pack_bf16x2(v[0], v[1]);
             o.y = pack_bf16x2(v[2], v[3]);
@@ -307,14 +314,13 @@ __device__ __forceinline__ void lgemm_epilogue(const LGemmArgs& g, uint32_t tmem
             *(uint4*)(g.out_h + cm_off(row, n0 + q * 8, g.K, LR_TM)) = o;
         }
     } else if (row < g.C) {
-        const int cb = g.cur_buf[row];
         const int buf = g.prime ? cb : 1 - cb;
         float* dst = g.logits + ((size_t)buf * g.C + row) * g.Pp + n0;
         float v[32];
         float mx = -INFINITY;
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
-            v[j] = __uint_as_float(r[j]) + g.bias[n0 + j];
+            v[j] = __uint_as_float(r[j]) + bias[j];
             if (n0 + j < g.P) mx = fmaxf(mx, v[j]);
         }
 #pragma unroll
@@ -393,7 +399,7 @@ __global__ void __launch_bounds__(128) k_learned_gemm(LGemmArgs g)
     tc_fence_after();
     const bool all_ok = __syncthreads_and(done_ok && *s_ok);
     if (all_ok) {
-        lgemm_epilogue(g, tmem, warp, lane, mt, nt);
+        lgemm_epilogue(g, tmem, warp, lane, mt, nt, g.bias + nt * LR_TN, lgemm_cur_buf(g, mt));
     } else if (tid == 0) {
         atomicOr(g.status, STATUS_TIMEOUT);
     }
@@ -473,12 +479,12 @@ struct LChain {
 };
 
 __device__ __forceinline__ void learned_chain_load(const ChainState& S, const LearnArgs& L, int flags, int block, LWarp* sw,
-                                                   LChain& D)
+                                                   int64_t t, LChain& D)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = block * LR_WARPS + warp;
     const int n = S.n, H = L.H;
-    D.t_dev = *S.step;
+    D.t_dev = t;
     if (c >= S.C) return;
     LWarp& W = sw[warp];
     for (int i = lane; i < n; i += 32) {
@@ -619,7 +625,7 @@ __device__ __forceinline__ void learned_chain_step(const ChainState& S, const Le
 #pragma unroll
                 for (int j = 0; j < 8; ++j) zc[q][j] = acc ? D.zq[q][j] : zc[q][j];
             cb = acc ? nb : cb;
-            D.cb = cb;
+            if (acc && lane == 0) L.cur_buf[c] = (uint8_t)cb;
             __syncwarp();
         }
         // ---------------- start step ts: draw, swap, re-score, layer 1 ---------------------
@@ -788,10 +794,9 @@ __device__ __forceinline__ void learned_chain_step(const ChainState& S, const Le
     }
 }
 
-// Thread 0 adds the block's re-scored items, and the last of the `nblocks` blocks to finish
-// advances the step counter.
-__device__ __forceinline__ void learned_chain_commit(const ChainState& S, const LearnArgs& L, int flags, int block,
-                                                     int nblocks, LWarp* sw, int64_t* s_items, const LChain& D)
+// Returns the chain's re-scored items.
+__device__ __forceinline__ int64_t learned_chain_commit(const ChainState& S, const LearnArgs& L, int flags, int block,
+                                                        LWarp* sw, const LChain& D)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = block * LR_WARPS + warp;
@@ -834,7 +839,6 @@ __device__ __forceinline__ void learned_chain_commit(const ChainState& S, const 
                 if (lane == 0) S.best_score[c] = s2;
             }
             if (lane == 0) {
-                L.cur_buf[c] = (uint8_t)D.cb;
                 S.cur_score[c] = s2;
                 S.accepts[c] += 1;
             }
@@ -866,17 +870,23 @@ __device__ __forceinline__ void learned_chain_commit(const ChainState& S, const 
         }
         __syncwarp();
     }
-    if (lane == 0) s_items[warp] = items;
+    return items;
+}
+
+// Thread 0 adds the block's re-scored items, and the last of the `nblocks` blocks to finish
+// sets the step counter to t_end.
+__device__ __forceinline__ void learned_advance(const ChainState& S, const LearnArgs& L, int nblocks, int64_t* s_items,
+                                                int64_t items, int64_t t_end)
+{
+    if ((threadIdx.x & 31) == 0) s_items[threadIdx.x >> 5] = items;
     __syncthreads();
-    if (threadIdx.x == 0 && (flags & LF_FINISH)) {
+    if (threadIdx.x == 0) {
         int64_t tot = 0;
         for (int w = 0; w < LR_WARPS; ++w) tot += s_items[w];
         if (tot) atomicAdd((unsigned long long*)S.items_total, (unsigned long long)tot);
-        // the last block advances the step counter
         __threadfence();
         const uint32_t ticket = atomicAdd(L.done, 1u);
         if (ticket == (uint32_t)nblocks - 1) {
-            const int64_t t_end = D.t_dev + 1;
             *S.step = t_end;
             if (S.record_every > 0 && t_end > S.burn_in) {
                 const int64_t r = (t_end - 1 - S.burn_in) / S.record_every + 1;
@@ -906,9 +916,10 @@ __global__ void __launch_bounds__(32 * LR_WARPS) k_learned_chain(ChainState S, L
     griddep_launch();
     __syncthreads();
     LChain D;
-    learned_chain_load(S, L, flags, blockIdx.x, sw, D);
+    learned_chain_load(S, L, flags, blockIdx.x, sw, *S.step, D);
     learned_chain_step(S, L, flags, blockIdx.x, sreg, sw, &s_bar, staged, D);
-    learned_chain_commit(S, L, flags, blockIdx.x, gridDim.x, sw, s_items, D);
+    const int64_t items = learned_chain_commit(S, L, flags, blockIdx.x, sw, D);
+    if (flags & LF_FINISH) learned_advance(S, L, gridDim.x, s_items, items, D.t_dev + 1);
     if (threadIdx.x == 0 && staged) mbar_wait_bounded(&s_bar, 0, WAIT_TIMEOUT_NS);   // no copy left in flight
 }
 
@@ -917,20 +928,25 @@ __global__ void __launch_bounds__(32 * LR_WARPS) k_learned_chain(ChainState S, L
 // ---------------------------------------------------------------------------------
 // One cooperative launch runs many MH steps.  A step is three phases -- layer 2 on the
 // proposals' layer-1 outputs, the output layer, then the chains (finish the step, start
-// the next) -- separated by grid-wide barriers instead of kernel boundaries.  Every CTA
-// keeps its layer-2 or output-layer weight tile in shared memory and its TMEM columns for
-// the whole launch, and the chain CTAs keep the survivors staged; only the activations
+// the next) -- handed on through counters in global memory instead of kernel boundaries:
+// a phase waits for the CTAs of the phase before it that work on its 128 chains.  Every
+// CTA keeps its layer-2 or output-layer weight tile in shared memory and its TMEM columns
+// for the whole launch, and the chain CTAs keep the survivors staged; only the activations
 // and the chains' outputs pass through L2.  What the chains' phase does not owe the next
-// GEMM waits: its inputs are loaded before the barrier in front of it, its bookkeeping
-// written behind the arrival after it (256 chains, n = 60, H = 512: 37 -> 26 us a step; of
-// 50,000 cycles of the step's slowest chain 25,000 went to the exact score, the edge credit
-// and to code that only accepting chains run).  CTAs [0, n3) own output-layer tiles, CTAs
-// [n3, n3 + n2) layer-2 tiles, and CTAs [0, nc) four chains each.
+// GEMM waits: its inputs are loaded before the wait in front of it, its bookkeeping written
+// behind the arrival after it.  256 chains, n = 60, H = 512: 37 us a step with grid-wide
+// barriers and everything between them (of 50,000 cycles of the step's slowest chain 25,000
+// went to the exact score, the edge credit and to code that only accepting chains run), 26
+// with those out of the way, 23 with a counter a phase and 128 chains.
+// CTAs [0, n3) own output-layer tiles, CTAs [n3, n3 + n2) layer-2 tiles; a block of four
+// chains goes to a CTA with an output tile of the same 128 chains (nt3 >= 32), else block b
+// to CTA b.
+static constexpr int LR_SYNC = 32;       // a counter a 128-byte line
 struct PersistArgs {
     int iters;
     int n2, n3, nc;
     int nt2, nt3;                 // N tiles of layer 2 (H / 32) and of the output layer (NT)
-    uint32_t* gsync;              // grid barrier counter, zero at launch
+    uint32_t* gsync;              // [M tiles][3] counters, LR_SYNC words apart, zero at launch
     uint32_t a_off, b_off, bar_off;   // dynamic shared memory: A tile, B tile, barriers
     int staged;                   // chain CTAs stage the survivors at [0, L.sreg_bytes)
 };
@@ -942,11 +958,11 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p)
     return v;
 }
 
-// grid-wide barrier number k (1, 2, ...) of the launch in two halves: every CTA's writes
-// before its arrival are visible after the wait, to generic loads and to the bulk copies
-// (async proxy) issued after it.  Bounded: false once the wait has run out (status gets
+// Hands a CTA's work on: its writes before the arrival are visible, to generic loads and to
+// the bulk copies (async proxy), after a wait for a count that includes it, and so on
+// through further hand-overs.  Waits are bounded: false once one has run out (status gets
 // STATUS_TIMEOUT).
-__device__ __forceinline__ void grid_arrive(uint32_t* counter)
+__device__ __forceinline__ void phase_arrive(uint32_t* counter)
 {
     asm volatile("fence.proxy.async.global;" ::: "memory");
     __syncthreads();
@@ -955,7 +971,7 @@ __device__ __forceinline__ void grid_arrive(uint32_t* counter)
         atomicAdd(counter, 1u);
     }
 }
-__device__ __forceinline__ bool grid_wait(uint32_t* counter, uint32_t target, uint32_t* status, int* s_ok)
+__device__ __forceinline__ bool phase_wait(const uint32_t* counter, uint32_t target, uint32_t* status, int* s_ok)
 {
     if (threadIdx.x == 0) {
         bool ok = true;
@@ -980,9 +996,11 @@ __device__ __forceinline__ bool grid_wait(uint32_t* counter, uint32_t target, ui
 // one GEMM tile of a phase: A (128 rows x K) by bulk copies, one mbarrier per 64-wide K
 // block (phase `parity`), MMAs into `tmem` as the blocks land, commit, epilogue
 __device__ __forceinline__ bool persist_gemm(const LGemmArgs& g, int mt, int nt, uint8_t* sA, const uint8_t* sB,
-                                             uint64_t* bar, uint32_t parity, uint32_t tmem, int* s_okg)
+                                             uint64_t* bar, uint32_t parity, uint32_t tmem, int* s_okg,
+                                             const float* bias)
 {
     const int KB = g.K >> 6, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int cb = lgemm_cur_buf(g, mt);
     if (tid == 0) {
         *s_okg = 1;
         const uint64_t pol = l2_policy_evict_last();
@@ -1013,7 +1031,7 @@ __device__ __forceinline__ bool persist_gemm(const LGemmArgs& g, int mt, int nt,
     const bool done_ok = mbar_wait_bounded(&bar[KB], parity, WAIT_TIMEOUT_NS);
     tc_fence_after();
     const bool all_ok = __syncthreads_and(done_ok && *s_okg);
-    if (all_ok) lgemm_epilogue(g, tmem, warp, lane, mt, nt);
+    if (all_ok) lgemm_epilogue(g, tmem, warp, lane, mt, nt, bias, cb);
     else if (tid == 0) atomicOr(g.status, STATUS_TIMEOUT);
     tc_fence_before();
     return all_ok;
@@ -1027,14 +1045,25 @@ __global__ void __launch_bounds__(32 * LR_WARPS, 1)
     __shared__ LWarp sw[LR_WARPS];
     __shared__ int64_t s_items[LR_WARPS];
     __shared__ uint32_t s_tslot;
-    __shared__ int s_okg, s_okb;                       // GEMM and grid-barrier outcomes
+    __shared__ int s_okg, s_okb;                       // GEMM and wait outcomes
+    __shared__ float s_bias[LR_TN];
     const int cta = blockIdx.x, tid = threadIdx.x;
-    const bool is3 = cta < P.n3, is2 = !is3 && cta < P.n3 + P.n2, isc = cta < P.nc;
+    const bool is3 = cta < P.n3, is2 = !is3 && cta < P.n3 + P.n2;
     const bool gemm = is3 || is2;
     const LGemmArgs& g = is3 ? g3 : g2;
     const int tile = is3 ? cta : cta - P.n3;
     const int ntiles = is3 ? P.nt3 : P.nt2;
     const int mt = gemm ? tile / ntiles : 0, nt = gemm ? tile - mt * ntiles : 0;
+    constexpr int per = LR_TM / LR_WARPS;              // chain blocks of an M tile
+    const int cblock = P.nt3 < per ? cta : cta % P.nt3 < per ? cta / P.nt3 * per + cta % P.nt3 : P.nc;
+    const bool isc = cblock < P.nc;
+    const int cmt = cblock / per;
+    const uint32_t nc_mt = (uint32_t)min(per, P.nc - mt * per);        // chain blocks of the GEMM's M tile
+    uint32_t* sync2 = P.gsync + (size_t)(3 * mt) * LR_SYNC;            // layer-2 tiles done, ...
+    uint32_t* sync3 = sync2 + LR_SYNC;                                 // output tiles done,
+    uint32_t* syncc = sync3 + LR_SYNC;                                 // chain blocks done, of the M tile
+    uint32_t* csync3 = P.gsync + (size_t)(3 * cmt + 1) * LR_SYNC;      // the same of the chains' M tile
+    uint32_t* csyncc = csync3 + LR_SYNC;
     const int KB = g2.K >> 6;
     uint8_t* sA = psm + P.a_off;
     uint8_t* sB = psm + P.b_off;
@@ -1060,6 +1089,8 @@ __global__ void __launch_bounds__(32 * LR_WARPS, 1)
             bulk_g2s(psm, L.sreg, L.sreg_bytes, &bar[KB + 2], l2_policy_evict_last());
         }
     }
+    if (gemm && tid < LR_TN) s_bias[tid] = g.bias[nt * LR_TN + tid];
+    const int64_t t0 = *S.step;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1069,25 +1100,31 @@ __global__ void __launch_bounds__(32 * LR_WARPS, 1)
     if (!__syncthreads_and(ok)) {
         if (tid == 0) atomicOr(g2.status, STATUS_TIMEOUT);
     } else {
-        const uint32_t G = (uint32_t)gridDim.x;
-        uint32_t nb = 0;                                // barriers passed
-        for (int it = 0; it < P.iters; ++it) {
-            const uint32_t parity = (uint32_t)(it & 1);
-            if (is2 && !persist_gemm(g2, mt, nt, sA, sB, bar, parity, tmem, &s_okg)) ok = false;
-            grid_arrive(P.gsync);
-            if (!grid_wait(P.gsync, G * ++nb, g2.status, &s_okb) || !ok) break;
-            if (is3 && !persist_gemm(g3, mt, nt, sA, sB, bar, parity, tmem, &s_okg)) ok = false;
-            grid_arrive(P.gsync);
-            LChain D;
-            if (isc) learned_chain_load(S, L, LF_FINISH | LF_START, cta, sw, D);
-            if (!grid_wait(P.gsync, G * ++nb, g2.status, &s_okb) || !ok) break;
-            if (isc) learned_chain_step(S, L, LF_FINISH | LF_START, cta, psm, sw, &bar[KB + 2], staged, D);
-            if (it + 1 < P.iters) grid_arrive(P.gsync);
-            // the state's bookkeeping while layer 2 runs on other CTAs; this CTA's next arrival
-            // comes after it
-            if (isc) learned_chain_commit(S, L, LF_FINISH | LF_START, cta, P.nc, sw, s_items, D);
-            if (it + 1 < P.iters && !grid_wait(P.gsync, G * ++nb, g2.status, &s_okb)) break;
+        int64_t items = 0;
+        int it = 0;
+        for (; it < P.iters; ++it) {
+            const uint32_t parity = (uint32_t)(it & 1), n_done = (uint32_t)it;
+            if (is2) {
+                if (!phase_wait(syncc, n_done * nc_mt, g2.status, &s_okb)) break;
+                if (!persist_gemm(g2, mt, nt, sA, sB, bar, parity, tmem, &s_okg, s_bias)) break;
+                phase_arrive(sync2);
+            }
+            if (is3) {
+                if (!phase_wait(sync2, (n_done + 1) * (uint32_t)P.nt2, g2.status, &s_okb)) break;
+                if (!persist_gemm(g3, mt, nt, sA, sB, bar, parity, tmem, &s_okg, s_bias)) break;
+                phase_arrive(sync3);
+            }
+            if (isc) {
+                LChain D;
+                learned_chain_load(S, L, LF_FINISH | LF_START, cblock, sw, t0 + it, D);
+                if (!phase_wait(csync3, (n_done + 1) * (uint32_t)P.nt3, g2.status, &s_okb)) break;
+                learned_chain_step(S, L, LF_FINISH | LF_START, cblock, psm, sw, &bar[KB + 2], staged, D);
+                phase_arrive(csyncc);
+                // the state's bookkeeping while layer 2 runs on other CTAs
+                items += learned_chain_commit(S, L, LF_FINISH | LF_START, cblock, sw, D);
+            }
         }
+        if (isc) learned_advance(S, L, P.nc, s_items, items, t0 + it);
     }
     if (tid == 0 && staged) mbar_wait_bounded(&bar[KB + 2], 0, WAIT_TIMEOUT_NS);   // no copy left in flight
     tc_fence_before();
@@ -1123,7 +1160,7 @@ struct LearnedPath {
     bool primed = false;
     bool pdl = true;
     cudaGraphExec_t exec = nullptr;
-    uint32_t* gsync = nullptr;           // grid barrier counter of the persistent launch
+    uint32_t* gsync = nullptr;           // counters of the persistent launch
     int persist = -1;                    // persistent launch: -1 not checked, 0 no, 1 yes
     PersistArgs pa{};
     size_t persist_smem = 0;
@@ -1195,7 +1232,7 @@ static int learned_alloc(bn_chains* ch)
                  o_lg = take(4 * 2 * Cs * Pp), o_part = take(8 * 2 * Cs * lp->NT), o_cb = take(Cs),
                  o_since = take(8 * Cs * n), o_prank = take(4 * Cs * n), o_pkey = take(8 * Cs * n), o_pab = take(2 * Cs),
                  o_pair = take(4 * Cs), o_lqf = take(4 * Cs), o_pu = take(8 * Cs), o_dp = take(8 * Cs),
-                 o_done = take(4), o_bound = take(4), o_status = take(4), o_gsync = take(4);
+                 o_done = take(4), o_bound = take(4), o_status = take(4), o_gsync = take(sizeof(uint32_t) * 3 * LR_SYNC * (size_t)lp->Mt);
     // survivors region [masks | keys | ranks | node offsets], each part 16-byte aligned
     const size_t r_key = (size_t)round_up((int64_t)(8 * alive), 16), r_rk = r_key + (size_t)round_up((int64_t)(8 * alive), 16),
                  r_off = r_rk + (size_t)round_up((int64_t)(4 * alive), 16),
@@ -1484,7 +1521,7 @@ static int launch_persist(bn_chains* ch, int iters, cudaStream_t s)
     LearnedPath* lp = ch->lp;
     PersistArgs P = lp->pa;
     P.iters = iters;
-    BN_CUDA(cudaMemsetAsync(lp->gsync, 0, sizeof(uint32_t), s));
+    BN_CUDA(cudaMemsetAsync(lp->gsync, 0, sizeof(uint32_t) * 3 * LR_SYNC * (size_t)lp->Mt, s));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)std::max(P.n2 + P.n3, P.nc), 1, 1);
     cfg.blockDim = dim3(32 * LR_WARPS, 1, 1);
