@@ -104,8 +104,11 @@ __device__ __forceinline__ uint32_t warp_walk(const uint64_t* m, uint32_t js, ui
 // kept-set test leaves ~3 nodes per step: measured on GB300 at n = 60, 1.66 us per step
 // with warp walks always against 1.70 us with lane walks above 8 nodes and 1.73 us above
 // 3); with more, every lane first walks its own nodes for 16 survivors and the warp then
-// walks those still open (every span node re-scored: uncached networks, learned steps).
+// walks those still open (every span node re-scored: uncached networks).  ROUNDS: it walks
+// ROUNDS * WALK_PROBE survivors, the loads of a round independent (learned steps at n = 60:
+// 4 rounds 23.6 us a step, 1 24.6, 8 23.8, all of them 27.5, the 16 one by one 24.9).
 constexpr int WALK_PROBE = 8;   // survivors each lane tests of its own nodes before the warp walks
+template <int ROUNDS = 0>
 __device__ __forceinline__ void span_walk(const uint64_t* m, uint32_t (&j)[2], const uint32_t (&j1)[2],
                                           const uint64_t (&npc)[2], const bool (&act)[2], int lane,
                                           int warp_max)
@@ -153,6 +156,23 @@ __device__ __forceinline__ void span_walk(const uint64_t* m, uint32_t (&j)[2], c
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (!act[h]) continue;
+        if (ROUNDS) {
+            // (loads of a round independent, no branch between them)
+            bool found = false;
+            for (int t = 0; t < ROUNDS && !found; ++t) {
+                uint64_t pm[WALK_PROBE];
+#pragma unroll
+                for (int r = 0; r < WALK_PROBE; ++r) pm[r] = j[h] + r < j1[h] ? m[j[h] + r] : ~0ull;
+                int first = WALK_PROBE;
+#pragma unroll
+                for (int r = WALK_PROBE - 1; r >= 0; --r)
+                    if ((pm[r] & npc[h]) == 0ull) first = r;
+                j[h] += first;
+                found = first < WALK_PROBE;
+            }
+            open[h] = !found;
+            continue;
+        }
         uint32_t x = j[h];
         bool found = false;
         for (int r = 0; r < 4 && !found; ++r) {

@@ -741,7 +741,7 @@ __device__ __forceinline__ void learned_chain_step(const ChainState& S, const Le
                     act[h] = true;
                 }
             }
-            span_walk(smask, wj, wj1, wnpc, act, lane, 8);
+            span_walk<4>(smask, wj, wj1, wnpc, act, lane, 8);
             double dpart = 0.0;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -937,7 +937,7 @@ __global__ void __launch_bounds__(32 * LR_WARPS) k_learned_chain(ChainState S, L
 // behind the arrival after it.  256 chains, n = 60, H = 512: 37 us a step with grid-wide
 // barriers and everything between them (of 50,000 cycles of the step's slowest chain 25,000
 // went to the exact score, the edge credit and to code that only accepting chains run), 26
-// with those out of the way, 23 with a counter a phase and 128 chains.
+// with those out of the way, 22 with a counter a phase and 128 chains.
 // CTAs [0, n3) own output-layer tiles, CTAs [n3, n3 + n2) layer-2 tiles; a block of four
 // chains goes to a CTA with an output tile of the same 128 chains (nt3 >= 32), else block b
 // to CTA b.
@@ -960,8 +960,9 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p)
 
 // Hands a CTA's work on: its writes before the arrival are visible, to generic loads and to
 // the bulk copies (async proxy), after a wait for a count that includes it, and so on
-// through further hand-overs.  Waits are bounded: false once one has run out (status gets
-// STATUS_TIMEOUT).
+// through further hand-overs.  The acquiring load and the block barrier order the CTA's later
+// reads; a fence behind it would cost 0.4 us a wait.  Waits are bounded: false once one has
+// run out (status gets STATUS_TIMEOUT).
 __device__ __forceinline__ void phase_arrive(uint32_t* counter)
 {
     asm volatile("fence.proxy.async.global;" ::: "memory");
@@ -984,7 +985,6 @@ __device__ __forceinline__ bool phase_wait(const uint32_t* counter, uint32_t tar
                 }
             }
         }
-        __threadfence();
         asm volatile("fence.proxy.async.global;" ::: "memory");
         if (!ok) atomicOr(status, STATUS_TIMEOUT);
         *s_ok = ok ? 1 : 0;

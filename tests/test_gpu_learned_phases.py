@@ -10,7 +10,7 @@ import synth
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,H,C", [(47, 128, 1), (47, 128, 127), (47, 64, 128), (47, 128, 129), (48, 64, 301), (30, 64, 259)])
+@pytest.mark.parametrize("n,H,C", [(47, 128, 1), (47, 128, 127), (47, 128, 128), (47, 128, 129), (48, 128, 301), (30, 128, 259)])
 def test_phases_equal_graph_launch(gpu, n, H, C):
     rng = np.random.default_rng(n + C)
     k, steps = 2, 300
