@@ -214,14 +214,15 @@ ROOF_SLICED_B = 32         # the batched full-table pass of roofline_hbm: one 32
 ISSUE_PER_SM = 4           # warp schedulers per SM, one warp instruction per clock each
 # ncu smsp__inst_executed.sum of k_chain_spec<1> at this workload (256 chains, 1,000-step
 # launches; all four warps of a chain, the dropped speculative evaluations included), per
-# chain per committed MH iteration; and dram__bytes_read.sum + dram__bytes_write.sum per
-# launch of the full-table k_scan<1024,0> (256 items per node, the sampler's step)
-FUSED_INST_PER_CHAIN_STEP = 760.0
-FUSED_TRAFFIC_BYTES = 2.146e6    # ncu dram bytes read + written per 1,000-step launch of k_chain_spec<1>
-BUILD_INST_PER_ENTRY = 649.0     # ncu smsp__inst_executed.sum of k_build<4,1,0> per entry at n=60, m=1000
-SCAN_TRAFFIC_BYTES = 121.5e6
+# chain per committed MH iteration
+FUSED_INST_PER_CHAIN_STEP = 752.0
+FUSED_TRAFFIC_BYTES = 1.902e6    # ncu dram bytes read + written per 1,000-step launch of k_chain_spec<1>
+BUILD_INST_PER_ENTRY = 86.9      # ncu smsp__inst_executed.sum of the counting and assembling kernels
+                                 # (k_joint_tc, k_joint, k_tc_rows, k_minor_rows, k_assemble) at n=60,
+                                 # m=1000, per table entry
+SCAN_TRAFFIC_BYTES = 117.7e6     # ncu dram bytes read + written per launch of k_scan_sliced<8,0> (a sampler step)
 NODES_TRAFFIC_BYTES = 124.2e6    # ncu dram bytes read + written per launch of k_scan_nodes at one order
-SLICED_TRAFFIC_BYTES = 120.37e6  # ncu dram bytes read + written per launch of k_scan_sliced<1,0> at 32 orders
+SLICED_TRAFFIC_BYTES = 117.64e6  # ncu dram bytes read + written per launch of k_scan_sliced<1,0> at 32 orders
 
 
 def _flush_l2(torch, flush, stream):
@@ -437,9 +438,9 @@ def _config_n20(bn, torch, synth, seed):
 
 def _config_n40(bn, torch, synth, seed, stream, flush, test_rate, hbm_peak):
     """40 ternary nodes, m = 2000, k = 4 (3.69 M entries): 512 chains stepped by the
-    full-table scan, each step's three kernels replayed from a CUDA graph, on the tiling
-    the autotuner picks for 512 items per node; the same chains on the pruned table's
-    fused sampler beside it."""
+    full-table scan (bit-sliced at this size), each step's three kernels replayed from a
+    CUDA graph; the same chains on the pruned table's fused sampler beside it.  The tiling
+    the autotuner picks for 512 items per node is that of the mask-test scan."""
     data, arity, k, R, _ = synth.workload("n40_k4_m2000")
     t = bn.build_scores(data, arity, k, R=R)
     S = bn.table_info(t)["sets_per_node"]
@@ -559,9 +560,12 @@ def main():
     for x in hbm_leg:
         B, us = x["orders"], x["scan_us"]
         tests = float(n) * S * B                 # (entry, order) consistency tests of one pass
-        x.update({"kernel": "k_scan_nodes" if n * ((B + 7) // 8) <= 1024 else "k_scan",
-                  "achieved_gbs": hbm_bytes / (us / 1e6) / 1e9, "frac": hbm_bytes / (us / 1e6) / 1e9 / hbm_peak,
-                  "tests_per_s": tests / (us / 1e6), "test_frac": tests / (us / 1e6) / test_rate})
+        nodes = B < 4                            # from four orders on the full mode scans bit-sliced
+        by = hbm_bytes if nodes else sliced_bytes
+        x.update({"kernel": "k_scan_nodes" if nodes else "k_scan_sliced",
+                  "achieved_gbs": by / (us / 1e6) / 1e9, "frac": by / (us / 1e6) / 1e9 / hbm_peak,
+                  "tests_per_s": tests / (us / 1e6),
+                  "test_frac": tests / (us / 1e6) / test_rate if nodes else None})
     sliced_leg = score_sweep(bn.SCAN_SLICED, SLICED_B)
     for x in sliced_leg:
         us = x["scan_us"]
@@ -592,7 +596,7 @@ def main():
     sum_score = {"orders": 1, "call_us": float(np.median(sum_times)),
                  "max_score_scan_us": hbm_leg[0]["scan_us"],
                  "note": "bn_score_orders_sum: FP64 log10-sum-exp10 over the consistent parent sets of "
-                         "every node (one exp10 per consistent set), against the max-based scan of the "
+                         "every node (integer exponentials of the entries near the best one), against the max-based scan of the "
                          "same order (roofline_hbm)"}
 
     with torch.cuda.stream(stream):
@@ -795,19 +799,20 @@ def main():
                              "chains' state only (the table stays in shared memory)"}
         avg_full = scan_ms_full / max(scan_l_full, 1)
         tests = items_prof * S / max(scan_l_full, 1)                 # (entry, item) tests per launch
-        roof_scan = {"kernel": "k_scan (full table, autotuned tiling, one launch per sampler step of all chains)",
-                     "bound": "alu", "unit": "tests/s", "achieved": tests / (avg_full / 1000.0),
-                     "peak": test_rate, "frac": tests / (avg_full / 1000.0) / test_rate,
-                     "traffic": SCAN_TRAFFIC_BYTES,
-                     "peak_source": "measured in this run: bn_measure_test_rate (the scan's own inner loop over "
-                                    "1,024 entries resident in shared memory, 8 x 256 threads per SM, CUDA events)",
+        roof_scan = {"kernel": "k_scan_sliced<8,0> (full table, one launch per sampler step of all chains)",
+                     "bound": "hbm", "unit": "GB/s", "achieved": 4 * n * S / (avg_full / 1000.0) / 1e9,
+                     "peak": hbm_peak, "frac": 4 * n * S / (avg_full / 1000.0) / 1e9 / hbm_peak,
+                     "traffic": SCAN_TRAFFIC_BYTES, "peak_source": peak_src,
                      "per_launch": {"tests": tests, "avg_ms": avg_full, "launches": scan_l_full,
-                                    "hbm_bytes_algorithmic": 4 * n * S + 8 * S,
-                                    "hbm_frac_of_measured": (4 * n * S + 8 * S) / (avg_full / 1000.0) / 1e9 / hbm_peak},
+                                    "tests_per_s": tests / (avg_full / 1000.0),
+                                    "tests_per_s_over_mask_test_rate": tests / (avg_full / 1000.0) / test_rate,
+                                    "hbm_bytes_algorithmic": 4 * n * S},
                      "share_of_step": avg_full / (ms_full / args.steps),
                      "note": "the paper's scan (a6) over the full table for a step of all chains' orders "
-                             "(full_scan): the table is read once per 256 orders, so the consistency tests, "
-                             "not HBM, bound it; traffic = ncu dram bytes read + written per launch"}
+                             "(full_scan), 32 orders per AND of parent words; the table is read once per step; "
+                             "bound in practice by the per-entry tests of eight groups of orders and the recording "
+                             "of hits; test_rate = the mask-test scan's measured in-core rate, which this scan "
+                             "exceeds; traffic = ncu dram bytes read + written per launch"}
         cpu = cpu1 = None
         if world == 1 and not args.no_cpu_baseline:
             nt = os.cpu_count() or 1
@@ -837,16 +842,19 @@ def main():
                                            "parent sets), each over its surviving entries in score order"},
             "roofline": roof_head,
             "roofline_scan": roof_scan,
-            "roofline_build": {"kernel": "k_build<4,1,0> (counting + local score + prior of every entry, n=60)",
+            "roofline_build": {"kernel": "k_joint_tc (tensor-core counts of the sets of 4 and 5 nodes), k_joint, "
+                                         "k_assemble (every entry, n=60)",
                                "bound": "alu", "unit": "warp instructions/s",
                                "achieved": BUILD_INST_PER_ENTRY * n * S / (build_kernel_ms / 1000.0),
                                "peak": issue_peak,
                                "frac": BUILD_INST_PER_ENTRY * n * S / (build_kernel_ms / 1000.0) / issue_peak,
                                "traffic": None, "kernel_ms": build_kernel_ms,
                                "row_visits_per_s": n * S * data.shape[0] / (build_kernel_ms / 1000.0),
-                               "note": "issue-bound: warp instructions per entry = ncu smsp__inst_executed.sum of "
-                                       "this kernel at this workload (649); peak as for roofline; DRAM carries only "
-                                       "the 8 B written per entry"},
+                               "note": "warp instructions per entry = ncu smsp__inst_executed.sum of these kernels at "
+                                       "this workload; peak as for roofline; k_joint_tc is bound by the "
+                                       "shared-memory port (indicators written and read by the products, lookups); "
+                                       "row_visits_per_s counts a row per entry, as if every entry were counted "
+                                       "alone"},
             "roofline_hbm": {"kernel": f"k_scan_sliced (bn_score_orders, BN_SCAN_SLICED: every entry of the full "
                                        f"table, {roof_b} orders)", "bound": "hbm",
                              "achieved": roof_sl["achieved_gbs"], "peak": hbm_peak, "unit": "GB/s",
@@ -865,9 +873,9 @@ def main():
                              "test_rate_peak": test_rate, "pruned_table": pruned_scoring,
                              "note": "bn_score_orders on B random orders of the full n=60 table: scan kernel time "
                                      "(CUDA events around its launch, L2 flushed before every call). by_orders: "
-                                     "BN_SCAN_FULL (one 64-bit mask test per entry and order), HBM fraction on 4 B "
-                                     "per (node, entry) + 8 B per entry, test fraction of the measured "
-                                     "consistency-test peak; sliced: BN_SCAN_SLICED (entries in score order, 32 "
+                                     "BN_SCAN_FULL (up to three orders one 64-bit mask test per entry and order, HBM "
+                                     "fraction on 4 B per (node, entry) + 8 B per entry, test fraction of the "
+                                     "measured consistency-test peak; from four on the bit-sliced pass); sliced: BN_SCAN_SLICED (entries in score order, 32 "
                                      "orders per AND of parent words; every entry read), HBM fraction on 4 B per "
                                      "(node, entry); sorted: BN_SCAN_SORTED (the same, nothing below the empty set "
                                      "read, stopping once every order has its entry; entries_at_most = the entries "

@@ -466,7 +466,7 @@ int bn_chains_set_proposal(bn_chains* c, bn_mlp* m, int mode, double eps_mix, vo
  * same either way):
  *   BN_LEARNED_LAUNCH_AUTO   (default) one cooperative persistent kernel runs up to 256
  *                            steps per launch -- per step the layer-2 tiles, the output-layer
- *                            tiles and the chains, separated by grid-wide barriers, with the
+ *                            tiles and the chains, handed on by device counters, with the
  *                            weight tiles resident in shared memory and TMEM -- when all its
  *                            CTAs fit on the GPU at once (at most 256 chains at H = 512);
  *                            otherwise as BN_LEARNED_LAUNCH_GRAPH

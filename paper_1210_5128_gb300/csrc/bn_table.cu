@@ -205,7 +205,7 @@ __global__ void k_pad_keys(int64_t* __restrict__ keys, int n, int64_t S, int64_t
 // C(60, 5) = 5.5 M tables instead of 29.4 M at n = 60, k = 4; k_assemble forms the entries.
 // Measured at n = 60, k = 4, m = 1000, ternary: 20.0 ms with one count table per entry,
 // 4.51 ms for k_joint over all of them; with the sets of four and five nodes on the tensor
-// cores (bn_joint_tc.cu) 2.90 ms for those, 0.03 for k_joint and 0.34 for k_assemble.
+// cores (bn_joint_tc.cu) 2.90 ms for those, 0.08 for k_joint and 0.34 for k_assemble.
 // ---------------------------------------------------------------------------------
 struct JointArgs {
     const uint32_t* packed;
