@@ -331,15 +331,17 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_scan(ScanArgs A)
     if (active && sub == 0 && b != SPOS_NONE) atomicMin(&A.list_best[(size_t)node * A.cap + item], b);
 }
 
-static constexpr size_t SCAN_BIN_BYTES = 8 * 65 * (MAXK + 1);   // binomial table (UNRANK)
+// binomial table (UNRANK): tables made from scores have parent sets of up to n - 1 nodes
+static constexpr size_t scan_bin_bytes(int k) { return (size_t)8 * 65 * (k + 1); }
 
 template <int SUB, bool UNRANK>
 static int scan_variant(const ScanArgs& A, dim3 grid, cudaStream_t s)
 {
     static unsigned long long ctx[64] = {0};
-    const size_t smem = ScanCfg<SUB>::SMEM + (UNRANK ? SCAN_BIN_BYTES : 0);
+    const size_t smem = ScanCfg<SUB>::SMEM + (UNRANK ? scan_bin_bytes(A.k) : 0);
     if (first_in_context(ctx))
-        BN_CUDA(cudaFuncSetAttribute(k_scan<SUB, UNRANK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        BN_CUDA(cudaFuncSetAttribute(k_scan<SUB, UNRANK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(ScanCfg<SUB>::SMEM + (UNRANK ? scan_bin_bytes(MAXN - 1) : 0))));
     k_scan<SUB, UNRANK><<<grid, SCAN_THREADS, smem, s>>>(A);
     BN_LAUNCH_CHECK("k_scan");
     return BN_OK;
