@@ -221,6 +221,31 @@ __global__ void k_accept(ChainState S)
         if (S.changed && lane == 0) S.changed[c] = moved ? 1 : 0;
     }
     __syncthreads();
+    // every thread has read the step: the last block to come here advances it and clears the
+    // work lists (the scan has read them), beside the sums and not behind the edge counts
+    if (warp == 1) {
+        uint32_t ticket = 0;
+        if (lane == 0) {
+            __threadfence();
+            ticket = atomicAdd(S.done, 1u);
+        }
+        if (__shfl_sync(0xffffffffu, ticket, 0) == gridDim.x - 1) {
+            uint32_t items = 0;
+            for (int i = lane; i < n; i += 32) {
+                items += S.list_count[i];
+                S.list_count[i] = 0;
+            }
+            items = __reduce_add_sync(0xffffffffu, items);
+            if (lane == 0) {
+                *S.items_total += items;
+                if (t >= S.burn_in && S.record_every > 0 && ((t - S.burn_in) % S.record_every) == 0 &&
+                    (t - S.burn_in) / S.record_every < S.record_cap)
+                    *S.rec_count = (t - S.burn_in) / S.record_every + 1;
+                *S.step = t + 1;
+                *S.done = 0;
+            }
+        }
+    }
     // the sums of the block's eight chains on eight lanes of one warp: an FP64 instruction
     // holds the pipe for the whole warp whatever lanes are on
     if (threadIdx.x < 8 && blockIdx.x * 8 + (int)threadIdx.x < S.C) {
@@ -285,31 +310,6 @@ __global__ void k_accept(ChainState S)
                     }
                 }
             }
-        }
-    }
-    // the last block to finish advances the step and clears the work lists
-    __shared__ int s_last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(S.done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (s_last && warp == 0) {
-        uint32_t items = 0;
-        for (int i = lane; i < n; i += 32) {
-            items += S.list_count[i];
-            S.list_count[i] = 0;
-        }
-        items = __reduce_add_sync(0xffffffffu, items);
-        if (lane == 0) {
-            *S.items_total += items;
-            if (t >= S.burn_in && S.record_every > 0 && ((t - S.burn_in) % S.record_every) == 0 &&
-                (t - S.burn_in) / S.record_every < S.record_cap)
-                *S.rec_count = (t - S.burn_in) / S.record_every + 1;
-            *S.step = t + 1;
-            *S.done = 0;
-            __threadfence();
         }
     }
 }
