@@ -460,12 +460,14 @@ __global__ void __launch_bounds__(TJ_THREADS, 1) k_joint_tc(TcJointArgs A)
 
 bool joint_tc_plan(int n, int m, int size, int luts, const uint8_t* ar, TcPlan* P)
 {
-    // Few sets: the set-up costs what the products save (26 nodes, 65,780 sets: build 347 us
-    // against 365; 20 nodes, 15,504 sets: equal).  The lgamma tables have to fit beside the stages.
+    // Few sets: the set-up costs what the products save (k = 4, m = 1000: 26 nodes, 65,780 sets,
+    // build 347 us against 365; 28 nodes with nearly constant columns 423 against 397; k = 3:
+    // 30 nodes, 27,405 sets, m = 64, 240 against 211; 40 nodes, 91,390 sets, m = 1000, 336
+    // against 400).  The lgamma tables have to fit beside the stages.
     const int lowk = size - 2;
     if ((size != 4 && size != 5) || n <= size || n > MAXN || m < 64 || luts * (m + 1) > TJ_LUT_ROWS) return false;
     const int64_t sets = (int64_t)h_binom.v[n][size];
-    if (sets < 20000) return false;
+    if (sets < 60000) return false;
     std::vector<uint32_t>&pairs = P->pairs, &rowinfo = P->rowinfo, &mt_first = P->mt_first, &nt_start = P->nt_start;
     // pairs d < e with room for a low set below d, d falling; 32-row blocks, no pair astride
     std::vector<int> tile_d;

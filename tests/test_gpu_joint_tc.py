@@ -17,11 +17,12 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,k,m,arities,kind", [
-    (22, 4, 64, (2, 3, 4), 0), (22, 4, 127, (3,), 1), (22, 4, 128, (2,), 1), (23, 4, 129, (4,), 0),
-    (21, 4, 300, (3,), 0), (24, 4, 1000, (2, 4), 0), (30, 3, 65, (2, 3, 4), 0), (30, 3, 500, (4,), 1),
-    (28, 3, 255, (2,), 0), (29, 4, 1574, (2, 3, 4), 0), (28, 4, 2099, (2, 3), 0), (27, 4, 3149, (3,), 1),
-    (27, 4, 1575, (2, 3, 4), 0), (28, 3, 6299, (2, 3), 0), (28, 3, 6300, (3,), 0),
-    (33, 3, 3599, (3, 4), 0), (30, 3, 3600, (2, 3), 0)])
+    (26, 4, 64, (2, 3, 4), 0), (27, 4, 127, (3,), 1), (26, 4, 128, (2,), 1), (27, 4, 129, (4,), 0),
+    (26, 4, 300, (3,), 0), (28, 4, 1000, (2, 4), 0), (37, 3, 65, (2, 3, 4), 0), (38, 3, 500, (4,), 1),
+    (37, 3, 255, (2,), 0), (29, 4, 1574, (2, 3, 4), 0), (28, 4, 2099, (2, 3), 0), (27, 4, 3149, (3,), 1),
+    (27, 4, 1575, (2, 3, 4), 0), (37, 3, 6299, (2, 3), 0), (37, 3, 6300, (3,), 0),
+    (36, 4, 300, (2, 3, 4), 0), (36, 4, 257, (2, 4), 0), (37, 4, 200, (3,), 1), (36, 4, 64, (2,), 0),
+    (36, 4, 1574, (2, 3, 4), 0), (39, 3, 3599, (3, 4), 0), (37, 3, 3600, (2, 3), 0), (25, 4, 500, (3,), 0), (36, 3, 500, (2, 3), 0)])
 def test_tensor_core_counts(gpu, n, k, m, arities, kind):
     rng = np.random.default_rng(n * 1000 + m)
     ar = rng.choice(arities, n).astype(np.uint8)
