@@ -862,6 +862,9 @@ __device__ __forceinline__ int64_t learned_chain_commit(const ChainState& S, con
             }
         }
         if (flags & LF_FLUSH) {
+            // an accepted step's dwell starts and edge counts were written by the lanes of its
+            // two positions; here a node's are read by lane i
+            __syncwarp();
             for (int i = lane; i < n; i += 32) {
                 const size_t si = (size_t)c * n + i;
                 credit_edges(S, c, i, W.rank[i], L.since[si], tf + 1);
