@@ -66,18 +66,6 @@ unsigned long long context_id()
     return 0;
 }
 
-bool first_in_context(unsigned long long* slots)
-{
-    static std::mutex mu;
-    const int d = device_id();
-    if (d < 0 || d >= 64) return true;
-    const unsigned long long id = context_id();
-    std::lock_guard<std::mutex> g(mu);
-    if (id != 0 && slots[d] == id) return false;
-    slots[d] = id;
-    return true;
-}
-
 int sm_count()
 {
     static std::mutex mu;

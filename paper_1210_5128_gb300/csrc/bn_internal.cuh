@@ -7,6 +7,7 @@
 #include <initializer_list>
 
 #include "bn.h"
+#include "bn_once.cuh"
 
 namespace bn {
 
@@ -25,10 +26,9 @@ int sm_count();                      // SMs of the current device
 int device_id();
 // Identity of the calling thread's current CUDA context (0 when the driver cannot say).
 unsigned long long context_id();
-// True the first time it is called in the current context of the current device with
-// this call site's `slots` (64 zero-initialised entries): per-context set-up, such as a
-// kernel's shared-memory attribute, which a context destroyed and created again loses.
-bool first_in_context(unsigned long long* slots);
+// Runs a call site's set-up once per context (bn_once.cuh) in the calling thread's current one.
+template <class F>
+int once_in_context(ContextOnce& once, F set_up) { return once.run(device_id(), context_id(), set_up); }
 
 // Device memory from the library's own pool of the current device (bn_api.cu).  dev_alloc /
 // dev_free are ordered by stream s; obj_alloc's memory is usable on every stream when it

@@ -530,11 +530,14 @@ bool joint_tc_plan(int n, int m, int size, int luts, const uint8_t* ar, TcPlan* 
 template <int NH>
 static int launch(const TcJointArgs& A, cudaStream_t s)
 {
-    static unsigned long long ctx[64] = {0};
+    static ContextOnce once;
     constexpr size_t fixed = (size_t)TJ_STAGES * (TJ_A_BYTES + TJ_B_BYTES) + 1024 + 16;
-    if (first_in_context(ctx))
+    const int rc = once_in_context(once, [&]() -> int {
         BN_CUDA(cudaFuncSetAttribute(k_joint_tc<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)(fixed + 12 * (size_t)TJ_LUT_ROWS)));
+        return BN_OK;
+    });
+    if (rc) return rc;
     const size_t smem = fixed + 12 * (size_t)(1 + NH) * A.m1;
     k_joint_tc<NH><<<std::min<uint32_t>((uint32_t)sm_count(), A.items), TJ_THREADS, smem, s>>>(A);
     BN_LAUNCH_CHECK("k_joint_tc");

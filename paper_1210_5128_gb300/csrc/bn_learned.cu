@@ -1353,12 +1353,14 @@ static int learned_weights(bn_chains* ch, cudaStream_t s)
     lp->g3.mode = 1;
     lp->g3.logits = (float*)lp->L.logits;
     lp->g3.part = (float2*)lp->L.part;
-    static unsigned long long ctx[64] = {0};
-    if (first_in_context(ctx)) {
+    static ContextOnce once;
+    const int rc = once_in_context(once, [&]() -> int {
         BN_CUDA(cudaFuncSetAttribute(k_learned_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)lgemm_smem(LR_MAX_H)));
         BN_CUDA(cudaFuncSetAttribute(k_learned_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, LR_STAGE_MAX));
-    }
+        return BN_OK;
+    });
+    if (rc) return rc;
     if (lp->exec) {
         cudaGraphExecDestroy(lp->exec);
         lp->exec = nullptr;

@@ -1494,16 +1494,16 @@ int build_survivor_cache(bn_table* t, cudaStream_t s)
 
 static int fused_smem_setup(int cap, size_t* smem)
 {
-    static unsigned long long ctx[64] = {0};
+    static ContextOnce once;
     const size_t mx = surv_cache_stride(SURV_CAP_MAX);
-    if (first_in_context(ctx)) {
+    *smem = surv_cache_stride(cap);
+    return once_in_context(once, [&]() -> int {
         BN_CUDA(cudaFuncSetAttribute(k_chain_fused<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
         BN_CUDA(cudaFuncSetAttribute(k_chain_spec<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)surv_cache_stride(SPEC_CAP_MAX)));
         BN_CUDA(cudaFuncSetAttribute(k_batch_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
-    }
-    *smem = surv_cache_stride(cap);
-    return BN_OK;
+        return BN_OK;
+    });
 }
 
 __global__ void k_batch_advance(const ChainState* __restrict__ Ss, const int* __restrict__ iters, int nnet)
@@ -1778,17 +1778,18 @@ static bool spec_staged(const bn_chains* ch)
 {
     const int64_t total = ch->t->alive_total;
     if (!ch->t->gcache) return total <= SURV_CAP_MAX;
-    static unsigned long long ctx[64] = {0};
+    static ContextOnce once;
     static int by_regs[64] = {0};
     const int d = device_id();
-    if (first_in_context(ctx) && d >= 0 && d < 64) {
+    once_in_context(once, [&]() -> int {
         int nb = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chain_spec<2>, 32 * SPEC_WARPS, 0) != cudaSuccess) {
             cudaGetLastError();
             nb = 4;
         }
-        by_regs[d] = std::max(1, nb);
-    }
+        if (d >= 0 && d < 64) by_regs[d] = std::max(1, nb);
+        return BN_OK;
+    });
     const int want = (ch->S.C + sm_count() - 1) / sm_count();
     const int per_sm = std::min(want, d >= 0 && d < 64 && by_regs[d] > 0 ? by_regs[d] : 4);
     const int64_t room = 227 * 1024 / per_sm - 1024 - (int64_t)(sizeof(FusedSmem) + sizeof(SpecBatch) + sizeof(SpecChain) +

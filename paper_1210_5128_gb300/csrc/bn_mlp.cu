@@ -176,9 +176,12 @@ static int gemm_split(int M, int N, int K, size_t ws_elems)
 
 static int gemm_launch(const GemmArgs& a, const GemmArgs* b, cudaStream_t s)
 {
-    static unsigned long long ctx[64] = {0};
-    if (first_in_context(ctx))
+    static ContextOnce once;
+    const int rc = once_in_context(once, [&]() -> int {
         BN_CUDA(cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
+        return BN_OK;
+    });
+    if (rc) return rc;
     auto blocks = [](const GemmArgs& g) { return (g.M / TC_BM) * (g.N / TC_BN) * g.ksplit; };
     GemmPair gp{{a, b ? *b : a}, blocks(a)};
     k_gemm_tc<<<(unsigned)(gp.blocks0 + (b ? blocks(*b) : 0)), 128, TC_SMEM, s>>>(gp);

@@ -337,11 +337,14 @@ static constexpr size_t scan_bin_bytes(int k) { return (size_t)8 * 65 * (k + 1);
 template <int SUB, bool UNRANK>
 static int scan_variant(const ScanArgs& A, dim3 grid, cudaStream_t s)
 {
-    static unsigned long long ctx[64] = {0};
+    static ContextOnce once;
     const size_t smem = ScanCfg<SUB>::SMEM + (UNRANK ? scan_bin_bytes(A.k) : 0);
-    if (first_in_context(ctx))
+    const int rc = once_in_context(once, [&]() -> int {
         BN_CUDA(cudaFuncSetAttribute(k_scan<SUB, UNRANK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)(ScanCfg<SUB>::SMEM + (UNRANK ? scan_bin_bytes(MAXN - 1) : 0))));
+        return BN_OK;
+    });
+    if (rc) return rc;
     k_scan<SUB, UNRANK><<<grid, SCAN_THREADS, smem, s>>>(A);
     BN_LAUNCH_CHECK("k_scan");
     return BN_OK;
@@ -581,12 +584,15 @@ static int launch_scan_nodes(const bn_table* t, int B, const uint64_t* list_pc, 
         ns_table_row<8>(launch[3], kern[3]);
     });
     const size_t smem = ns_smem(t->n);
-    static unsigned long long ctx[64] = {0};
-    if (first_in_context(ctx))
+    static ContextOnce ctx_once;
+    const int rc = once_in_context(ctx_once, [&]() -> int {
         for (int a = 0; a < 4; ++a)
             for (int r = 0; r < NS_RMAX; ++r)
                 BN_CUDA(cudaFuncSetAttribute(kern[a][r], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)ns_smem(MAXN)));
+        return BN_OK;
+    });
+    if (rc) return rc;
     const NsShape sh = ns_shape(t->n, B, t->Sp);
     // whole waves: as many blocks per SM as its 2,048 threads and shared memory hold (at
     // most four)
@@ -841,9 +847,12 @@ int launch_score_small(const bn_table* t, const uint8_t* orders, int B, uint32_t
                 best_rank, score, status};
     const unsigned grid = (unsigned)((B + ob - 1) / ob);
     if (t->scan_mode == BN_SCAN_PRUNED) {
-        static unsigned long long ctx[64] = {0};
-        if (first_in_context(ctx))
+        static ContextOnce once;
+        const int rc = once_in_context(once, [&]() -> int {
             BN_CUDA(cudaFuncSetAttribute(k_score_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * SC_SURVIVORS));
+            return BN_OK;
+        });
+        if (rc) return rc;
         k_score_small<true><<<grid, SC_THREADS, sizeof(uint64_t) * (size_t)t->alive_total, s>>>(A);
     } else
         k_score_small<false><<<grid, SC_THREADS, 0, s>>>(A);

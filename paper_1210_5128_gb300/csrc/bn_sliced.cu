@@ -433,16 +433,18 @@ template <int G, bool CUT>
 static int sliced_launch(const bn_table* t, const uint32_t* list_count, const uint64_t* list_pc,
                          uint32_t* list_best, int cap, int sets, uint32_t* status, cudaStream_t s)
 {
-    static unsigned long long ctx[64] = {0};
+    static ContextOnce once;
     static int resident[64] = {0};
     const int d = device_id();
-    if (first_in_context(ctx)) {
+    const int rc = once_in_context(once, [&]() -> int {
         BN_CUDA(cudaFuncSetAttribute(k_scan_sliced<G, CUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sl_smem(G)));
         int nb = 0;
         BN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_scan_sliced<G, CUT>, SL_THREADS, sl_smem(G)));
         if (d >= 0 && d < 64) resident[d] = std::max(1, nb);
-    }
+        return BN_OK;
+    });
+    if (rc) return rc;
     const int per_sm = (d >= 0 && d < 64 && resident[d] > 0) ? resident[d] : 1;
     const int64_t want = (int64_t)sm_count() * per_sm;
     int64_t nchunk, per = 0;

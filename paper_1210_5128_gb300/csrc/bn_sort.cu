@@ -670,13 +670,15 @@ static int rank_by_buckets(bn_table* t, cudaStream_t s)
          (rc = tmp.get(&A.tile_base, (size_t)per * A.tiles * A.NB)) || (rc = tmp.get(&A.bid, (size_t)per * S)) ||
          (rc = tmp.get(&A.bx, (size_t)per * S)) || (rc = tmp.get(&A.br, (size_t)per * S))))
         return rc;
-    static unsigned long long ctx[64] = {0};
-    if (first_in_context(ctx)) {
+    static ContextOnce once;
+    rc = once_in_context(once, [&]() -> int {
         BN_CUDA(cudaFuncSetAttribute(k_bs_split, cudaFuncAttributeMaxDynamicSharedMemorySize, BS_SAMPLES * 12));
         BN_CUDA(cudaFuncSetAttribute(k_bs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SCATTER_SMEM));
         BN_CUDA(cudaFuncSetAttribute(k_bs_sort<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SMEM));
         BN_CUDA(cudaFuncSetAttribute(k_bs_sort<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SMEM));
-    }
+        return BN_OK;
+    });
+    if (rc) return rc;
     for (A.node0 = 0; A.node0 < t->n; A.node0 += per) {
         const int nb = std::min(per, t->n - A.node0);
         if (whole) {

@@ -631,10 +631,19 @@ struct Temps {
     ~Temps() { release(); }
 };
 
+static constexpr size_t JOINT_SMEM = 220 * 1024;       // of a block of k_joint, at most
+
 template <int KT, bool SMEM_DATA, bool MINOR>
 static int launch_joint(const JointArgs& A, size_t smem, int grid, int threads, cudaStream_t s)
 {
-    BN_CUDA(cudaFuncSetAttribute(k_joint<KT, SMEM_DATA, MINOR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // (the limit of every build: one thread's smaller build must not lower another's)
+    static ContextOnce once;
+    const int rc = once_in_context(once, [&]() -> int {
+        BN_CUDA(cudaFuncSetAttribute(k_joint<KT, SMEM_DATA, MINOR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)JOINT_SMEM));
+        return BN_OK;
+    });
+    if (rc) return rc;
     k_joint<KT, SMEM_DATA, MINOR><<<grid, threads, smem, s>>>(A);
     BN_LAUNCH_CHECK("k_joint");
     return BN_OK;
@@ -877,7 +886,7 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
     int nwarps = BUILD_THREADS / 32;
     const size_t data_bytes = sizeof(uint32_t) * (size_t)n * mw;
     const size_t per_hist = sizeof(uint32_t) * (size_t)A.cells_cap, per_base = (size_t)mw * 32;
-    const size_t LIM = 220 * 1024;
+    const size_t LIM = JOINT_SMEM;
     bool base = m <= LIST_ROWS;
     while (base && nwarps > 2 && nwarps * (per_hist + per_base) > LIM) nwarps /= 2;
     if (!base || nwarps * (per_hist + per_base) > LIM) {
