@@ -1502,8 +1502,17 @@ static int persist_setup(bn_chains* ch)
     size_t smem = layout(sreg > 0);
     if (smem + static_smem > (size_t)optin) smem = layout(false);     // survivors from global memory
     if (smem + static_smem > (size_t)optin) return BN_OK;
-    if (cudaFuncSetAttribute(k_learned_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess) {
+    // the most a block can have: another chain set's smaller layout must not lower it
+    static ContextOnce once;
+    const int rc = once_in_context(once, [&]() -> int {
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaFuncGetAttributes(&fa, k_learned_persist);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_learned_persist, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     optin - (int)fa.sharedSizeBytes);
+        return e == cudaSuccess ? BN_OK : BN_ECUDA;
+    });
+    if (rc) {
         cudaGetLastError();
         return BN_OK;
     }
