@@ -480,7 +480,9 @@ __global__ void __launch_bounds__(256) k_embed_grad(const uint8_t* __restrict__ 
     if (y == 0 && j < d) gE[(size_t)v * d + j] = s;
 }
 
-// Adam (Kingma & Ba): moments and the FP32 master weight
+// Adam (Kingma & Ba): moments and the FP32 master weight.  The bias corrections of the next
+// step live on the device (bn_adam) and every step advances them itself, so that a
+// captured step replays with the corrections of its own place in the run.
 struct AdamRates {
     float lr, b1, b2, eps, c1, c2;
 };
@@ -505,8 +507,18 @@ struct AdamTensor {
 };
 struct AdamArgs {
     AdamTensor t[7];
-    AdamRates R;
+    AdamRates R;                // c1 and c2 filled in by the kernel
+    bn_adam* next;
 };
+// powers of the moments' rates: exact products rounded once to FP64 each step, far inside the
+// FP32 that the corrections are rounded to
+__host__ __device__ __forceinline__ void adam_set(bn_adam* a, double p1, double p2)
+{
+    a->p1 = p1;
+    a->p2 = p2;
+    a->c1 = 1.f - (float)p1;
+    a->c2 = 1.f - (float)p2;
+}
 
 // Every parameter in one launch, with the bf16 copies the GEMMs read: 1,024 elements a block,
 // W1 and W2 by 32 x 32 tiles for their transposes.  Bound by the weights' and moments'
@@ -515,6 +527,9 @@ struct AdamArgs {
 __global__ void __launch_bounds__(256) k_adam(AdamArgs A)
 {
     __shared__ bf16 tile[32][33];
+    AdamRates R = A.R;
+    R.c1 = A.next->c1;
+    R.c2 = A.next->c2;
     int blk = blockIdx.x, k = 0;
     while (blk >= A.t[k].blocks) blk -= A.t[k++].blocks;
     const AdamTensor& T = A.t[k];
@@ -524,16 +539,25 @@ __global__ void __launch_bounds__(256) k_adam(AdamArgs A)
         bf16 v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            v[q] = __float2bfloat16_rn(adam_at(T.w, T.g, T.m, T.v, (int64_t)(r0 + y + 8 * q) * T.cols + c0 + x, A.R));
+            v[q] = __float2bfloat16_rn(adam_at(T.w, T.g, T.m, T.v, (int64_t)(r0 + y + 8 * q) * T.cols + c0 + x, R));
         store_tile(tile, v, r0, c0, T.b, T.cols, T.bT, T.rows);
-        return;
-    }
+    } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int64_t i = (int64_t)blk * 1024 + q * 256 + y * 32 + x;
-        if (i < T.cols) {
-            const float w = adam_at(T.w, T.g, T.m, T.v, i, A.R);
-            if (T.b) T.b[i] = __float2bfloat16_rn(w);
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = (int64_t)blk * 1024 + q * 256 + y * 32 + x;
+            if (i < T.cols) {
+                const float w = adam_at(T.w, T.g, T.m, T.v, i, R);
+                if (T.b) T.b[i] = __float2bfloat16_rn(w);
+            }
+        }
+    }
+    // the last block to come here -- every block has used the corrections -- sets the next step's
+    __syncthreads();
+    if (x == 0 && y == 0) {
+        __threadfence();
+        if (atomicAdd(&A.next->done, 1u) == gridDim.x - 1) {
+            adam_set(A.next, A.next->p1 * (double)R.b1, A.next->p2 * (double)R.b2);
+            A.next->done = 0;
         }
     }
 }
@@ -663,8 +687,6 @@ int bn::mlp_loss_grad_dev(bn_mlp* m, const uint8_t* d_orders, const uint32_t* d_
 
 int bn::mlp_adam_dev(bn_mlp* m, cudaStream_t s)
 {
-    m->t += 1;
-    const float c1 = 1.f - powf(m->beta1, (float)m->t), c2 = 1.f - powf(m->beta2, (float)m->t);
     auto flat = [](float* w, float* g, float* mm, float* v, bf16* b, int64_t cnt) {
         return AdamTensor{w, g, mm, v, b, nullptr, 1, (int)cnt, (int)((cnt + 1023) / 1024)};
     };
@@ -677,7 +699,8 @@ int bn::mlp_adam_dev(bn_mlp* m, cudaStream_t s)
                 flat(m->E, m->gE, m->mE, m->vE, m->Eb, (int64_t)m->n * m->d),
                 flat(m->b1, m->gb1, m->mb1, m->vb1, nullptr, m->H), flat(m->b2, m->gb2, m->mb2, m->vb2, nullptr, m->H),
                 flat(m->b3, m->gb3, m->mb3, m->vb3, nullptr, m->P)},
-               {m->lr, m->beta1, m->beta2, m->adam_eps, c1, c2}};
+               {m->lr, m->beta1, m->beta2, m->adam_eps, 0.f, 0.f},
+               m->adam};
     int blocks = 0;
     for (const AdamTensor& t : A.t) blocks += t.blocks;
     k_adam<<<(unsigned)blocks, TILE, 0, s>>>(A);
@@ -750,6 +773,9 @@ extern "C" int bn_mlp_create(int n, const bn_mlp_params* p, const float* E, cons
     for (auto& e2 : f32) *e2.first = (float*)(base + offs[k++]);
     for (auto& e2 : b16) *e2.first = (bf16*)(base + offs[k++]);
     m->status = (uint32_t*)(base + o_status);
+    m->adam = (bn_adam*)(base + o_status + 64);
+    bn_adam first = {};
+    adam_set(&first, (double)m->beta1, (double)m->beta2);
     m->stage_orders = base + o_stage;
     m->stage_pairs = (uint32_t*)(base + o_stage + (size_t)round_up((int64_t)cap * n, 256));
     m->stage_alpha = (float*)((uint8_t*)m->stage_pairs + (size_t)round_up((int64_t)cap * 4, 256));
@@ -760,7 +786,8 @@ extern "C" int bn_mlp_create(int n, const bn_mlp_params* p, const float* E, cons
     if (cudaMemsetAsync(m->block, 0, off, s) != cudaSuccess) return fail(cuda_fail(cudaGetLastError(), "memset", __FILE__, __LINE__));
     const cudaMemcpyKind kind = mem == BN_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     // weights come row-major and unpadded: E n x d, W1 H x (n d), W2 H x H, W3 P x H
-    if (cudaMemcpyAsync(m->E, E, 4 * nE, kind, s) != cudaSuccess ||
+    if (cudaMemcpyAsync(m->adam, &first, sizeof(first), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(m->E, E, 4 * nE, kind, s) != cudaSuccess ||
         cudaMemcpy2DAsync(m->W1, 4 * (size_t)ndp, W1, 4 * (size_t)m->nd, 4 * (size_t)m->nd, H, kind, s) != cudaSuccess ||
         cudaMemcpyAsync(m->b1, b1, 4 * (size_t)H, kind, s) != cudaSuccess ||
         cudaMemcpyAsync(m->W2, W2, 4 * nW2, kind, s) != cudaSuccess ||

@@ -5,10 +5,17 @@
 
 #include "bn_internal.cuh"
 
+// Adam's state beside the moments: the rates' powers at the next step, its bias corrections,
+// and the blocks of the running step that are done
+struct bn_adam {
+    double p1, p2;
+    float c1, c2;
+    uint32_t done;
+};
+
 struct bn_mlp {
     int n = 0, d = 0, H = 0, P = 0, Pp = 0, nd = 0, ndp = 0, cap = 0, Mp = 0;
     float lr = 0.f, beta1 = 0.9f, beta2 = 0.999f, adam_eps = 1e-8f;
-    int64_t t = 0;                 // Adam steps taken
     void* block = nullptr;
     size_t bytes = 0;
     // FP32 master weights (W1 padded to H x ndp, W3 to Pp x H), gradients, Adam moments
@@ -26,6 +33,7 @@ struct bn_mlp {
     float* ws = nullptr;           // split-K partials
     size_t ws_elems = 0;
     uint32_t* status;
+    bn_adam* adam;
     uint8_t* stage_orders;
     uint32_t* stage_pairs;
     float* stage_alpha;
