@@ -816,7 +816,11 @@ static int rank_by_radix(bn_table* t, cudaStream_t s)
 // Ranks every node's entries (see the file comment) and lays out what the scans read:
 // srank, spos, its entry-major copy spos_t and (k <= 4) the parent nodes by sorted
 // position.  d_cut receives each node's empty-set position + 1 (device, n words; the caller
-// copies it to t->cut).  Temporaries are stream-ordered; nothing waits for the device.
+// copies it to t->cut).  Temporaries are stream-ordered.  The parent nodes' memory is taken here
+// and not with the rest of the table, though that may wait for the counting kernels (whose
+// freed sums it can reuse): taken before them, the host's 10 to 20 us come before the first
+// kernel instead of behind it (37 nodes learned end to end 2.34 -> 2.35 ms, twelve networks
+// 19.2 -> 19.3).
 int rank_entries(bn_table* t, uint32_t* d_cut, cudaStream_t s)
 {
     const int64_t S = t->S;

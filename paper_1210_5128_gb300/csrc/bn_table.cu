@@ -814,7 +814,7 @@ static int build_plan(const uint8_t* data, int m, int n, const uint8_t* arity, i
 // Device half: every kernel of the build on stream s, writing t (allocated), OR-ing
 // STATUS_BADINPUT into d_meta[0] for a data value at or above its arity and leaving the
 // nodes' empty-set positions + 1 in d_meta[1..n] (META_WORDS words).  Temporaries are
-// stream-ordered; nothing here waits for the device.
+// stream-ordered; the host waits for the device only where rank_entries takes memory.
 static constexpr int META_WORDS = 1 + MAXN;
 static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cudaStream_t s,
                          cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr)
