@@ -36,6 +36,7 @@ static constexpr int SUM_OB = 8;          // orders per block
 static constexpr int SUM_THREADS = 256;
 static constexpr int SUM_WARPS = SUM_THREADS / 32;
 static constexpr int SUM_BATCH = 256;     // orders whose partials are held at a time
+static constexpr int SUM_SLICE = 65535 * 256;   // orders whose lists are: as many as every scan's grid takes
 
 struct SumScanArgs {
     const int64_t* keys;
@@ -299,7 +300,7 @@ extern "C" int bn_score_orders_sum(const bn_table* t, const uint8_t* orders, int
     // short runs where there are few: a warp's steps are its latency
     const int run = t->S >= 65536 ? 1024 : 256;
     const int nchunk = (int)((t->S + SUM_WARPS * run - 1) / (SUM_WARPS * run));
-    const int batch = std::min(B, SUM_BATCH);
+    const int batch = std::min(B, SUM_BATCH), slice = std::min(B, SUM_SLICE);
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
@@ -307,8 +308,8 @@ extern "C" int bn_score_orders_sum(const bn_table* t, const uint8_t* orders, int
         return o;
     };
     const size_t o_orders = take(mem == BN_MEM_HOST ? (size_t)B * n : 0);
-    const size_t o_pc = take(sizeof(uint64_t) * (size_t)n * B);
-    const size_t o_best = take(sizeof(uint32_t) * (size_t)n * B);
+    const size_t o_pc = take(sizeof(uint64_t) * (size_t)n * slice);
+    const size_t o_best = take(sizeof(uint32_t) * (size_t)n * slice);
     const size_t o_cnt = take(sizeof(uint32_t) * n);
     const size_t o_st = take(sizeof(uint32_t));
     const size_t o_part = take(sizeof(double) * (size_t)n * batch * nchunk);
@@ -338,22 +339,26 @@ extern "C" int bn_score_orders_sum(const bn_table* t, const uint8_t* orders, int
     double* d_os = mem == BN_MEM_HOST ? (order_score ? (double*)(base + o_os) : nullptr) : order_score;
     double* d_ns = mem == BN_MEM_HOST ? (node_score ? (double*)(base + o_ns) : nullptr) : node_score;
     BN_CUDA(cudaMemsetAsync(d_st, 0, sizeof(uint32_t), s));
-    int rc = launch_pred_lists(d_orders, B, n, d_pc, d_best, d_cnt, d_st, s);
-    if (rc) return rc;
-    // the best consistent entries, by the fastest scan the table has (all give the same)
-    if (t->amask) rc = launch_scan_pruned(t, d_cnt, d_pc, d_best, B, s);
-    else if (t->sset) rc = launch_scan_sliced(t, d_cnt, d_pc, d_best, B, true, d_st, s);
-    else rc = launch_scan(t, plan_scan(t, B), d_cnt, d_pc, d_best, B, d_st, s);
-    if (rc) return rc;
     const double reach = std::log10((double)t->S) + 60.0 * 0.30102999566398120;
-    for (int b0 = 0; b0 < B; b0 += batch) {
-        SumScanArgs A{t->keys, t->pst, t->srank, t->S, t->Sp, n, B, b0, std::min(B, b0 + batch), run, nchunk, reach, d_pc,
-                      d_best, d_part};
-        const int groups = (A.b1 - b0 + SUM_OB - 1) / SUM_OB;
-        k_sum_window<<<dim3((unsigned)nchunk, (unsigned)n, (unsigned)groups), SUM_THREADS, 0, s>>>(A);
-        BN_LAUNCH_CHECK("k_sum_window");
-        k_sum_finish<<<(unsigned)(A.b1 - b0), SUM_THREADS, 0, s>>>(A, d_ns, d_os);
-        BN_LAUNCH_CHECK("k_sum_finish");
+    for (int64_t s0 = 0; s0 < B; s0 += slice) {
+        const int Bs = (int)std::min<int64_t>(slice, B - s0);
+        int rc = launch_pred_lists(d_orders + (size_t)s0 * n, Bs, n, d_pc, d_best, d_cnt, d_st, s);
+        if (rc) return rc;
+        // the best consistent entries, by the fastest scan the table has (all give the same)
+        if (t->amask) rc = launch_scan_pruned(t, d_cnt, d_pc, d_best, Bs, s);
+        else if (t->sset) rc = launch_scan_sliced(t, d_cnt, d_pc, d_best, Bs, true, d_st, s);
+        else rc = launch_scan(t, plan_scan(t, Bs), d_cnt, d_pc, d_best, Bs, d_st, s);
+        if (rc) return rc;
+        for (int b0 = 0; b0 < Bs; b0 += batch) {
+            SumScanArgs A{t->keys, t->pst, t->srank, t->S, t->Sp, n, Bs, b0, std::min(Bs, b0 + batch), run, nchunk, reach,
+                          d_pc, d_best, d_part};
+            const int groups = (A.b1 - b0 + SUM_OB - 1) / SUM_OB;
+            k_sum_window<<<dim3((unsigned)nchunk, (unsigned)n, (unsigned)groups), SUM_THREADS, 0, s>>>(A);
+            BN_LAUNCH_CHECK("k_sum_window");
+            k_sum_finish<<<(unsigned)(A.b1 - b0), SUM_THREADS, 0, s>>>(A, d_ns ? d_ns + (size_t)s0 * n : nullptr,
+                                                                      d_os ? d_os + s0 : nullptr);
+            BN_LAUNCH_CHECK("k_sum_finish");
+        }
     }
     if (mem == BN_MEM_HOST) {
         if (order_score) BN_CUDA(cudaMemcpyAsync(order_score, d_os, sizeof(double) * B, cudaMemcpyDeviceToHost, s));
