@@ -21,13 +21,14 @@
 // arithmetic (exp10_fx), relative to the first entry ref of a stretch of the list no longer
 // than one decade; a consistent order adds it as an integer, and only the stretch's sums
 // are brought to FP64 and scaled by 10^(ref - m) -- one exp10 on eight lanes per 1,024
-// entries.  Every term is good to 2^-55 of itself, as from FP64.  Steps of 32 entries that
+// entries.  Every term is good to 2^-55 of itself.  Steps of 32 entries that
 // span more than a decade or two binades of scores (short lists, the ends of long ones)
 // take FP64 exponentials per (entry, order).  8 orders at n = 60: 484 us with one exp10 per
 // (entry, order), 208 so; 6.1 ms with every entry's.
 #include <algorithm>
 #include <cmath>
 
+#include "bn_fx.cuh"
 #include "bn_table.cuh"
 
 namespace bn {
@@ -57,53 +58,7 @@ __device__ __forceinline__ int64_t sorted_key(const SumScanArgs& A, int i, int64
     return A.keys[(size_t)i * A.Sp + A.srank[(size_t)i * A.Sp + p]];
 }
 
-// 2^(-j / 64), 2^(-j / 4096) and 2^(-j / 262144), j < 64, with 63 fractional bits, from the
-// exponential series in integer arithmetic
-struct Exp2Tables {
-    uint64_t v[3][64];
-};
-constexpr uint64_t LN2_64 = 0xB17217F7D1CF79ACull;        // ln 2 in 2^-64
-constexpr uint64_t mulhi_c(uint64_t a, uint64_t b) { return (uint64_t)(((unsigned __int128)a * b) >> 64); }
-constexpr Exp2Tables make_exp2()
-{
-    Exp2Tables T{};
-    for (int t = 0; t < 3; ++t)
-        for (int j = 0; j < 64; ++j) {
-            // e^-z, z = ln 2 * j / 64^(t + 1), as sum (-z)^k / k! in 2^-64 with 128-bit sums
-            const uint64_t x = (uint64_t)j << (58 - 6 * t);                  // j / 64^(t + 1) in 2^-64
-            const uint64_t z = mulhi_c(x, LN2_64);
-            unsigned __int128 pos = (unsigned __int128)1 << 64, neg = 0;
-            uint64_t term = z;
-            for (int k = 1; k < 24; ++k) {
-                if (k & 1) neg += term;
-                else pos += term;
-                term = mulhi_c(term, z) / (uint64_t)(k + 1);
-            }
-            T.v[t][j] = (uint64_t)((pos - neg + 1) >> 1);
-        }
-    return T;
-}
 static __device__ const Exp2Tables g_exp2 = make_exp2();
-
-// 10^-d in 2^-58 for d in [0, 1] given in 2^-60: d log2 10 = whole + three table digits of
-// six bits + a rest below 2^-18, whose 2^-r = 1 - z + z^2 / 2 up to z^3 / 6 < 2^-58
-__device__ __forceinline__ uint64_t exp10_fx(uint64_t d, const uint64_t (&T)[3][64])
-{
-    constexpr uint64_t LOG2_10 = 0x6A4D3C25E68DC57Full;                      // log2 10 in 2^-61
-    const uint64_t y = __umul64hi(d, LOG2_10);                               // in 2^-57
-    const uint32_t whole = (uint32_t)(y >> 57);
-    const uint64_t t1 = T[0][(y >> 51) & 63], t2 = T[1][(y >> 45) & 63], t3 = T[2][(y >> 39) & 63];
-    const uint64_t r = y & ((1ull << 39) - 1);                               // in 2^-57, below 2^-18
-    const uint64_t z = __umul64hi(r << 25, LN2_64);                          // in 2^-82, below 2^63.5
-    const uint32_t zh = (uint32_t)(z >> 32);                                 // z in 2^-50
-    const uint64_t sq = (uint64_t)zh * zh;                                   // z^2 in 2^-100
-    // 1 - z + z^2 / 2 in 2^-63
-    const uint64_t e = (1ull << 63) - (z >> 19) + (sq >> 38);
-    uint64_t p = __umul64hi(t1, t2) << 1;                                    // 2^-63 each
-    p = __umul64hi(p, t3) << 1;
-    p = __umul64hi(p, e);                                                    // 2^-62
-    return (p >> 4) >> whole;                                                // 2^-58
-}
 
 __global__ void __launch_bounds__(SUM_THREADS) k_sum_window(SumScanArgs A)
 {
@@ -175,7 +130,7 @@ __global__ void __launch_bounds__(SUM_THREADS) k_sum_window(SumScanArgs A)
                 sum[b] = 0;
             }
             if (lane < nb && my_m > -INFINITY) {
-                const double t = __fma_rn((double)top, 0x1p44, (double)mine) * 0x1p-58;
+                const double t = __fma_rn((double)top, 0x1p44, (double)mine) * 0x1p-59;
                 if (t != 0.0) acc += t * exp10(key_to_double(ref) - my_m);
             }
             held = 0;
