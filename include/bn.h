@@ -28,6 +28,9 @@
  *     S(n-1, k) = sum_{j<=k} C(n-1, j) sets per node (Sec. III.B).
  *   - Ties between equal local scores always go to the lowest rank.
  *   - Orders are arrays of n node ids, position -> node.
+ *   - Device memory: objects and scratch come from a pool of the library's own, which keeps
+ *     up to 2 GiB per device mapped after they are freed, for the next calls; other
+ *     allocators in the process cannot use it until bn_release_memory gives it back.
  */
 #ifndef BN_H
 #define BN_H
@@ -493,6 +496,10 @@ int bn_gemm_bf16(const uint16_t* A, const uint16_t* B, float* C, int M, int N, i
  * status word.  Returns BN_ETIMEOUT when both waits ran out as intended (the context
  * stays usable), BN_ECUDA otherwise. */
 int bn_selftest_timeout(int64_t timeout_ns, void* stream);
+
+/* Give the memory that no live object uses back to the current device (see "Device memory"
+ * above); waits for the device's work.  The next calls map memory anew.  Errors: BN_ECUDA. */
+int bn_release_memory(void);
 
 /* Measured peak rate of the scan's consistency test on this GPU (the paper has no
  * counterpart; it is the denominator of the full-table scan's roofline): a kernel that

@@ -29,7 +29,7 @@ OUT = dict(orders=1, scores=2, ranks=3, best_orders=4, best_scores=5, best_ranks
 ABI = ["bn_build_scores", "bn_table_from_scores", "bn_table_info", "bn_table_scores",
        "bn_table_free", "bn_score_orders", "bn_unrank", "bn_rank", "bn_chains_create",
        "bn_chains_step", "bn_chains_step_profiled", "bn_chains_read", "bn_chains_free",
-       "bn_mcmc_run", "bn_last_error", "bn_version", "bn_kernel_launches"]
+       "bn_mcmc_run", "bn_last_error", "bn_version", "bn_kernel_launches", "bn_release_memory"]
 
 
 class BNError(RuntimeError):
@@ -139,6 +139,12 @@ def last_error() -> str:
 
 def version() -> str:
     return lib().bn_version().decode()
+
+
+def release_memory():
+    """Give device memory that no live object uses back to the device (bn_release_memory): up
+    to 2 GiB stay mapped for later calls otherwise."""
+    _check(lib().bn_release_memory())
 
 
 def kernel_launches() -> int:

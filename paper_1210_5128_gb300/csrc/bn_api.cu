@@ -82,7 +82,7 @@ int sm_count()
 
 // ---------------------------------------------------------------------------------
 // Memory.  Tables, chains and scratch come from one stream-ordered pool per device that keeps
-// up to POOL_KEEP bytes mapped between calls: mapping and unmapping a table's memory took
+// up to POOL_KEEP bytes mapped between calls (bn_release_memory gives them back): mapping and unmapping a table's memory took
 // as long as a fifth of the build it was for (60 nodes: 1.8 ms of a 9.3 ms call; 37 nodes:
 // 1.1 of 3.2).  What is above POOL_KEEP goes back to the device at the next
 // synchronisation, and all of it when an allocation of the library's own fails.
@@ -275,6 +275,16 @@ int bn_selftest_timeout(int64_t timeout_ns, void* stream)
     if (h == (bn::STATUS_TIMEOUT | (bn::STATUS_TIMEOUT << 1)))
         return bn::set_error(BN_ETIMEOUT, "bn_selftest_timeout: both bounded waits gave up as intended");
     return bn::set_error(BN_ECUDA, "bn_selftest_timeout: unexpected status %u", h);
+}
+
+int bn_release_memory(void)
+{
+    bn::t_err[0] = 0;
+    const bn::DevPool P = bn::dev_pool();
+    if (!P.pool) return BN_OK;
+    BN_CUDA(cudaDeviceSynchronize());                  // frees queued on any stream have happened
+    BN_CUDA(cudaMemPoolTrimTo(P.pool, 0));
+    return BN_OK;
 }
 
 const char* bn_last_error(void) { return bn::t_err; }
