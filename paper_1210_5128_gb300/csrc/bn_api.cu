@@ -4,7 +4,6 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
-#include <vector>
 
 #include <cuda.h>
 
@@ -184,11 +183,8 @@ struct SlotEntry {
     uint8_t* p;
 };
 static std::mutex g_slot_mu;
-static std::vector<SlotEntry>& slot_list()
-{
-    static std::vector<SlotEntry>* v = new std::vector<SlotEntry>();     // never destroyed: calls may outlive statics
-    return *v;
-}
+static SlotEntry g_slots[SLOT_KEEP];               // (plain memory: a slot's end cannot throw, and
+static size_t g_slot_count = 0;                    // calls may outlive the statics' destruction)
 
 HostSlot::HostSlot()
 {
@@ -196,11 +192,10 @@ HostSlot::HostSlot()
     uint8_t* p = nullptr;
     if (ctx) {
         std::lock_guard<std::mutex> g(g_slot_mu);
-        auto& v = slot_list();
-        for (size_t i = v.size(); i-- > 0;)
-            if (v[i].ctx == ctx) {
-                p = v[i].p;
-                v.erase(v.begin() + (ptrdiff_t)i);
+        for (size_t i = g_slot_count; i-- > 0;)
+            if (g_slots[i].ctx == ctx) {
+                p = g_slots[i].p;
+                g_slots[i] = g_slots[--g_slot_count];
                 break;
             }
     }
@@ -218,9 +213,8 @@ HostSlot::~HostSlot()
     if (!status) return;
     if (ctx) {
         std::lock_guard<std::mutex> g(g_slot_mu);
-        auto& v = slot_list();
-        if (v.size() < SLOT_KEEP) {
-            v.push_back({ctx, (uint8_t*)status});
+        if (g_slot_count < SLOT_KEEP) {
+            g_slots[g_slot_count++] = {ctx, (uint8_t*)status};
             return;
         }
     }
