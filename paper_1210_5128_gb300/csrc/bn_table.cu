@@ -288,8 +288,8 @@ __device__ __forceinline__ void minor_cells(uint32_t* hist, const uint32_t* pre,
 // lowest node is not in its most frequent state -- about half -- and the frequent state's
 // cells are what is left of the configurations' counts.  A visit is two 16-bit loads (the
 // list ascends, so the second is nearly consecutive over the lanes), a multiply-add and a
-// shared atomic; the hottest cells take no atomics at all.  Without MINOR (more rows than a
-// list entry names, or no room) every row's cell is formed from all nodes.  Shared memory
+// shared atomic; the hottest cells take no atomics at all.  Without MINOR (few sets, or many
+// rows: the rule is in build_enqueue) every row's cell is formed from all nodes.  Shared memory
 // holds the warps' histograms, the rows' offsets (MINOR), then (SMEM_DATA) the packed data.
 // n = 60, k = 4, m = 1000: 4.51 ms against 5.05 with every row visited; 628 warp
 // instructions a set at two thirds of the issue slots, and the shared-memory pipe 72 % busy
@@ -880,24 +880,6 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
     uint32_t* d_len = nullptr;
     Temps sums(s);
     if ((rc = sums.get(&A.G, (size_t)A.S1)) || (rc = sums.get(&A.H, (size_t)A.S0 * P.nv))) return rc;
-    // Shared memory: the histograms, the rows' offsets and the packed data as long as two
-    // blocks fit an SM with them; fewer warps a block, then every row of every set, when a
-    // block alone does not fit (counts of thousands of cells).
-    int nwarps = BUILD_THREADS / 32;
-    const size_t data_bytes = sizeof(uint32_t) * (size_t)n * mw;
-    const size_t per_hist = sizeof(uint32_t) * (size_t)A.cells_cap, per_base = (size_t)mw * 32;
-    const size_t LIM = JOINT_SMEM;
-    bool base = m <= LIST_ROWS;
-    while (base && nwarps > 2 && nwarps * (per_hist + per_base) > LIM) nwarps /= 2;
-    if (!base || nwarps * (per_hist + per_base) > LIM) {
-        base = false;
-        nwarps = BUILD_THREADS / 32;
-        while (nwarps > 1 && nwarps * per_hist > LIM) nwarps /= 2;
-    }
-    size_t smem = nwarps * (per_hist + (base ? per_base : 0));
-    const bool smem_data = smem + data_bytes <= LIM / 2;
-    if (smem_data) smem += data_bytes;
-    const int per_sm = std::max(1, std::min(2048 / (32 * nwarps), (int)((224 * 1024) / std::max<size_t>(smem + 1024, 1))));
     // the largest sets -- nearly all of them -- and those of four nodes on the tensor cores
     // where they are many and one set of lgamma tables serves them all (K2; BDeu with one arity)
     TcPlan tcp[2];                    // k + 1 nodes; four nodes where they are parent sets too
@@ -917,8 +899,33 @@ static int build_enqueue(const BuildPlan& P, bn_table* t, uint32_t* d_meta, cuda
             return rc;
     }
     if (tc[0]) A.S1 = tc[1] ? num_sets_host(n, k - 1) : A.S0;
+    // Shared memory of a block: the histograms, with `base` the rows' offsets, and the packed
+    // data as long as two blocks fit an SM with them
+    const int nwarps = BUILD_THREADS / 32;
+    const size_t data_bytes = sizeof(uint32_t) * (size_t)n * mw;
+    const size_t per_hist = sizeof(uint32_t) * (size_t)A.cells_cap, per_base = (size_t)mw * 32;
+    static_assert(sizeof(uint32_t) * MAX_CELLS * (BUILD_THREADS / 32) <= JOINT_SMEM, "the histograms of a block fit");
+    size_t smem = 0;
+    bool smem_data = false;
+    int per_sm = 1;
+    auto shape = [&](bool base) {
+        smem = nwarps * (per_hist + (base ? per_base : 0));
+        smem_data = smem + data_bytes <= JOINT_SMEM / 2;
+        if (smem_data) smem += data_bytes;
+        per_sm = std::max(1, std::min(2048 / (32 * nwarps), (int)((224 * 1024) / std::max<size_t>(smem + 1024, 1))));
+        return (int64_t)sm_count() * per_sm * nwarps;               // resident warps
+    };
+    // The rows' offsets pay while two blocks an SM hold them and, up to k = 4, a warp keeps
+    // them for a few sets (five a unit) and there are not many rows: beyond, fewer warps are
+    // resident, with 16,000 rows a quarter of those without.  us of k_joint with and without,
+    // two to four states, BDeu: 37 nodes, k = 4, m = 1,000 480 / 593, 2,500 920 / 960, 4,000
+    // 1,742 / 1,390, 8,000 5,262 / 2,532; 30 nodes, m = 900 (4 sets a unit) 312 / 268, 1,000
+    // (5) 233 / 271; k = 3, ternary, m = 1,000 67 / 63, 16,000 1,088 / 360.  k = 5, binary, 24
+    // nodes: m = 1,000 277 / 302, 5,000 614 / 896.
+    bool base = m > 0 && m <= LIST_ROWS && nwarps * (per_hist + per_base) <= JOINT_SMEM / 2;
+    if (base && k <= 4) base = m <= 2500 && A.S1 >= 5 * 8 * shape(true);
+    const int64_t warps = shape(base);
     // 8 to 64 sets a unit: about eight units a resident warp where there are enough sets
-    const int64_t warps = (int64_t)sm_count() * per_sm * nwarps;
     A.range = (int)std::max<int64_t>(4, std::min<int64_t>(64, A.S1 / (8 * warps)));
     const int64_t units = (A.S1 + A.range - 1) / A.range;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count() * per_sm, (units + nwarps - 1) / nwarps));
