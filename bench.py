@@ -18,7 +18,9 @@ measured on the same table.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-Prints one JSON line (rank 0).  Under torchrun every rank runs its own replica of the
+Prints one short JSON line (rank 0): the headline, its end-to-end number, its roofline and the
+clocks.  Everything measured, the other legs included, goes to the file --legs names
+(bench_legs.json beside this file).  Under torchrun every rank runs its own replica of the
 table and its own chains (independent chains, no data exchange); the value is the sum
 over ranks of order evaluations divided by the slowest rank's time.
 """
@@ -64,6 +66,7 @@ def parse():
     ap.add_argument("--batch-ess-steps", type=int, default=4000)
     ap.add_argument("--batch-train", type=int, default=300)
     ap.add_argument("--no-accuracy", action="store_true", help="skip the ROC and noise study")
+    ap.add_argument("--legs", default=os.path.join(ROOT, "bench_legs.json"), help="file for everything measured")
     ap.add_argument("--no-configs", action="store_true", help="skip the n=20 and n=40 configurations")
     return ap.parse_args()
 
@@ -201,10 +204,29 @@ def config_dict(chains, scan="pruned"):
                         f"k=4 (489,406 parent sets/node, 29.36M FP64 entries, 235 MB), {chains} chains, "
                         "uniform swap proposal",
             "chains": chains, "n": 60, "k": 4, "m": 1000, "scan": scan,
-            "l2": "flushed: a 512 MB buffer is written and another read before every timed step (outside "
-                  "its events); "
-                  "the table is 235 MB of FP64 entries, the full scan streams 117 MB of sorted positions "
-                  "plus the 3.9 MB mask table per pass"}
+            "l2": "flushed: a 512 MB buffer is written and another read before every timed step"}
+
+
+HEAD_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks")
+
+
+def emit(line, path):
+    """Prints the headline of `line` as one JSON line, short enough to be kept whole, and writes
+    all of it to `path`."""
+    head = {k: line[k] for k in HEAD_KEYS}
+    head["e2e"] = {k: v for k, v in line["e2e"].items() if k != "note"}
+    r = line["roofline"]
+    head["roofline"] = {k: r[k] for k in ("bound", "unit", "achieved", "peak", "frac")}
+    if line.get("cpu_baseline"):
+        head["cpu_baseline"] = {k: line["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind")}
+    try:
+        with open(path, "w") as f:
+            json.dump(line, f, indent=1)
+        head["legs"] = os.path.basename(path)
+    except OSError as e:
+        print(f"bench.py: {path}: {e}", file=sys.stderr)
+    print(json.dumps(head), flush=True)
 
 
 L2_FLUSH_BYTES = 512 << 20 # written, then another buffer read, between timed steps (L2 is 129 MB)
@@ -907,7 +929,7 @@ def main():
             "table_entries_per_s": n * S / build_s,
             "table_row_visits_per_s": n * S * data.shape[0] / build_s,
         }
-        print(json.dumps(line), flush=True)
+        emit(line, args.legs)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()
