@@ -84,8 +84,8 @@ int bn_build_scores(const uint8_t* data, int m, int n, const uint8_t* arity, int
                     void* stream, bn_table** out);
 
 /* bn_build_scores with the device time of its counting and scoring kernels (the table
- * build of Eq. (3)-(4)) measured by CUDA events on `stream` around those launches: *build_ms receives it (build_ms may be NULL).  Outputs and errors as
- * bn_build_scores. */
+ * build of Eq. (3)-(4)) measured by CUDA events on `stream` around those launches:
+ * *build_ms receives it (build_ms may be NULL).  Outputs and errors as bn_build_scores. */
 int bn_build_scores_profiled(const uint8_t* data, int m, int n, const uint8_t* arity, int k,
                              const double* R, const bn_score_params* params, int mem,
                              void* stream, bn_table** out, double* build_ms);

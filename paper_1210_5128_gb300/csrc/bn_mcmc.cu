@@ -334,7 +334,7 @@ struct FusedArgs {
     int staged;          // 1: the network's survivors fit the warp's shared-memory cache
     int cap;             // survivors per warp cache (shared-memory layout of the launch;
                          // the table's survivor count for a global-memory cache)
-    const uint8_t* gcache;   // not staged: the same cache in global memory, or null
+    const uint8_t* gcache;   // the same cache in global memory (staged: copied from it), or null
     const uint16_t* gfirst;  // with gcache: [node][v] first survivor of the node whose set
                              // contains node v (the node's survivor count if none)
     double margin_x;     // bound on |ln10 (dpart - (s' - s))| (rounding of the two sums)
@@ -466,7 +466,7 @@ __device__ __forceinline__ void fill_surv_cache(const ChainState& S, const Fused
 }
 
 // The survivors in the cache layout above, in global memory (one thread per survivor; the
-// prefix ORs one thread per node, in a second launch)
+// prefix ORs follow in k_gcache_index)
 __global__ void k_gcache_fill(const int64_t* __restrict__ keys, const uint32_t* __restrict__ srank, int64_t Sp,
                               int n, const uint64_t* __restrict__ amask, const uint32_t* __restrict__ aspos,
                               const uint32_t* __restrict__ aoff, uint32_t total, int cap, uint8_t* __restrict__ cache)

@@ -523,7 +523,7 @@ __host__ __device__ __forceinline__ void adam_set(bn_adam* a, double p1, double 
 // Every parameter in one launch, with the bf16 copies the GEMMs read: 1,024 elements a block,
 // W1 and W2 by 32 x 32 tiles for their transposes.  Bound by the weights' and moments'
 // traffic, 24 bytes a parameter and step; seven launches for the step and four for the
-// copies took 61 us of kernels at n = 60, H = 512, this one 18.
+// copies took 61 us of kernels at n = 60, H = 512, this one 19.
 __global__ void __launch_bounds__(256) k_adam(AdamArgs A)
 {
     __shared__ bf16 tile[32][33];
