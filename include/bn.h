@@ -421,7 +421,9 @@ typedef struct {
 int bn_mlp_create(int n, const bn_mlp_params* p, const float* E, const float* W1,
                   const float* b1, const float* W2, const float* b2, const float* W3,
                   const float* b3, int mem, void* stream, bn_mlp** out);
-/* logits of B <= batch_cap orders: B x P float32 */
+/* logits of B <= batch_cap orders: B x P float32.  Here and in bn_mlp_loss_grad an order
+ * that names a node at or above n, or a pair at or above P, is BN_EINVAL (the outputs are
+ * then not meaningful; the network's weights are untouched). */
 int bn_mlp_forward(bn_mlp* m, const uint8_t* orders, int B, float* logits, int mem,
                    void* stream);
 /* loss and gradients (kept inside; read them with bn_mlp_read) of B logged steps:

@@ -250,10 +250,11 @@ __device__ __forceinline__ void store_tile(bf16 (&tile)[32][33], const bf16 (&v)
 }
 
 // x rows: X[r][p*d + j] = E[order_r(p)][j] (bf16), zero padding; XT and inv (the inverse
-// orders: inv[r * 64 + v] = position of node v in order r) for training
+// orders: inv[r * 64 + v] = position of node v in order r) for training.  An entry that is no
+// node counts as zero and sets STATUS_BADINPUT.
 __global__ void __launch_bounds__(256) k_embed(const uint8_t* __restrict__ orders, int B, int n, int d, int ndp, int Mp,
                                                const bf16* __restrict__ Eb, bf16* __restrict__ X, bf16* __restrict__ XT,
-                                               uint8_t* __restrict__ inv)
+                                               uint8_t* __restrict__ inv, uint32_t* status)
 {
     __shared__ bf16 tile[32][33];
     const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, col = c0 + threadIdx.x;
@@ -265,8 +266,12 @@ __global__ void __launch_bounds__(256) k_embed(const uint8_t* __restrict__ order
         v[k] = __float2bfloat16_rn(0.f);
         if (r < B && p < n) {
             const int o = orders[(size_t)r * n + p];
-            v[k] = Eb[(size_t)o * d + j];
-            if (inv && j == 0) inv[(size_t)r * 64 + o] = (uint8_t)p;
+            if (o < n) {
+                v[k] = Eb[(size_t)o * d + j];
+                if (inv && j == 0) inv[(size_t)r * 64 + o] = (uint8_t)p;
+            } else {
+                atomicOr(status, STATUS_BADINPUT);
+            }
         }
     }
     store_tile(tile, v, r0, c0, X, ndp, XT, Mp);
@@ -303,17 +308,19 @@ __global__ void __launch_bounds__(256) k_bias(Product in, float* __restrict__ Z,
 
 // output layer gradient of the BCE loss (one logit per row): block per row.  The row's
 // d loss / d logit and loss term go to grow[r] and lrow[r]; k_out_grad_w and k_loss_sum
-// sum them in row order, so the gradients and the loss do not depend on scheduling.
+// sum them in row order, so the gradients and the loss do not depend on scheduling.  A pair
+// that does not exist counts as pair 0 here and nowhere in gW3, and sets STATUS_BADINPUT.
 __global__ void k_out_grad(const float* __restrict__ L, int ldl, const uint32_t* __restrict__ pairs,
-                           const float* __restrict__ alpha, int B, int Mp, int H, const float* __restrict__ Z2,
+                           const float* __restrict__ alpha, int B, int P, int Mp, int H, const float* __restrict__ Z2,
                            const bf16* __restrict__ W3b, bf16* __restrict__ dZ2, bf16* __restrict__ dZ2T,
-                           float* __restrict__ grow, float* __restrict__ lrow)
+                           float* __restrict__ grow, float* __restrict__ lrow, uint32_t* status)
 {
     const int r = blockIdx.x;
     float g = 0.f;
     int p = 0;
     if (r < B) {
-        p = (int)pairs[r];
+        p = pairs[r] < (uint32_t)P ? (int)pairs[r] : 0;
+        if (threadIdx.x == 0 && pairs[r] >= (uint32_t)P) atomicOr(status, STATUS_BADINPUT);
         const float l = L[(size_t)r * ldl + p];
         const float s = 1.f / (1.f + expf(-l));
         const float a = alpha[r];
@@ -365,7 +372,7 @@ __device__ __forceinline__ void colsum_block(float (&s_t)[CS_ROWS][33], const bf
 // column sums of dZ2 (gb2), the last block the batch loss (per thread a strided run, then a
 // fixed shared-memory tree).
 __global__ void __launch_bounds__(256) k_out_sums(const uint32_t* __restrict__ pairs, const float* __restrict__ grow,
-                                                  const float* __restrict__ lrow, int B, int H,
+                                                  const float* __restrict__ lrow, int B, int P, int H,
                                                   const bf16* __restrict__ H2, const bf16* __restrict__ dZ2,
                                                   float* __restrict__ gW3, float* __restrict__ gb3,
                                                   float* __restrict__ gb2, float* __restrict__ loss)
@@ -395,7 +402,7 @@ __global__ void __launch_bounds__(256) k_out_sums(const uint32_t* __restrict__ p
     const uint32_t p = pairs[r];
     bool dup = false;
     for (int q = tid; q < r; q += 256) dup |= pairs[q] == p;
-    if (__syncthreads_or(dup)) return;                                  // block-uniform
+    if (__syncthreads_or(dup) || p >= (uint32_t)P) return;              // block-uniform
     float sb = 0.f;
     for (int c0 = 0; c0 < H; c0 += 256) {
         const int c = c0 + tid;
@@ -619,7 +626,7 @@ static int mlp_forward(bn_mlp* m, const uint8_t* d_orders, int B, bool train, cu
     if (Mp > m->cap) return set_error(BN_EINVAL, "mlp: batch %d above capacity %d", B, m->cap);
     m->Mp = Mp;
     k_embed<<<tiles_of(Mp, m->ndp), TILE, 0, s>>>(d_orders, B, m->n, m->d, m->ndp, Mp, m->Eb, m->X, train ? m->XT : nullptr,
-                                                 train ? m->inv : nullptr);
+                                                 train ? m->inv : nullptr, m->status);
     BN_LAUNCH_CHECK("k_embed");
     int rc;
     Product z;
@@ -666,10 +673,10 @@ int bn::mlp_loss_grad_dev(bn_mlp* m, const uint8_t* d_orders, const uint32_t* d_
     int rc = mlp_forward(m, d_orders, B, true, s);
     if (rc) return rc;
     const int Mp = m->Mp, H = m->H;
-    k_out_grad<<<Mp, 256, 0, s>>>(m->L, m->Pp, d_pairs, d_alpha, B, Mp, H, m->Z2, m->W3b, m->dZ2, m->dZ2T,
-                                  m->grow, m->lrow);
+    k_out_grad<<<Mp, 256, 0, s>>>(m->L, m->Pp, d_pairs, d_alpha, B, m->P, Mp, H, m->Z2, m->W3b, m->dZ2, m->dZ2T,
+                                  m->grow, m->lrow, m->status);
     BN_LAUNCH_CHECK("k_out_grad");
-    k_out_sums<<<(unsigned)(B + H / 32 + 1), 256, 0, s>>>(d_pairs, m->grow, m->lrow, B, H, m->H2, m->dZ2, m->gW3, m->gb3,
+    k_out_sums<<<(unsigned)(B + H / 32 + 1), 256, 0, s>>>(d_pairs, m->grow, m->lrow, B, m->P, H, m->H2, m->dZ2, m->gW3, m->gb3,
                                                         m->gb2, m->loss);
     BN_LAUNCH_CHECK("k_out_sums");
     Product dH, dX;
@@ -816,6 +823,11 @@ static int check_status(bn_mlp* m, cudaStream_t s, const char* who)
     BN_CUDA(cudaMemcpyAsync(&st, m->status, 4, cudaMemcpyDeviceToHost, s));
     BN_CUDA(cudaStreamSynchronize(s));
     if (st & STATUS_TIMEOUT) return set_error(BN_ETIMEOUT, "%s: a bounded device wait expired", who);
+    if (st & STATUS_BADINPUT) {
+        BN_CUDA(cudaMemsetAsync(m->status, 0, 4, s));       // the next call's inputs are its own
+        BN_CUDA(cudaStreamSynchronize(s));
+        return set_error(BN_EINVAL, "%s: an order names a node or a row a swap pair that does not exist", who);
+    }
     return BN_OK;
 }
 
