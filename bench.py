@@ -240,8 +240,8 @@ ISSUE_PER_SM = 4           # warp schedulers per SM, one warp instruction per cl
 FUSED_INST_PER_CHAIN_STEP = 752.0
 FUSED_TRAFFIC_BYTES = 1.902e6    # ncu dram bytes read + written per 1,000-step launch of k_chain_spec<1>
 BUILD_INST_PER_ENTRY = 86.9      # ncu smsp__inst_executed.sum of the counting and assembling kernels
-                                 # (k_joint_tc, k_joint, k_tc_rows, k_minor_rows, k_assemble) at n=60,
-                                 # m=1000, per table entry
+                                 # (k_joint_tc, k_joint, k_tc_rows, k_assemble) at n=60, m=1000, per
+                                 # table entry
 SCAN_TRAFFIC_BYTES = 117.7e6     # ncu dram bytes read + written per launch of k_scan_sliced<8,0> (a sampler step)
 NODES_TRAFFIC_BYTES = 124.2e6    # ncu dram bytes read + written per launch of k_scan_nodes at one order
 SLICED_TRAFFIC_BYTES = 117.64e6  # ncu dram bytes read + written per launch of k_scan_sliced<1,0> at 32 orders
