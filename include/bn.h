@@ -472,11 +472,12 @@ int bn_chains_set_proposal(bn_chains* c, bn_mlp* m, int mode, double eps_mix, vo
  *   BN_LEARNED_LAUNCH_AUTO   (default) one cooperative persistent kernel runs up to 256
  *                            steps per launch -- per step the layer-2 tiles, the output-layer
  *                            tiles and the chains, handed on by device counters, with the
- *                            weight tiles resident in shared memory and TMEM -- when all its
- *                            CTAs fit on the GPU at once (at most 256 chains at H = 512);
- *                            otherwise as BN_LEARNED_LAUNCH_GRAPH
+ *                            weight tiles resident in shared memory and TMEM -- when that
+ *                            fits on the GPU; otherwise as BN_LEARNED_LAUNCH_GRAPH
  *   BN_LEARNED_LAUNCH_GRAPH  three kernels per step (chains, layer 2, output layer),
  *                            chained by programmatic dependent launch in a CUDA graph
+ * A set whose CTAs do not fit on the GPU at once (more than 256 chains at n = 60, H = 512)
+ * is stepped in groups that do, one after another for all steps of the call.
  * Errors: BN_EINVAL. */
 #define BN_LEARNED_LAUNCH_AUTO  0
 #define BN_LEARNED_LAUNCH_GRAPH 1

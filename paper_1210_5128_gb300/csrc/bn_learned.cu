@@ -1,7 +1,7 @@
 // bn_learned.cu -- the MH sampler with the learned swap proposal, built for latency.
 //
-// One MH step of every chain is three kernels, chained by programmatic dependent launch
-// and captured as a CUDA graph:
+// One MH step of a group of chains (LearnGroup) is three kernels, chained by programmatic
+// dependent launch and captured as a CUDA graph, or three phases of k_learned_persist:
 //   k_learned_chain  one warp per chain: finishes the previous step (reverse proposal
 //                    probability from the network's outputs on the proposed order, the
 //                    exact MH test, state update, best graph, dwell-time edge counts,
@@ -48,6 +48,7 @@ enum { LF_FINISH = 1, LF_START = 2, LF_FLUSH = 4 };
 
 struct LearnArgs {
     int H, P, Pp, NT;
+    int c0;                   // the set's chain that is chain 0 here (LearnGroup)
     float eps;
     float scale;              // 2^-shift: fixed-point layer-1 sums to float
     const int32_t* T;         // [n][n][H] fixed point of W1_p E[v]
@@ -515,7 +516,7 @@ __device__ __forceinline__ void learned_chain_load(const ChainState& S, const Le
         }
     }
     if (flags & LF_START)
-        D.x = philox4x64((uint64_t)(fin ? D.t_dev + 1 : D.t_dev), (uint64_t)c, 0, 0, S.seed, 0);
+        D.x = philox4x64((uint64_t)(fin ? D.t_dev + 1 : D.t_dev), (uint64_t)(L.c0 + c), 0, 0, S.seed, 0);
     __syncwarp();
 }
 
@@ -1146,27 +1147,42 @@ __global__ void k_gather_logits(const float* __restrict__ logits, const uint8_t*
     out[idx] = logits[((size_t)cur_buf[c] * C + c) * Pp + j];
 }
 
+// A set is stepped in groups of whole M tiles whose grids are resident at once, one group
+// after another for all steps of the call (the chains are independent): the persistent
+// launch needs that, and the three kernels of a step are not run on larger grids either:
+// several waves of output tiles (896 at 2,048 chains), overlapped by programmatic launch,
+// ended three times in an illegal address, with every address in range by calculation and
+// the cause not found.  A group is the chains [c0, c0 + C) with its own part of every
+// per-chain array.
+struct LearnGroup {
+    int c0 = 0, C = 0, Mt = 0;
+    LearnArgs L{};
+    LGemmArgs g2{}, g3{};
+    PersistArgs pa{};
+    cudaGraphExec_t exec = nullptr;
+};
+
 struct LearnedPath {
     void* block = nullptr;
     size_t bytes = 0;
     int C = 0, n = 0, H = 0, d = 0, P = 0, Pp = 0, NT = 0, Mt = 0;
     int64_t alive = 0;
     int shift = 0;
-    LearnArgs L{};
-    LGemmArgs g2{}, g3{};
+    LearnArgs L{};                       // of the whole set
     uint8_t *wp2 = nullptr, *wp3 = nullptr, *h2 = nullptr;
     uint32_t* bound = nullptr;
     uint32_t* status = nullptr;
+    int64_t* step0 = nullptr;            // the step the call began at (sets of several groups)
     const bn_table* table = nullptr;
     const uint64_t* amask = nullptr;     // the table's survivors the path was built from
     bool weights_ok = false;
     bool primed = false;
     bool pdl = true;
-    cudaGraphExec_t exec = nullptr;
     uint32_t* gsync = nullptr;           // counters of the persistent launch
-    int persist = -1;                    // persistent launch: -1 not checked, 0 no, 1 yes
+    int persist_slots = 0;               // CTAs of the persistent launch resident at once (0: not possible)
     PersistArgs pa{};
     size_t persist_smem = 0;
+    std::vector<LearnGroup> groups;
 };
 
 }  // namespace bn
@@ -1192,10 +1208,58 @@ void bn::learned_invalidate(LearnedPath* lp, bool weights)
 void bn::learned_free(LearnedPath* lp)
 {
     if (!lp) return;
-    if (lp->exec) cudaGraphExecDestroy(lp->exec);
+    for (LearnGroup& G : lp->groups)
+        if (G.exec) cudaGraphExecDestroy(G.exec);
     obj_free({lp->block});
     delete lp;
 }
+
+// the group's view of the set's state
+static ChainState group_state(const ChainState& A, const LearnGroup& G)
+{
+    ChainState S = A;
+    const size_t c0 = (size_t)G.c0, cn = c0 * A.n;
+    S.C = G.C;
+    S.cur_order += cn;
+    S.cur_rank += cn;
+    S.cur_key += cn;
+    S.cur_score += c0;
+    S.best_order += cn;
+    S.best_rank += cn;
+    S.best_score += c0;
+    S.accepts += c0;
+    S.edge += cn * A.n;
+    S.trace_score += c0 * A.trace_cap;
+    S.trace_accept += c0 * A.trace_cap;
+    S.rec_bits += cn * A.n * A.rec_words;
+    return S;
+}
+
+// its view of the path's buffers (c0 is a multiple of LR_TM); the two buffers of logits and
+// partials lie together per group
+static LearnArgs group_args(const LearnArgs& A, int n, int c0)
+{
+    LearnArgs L = A;
+    const size_t c = (size_t)c0, cn = c * n;
+    L.c0 = c0;
+    L.h1 += c * A.H * 2;
+    L.z1 += c * A.H;
+    L.z1p += c * A.H;
+    L.logits += 2 * c * A.Pp;
+    L.part += 2 * c * A.NT;
+    L.cur_buf += c;
+    L.since += cn;
+    L.prank += cn;
+    L.pkey += cn;
+    L.pab += 2 * c;
+    L.ppair += c;
+    L.plqf += c;
+    L.pu += c;
+    L.pdpart += c;
+    return L;
+}
+
+static int learned_group(LearnedPath* lp);
 
 // device buffers of the path (sizes from the chains, the network and the table)
 static int learned_alloc(bn_chains* ch)
@@ -1235,7 +1299,7 @@ static int learned_alloc(bn_chains* ch)
                  o_lg = take(4 * 2 * Cs * Pp), o_part = take(8 * 2 * Cs * lp->NT), o_cb = take(Cs),
                  o_since = take(8 * Cs * n), o_prank = take(4 * Cs * n), o_pkey = take(8 * Cs * n), o_pab = take(2 * Cs),
                  o_pair = take(4 * Cs), o_lqf = take(4 * Cs), o_pu = take(8 * Cs), o_dp = take(8 * Cs),
-                 o_done = take(4), o_bound = take(4), o_status = take(4), o_gsync = take(sizeof(uint32_t) * 3 * LR_SYNC * (size_t)lp->Mt);
+                 o_done = take(4), o_bound = take(4), o_status = take(4), o_step0 = take(8), o_gsync = take(sizeof(uint32_t) * 3 * LR_SYNC * (size_t)lp->Mt);
     // survivors region [masks | keys | ranks | node offsets], each part 16-byte aligned
     const size_t r_key = (size_t)round_up((int64_t)(8 * alive), 16), r_rk = r_key + (size_t)round_up((int64_t)(8 * alive), 16),
                  r_off = r_rk + (size_t)round_up((int64_t)(4 * alive), 16),
@@ -1287,7 +1351,13 @@ static int learned_alloc(bn_chains* ch)
     lp->h2 = B + o_h2;
     lp->bound = (uint32_t*)(B + o_bound);
     lp->status = (uint32_t*)(B + o_status);
+    lp->step0 = (int64_t*)(B + o_step0);
     lp->gsync = (uint32_t*)(B + o_gsync);
+    const int rc = learned_group(lp);
+    if (rc) {
+        learned_free(lp);
+        return rc;
+    }
     ch->lp = lp;
     return BN_OK;
 }
@@ -1332,51 +1402,46 @@ static int learned_weights(bn_chains* ch, cudaStream_t s)
     BN_LAUNCH_CHECK("k_surv_compact");
     lp->L.b1 = m->b1;
     lp->L.eps = ch->S.eps_mix;
-    LGemmArgs g{};
-    g.K = H;
-    g.C = lp->C;
-    g.P = lp->P;
-    g.Pp = lp->Pp;
-    g.NT = lp->NT;
-    g.cur_buf = lp->L.cur_buf;
-    g.status = lp->status;
-    lp->g2 = g;
-    lp->g2.A = lp->L.h1;
-    lp->g2.B = lp->wp2;
-    lp->g2.bias = m->b2;
-    lp->g2.mode = 0;
-    lp->g2.out_h = lp->h2;
-    lp->g3 = g;
-    lp->g3.A = lp->h2;
-    lp->g3.B = lp->wp3;
-    lp->g3.bias = m->b3;
-    lp->g3.mode = 1;
-    lp->g3.logits = (float*)lp->L.logits;
-    lp->g3.part = (float2*)lp->L.part;
-    static ContextOnce once;
-    const int rc = once_in_context(once, [&]() -> int {
-        BN_CUDA(cudaFuncSetAttribute(k_learned_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)lgemm_smem(LR_MAX_H)));
-        BN_CUDA(cudaFuncSetAttribute(k_learned_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, LR_STAGE_MAX));
-        return BN_OK;
-    });
-    if (rc) return rc;
-    if (lp->exec) {
-        cudaGraphExecDestroy(lp->exec);
-        lp->exec = nullptr;
+    for (LearnGroup& G : lp->groups) {
+        G.L = group_args(lp->L, n, G.c0);
+        LGemmArgs g{};
+        g.K = H;
+        g.C = G.C;
+        g.P = lp->P;
+        g.Pp = lp->Pp;
+        g.NT = lp->NT;
+        g.cur_buf = G.L.cur_buf;
+        g.status = lp->status;
+        G.g2 = g;
+        G.g2.A = G.L.h1;
+        G.g2.B = lp->wp2;
+        G.g2.bias = m->b2;
+        G.g2.mode = 0;
+        G.g2.out_h = lp->h2 + (size_t)G.c0 * H * 2;
+        G.g3 = g;
+        G.g3.A = G.g2.out_h;
+        G.g3.B = lp->wp3;
+        G.g3.bias = m->b3;
+        G.g3.mode = 1;
+        G.g3.logits = (float*)G.L.logits;
+        G.g3.part = (float2*)G.L.part;
+        if (G.exec) {
+            cudaGraphExecDestroy(G.exec);
+            G.exec = nullptr;
+        }
     }
     lp->weights_ok = true;
     lp->primed = false;
     return BN_OK;
 }
 
-static int launch_gemm(LearnedPath* lp, const LGemmArgs& g, int prime, cudaStream_t s)
+static int launch_gemm(LearnedPath* lp, const LearnGroup& G, const LGemmArgs& g, int prime, cudaStream_t s)
 {
     LGemmArgs a = g;
     a.prime = prime;
     const unsigned nx = (unsigned)(g.mode == 0 ? lp->H / LR_TN : lp->NT);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nx, (unsigned)lp->Mt, 1);
+    cfg.gridDim = dim3(nx, (unsigned)G.Mt, 1);
     cfg.blockDim = dim3(128, 1, 1);
     cfg.dynamicSmemBytes = lgemm_smem(lp->H);
     cfg.stream = s;
@@ -1390,11 +1455,11 @@ static int launch_gemm(LearnedPath* lp, const LGemmArgs& g, int prime, cudaStrea
     return BN_OK;
 }
 
-static int launch_chain(bn_chains* ch, int flags, cudaStream_t s)
+static int launch_chain(bn_chains* ch, const LearnGroup& G, int flags, cudaStream_t s)
 {
     LearnedPath* lp = ch->lp;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((lp->C + LR_WARPS - 1) / LR_WARPS), 1, 1);
+    cfg.gridDim = dim3((unsigned)((G.C + LR_WARPS - 1) / LR_WARPS), 1, 1);
     cfg.blockDim = dim3(32 * LR_WARPS, 1, 1);
     cfg.dynamicSmemBytes = lp->L.sreg_bytes;
     cfg.stream = s;
@@ -1403,18 +1468,18 @@ static int launch_chain(bn_chains* ch, int flags, cudaStream_t s)
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = lp->pdl ? 1 : 0;
-    BN_CUDA(cudaLaunchKernelEx(&cfg, k_learned_chain, ch->S, lp->L, flags));
+    BN_CUDA(cudaLaunchKernelEx(&cfg, k_learned_chain, group_state(ch->S, G), G.L, flags));
     BN_LAUNCH_CHECK("k_learned_chain");
     return BN_OK;
 }
 
 // one step's network on the proposals, then finish it and start the next
-static int launch_iter(bn_chains* ch, int flags, cudaStream_t s)
+static int launch_iter(bn_chains* ch, const LearnGroup& G, int flags, cudaStream_t s)
 {
     int rc;
-    if ((rc = launch_gemm(ch->lp, ch->lp->g2, 0, s))) return rc;
-    if ((rc = launch_gemm(ch->lp, ch->lp->g3, 0, s))) return rc;
-    return launch_chain(ch, flags, s);
+    if ((rc = launch_gemm(ch->lp, G, G.g2, 0, s))) return rc;
+    if ((rc = launch_gemm(ch->lp, G, G.g3, 0, s))) return rc;
+    return launch_chain(ch, G, flags, s);
 }
 
 // the current orders' layer-1 sums and network outputs
@@ -1424,8 +1489,8 @@ static int learned_prime(bn_chains* ch, cudaStream_t s)
     k_learned_prime<<<(lp->C + LR_WARPS - 1) / LR_WARPS, 32 * LR_WARPS, 0, s>>>(ch->S, lp->L);
     BN_LAUNCH_CHECK("k_learned_prime");
     int rc;
-    if ((rc = launch_gemm(lp, lp->g2, 1, s))) return rc;
-    if ((rc = launch_gemm(lp, lp->g3, 1, s))) return rc;
+    for (const LearnGroup& G : lp->groups)
+        if ((rc = launch_gemm(lp, G, G.g2, 1, s)) || (rc = launch_gemm(lp, G, G.g3, 1, s))) return rc;
     lp->primed = true;
     return BN_OK;
 }
@@ -1440,23 +1505,23 @@ int bn::learned_setup(bn_chains* ch, cudaStream_t s)
 }
 
 // the G-iteration graph of the steady state (captured once per set-up)
-static int learned_graph(bn_chains* ch, cudaStream_t s)
+static int learned_graph(bn_chains* ch, LearnGroup& G, cudaStream_t s)
 {
     LearnedPath* lp = ch->lp;
-    if (lp->exec) return BN_OK;
+    if (G.exec) return BN_OK;
     for (int attempt = 0; attempt < 2; ++attempt) {
         cudaGraph_t g = nullptr;
         BN_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
         int rc = BN_OK;
         const int64_t l0 = bn_kernel_launches();
-        for (int i = 0; i < LR_GRAPH_ITERS && rc == BN_OK; ++i) rc = launch_iter(ch, LF_FINISH | LF_START, s);
+        for (int i = 0; i < LR_GRAPH_ITERS && rc == BN_OK; ++i) rc = launch_iter(ch, G, LF_FINISH | LF_START, s);
         count_launches(-(bn_kernel_launches() - l0));       // captured, not run
         cudaError_t ce = cudaStreamEndCapture(s, &g);
         if (rc == BN_OK && ce == cudaSuccess) {
-            cudaError_t ie = cudaGraphInstantiate(&lp->exec, g, 0);
+            cudaError_t ie = cudaGraphInstantiate(&G.exec, g, 0);
             cudaGraphDestroy(g);
             if (ie == cudaSuccess) return BN_OK;
-            lp->exec = nullptr;
+            G.exec = nullptr;
         } else if (g) {
             cudaGraphDestroy(g);
         }
@@ -1467,19 +1532,13 @@ static int learned_graph(bn_chains* ch, cudaStream_t s)
     return set_error(BN_ECUDA, "learned proposal: graph capture failed");
 }
 
-// the persistent launch's plan: CTAs per role, shared-memory layout, and whether every
-// CTA can be resident at once (a cooperative launch needs that)
-static int persist_setup(bn_chains* ch)
+// the persistent launch's shared-memory layout and how many of its CTAs can be resident at
+// once (a cooperative launch needs all of them)
+static void persist_plan(LearnedPath* lp)
 {
-    LearnedPath* lp = ch->lp;
-    if (lp->persist >= 0) return BN_OK;
-    lp->persist = 0;
     PersistArgs& P = lp->pa;
     P.nt2 = lp->H / LR_TN;
     P.nt3 = lp->NT;
-    P.n2 = P.nt2 * lp->Mt;
-    P.n3 = P.nt3 * lp->Mt;
-    P.nc = (lp->C + LR_WARPS - 1) / LR_WARPS;
     P.gsync = lp->gsync;
     const size_t sreg = lp->L.sreg_bytes;
     const size_t a_bytes = (size_t)LR_TM * lp->H * 2, b_bytes = (size_t)LR_TN * lp->H * 2;
@@ -1488,7 +1547,7 @@ static int persist_setup(bn_chains* ch)
     int optin = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
         cudaGetLastError();
-        return BN_OK;
+        return;
     }
     const size_t static_smem = sizeof(LWarp) * LR_WARPS + 64 + 1024;   // + alignment slack
     auto layout = [&](bool stage) {
@@ -1501,7 +1560,7 @@ static int persist_setup(bn_chains* ch)
     };
     size_t smem = layout(sreg > 0);
     if (smem + static_smem > (size_t)optin) smem = layout(false);     // survivors from global memory
-    if (smem + static_smem > (size_t)optin) return BN_OK;
+    if (smem + static_smem > (size_t)optin) return;
     // the most a block can have: another chain set's smaller layout must not lower it
     static ContextOnce once;
     const int rc = once_in_context(once, [&]() -> int {
@@ -1512,32 +1571,66 @@ static int persist_setup(bn_chains* ch)
                                      optin - (int)fa.sharedSizeBytes);
         return e == cudaSuccess ? BN_OK : BN_ECUDA;
     });
-    if (rc) {
-        cudaGetLastError();
-        return BN_OK;
-    }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_learned_persist, 32 * LR_WARPS, smem) != cudaSuccess) {
+    if (rc || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_learned_persist, 32 * LR_WARPS, smem) != cudaSuccess) {
         cudaGetLastError();
-        return BN_OK;
+        return;
     }
-    const int grid = std::max(P.n2 + P.n3, P.nc);
-    if ((int64_t)per_sm * sm_count() < grid) return BN_OK;
     lp->persist_smem = smem;
-    lp->persist = 1;
+    lp->persist_slots = per_sm * sm_count();
+}
+
+// The set's groups, as equal as whole tiles allow.  A group's GEMM tiles fit at once: by the
+// persistent launch's room, or, where that is not possible, the GEMM kernel's, at most two
+// CTAs an SM; and so do the chains' blocks, of either launch.
+static int learned_group(LearnedPath* lp)
+{
+    static ContextOnce once;
+    const int rc = once_in_context(once, [&]() -> int {
+        BN_CUDA(cudaFuncSetAttribute(k_learned_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)lgemm_smem(LR_MAX_H)));
+        BN_CUDA(cudaFuncSetAttribute(k_learned_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, LR_STAGE_MAX));
+        return BN_OK;
+    });
+    if (rc) return rc;
+    persist_plan(lp);
+    int og = 0, oc = 0;
+    BN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&og, k_learned_gemm, 128, lgemm_smem(lp->H)));
+    BN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&oc, k_learned_chain, 32 * LR_WARPS, lp->L.sreg_bytes));
+    const int per_tile = lp->H / LR_TN + lp->NT, blocks = LR_TM / LR_WARPS;
+    int slots = lp->persist_slots;
+    if (slots < std::max(per_tile, blocks)) slots = std::min(2, og) * sm_count();
+    const int cslots = std::min(slots, std::min(2, oc) * sm_count());
+    const bool whole = lp->Mt * per_tile <= slots && (lp->C + LR_WARPS - 1) / LR_WARPS <= cslots;
+    const int fit = whole ? lp->Mt : std::max(1, std::min(slots / per_tile, cslots / blocks));
+    const int count = (lp->Mt + fit - 1) / fit;
+    lp->groups.resize((size_t)count);
+    for (int q = 0, t0 = 0; q < count; ++q) {
+        LearnGroup& G = lp->groups[(size_t)q];
+        G.Mt = lp->Mt / count + (q < lp->Mt % count ? 1 : 0);
+        G.c0 = t0 * LR_TM;
+        G.C = std::min(G.Mt * LR_TM, lp->C - G.c0);
+        t0 += G.Mt;
+        G.pa = lp->pa;
+        G.pa.n2 = G.pa.nt2 * G.Mt;
+        G.pa.n3 = G.pa.nt3 * G.Mt;
+        G.pa.nc = (G.C + LR_WARPS - 1) / LR_WARPS;
+    }
     return BN_OK;
 }
 
+static unsigned persist_grid(const PersistArgs& P) { return (unsigned)std::max(P.n2 + P.n3, P.nc); }
+
 // `iters` learned steps (each: layer 2, output layer, finish + start) in one cooperative
 // launch
-static int launch_persist(bn_chains* ch, int iters, cudaStream_t s)
+static int launch_persist(bn_chains* ch, const LearnGroup& G, int iters, cudaStream_t s)
 {
     LearnedPath* lp = ch->lp;
-    PersistArgs P = lp->pa;
+    PersistArgs P = G.pa;
     P.iters = iters;
-    BN_CUDA(cudaMemsetAsync(lp->gsync, 0, sizeof(uint32_t) * 3 * LR_SYNC * (size_t)lp->Mt, s));
+    BN_CUDA(cudaMemsetAsync(lp->gsync, 0, sizeof(uint32_t) * 3 * LR_SYNC * (size_t)G.Mt, s));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::max(P.n2 + P.n3, P.nc), 1, 1);
+    cfg.gridDim = dim3(persist_grid(P), 1, 1);
     cfg.blockDim = dim3(32 * LR_WARPS, 1, 1);
     cfg.dynamicSmemBytes = lp->persist_smem;
     cfg.stream = s;
@@ -1546,42 +1639,55 @@ static int launch_persist(bn_chains* ch, int iters, cudaStream_t s)
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    BN_CUDA(cudaLaunchKernelEx(&cfg, k_learned_persist, ch->S, lp->L, lp->g2, lp->g3, P));
+    BN_CUDA(cudaLaunchKernelEx(&cfg, k_learned_persist, group_state(ch->S, G), G.L, G.g2, G.g3, P));
     BN_LAUNCH_CHECK("k_learned_persist");
     return BN_OK;
 }
 
 static constexpr int LR_PERSIST_ITERS = 256;   // learned steps per persistent launch
 
+// a group's steps of one call
+static int group_step(bn_chains* ch, LearnGroup& G, int64_t steps, cudaStream_t s)
+{
+    LearnedPath* lp = ch->lp;
+    int rc;
+    if ((rc = launch_chain(ch, G, LF_START, s))) return rc;
+    int64_t mid = steps - 1;
+    if (ch->learned_launch == BN_LEARNED_LAUNCH_AUTO && persist_grid(G.pa) <= (unsigned)lp->persist_slots) {
+        for (; mid > 0;) {
+            const int k = (int)std::min<int64_t>(mid, LR_PERSIST_ITERS);
+            if ((rc = launch_persist(ch, G, k, s))) return rc;
+            mid -= k;
+        }
+    }
+    if (mid >= LR_GRAPH_ITERS) {
+        if ((rc = learned_graph(ch, G, s))) return rc;
+        for (; mid >= LR_GRAPH_ITERS; mid -= LR_GRAPH_ITERS) {
+            BN_CUDA(cudaGraphLaunch(G.exec, s));
+            count_launches(3 * LR_GRAPH_ITERS);
+        }
+    }
+    for (; mid > 0; --mid)
+        if ((rc = launch_iter(ch, G, LF_FINISH | LF_START, s))) return rc;
+    if ((rc = launch_gemm(lp, G, G.g2, 0, s)) || (rc = launch_gemm(lp, G, G.g3, 0, s))) return rc;
+    return launch_chain(ch, G, LF_FINISH | LF_FLUSH, s);
+}
+
 int bn::learned_step(bn_chains* ch, int64_t steps, cudaStream_t s)
 {
     int rc = learned_setup(ch, s);
     if (rc) return rc;
     if (steps <= 0) return BN_OK;
-    if ((rc = launch_chain(ch, LF_START, s))) return rc;
-    int64_t mid = steps - 1;
-    if (ch->learned_launch == BN_LEARNED_LAUNCH_AUTO && mid > 0 && (rc = persist_setup(ch))) return rc;
-    if (ch->learned_launch == BN_LEARNED_LAUNCH_AUTO && ch->lp->persist == 1) {
-        for (; mid > 0;) {
-            const int k = (int)std::min<int64_t>(mid, LR_PERSIST_ITERS);
-            if ((rc = launch_persist(ch, k, s))) return rc;
-            mid -= k;
-        }
+    LearnedPath* lp = ch->lp;
+    // every group counts the same steps on the set's counter
+    const bool several = lp->groups.size() > 1;
+    if (several) BN_CUDA(cudaMemcpyAsync(lp->step0, ch->S.step, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    for (LearnGroup& G : lp->groups) {
+        if (G.c0 > 0) BN_CUDA(cudaMemcpyAsync(ch->S.step, lp->step0, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+        if ((rc = group_step(ch, G, steps, s))) return rc;
     }
-    if (mid >= LR_GRAPH_ITERS) {
-        if ((rc = learned_graph(ch, s))) return rc;
-        for (; mid >= LR_GRAPH_ITERS; mid -= LR_GRAPH_ITERS) {
-            BN_CUDA(cudaGraphLaunch(ch->lp->exec, s));
-            count_launches(3 * LR_GRAPH_ITERS);
-        }
-    }
-    for (; mid > 0; --mid)
-        if ((rc = launch_iter(ch, LF_FINISH | LF_START, s))) return rc;
-    if ((rc = launch_gemm(ch->lp, ch->lp->g2, 0, s)) || (rc = launch_gemm(ch->lp, ch->lp->g3, 0, s)) ||
-        (rc = launch_chain(ch, LF_FINISH | LF_FLUSH, s)))
-        return rc;
     uint32_t st = 0;
-    BN_CUDA(cudaMemcpyAsync(&st, ch->lp->status, 4, cudaMemcpyDeviceToHost, s));
+    BN_CUDA(cudaMemcpyAsync(&st, lp->status, 4, cudaMemcpyDeviceToHost, s));
     BN_CUDA(cudaStreamSynchronize(s));
     if (st & STATUS_TIMEOUT) return set_error(BN_ETIMEOUT, "learned proposal: a bounded device wait expired");
     return BN_OK;
@@ -1598,8 +1704,11 @@ int bn::learned_read_logits(const bn_chains* ch, float* out, int mem, cudaStream
         BN_CUDA(dev_alloc((void**)&tmp, 4 * (size_t)cnt, s));
         d = tmp;
     }
-    k_gather_logits<<<blocks_of(cnt), 256, 0, s>>>(lp->L.logits, lp->L.cur_buf, lp->C, lp->P, lp->Pp, d);
-    BN_LAUNCH_CHECK("k_gather_logits");
+    for (const LearnGroup& G : lp->groups) {
+        k_gather_logits<<<blocks_of((int64_t)G.C * lp->P), 256, 0, s>>>(G.L.logits, G.L.cur_buf, G.C, lp->P, lp->Pp,
+                                                                         d + (int64_t)G.c0 * lp->P);
+        BN_LAUNCH_CHECK("k_gather_logits");
+    }
     if (mem == BN_MEM_HOST) {
         BN_CUDA(cudaMemcpyAsync(out, tmp, 4 * (size_t)cnt, cudaMemcpyDeviceToHost, s));
         dev_free(tmp, s);
